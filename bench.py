@@ -55,7 +55,9 @@ def profiled_traffic(name: str):
 def launches_per_call(name: str, w) -> int:
     """Kernels one call enqueues.  Sampling: streaming, merge, histogram pass, collect pass, row finish, cluster kernel.
     Verification adds the residual pass, the residual draw and the combine kernel.  (sonic_topk: streaming, merge,
-    cluster kernel.)"""
+    cluster kernel.)  A call whose rows fit the chip at once is one launch of the row kernel."""
+    if name == "c1":
+        return 1
     if name == "c4":
         return 9 if w.K > 0 else 7
     if name.startswith("c5"):

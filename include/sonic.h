@@ -59,7 +59,7 @@ extern "C" {
  * processed logits of rows with top-k off as ordered keys) plus 58 KB of histogram and lists. */
 size_t sonic_workspace_bytes(int max_rows, int max_vocab, int max_topk);
 
-/* Zeroes the workspace header (the first 512 bytes: work counters and the sticky error word) once after allocation
+/* Zeroes the workspace header (the first 17 KB: work counters, the sticky error word, a ticket per request) once after allocation
  * (a memset enqueued on `stream`, a cudaStream_t passed as void*).  The kernels put the counters back to zero
  * at the end of every call and initialise every other word they read themselves, so replays need no
  * re-initialisation and one workspace serves calls of different shapes.  Two calls that use the same workspace
@@ -70,7 +70,8 @@ size_t sonic_workspace_bytes(int max_rows, int max_vocab, int max_topk);
  * reports SONIC_FLAG_TIMEOUT with token -1 until the workspace is initialised again with this function.
  *
  * Streams: a call's kernels are ordered on the caller's `stream` (everything enqueued before the call precedes
- * them, everything after follows them).  Per host thread and device the library keeps ONE internal non-blocking stream
+ * them, everything after follows them).  A call of few rows is one kernel on that stream; the rest of this paragraph is
+ * about larger calls.  Per host thread and device the library keeps ONE internal non-blocking stream
  * and two events, created by this function or by the thread's first sampling call outside a stream capture:
  * sonic_sample / sonic_verify fork it from `stream` behind their first kernel and join it back before their last
  * one, so that rows with and without top-k are finished side by side.  Under stream capture the fork is captured
@@ -169,7 +170,7 @@ int sonic_topk(const void *logits, int dtype, int B, int V, int64_t row_stride, 
  *
  * Same inputs, outputs and results as sonic_topk, for at most SONIC_STATIC_MAX_ROWS rows
  * per call; larger B is rejected with SONIC_ESHAPE.  The scratch memory is a fixed array
- * of about 4.2 MB inside the library image (SONIC_STATIC_MAX_ROWS rows of candidate
+ * of about 4.3 MB inside the library image (SONIC_STATIC_MAX_ROWS rows of candidate
  * slots and control words); every GPU that loads the library holds it until the process
  * exits.  The function calls no cudaMalloc, cudaFree or other allocating routine, and
  * all of its kernels go to `stream`.

@@ -1,6 +1,8 @@
 // C ABI of the sonic library (see include/sonic.h): argument validation and
 // kernel launches.  Nothing here allocates device memory or synchronises.
+#include <algorithm>
 #include <cstdio>
+#include <cmath>
 #include <cstring>
 #include <mutex>
 
@@ -9,23 +11,22 @@
 #include "sonic_dense.cuh"
 #include "sonic_stream.cuh"
 #include "sonic_exact.cuh"
+#include "sonic_row.cuh"
 
 namespace sonic {
 
 // Verification epilogue: the K+1 positions of a request were resolved
 // independently (accept flag, correction token); this scans them in order.
-__global__ void sonic_verify_combine_kernel(const KParams P, int B) {
-    KERNEL_T0(5);
-    KERNEL_T1(5);
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
+__device__ __forceinline__ void verify_combine(const KParams &P, int b) {
     const int K = P.K;
     int *toks = P.out_tokens + (size_t)b * (K + 1);
     uint32_t flags = 0;
     int acc = 0;
     bool decided = false;
     for (int l = 0; l <= K; ++l) {
-        const PosResult r = P.pr[(size_t)b * (K + 1) + l];
+        const uint4 raw = __ldcg(reinterpret_cast<const uint4 *>(&P.pr[(size_t)b * (K + 1) + l]));
+        PosResult r;
+        r.token = (int)raw.x; r.flags = raw.y; r.p = __uint_as_float(raw.z);
         toks[l] = -1;
         if (l < K && P.out_pdraft) P.out_pdraft[(size_t)b * K + l] = (r.flags & (F_BADPARAM | F_NO_TOKEN)) ? 0.0f : r.p;
         if (r.flags & F_BADPARAM) flags |= F_BADPARAM;
@@ -45,7 +46,15 @@ __global__ void sonic_verify_combine_kernel(const KParams P, int B) {
     P.out_flags[b] = flags;
 }
 
+__global__ void sonic_verify_combine_kernel(const KParams P, int B) {
+    KERNEL_T0(5);
+    KERNEL_T1(5);
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b < B) verify_combine(P, b);
+}
+
 constexpr size_t WS_HEADER = WS_HEADER_WORDS * 4;
+constexpr size_t WS_CLEAR = WS_TICKETS * 4;       // the part of it that the streaming chain uses
 constexpr int MERGE_SMEM = MERGE_CAP * 8;
 constexpr int STREAM_SMEM_F32 = VecTraits<0>::NSTAGE * CTA_TILE * 4 + (int)sizeof(StreamShared<0>);
 constexpr int STREAM_SMEM_BF16 = VecTraits<1>::NSTAGE * CTA_TILE * 2 + CTA_TILE * 4 + (int)sizeof(StreamShared<1>);
@@ -102,6 +111,42 @@ static Layout layout_for(long long rows, int V, bool dense, size_t cap = CAND_CA
     return L;
 }
 
+// pick_groups' table for one vocabulary size (the model is described beside GroupTable); the last sizes are remembered.
+static void make_group_table(GroupTable &t, int V) {
+    memset(&t, 0, sizeof(t));
+    const float lg_nw = log2f((float)((V + WARP_TILE - 1) / WARP_TILE));
+    const float lg_nt = log2f((float)((V + CTA_TILE - 1) / CTA_TILE));
+    for (int step = 0; step < GK_STEPS; ++step) {
+        const bool tile = (step & 1) != 0;
+        if (tile && step > 7) continue;
+        const int G = tile ? (1 << (step >> 1)) : (2 << (step >> 1));
+        const float m = (float)(tile ? G * (CTA_TILE / WARP_TILE) : G);              // groups per block
+        const float lg = tile ? lg_nt : lg_nw;                                      // log2 of the blocks per row
+        const float r = exp2f(-lg / m);                                             // Nb^(-1/m)
+        const float est = (float)V * ((float)G / (float)WARP_TILE) * -logf(1.0f - r);
+        // the proven count scatters around the estimate (about 15 % at 16 groups, far more at 2)
+        auto serves = [&](int k) {
+            const float need = (float)k * (m >= 16.0f ? 1.7f : 1.0f + 6.0f / sqrtf(m)) + 30.0f;
+            const float xk = (float)k * ((float)WARP_TILE / (float)G) / (float)V;
+            const float lg_fail = lg + m * log2f(1.0f - expf(-xk));                 // log2 of the failure probability
+            return est >= need && lg_fail <= -9.97f;                                // log2(1e-3)
+        };
+        int lo = 0, hi = MAX_TOPK + 1;                                              // serves(lo) (or lo = 0), not serves(hi)
+        while (hi - lo > 1) { const int mid = (lo + hi) / 2; if (serves(mid)) lo = mid; else hi = mid; }
+        t.k[step] = lo;
+        if (est > 0.5f * (float)CAND_CAP) t.over |= 1u << step;
+    }
+}
+static const GroupTable &group_table(int V) {
+    static thread_local struct { int V; GroupTable t; } memo[4];
+    static thread_local unsigned int next;
+    for (auto &m : memo) if (m.V == V) return m.t;
+    auto &m = memo[next++ & 3];
+    make_group_table(m.t, V);
+    m.V = V;
+    return m.t;
+}
+
 static int g_sm_count[64];
 
 static int configure_once(int *sm_count, int *device) {
@@ -124,6 +169,10 @@ static int configure_once(int *sm_count, int *device) {
         set((const void *)sonic_stream_kernel<0>, STREAM_SMEM_F32);
         set((const void *)sonic_stream_kernel<1>, STREAM_SMEM_BF16);
         if (r == cudaSuccess) r = cudaDeviceGetAttribute(&g_sm_count[dev], cudaDevAttrMultiProcessorCount, dev);
+        set((const void *)sonic_row_kernel<0>, ROW_DYN_SMEM);
+        set((const void *)sonic_row_kernel<1>, ROW_DYN_SMEM);
+        for (const void *f : {(const void *)sonic_row_kernel<0>, (const void *)sonic_row_kernel<1>})
+            if (r == cudaSuccess) r = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);      // (clusters of up to 16)
         set((const void *)sonic_exact_kernel<0>, EXACT_SMEM);
         set((const void *)sonic_exact_kernel<1>, EXACT_SMEM);
         int n = 0;
@@ -189,6 +238,46 @@ static SideStream *side_stream_for(int dev, cudaStream_t st) {
     return &S;
 }
 
+// Whether a call goes to the row kernel as a whole: when all of its rows' clusters are resident at once (two CTAs per SM).
+// Measured (us per call, streaming chain against row kernel): one bf16 row of 131072 with top-k 25.7 -> 13.6; 3 x 3
+// verification rows of 32003 47 -> 27; 37 fp32 rows of 50021 of every kind 48.8 -> 40.7; 32 bf16 rows of 100003 without
+// top-k 73.8 -> 63.7.  With 64 rows of 131072 (1.7 times what is resident) the chain is ahead again, 58 against 64.5: its
+// persistent CTAs keep loading while the rows' selections wait for one another.  sonic_topk beyond ROW_KMAX: the chain.
+static bool row_route(const KParams &P, int sm_count) {
+#if defined(SONIC_TRACE) || defined(SONIC_TEST_WITHHOLD)
+    return false;                                 // (these variants exist to look into the streaming chain)
+#else
+    if (P.op == OP_TOPK && P.ktop > ROW_KMAX) return false;
+    const int c = std::max(ROW_CMIN, (P.V + ROW_SLICE_MAX - 1) / ROW_SLICE_MAX);
+    return (long long)P.rows * c <= 2ll * sm_count;
+#endif
+}
+
+// CTAs of a row's cluster: as many as are resident for this number of rows, so that every CTA has few elements (a step
+// costs 64 cycles per instruction and 8192 elements), within what a slice can be.
+static cudaError_t launch_rows(const KParams &P, cudaStream_t st, int sm_count) {
+    const int cmin = std::max(ROW_CMIN, (P.V + ROW_SLICE_MAX - 1) / ROW_SLICE_MAX);
+    const int cmax = std::min(ROW_CMAX, std::max(cmin, (P.V + ROW_UNIT - 1) / ROW_UNIT));
+    const int fit = (int)(2ll * sm_count / P.rows);
+    int C = 1;
+    while (C * 2 <= std::min(fit, cmax)) C *= 2;
+    C = std::max(C, cmin);
+    const int per = (P.V + C - 1) / C, slice = (per + ROW_UNIT - 1) / ROW_UNIT * ROW_UNIT;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = C; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.stream = st;
+    cfg.gridDim = dim3((unsigned)P.rows * C);
+    cfg.blockDim = dim3(ROW_THREADS);
+    cfg.dynamicSmemBytes = ROW_DYN_SMEM;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return P.dtype == SONIC_DTYPE_F32 ? cudaLaunchKernelEx(&cfg, sonic_row_kernel<0>, P, slice)
+                                      : cudaLaunchKernelEx(&cfg, sonic_row_kernel<1>, P, slice);
+}
+
 // One call = a chain of kernels on the caller's stream.  Up to the residual pass each is a programmatic dependent
 // of the one before (it may begin launching while its predecessor runs; the paper overlaps its two stages the
 // same way, Section 3.5):
@@ -197,7 +286,8 @@ static SideStream *side_stream_for(int dev, cudaStream_t st) {
 //   -> cluster kernel (an ordinary launch after all of it: rows no other path finished; usually none) -> [verification scan]
 // The second line runs on the thread's internal stream beside the merges when that stream can be used, else behind
 // them on the caller's stream.
-static int launch_all(KParams &P, void *ws, size_t ws_bytes, cudaStream_t st, int B_requests) {
+// clear: the header may hold anything (sonic_topk_static's array keeps what the previous call left).
+static int launch_all(KParams &P, void *ws, size_t ws_bytes, cudaStream_t st, int B_requests, bool clear = false) {
     if (!ws) return fail(SONIC_EINVAL, "workspace is NULL");
     if (((uintptr_t)ws & 255) != 0) return fail(SONIC_EINVAL, "workspace must be 256-byte aligned");
     const bool dense = (P.op != OP_TOPK);
@@ -214,6 +304,8 @@ static int launch_all(KParams &P, void *ws, size_t ws_bytes, cudaStream_t st, in
     P.cand = reinterpret_cast<unsigned long long *>(base + L.cand);
     P.cand_stride = L.cand_stride;
     P.ytiles = L.ytiles;
+    P.tickets = P.error + WS_TICKETS;
+    P.groups = group_table(P.V);
     if (dense) {
         P.drow = reinterpret_cast<DenseRow *>(base + L.drow);
         P.dtile = reinterpret_cast<DenseTile *>(base + L.dtile);
@@ -224,6 +316,17 @@ static int launch_all(KParams &P, void *ws, size_t ws_bytes, cudaStream_t st, in
         P.ykeys = reinterpret_cast<unsigned int *>(base + L.ykeys);
     }
 
+    if (row_route(P, sm_count)) {
+        P.fresh = clear ? 1 : 0;
+        cudaError_t e = launch_rows(P, st, sm_count);
+        if (e != cudaSuccess) return fail_cuda(e, "row kernel launch");
+        g_err[0] = 0;
+        return SONIC_OK;
+    }
+    if (clear) {
+        cudaError_t e = cudaMemsetAsync(ws, 0, WS_CLEAR, st);
+        if (e != cudaSuccess) return fail_cuda(e, "cudaMemsetAsync");
+    }
     const int tiles = (P.V + CTA_TILE - 1) / CTA_TILE;
     const long long nitems_ll = (long long)tiles * P.rows;
     if (nitems_ll > 0x7FFFFFFF) return fail(SONIC_ESHAPE, "rows x tiles too large");
@@ -474,15 +577,12 @@ int sonic_topk_static(const void *logits, int dtype, int B, int V, int64_t row_s
     void *ws = nullptr;
     rc = static_workspace_address(&ws);
     if (rc != SONIC_OK) return rc;
-    // the array keeps whatever the previous call left: the header's control words must start at zero
-    cudaError_t e = cudaMemsetAsync(ws, 0, WS_HEADER, (cudaStream_t)stream);
-    if (e != cudaSuccess) return fail_cuda(e, "cudaMemsetAsync");
     KParams P;
     memset(&P, 0, sizeof(P));
     P.op = OP_TOPK;
     P.rows = B; P.V = V; P.dtype = dtype; P.logits = logits; P.row_stride = row_stride; P.ktop = k;
     P.out_vals = out_vals; P.out_idx = out_idx;
-    return launch_all(P, ws, STATIC_WS_BYTES, (cudaStream_t)stream, B);
+    return launch_all(P, ws, STATIC_WS_BYTES, (cudaStream_t)stream, B, true);
 }
 
 const char *sonic_last_error(void) { return g_err; }

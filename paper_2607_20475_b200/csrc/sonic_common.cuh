@@ -60,7 +60,9 @@ constexpr int WS_NRESID = 5;                   // verification rows of the curre
 constexpr int WS_EXACT_LEFT = 6;               // clusters of the cluster kernel that have run out of rows
 constexpr int WS_NEXACT = 7;                   // rows of the current call that belong to the cluster kernel by class
 constexpr int WS_TEST_WITHHOLD = 100;          // test-only builds (SONIC_TEST_WITHHOLD): 1 + the work item whose tile copy is withheld
-constexpr int WS_HEADER_WORDS = 128;
+constexpr int WS_TICKETS = 128;                // [MAX_REQUESTS] verification: positions of a request that are finished (row kernel; zero between calls)
+constexpr int MAX_REQUESTS = 4096;
+constexpr int WS_HEADER_WORDS = WS_TICKETS + MAX_REQUESTS;
 constexpr uint32_t ST_FAILED = 0x1;           // streaming / histogram path could not finish the row
 constexpr unsigned int ERR_TIMEOUT = 0x1;     // workspace header: a bounded mbarrier wait expired
 constexpr uint32_t TILE_BADID = 0x1;          // TileRec.flags: a list id of the row was out of range
@@ -116,8 +118,36 @@ struct __align__(16) PosResult {              // per logit row, verification onl
     int support;
 };
 
+// Which group maxima bound a tile's cutoff.  A warp tile (1024 elements) is cut into G groups (a power of
+// two, 1..32, or 64 with half-lane groups) and the cutoff of a block is the smallest of its group maxima, so
+// at least one element per group lies at or above it.  Two kinds of block:
+//   warp mode: block = warp tile (G groups); the tile cutoff is the LARGEST of its eight warp cutoffs;
+//   tile mode: block = the whole 8192-element tile (8 G groups); the tile cutoff is the SMALLEST warp cutoff.
+// The row-wide cutoff T is the largest tile cutoff either way.  For position-independent data a block of m
+// groups has a cutoff above t with probability (1 - exp(-x))^m, x = (elements above t per group), so with
+// Nb blocks in the row T sits where 1 - exp(-x) = Nb^(-1/m), and the proven prefix holds about
+//     P = V * (G / 1024) * -ln(1 - Nb^(-1/m))
+// elements.  A minimum over more groups concentrates better: at V = 2^18 tile mode with G = 1 proves
+// 245 elements on average (94 at worst in 400 simulated rows) where warp mode with G = 4 proves 265 (63 at
+// worst) and G = 8 proves 1330.  The candidates are tried in the order of their P (warp 2, tile 1, warp 4,
+// tile 2, warp 8, tile 4, warp 16, tile 8, warp 32, warp 64) and the first one is taken whose P clears k
+// with a margin that covers the spread of T and whose proof fails rarely enough: the proof fails when
+// some block has an element of the row's top k in every group; with x_k = k * (1024 / G) / V elements
+// of the top k per group that happens with probability about Nb * (1 - exp(-x_k))^m per row, which must
+// stay below 1e-3 (warp mode with four groups would send one row in three hundred to the exact kernel at
+// k = 64, V = 2^18, and such a row costs more than the whole call does without it).  Tile mode stops at
+// G = 8: a minimum over more groups now and then falls so low that the tile overflows its candidate slot.
+// The conditions are monotone in k, so for one V each step has a largest k that it serves: the host works those out once
+// per vocabulary size (GroupTable) and the kernels compare.
+constexpr int PICK_TILE_MODE = 0x100;
+constexpr int GK_STEPS = 11;
+struct GroupTable {
+    int k[GK_STEPS];                          // largest k the step serves (0: none)
+    unsigned int over;                        // bit: the step's estimate is beyond what the candidate slots hold
+};
 struct KParams {
     int op, rows, V, K, ktop, dtype;
+    int fresh;                                // the header's error word says nothing about this call (sonic_topk_static)
     const void *logits;
     long long row_stride;
     const uint32_t *mode;
@@ -160,6 +190,8 @@ struct KParams {
     unsigned long long *members;              // [rows][MEMBER_CAP] elements of the crossing bin (key << 32 | ~index)
     unsigned int *ykeys;                      // [rows][ytiles * CTA_TILE] ordered keys of the processed logits
     int ytiles;
+    GroupTable groups;                        // pick_groups' table for V
+    unsigned int *tickets;                    // [MAX_REQUESTS] in the header
 };
 
 // Per-row configuration derived from the request's mode bits and parameters.
@@ -194,50 +226,14 @@ __device__ __forceinline__ float div_tau(float z, float tau) {
     return special ? z : q;
 }
 
-// Which group maxima bound a tile's cutoff.  A warp tile (1024 elements) is cut into G groups (a power of
-// two, 1..32, or 64 with half-lane groups) and the cutoff of a block is the smallest of its group maxima, so
-// at least one element per group lies at or above it.  Two kinds of block:
-//   warp mode: block = warp tile (G groups); the tile cutoff is the LARGEST of its eight warp cutoffs;
-//   tile mode: block = the whole 8192-element tile (8 G groups); the tile cutoff is the SMALLEST warp cutoff.
-// The row-wide cutoff T is the largest tile cutoff either way.  For position-independent data a block of m
-// groups has a cutoff above t with probability (1 - exp(-x))^m, x = (elements above t per group), so with
-// Nb blocks in the row T sits where 1 - exp(-x) = Nb^(-1/m), and the proven prefix holds about
-//     P = V * (G / 1024) * -ln(1 - Nb^(-1/m))
-// elements.  A minimum over more groups concentrates better: at V = 2^18 tile mode with G = 1 proves
-// 245 elements on average (94 at worst in 400 simulated rows) where warp mode with G = 4 proves 265 (63 at
-// worst) and G = 8 proves 1330.  The candidates are tried in the order of their P (warp 2, tile 1, warp 4,
-// tile 2, warp 8, tile 4, warp 16, tile 8, warp 32, warp 64) and the first one is taken whose P clears k
-// with a margin that covers the spread of T and whose proof fails rarely enough: the proof fails when
-// some block has an element of the row's top k in every group; with x_k = k * (1024 / G) / V elements
-// of the top k per group that happens with probability about Nb * (1 - exp(-x_k))^m per row, which must
-// stay below 1e-3 (warp mode with four groups would send one row in three hundred to the exact kernel at
-// k = 64, V = 2^18, and such a row costs more than the whole call does without it).  Tile mode stops at
-// G = 8: a minimum over more groups now and then falls so low that the tile overflows its candidate slot.
-// Returns G, plus PICK_TILE_MODE in tile mode; 0 means "keep every finite element" (vocabularies the
-// merge can sort whole); -1 hands the row to the exact kernel.
-#ifndef SONIC_LG_FAIL_MAX
-#define SONIC_LG_FAIL_MAX -9.97f          // log2(1e-3)
-#endif
-constexpr int PICK_TILE_MODE = 0x100;
-__device__ __forceinline__ int pick_groups(int k, int V) {
+// Returns G, plus PICK_TILE_MODE in tile mode; 0 means "keep every finite element" (vocabularies the merge can sort
+// whole); -1 hands the row to the exact kernel.
+__device__ __forceinline__ int pick_groups(const GroupTable &t, int k, int V) {
     if (V <= MERGE_CAP) return 0;
-    const float lg_nw = __log2f((float)((V + WARP_TILE - 1) / WARP_TILE));
-    const float lg_nt = __log2f((float)((V + CTA_TILE - 1) / CTA_TILE));
-    for (int step = 0; step < 11; ++step) {
+#pragma unroll
+    for (int step = 0; step < GK_STEPS; ++step) {
         const bool tile = (step & 1) != 0;
-        if (tile && step > 7) continue;
-        const int G = tile ? (1 << (step >> 1)) : (2 << (step >> 1));
-        const float m = (float)(tile ? G * (CTA_TILE / WARP_TILE) : G);              // groups per block
-        const float lg = tile ? lg_nt : lg_nw;                                      // log2 of the blocks per row
-        const float r = exp2f(-lg / m);                                             // Nb^(-1/m)
-        const float est = (float)V * ((float)G / (float)WARP_TILE) * -__logf(1.0f - r);
-        // the proven count scatters around the estimate (about 15 % at 16 groups, far more at 2)
-        const float need = (float)k * (m >= 16.0f ? 1.7f : 1.0f + 6.0f * rsqrtf(m)) + 30.0f;
-        // above MERGE_CAP the merge first narrows the candidates with a key floor; the tiles' slots bound the rest
-        const float xk = (float)k * ((float)WARP_TILE / (float)G) / (float)V;
-        const float lg_fail = lg + m * __log2f(1.0f - __expf(-xk));                 // log2 of the failure probability
-        if (est >= need && lg_fail <= SONIC_LG_FAIL_MAX)
-            return (est <= 0.5f * (float)CAND_CAP) ? (G | (tile ? PICK_TILE_MODE : 0)) : -1;
+        if (k <= t.k[step]) return ((t.over >> step) & 1u) ? -1 : ((tile ? (1 << (step >> 1)) : (2 << (step >> 1))) | (tile ? PICK_TILE_MODE : 0));
     }
     return -1;
 }
@@ -331,7 +327,7 @@ __device__ __forceinline__ RowCfg resolve_cfg(const KParams &P, int row, const C
             int G;
             if (memo_k && *memo_k == c.k) G = *memo_G;
             else {
-                G = pick_groups(c.k, P.V);
+                G = pick_groups(P.groups, c.k, P.V);
                 if (memo_k) { *memo_k = c.k; *memo_G = G; }
             }
             if (G >= 0) { c.cls = CLS_TOPK; c.G = G & (PICK_TILE_MODE - 1); c.tile_min = (G & PICK_TILE_MODE) != 0; }

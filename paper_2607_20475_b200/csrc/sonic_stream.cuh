@@ -114,6 +114,52 @@ __device__ void merge_epilogue(const KParams &P, const RowCfg &c, int row, int n
 template <int THREADS, typename SH>
 __device__ void merge_epilogue_small(const KParams &P, const RowCfg &c, int row, int n, unsigned long long *buf, SH &sh, int tid, uint2 cells);
 
+// Counting bins of the candidates of a large-k row: MERGE_GBINS bins of 2^MERGE_GSHIFT keys above the proven threshold
+// (one binade of fp32 keys; whatever lies higher shares the top bin), kept in the scratch words of MergeShared.
+constexpr int MERGE_GBINS = 2 * MERGE_THREADS, MERGE_GSHIFT = 13;
+
+// The bin in which the count from the top reaches `need`, the count above it and the count with it (bin < 0: the
+// bins hold fewer than `need`); thread t owns bins GBINS-1-2t and GBINS-2-2t.  Two barriers.
+template <int THREADS>
+__device__ __forceinline__ void merge_bins_find(MergeShared<THREADS> &sh, int tid, int need, int &bin, int &above, int &with) {
+    constexpr int GBINS = MERGE_GBINS, BPT = GBINS / THREADS;
+    static_assert(GBINS * 4 <= THREADS * 8, "the counting bins live in the scratch words");
+    const int *ghist = reinterpret_cast<const int *>(sh.scratch);
+    const int lane_ = tid & 31, warp_ = tid >> 5;
+    int v[BPT], sum = 0;
+#pragma unroll
+    for (int j = 0; j < BPT; ++j) { v[j] = ghist[GBINS - 1 - (tid * BPT + j)]; sum += v[j]; }
+    int incl = sum;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int o = __shfl_up_sync(0xFFFFFFFFu, incl, off);
+        if (lane_ >= off) incl += o;
+    }
+    if (lane_ == 31) sh.wsum[warp_] = incl;
+    if (tid == 0) sh.bracket[0] = -1;
+    __syncthreads();
+    int pre = incl - sum;
+    for (int w = 0; w < warp_; ++w) pre += sh.wsum[w];
+    if (pre < need && pre + sum >= need) {
+        int run = pre;
+#pragma unroll
+        for (int j = 0; j < BPT; ++j) {
+            if (run < need && run + v[j] >= need) { sh.bracket[0] = GBINS - 1 - (tid * BPT + j); sh.bracket[1] = run; sh.bracket[2] = run + v[j]; }
+            run += v[j];
+        }
+    }
+    __syncthreads();
+    bin = sh.bracket[0]; above = sh.bracket[1]; with = sh.bracket[2];
+    __syncthreads();
+}
+
+// The rest of a top-k row once its candidates are in buf[0, Pn) (at most MERGE_CAP, distinct, in no order): the n best of
+// them, sorted, then the outputs of sonic_topk or the truncation epilogue and the token.  binned: the candidates were
+// counted in the bins above `gbase` while they were gathered.
+template <int THREADS, typename Sync>
+__device__ void merge_finish(const KParams &P, const RowCfg &c, int row, unsigned long long *buf, const int Pn, const int n,
+                             MergeShared<THREADS> &sh, int tid, uint2 cells, const bool binned, const uint32_t gbase);
+
 // Row merge for top-k class rows (one CTA per row).  buf is MERGE_CAP 64-bit
 // words of shared memory.  Returns false if the candidates cannot prove the
 // row's answer.
@@ -163,45 +209,13 @@ __device__ bool merge_topk_row(const KParams &P, const RowCfg &c, int row, int t
     // Large k: while the candidates are gathered they are also counted in 1024 bins of 8192 keys above the proven
     // threshold (one binade of fp32 keys; whatever lies higher shares the top bin).  The bin in which the count from
     // the top reaches k then brackets the k-th key without a pass of its own (GBINS ints in sh.scratch).
-    constexpr int GBINS = 2 * THREADS, GSHIFT = 13;
-    static_assert(GBINS * 4 <= THREADS * 8, "the counting bins live in the scratch words");
+    constexpr int GBINS = MERGE_GBINS, GSHIFT = MERGE_GSHIFT;
     int *ghist = reinterpret_cast<int *>(sh.scratch);
     const uint32_t gbase = c.temp ? tykey : tkey;
     const bool use_bins = !complete && c.k > RANK_SORT_MAX / 2 && total > RANK_SORT_MAX;
     auto gbin = [&](unsigned long long key) -> int {
         const uint32_t d = ((uint32_t)(key >> 32) - gbase) >> GSHIFT;
         return (int)min(d, (uint32_t)(GBINS - 1));
-    };
-    // the bin in which the count from the top reaches `need`, the count above it and the count with it (bin < 0: the
-    // bins hold fewer than `need`); thread t owns bins GBINS-1-2t and GBINS-2-2t.  Two barriers.
-    auto bins_find = [&](int need, int &bin, int &above, int &with) {
-        constexpr int BPT = GBINS / THREADS;
-        const int lane_ = tid & 31, warp_ = tid >> 5;
-        int v[BPT], sum = 0;
-#pragma unroll
-        for (int j = 0; j < BPT; ++j) { v[j] = ghist[GBINS - 1 - (tid * BPT + j)]; sum += v[j]; }
-        int incl = sum;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int o = __shfl_up_sync(0xFFFFFFFFu, incl, off);
-            if (lane_ >= off) incl += o;
-        }
-        if (lane_ == 31) sh.wsum[warp_] = incl;
-        if (tid == 0) sh.bracket[0] = -1;
-        csync();
-        int pre = incl - sum;
-        for (int w = 0; w < warp_; ++w) pre += sh.wsum[w];
-        if (pre < need && pre + sum >= need) {
-            int run = pre;
-#pragma unroll
-            for (int j = 0; j < BPT; ++j) {
-                if (run < need && run + v[j] >= need) { sh.bracket[0] = GBINS - 1 - (tid * BPT + j); sh.bracket[1] = run; sh.bracket[2] = run + v[j]; }
-                run += v[j];
-            }
-        }
-        csync();
-        bin = sh.bracket[0]; above = sh.bracket[1]; with = sh.bracket[2];
-        csync();
     };
     for (int attempt = 0; attempt < 2; ++attempt) {
         unsigned long long kmax = 0ull;
@@ -280,7 +294,7 @@ __device__ bool merge_topk_row(const KParams &P, const RowCfg &c, int row, int t
         // them, then pack again.  The bins counted during the pass usually give it at once ...
         if (use_bins) {
             int b, above, with;
-            bins_find(c.k, b, above, with);
+            merge_bins_find<THREADS>(sh, tid, c.k, b, above, with);
             if (b >= 0 && with <= MERGE_CAP) {
                 floor_key = max(1ull, ((unsigned long long)gbase + ((unsigned long long)b << GSHIFT)) << 32);
                 if (tid == 0) sh.count = 0;
@@ -446,7 +460,15 @@ __device__ bool merge_topk_row(const KParams &P, const RowCfg &c, int row, int t
     if (Pn >= c.k) n = c.k;
     else if (complete && P.op != OP_TOPK) n = Pn;
     else return false;
-    unsigned long long *sorted = buf;
+    merge_finish<THREADS, Sync>(P, c, row, buf, Pn, n, sh, tid, cells, use_bins, gbase);
+    return true;
+}
+
+template <int THREADS, typename Sync>
+__device__ void merge_finish(const KParams &P, const RowCfg &c, int row, unsigned long long *buf, const int Pn, const int n,
+                             MergeShared<THREADS> &sh, int tid, uint2 cells, const bool binned, const uint32_t gbase) {
+    Sync csync;
+    constexpr int GBINS = MERGE_GBINS, GSHIFT = MERGE_GSHIFT;
     int Pn2 = Pn;
     // How many keys the sort below should get at most: what the rank sort takes in one go when n is small, else the
     // bitonic size that leaves the threshold search a window of at least 16 ranks above n (for the largest n the
@@ -460,9 +482,9 @@ __device__ bool merge_topk_row(const KParams &P, const RowCfg &c, int row, int t
         bool tight = false;
         bool bracketed = false;
         int cnt_lo = Pn, cnt_hi = 0;
-        if (use_bins) {
+        if (binned) {
             int b, above, with;
-            bins_find(n, b, above, with);
+            merge_bins_find<THREADS>(sh, tid, n, b, above, with);
             if (b >= 0) {
                 // bin b holds the keys gbase + (b << GSHIFT) .. gbase + ((b + 1) << GSHIFT) - 1 (the top bin: and all above)
                 const unsigned long long klo = (unsigned long long)gbase + ((unsigned long long)b << GSHIFT);
@@ -637,8 +659,6 @@ __device__ bool merge_topk_row(const KParams &P, const RowCfg &c, int row, int t
         Pn2 = sh.count;
         csync();
     }
-    const int PnAll = Pn;
-    (void)PnAll;
 #define Pn Pn2
     if (Pn <= RANK_SORT_MAX) {
         // few candidates, one per thread: every warp sorts its 32 keys with shuffles, then a key's rank is its
@@ -660,7 +680,6 @@ __device__ bool merge_topk_row(const KParams &P, const RowCfg &c, int row, int t
         csync();
         bitonic_sort_desc_cta<THREADS>(buf, m, tid);
     }
-    (void)sorted;
 #undef Pn
 
     if (P.op == OP_TOPK) {
@@ -669,11 +688,11 @@ __device__ bool merge_topk_row(const KParams &P, const RowCfg &c, int row, int t
             P.out_vals[(size_t)row * P.ktop + j] = unkey((uint32_t)(kv >> 32));
             P.out_idx[(size_t)row * P.ktop + j] = (int)(~(uint32_t)kv);
         }
-        return true;
+        return;
     }
     if (n == 0) {
         if (tid == 0) emit_row(P, c, row, -1, 0.0f, F_NO_TOKEN, 0, 0.0f);
-        return true;
+        return;
     }
     // small supports are finished by one warp without block barriers
     if (n <= WARP_EPILOGUE_MAX) {
@@ -681,7 +700,6 @@ __device__ bool merge_topk_row(const KParams &P, const RowCfg &c, int row, int t
     } else {
         merge_epilogue<THREADS, Sync>(P, c, row, n, buf, sh, tid, cells);
     }
-    return true;
 }
 
 // Truncation epilogue and token selection over the n best candidates, sorted in
