@@ -55,7 +55,7 @@ __global__ void sonic_verify_combine_kernel(const KParams P, int B) {
 
 constexpr size_t WS_HEADER = WS_HEADER_WORDS * 4;
 constexpr size_t WS_CLEAR = WS_TICKETS * 4;       // the part of it that the streaming chain uses
-constexpr int MERGE_SMEM = MERGE_CAP * 8;
+constexpr int MERGE_SMEM = MERGE_CAP * 8 + MERGE_BUCKETS * 4;
 constexpr int STREAM_SMEM_F32 = VecTraits<0>::NSTAGE * CTA_TILE * 4 + (int)sizeof(StreamShared<0>);
 constexpr int STREAM_SMEM_BF16 = VecTraits<1>::NSTAGE * CTA_TILE * 2 + CTA_TILE * 4 + (int)sizeof(StreamShared<1>);
 constexpr int EXACT_CLUSTERS = 4;             // clusters of the cluster kernel (its rows are rare)

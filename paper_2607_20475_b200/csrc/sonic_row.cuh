@@ -96,6 +96,7 @@ constexpr int ROW_OFF_RX = ROW_SLICE_MAX * 4, ROW_OFF_H = ROW_OFF_RX + ROW_CMAX 
               ROW_OFF_CTL = ROW_OFF_MASK + ROW_SLICE_MAX / 8, ROW_DYN_SMEM = ROW_OFF_CTL + (int)sizeof(RowShared);
 static_assert(ROW_LAND * 8 >= ROW_BINS * ROW_COPIES * 8 && ROW_OFF_MASK - ROW_OFF_RX >= ROW_SLICE_MAX * 2, "areas share their place");
 static_assert(ROW_XBINS * 8 <= ROW_BINS * 4, "bins received");
+static_assert(ROW_CMAX * ROW_BINS >= MERGE_BUCKETS, "the sort's buckets take the place of the bins received");
 static_assert(ROW_DYN_SMEM + 1024 <= 233472 / 2, "two CTAs per SM");
 extern __shared__ __align__(128) unsigned char row_smem[];
 __device__ __forceinline__ float *row_y() { return reinterpret_cast<float *>(row_smem); }                                       // [slice] the CTA's part of the row
@@ -934,17 +935,13 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
         if (P.op == OP_TOPK) { for (int j = 0; j < P.ktop; ++j) { P.out_vals[(size_t)row * P.ktop + j] = -CUDART_INF_F; P.out_idx[(size_t)row * P.ktop + j] = -1; } }
         else emit(-1, 0.0f, F_TIMEOUT, 0, 0.0f);
     };
+    // A copy that never comes, or the workspace's sticky error: every CTA of the cluster learns of it with the first
+    // exchange, and all of them leave behind it (the values computed up to there are not used).
+    bool late = (err & ERR_TIMEOUT) != 0u;
     if (!mbar_wait(&sh.full, 0)) {
-        // the copy never came: every CTA of the cluster learns of it with the first exchange
         if (tid == 0) atomicOr(P.error, ERR_TIMEOUT);
-        cl_wait();
-        if (tid < x.ncta) *cl_map(&sh.late[x.rank], tid) = 1u;
-        cl_arrive();
-        cl_wait();
-        if (lead) emit_late();
-        return;
+        late = true;
     }
-    if (err & ERR_TIMEOUT) { if (lead) emit_late(); return; }
 
     // ---------------------------------------------------------------- logit processing
     // Penalties and biases commute with the mask (a masked logit stays -inf); they are applied to the raw values.
@@ -978,7 +975,8 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
         bad = __syncthreads_or(bad ? 1 : 0) != 0;                   // (every CTA reads the whole lists: all take the exit below or none)
     }
     if (bad) {
-        if (lead) emit(-1, 0.0f, F_BADPARAM | (c.cls == CLS_DENSE ? F_DENSE : 0u), 0, 0.0f);
+        if (lead && late) emit_late();
+        else if (lead) emit(-1, 0.0f, F_BADPARAM | (c.cls == CLS_DENSE ? F_DENSE : 0u), 0, 0.0f);
         return;
     }
     // Direct exchange of group maxima: the values stay undivided, only the candidates see the temperature.
@@ -1020,6 +1018,7 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
     const bool divide = c.temp && c.tau != 1.0f;
     process(divide && !direct, true);
     cl_wait();                                                      // every CTA of the cluster is running
+    if (late && tid < (greedy ? 1 : x.ncta)) *cl_map(&sh.late[x.rank], tid) = 1u;        // (a greedy row's other CTAs wait for nobody)
 
     RowSel s;
     s.vmin = P.op == OP_TOPK ? -CUDART_INF_F : -CUDART_MAX_NORMAL_F;
@@ -1096,7 +1095,7 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
                     buf[i] = v;
                 }
                 __syncthreads();
-                merge_finish<ROW_THREADS, BlockSync>(P, c, row, buf, n, min(c.k, n), sh.merge, tid, cells, false, 0u);
+                merge_finish<ROW_THREADS, BlockSync>(P, c, row, buf, reinterpret_cast<unsigned int *>(row_rx()), n, min(c.k, n), sh.merge, tid, cells);
             }
             if (finish_request && tid == 0) row_ticket(P, c.b);
             return;
@@ -1224,7 +1223,7 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
         unsigned long long *buf = reinterpret_cast<unsigned long long *>(row_smem);
         for (int i = tid; i < n; i += ROW_THREADS) buf[i] = row_land()[i];
         __syncthreads();
-        merge_finish<ROW_THREADS, BlockSync>(P, c, row, buf, n, min(c.k, n), sh.merge, tid, cells, false, 0u);
+        merge_finish<ROW_THREADS, BlockSync>(P, c, row, buf, reinterpret_cast<unsigned int *>(row_rx()), n, min(c.k, n), sh.merge, tid, cells);
         if (finish_request && tid == 0) row_ticket(P, c.b);
         return;
     }

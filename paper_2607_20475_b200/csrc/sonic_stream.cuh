@@ -99,12 +99,13 @@ struct MergeShared {
     unsigned int tkey;
     int n_p, n_m, pick;
     int found;
-    int wsum[THREADS / 32];                    // a block scan's warp totals
+    int wsum[THREADS / 32], wsum2[THREADS / 32];       // a block scan's warp totals
     int bracket[4];                            // the counting bins' answer: bin, count above it, count with it
     alignas(16) double scratch[THREADS];      // also read as int4
 };
 
 
+constexpr int MERGE_BUCKETS = 4096;           // buckets of the sort of larger candidate sets (16 KB behind the keys)
 constexpr int RANK_SORT_MAX = 512;            // at most this many candidates: sort by rank counting
 constexpr int WARP_EPILOGUE_MAX = 128;        // at most this many survivors of TopK: one warp finishes the row
 struct WarpSync { __device__ __forceinline__ void operator()() const { __syncwarp(); } };
@@ -153,19 +154,169 @@ __device__ __forceinline__ void merge_bins_find(MergeShared<THREADS> &sh, int ti
     __syncthreads();
 }
 
+// Sorts up to 256 distinct 64-bit keys (zeros pad) in descending order, one warp, eight keys per lane.
+__device__ __noinline__ void warp_sort_256(unsigned long long *a, int cnt, int lane) {
+    unsigned long long k[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) { const int e = j * 32 + lane; k[j] = (e < cnt) ? a[e] : 0ull; }
+#pragma unroll
+    for (int size = 2; size <= 256; size <<= 1) {
+#pragma unroll
+        for (int d = size >> 1; d > 0; d >>= 1) {
+            if (d >= 32) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int o = j ^ (d >> 5);
+                    if (o > j) {
+                        const bool desc = (((j * 32) & size) == 0);
+                        if ((k[j] < k[o]) == desc) { const unsigned long long t = k[j]; k[j] = k[o]; k[o] = t; }
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const unsigned long long o = __shfl_xor_sync(0xFFFFFFFFu, k[j], d);
+                    const int e = j * 32 + lane;
+                    const bool take_max = (((e & size) == 0) == ((e & d) == 0));
+                    k[j] = ((k[j] > o) == take_max) ? k[j] : o;
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) { const int e = j * 32 + lane; if (e < cnt) a[e] = k[j]; }
+}
+
+// Descending sort of n0 distinct 64-bit keys in buf (RANK_SORT_MAX < n0 <= MERGE_CAP), of which the first n are wanted:
+// 4096 buckets by distance from the smallest, one counting pass, one scan, one scatter;
+// what shares a bucket (a handful of keys for smooth values) is ranked by counting, a crowded bucket (ties of a
+// low-precision value) is sorted by a warp.  About 35 instructions per key in eight barrier-separated steps, where a
+// bitonic sort of 4096 keys goes through 78 compare-exchange steps, 21 of them behind block barriers.  A bucket beyond
+// 256 keys that the wanted ones reach into falls back to the bitonic sort.
+template <int THREADS>
+__device__ __forceinline__ void merge_bucket_sort(unsigned long long *buf, unsigned int *bins, const int n0, const int n, MergeShared<THREADS> &sh, int tid) {
+    constexpr int NB = MERGE_BUCKETS, ITEMS = MERGE_CAP / THREADS, BPT = NB / THREADS, FEW = 64, WARP_MAX = 256;
+    const int lane = tid & 31, warp = tid >> 5;
+    unsigned long long key[ITEMS];
+    uint32_t mx = 0u, mn = 0xFFFFFFFFu;
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) {
+        if (u * THREADS >= n0) break;
+        const int i = u * THREADS + tid;
+        key[u] = (i < n0) ? buf[i] : 0ull;
+        if (i < n0) { mx = max(mx, (uint32_t)(key[u] >> 32)); mn = min(mn, (uint32_t)(key[u] >> 32)); }
+    }
+    for (int i = tid; i < NB; i += THREADS) bins[i] = 0u;
+    mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+    mn = __reduce_min_sync(0xFFFFFFFFu, mn);
+    if (lane == 0) { sh.wsum[warp] = (int)mx; sh.wsum2[warp] = (int)mn; }
+    if (tid == 0) { sh.count = 0; sh.found = 0; }
+    __syncthreads();
+    mx = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)sh.wsum[lane & (THREADS / 32 - 1)]);
+    mn = __reduce_min_sync(0xFFFFFFFFu, (uint32_t)sh.wsum2[lane & (THREADS / 32 - 1)]);
+    // Bucket: 256 per octave of the distance above the smallest key.  The upper tail of a smooth distribution is dense at
+    // its lower end and thins out exponentially, so an octave holds at most a quarter of the keys (8 per bucket of 8192),
+    // and an outlier costs a few octaves of 16 instead of squashing everything else into a few buckets.
+    const float y0 = fmaxf(unkey(mn), -1.7e38f);
+    auto dist = [=](uint32_t key) -> int { return __float_as_int(fmaxf(fminf(unkey(key), 1.7e38f) - y0, 0.0f)) >> 15; };
+    const int top = dist(mx);
+    auto bucket = [=](unsigned long long k) -> int { return min(NB - 1, top - dist((uint32_t)(k >> 32))); };       // (monotone)
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) {
+        if (u * THREADS >= n0) break;
+        if (u * THREADS + tid < n0) atomicAdd(&bins[bucket(key[u])], 1u);
+    }
+    __syncthreads();
+    // exclusive scan of the buckets, BPT consecutive ones per thread
+    {
+        unsigned int v[BPT], sum = 0u;
+#pragma unroll
+        for (int j = 0; j < BPT; j += 4) {
+            const uint4 q = *reinterpret_cast<const uint4 *>(bins + tid * BPT + j);
+            v[j] = q.x; v[j + 1] = q.y; v[j + 2] = q.z; v[j + 3] = q.w;
+            sum += (q.x + q.y) + (q.z + q.w);
+        }
+        unsigned int incl = sum;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) { const unsigned int o = __shfl_up_sync(0xFFFFFFFFu, incl, off); if (lane >= off) incl += o; }
+        __syncthreads();                                            // (every thread has read the warps' extremes)
+        if (lane == 31) sh.wsum[warp] = (int)incl;
+        __syncthreads();
+        unsigned int run = incl - sum;
+        for (int w = 0; w < warp; ++w) run += (unsigned int)sh.wsum[w];
+#pragma unroll
+        for (int j = 0; j < BPT; ++j) {
+            if (v[j] > (unsigned int)FEW && run < (unsigned int)n) {
+                if (v[j] > (unsigned int)WARP_MAX) sh.found = 1;
+                else {
+                    const int at = atomicAdd(&sh.count, 1);
+                    reinterpret_cast<unsigned int *>(sh.scratch)[at] = run | (v[j] << 16);       // (more than MERGE_CAP / FEW never exist)
+                }
+            }
+            const unsigned int t = v[j]; v[j] = run; run += t;
+        }
+#pragma unroll
+        for (int j = 0; j < BPT; j += 4) *reinterpret_cast<uint4 *>(bins + tid * BPT + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+    }
+    __syncthreads();
+    if (sh.found) {
+        const int m = next_pow2(n0);
+        for (int i = n0 + tid; i < m; i += THREADS) buf[i] = 0ull;
+        __syncthreads();
+        bitonic_sort_desc_cta<THREADS>(buf, m, tid);
+        return;
+    }
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) {
+        if (u * THREADS >= n0) break;
+        if (u * THREADS + tid < n0) buf[atomicAdd(&bins[bucket(key[u])], 1u)] = key[u];
+    }
+    __syncthreads();
+    // bins[b] is now where bucket b ends: rank inside the bucket, for the wanted ones
+    int to[ITEMS];
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) {
+        if (u * THREADS >= n0) break;
+        const int i = u * THREADS + tid;
+        to[u] = -1;
+        if (i < n0) {
+            const unsigned long long k = buf[i];
+            const int b = bucket(k), first = b ? (int)bins[b - 1] : 0, cnt = (int)bins[b] - first;
+            if (first < n && cnt > 1 && cnt <= FEW) {
+                int r = first;
+#pragma unroll 4
+                for (int t = first; t < first + cnt; ++t) r += (buf[t] > k) ? 1 : 0;
+                to[u] = r;
+            }
+            key[u] = k;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) {
+        if (u * THREADS >= n0) break;
+        if (to[u] >= 0) buf[to[u]] = key[u];
+    }
+    const int crowded = sh.count;
+    for (int q = warp; q < crowded; q += THREADS / 32) {
+        const unsigned int e = reinterpret_cast<const unsigned int *>(sh.scratch)[q];
+        warp_sort_256(buf + (e & 0xFFFFu), (int)(e >> 16), lane);
+    }
+    __syncthreads();
+}
+
 // The rest of a top-k row once its candidates are in buf[0, Pn) (at most MERGE_CAP, distinct, in no order): the n best of
-// them, sorted, then the outputs of sonic_topk or the truncation epilogue and the token.  binned: the candidates were
-// counted in the bins above `gbase` while they were gathered.
+// them, sorted, then the outputs of sonic_topk or the truncation epilogue and the token.  bins: MERGE_BUCKETS words.
 template <int THREADS, typename Sync>
-__device__ void merge_finish(const KParams &P, const RowCfg &c, int row, unsigned long long *buf, const int Pn, const int n,
-                             MergeShared<THREADS> &sh, int tid, uint2 cells, const bool binned, const uint32_t gbase);
+__device__ void merge_finish(const KParams &P, const RowCfg &c, int row, unsigned long long *buf, unsigned int *bins, const int Pn, const int n,
+                             MergeShared<THREADS> &sh, int tid, uint2 cells);
 
 // Row merge for top-k class rows (one CTA per row).  buf is MERGE_CAP 64-bit
 // words of shared memory.  Returns false if the candidates cannot prove the
 // row's answer.
 template <int THREADS, typename Sync>
 __device__ bool merge_topk_row(const KParams &P, const RowCfg &c, int row, int tiles,
-                               unsigned long long *buf, MergeShared<THREADS> &sh, int tid, uint2 cells) {
+                               unsigned long long *buf, unsigned int *bins, MergeShared<THREADS> &sh, int tid, uint2 cells) {
     Sync csync;
     const int cap_t = (int)(P.cand_stride / (unsigned)tiles);
     const TileRec *rec = P.tiles + (size_t)row * MAX_TILES;
@@ -212,7 +363,7 @@ __device__ bool merge_topk_row(const KParams &P, const RowCfg &c, int row, int t
     constexpr int GBINS = MERGE_GBINS, GSHIFT = MERGE_GSHIFT;
     int *ghist = reinterpret_cast<int *>(sh.scratch);
     const uint32_t gbase = c.temp ? tykey : tkey;
-    const bool use_bins = !complete && c.k > RANK_SORT_MAX / 2 && total > RANK_SORT_MAX;
+    const bool use_bins = !complete && total > MERGE_CAP;
     auto gbin = [&](unsigned long long key) -> int {
         const uint32_t d = ((uint32_t)(key >> 32) - gbase) >> GSHIFT;
         return (int)min(d, (uint32_t)(GBINS - 1));
@@ -460,206 +611,14 @@ __device__ bool merge_topk_row(const KParams &P, const RowCfg &c, int row, int t
     if (Pn >= c.k) n = c.k;
     else if (complete && P.op != OP_TOPK) n = Pn;
     else return false;
-    merge_finish<THREADS, Sync>(P, c, row, buf, Pn, n, sh, tid, cells, use_bins, gbase);
+    merge_finish<THREADS, Sync>(P, c, row, buf, bins, Pn, n, sh, tid, cells);
     return true;
 }
 
 template <int THREADS, typename Sync>
-__device__ void merge_finish(const KParams &P, const RowCfg &c, int row, unsigned long long *buf, const int Pn, const int n,
-                             MergeShared<THREADS> &sh, int tid, uint2 cells, const bool binned, const uint32_t gbase) {
+__device__ void merge_finish(const KParams &P, const RowCfg &c, int row, unsigned long long *buf, unsigned int *bins, const int Pn, const int n,
+                             MergeShared<THREADS> &sh, int tid, uint2 cells) {
     Sync csync;
-    constexpr int GBINS = MERGE_GBINS, GSHIFT = MERGE_GSHIFT;
-    int Pn2 = Pn;
-    // How many keys the sort below should get at most: what the rank sort takes in one go when n is small, else the
-    // bitonic size that leaves the threshold search a window of at least 16 ranks above n (for the largest n the
-    // next size up would cost more than searching a narrow window).
-    int want_hi = (n + n / 2 + 16 <= RANK_SORT_MAX) ? n + n / 2 + 16 : next_pow2(n + 16);
-    if (want_hi > MERGE_CAP / 2) want_hi = next_pow2(n);
-    if (Pn > RANK_SORT_MAX && Pn > want_hi) {
-        // more proven candidates than that: search a key threshold that keeps between n and want_hi of them (any
-        // such threshold keeps the n best), then sort only those
-        unsigned long long lo = 0ull, hi = ~0ull;          // count(>= lo) >= n > count(>= hi)
-        bool tight = false;
-        bool bracketed = false;
-        int cnt_lo = Pn, cnt_hi = 0;
-        if (binned) {
-            int b, above, with;
-            merge_bins_find<THREADS>(sh, tid, n, b, above, with);
-            if (b >= 0) {
-                // bin b holds the keys gbase + (b << GSHIFT) .. gbase + ((b + 1) << GSHIFT) - 1 (the top bin: and all above)
-                const unsigned long long klo = (unsigned long long)gbase + ((unsigned long long)b << GSHIFT);
-                lo = klo << 32;
-                hi = (b == GBINS - 1 || klo + (1ull << GSHIFT) > 0xFFFFFFFFull) ? ~0ull : ((klo + (1ull << GSHIFT)) << 32);
-                cnt_hi = above;
-                cnt_lo = with;
-                bracketed = true;
-            }
-        }
-        if (!bracketed) {
-            // First bracket from the data itself: 31 of the keys, sorted, split the candidates into 32 buckets of
-            // about equal population wherever the keys crowd; one counting pass then places n within one bucket.
-            unsigned long long *sth = reinterpret_cast<unsigned long long *>(sh.scratch);          // [32] ascending, last = sentinel
-            int *hist = reinterpret_cast<int *>(sh.scratch + 32);                                  // [32]
-            unsigned long long *res = reinterpret_cast<unsigned long long *>(sh.scratch + 64);     // lo, hi, count(>= lo), count(>= hi)
-            if (tid < 32) {
-                unsigned long long k = (tid < 31) ? buf[(int)(((long long)(tid + 1) * Pn) >> 5)] : ~0ull;
-#pragma unroll
-                for (int kk = 2; kk <= 32; kk <<= 1) {
-#pragma unroll
-                    for (int jj = kk >> 1; jj > 0; jj >>= 1) {
-                        const unsigned long long o = __shfl_xor_sync(0xFFFFFFFFu, k, jj);
-                        const bool take_min = (((tid & kk) == 0) == ((tid & jj) == 0));
-                        k = ((k < o) == take_min) ? k : o;
-                    }
-                }
-                sth[tid] = k;
-                hist[tid] = 0;
-            }
-            csync();
-            for (int i = tid; i < Pn; i += THREADS) {
-                const unsigned long long key = buf[i];
-                int bkt = 0;                                   // number of sampled keys <= key
-#pragma unroll
-                for (int step = 16; step > 0; step >>= 1)
-                    if (bkt + step <= 31 && sth[bkt + step - 1] <= key) bkt += step;
-                atomicAdd(&hist[bkt], 1);
-            }
-            csync();
-            if (tid < 32) {
-                int suf = hist[tid];                           // -> number of keys in buckets >= tid
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int dn = __shfl_down_sync(0xFFFFFFFFu, suf, o);
-                    if (tid + o < 32) suf += dn;
-                }
-                // keys >= sth[q] are those of buckets q + 1 and above: the largest such q that still keeps n
-                const unsigned int okm = __ballot_sync(0xFFFFFFFFu, tid >= 1 && suf >= n);
-                if (okm) {
-                    const int l = 31 - __clz(okm);
-                    const int cnt = __shfl_sync(0xFFFFFFFFu, suf, l);
-                    const int above = (l < 31) ? __shfl_sync(0xFFFFFFFFu, suf, (l + 1) & 31) : 0;     // keys >= hi
-                    if (tid == 0) { res[0] = sth[l - 1]; res[1] = sth[l]; res[2] = (unsigned long long)cnt; res[3] = (unsigned long long)above; }
-                } else {
-                    const int above = __shfl_sync(0xFFFFFFFFu, suf, 1);
-                    if (tid == 0) { res[0] = 0ull; res[1] = sth[0]; res[2] = (unsigned long long)Pn; res[3] = (unsigned long long)above; }
-                }
-            }
-            csync();
-            lo = res[0]; hi = res[1];
-            cnt_lo = (int)res[2]; cnt_hi = (int)res[3];
-            csync();
-        }
-        {
-            tight = cnt_lo <= want_hi;
-            // The bucket [lo, hi) holds the boundary.  If it is small, its keys are collected and ranked, which gives
-            // the threshold that keeps exactly n (no search over key space, whose passes multiply when equal values
-            // differ only in their index bits).
-            const int in_bucket = cnt_lo - cnt_hi, need_here = n - cnt_hi;         // 1 <= need_here <= in_bucket
-            if (!tight && in_bucket <= THREADS) {
-                unsigned long long *list = reinterpret_cast<unsigned long long *>(sh.scratch);         // [THREADS]
-                if (tid == 0) sh.count = 0;
-                csync();
-                for (int i0 = 0; i0 < Pn; i0 += THREADS) {
-                    const int i = i0 + tid;
-                    const unsigned long long key = (i < Pn) ? buf[i] : 0ull;
-                    const bool inb = (i < Pn) && key >= lo && key < hi;
-                    const unsigned int mk = __ballot_sync(0xFFFFFFFFu, inb);
-                    int base = 0;
-                    if ((tid & 31) == 0 && mk) base = atomicAdd(&sh.count, __popc(mk));
-                    base = __shfl_sync(0xFFFFFFFFu, base, 0);
-                    if (inb) list[base + __popc(mk & ((1u << (tid & 31)) - 1u))] = key;
-                }
-                csync();
-                int rank;
-                const unsigned long long key = rank_keys<THREADS, Sync>(list, in_bucket, tid, rank);
-                csync();
-                if (key != 0ull && rank == need_here - 1) list[0] = key;      // exactly one thread (keys are distinct)
-                csync();
-                lo = list[0];
-                tight = true;                                   // count(>= lo) == n
-                csync();
-            }
-        }
-        // eight-way search: seven interior thresholds per pass.  The warps add their counts into one of two sets
-        // of totals in shared memory (the other set is cleared meanwhile), so a pass costs two block barriers
-        // and every thread reads just the seven totals.
-        int *tot2 = reinterpret_cast<int *>(sh.scratch);          // [2][8]
-        if (tid < 16) tot2[tid] = 0;
-        csync();
-        int pass = 0;
-        for (int it = 0; it < 24 && !tight && hi - lo > 1ull; ++it, ++pass) {
-            const unsigned long long step = (hi - lo) >> 3;
-            unsigned long long th[7];
-#pragma unroll
-            for (int q = 0; q < 7; ++q) th[q] = (step > 0) ? lo + step * (q + 1) : min(hi - 1ull, lo + 1ull + q);
-            int cnt[7] = {0, 0, 0, 0, 0, 0, 0};
-            for (int i = tid; i < Pn; i += THREADS) {
-                const unsigned long long key = buf[i];
-#pragma unroll
-                for (int q = 0; q < 7; ++q) cnt[q] += (key >= th[q]) ? 1 : 0;
-            }
-            int *tot = tot2 + (pass & 1) * 8;
-#pragma unroll
-            for (int q = 0; q < 7; ++q) {
-                cnt[q] = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned int)cnt[q]);
-                if ((tid & 31) == 0 && cnt[q]) atomicAdd(&tot[q], cnt[q]);
-            }
-            if (tid < 8) tot2[((pass + 1) & 1) * 8 + tid] = 0;     // the next pass's set (last read before the previous barrier)
-            csync();
-            const int4 a4 = reinterpret_cast<const int4 *>(tot)[0], b4 = reinterpret_cast<const int4 *>(tot)[1];
-            const int tots[7] = {a4.x, a4.y, a4.z, a4.w, b4.x, b4.y, b4.z};
-            bool done = false;
-#pragma unroll
-            for (int q = 6; q >= 0; --q) {                 // the highest threshold that still keeps n
-                if (!done && tots[q] >= n) {
-                    lo = th[q];
-                    if (q < 6) hi = th[q + 1];
-                    done = true;
-                    if (tots[q] <= want_hi) it = 1000;      // tight enough
-                }
-            }
-            if (!done) hi = th[0];
-            csync();
-        }
-        // keep the keys >= lo, packed to the front
-        if (tid == 0) sh.count = 0;
-        csync();
-        if (Pn <= MERGE_CAP / 2) {
-            // room for a copy: pack into the upper half without barriers, then move the survivors down
-            unsigned long long *up = buf + MERGE_CAP / 2;
-            for (int i0 = 0; i0 < Pn; i0 += THREADS) {
-                const int i = i0 + tid;
-                const unsigned long long key = (i < Pn) ? buf[i] : 0ull;
-                const bool keep = (i < Pn) && key >= lo;
-                const unsigned int mk = __ballot_sync(0xFFFFFFFFu, keep);
-                int base = 0;
-                if ((tid & 31) == 0 && mk) base = atomicAdd(&sh.count, __popc(mk));
-                base = __shfl_sync(0xFFFFFFFFu, base, 0);
-                if (keep) up[base + __popc(mk & ((1u << (tid & 31)) - 1u))] = key;
-            }
-            csync();
-            const int kept = sh.count;
-            for (int i = tid; i < kept; i += THREADS) buf[i] = up[i];
-        } else {
-            // in place (every position written is at or below one already read)
-            for (int i0 = 0; i0 < Pn; i0 += THREADS) {
-                const int i = i0 + tid;
-                const unsigned long long key = (i < Pn) ? buf[i] : 0ull;
-                const bool keep = (i < Pn) && key >= lo;
-                const unsigned int mk = __ballot_sync(0xFFFFFFFFu, keep);
-                csync();                                        // all reads of this trip precede its writes
-                int base = 0;
-                if ((tid & 31) == 0 && mk) base = atomicAdd(&sh.count, __popc(mk));
-                base = __shfl_sync(0xFFFFFFFFu, base, 0);
-                if (keep) buf[base + __popc(mk & ((1u << (tid & 31)) - 1u))] = key;
-                csync();
-            }
-        }
-        csync();
-        Pn2 = sh.count;
-        csync();
-    }
-#define Pn Pn2
     if (Pn <= RANK_SORT_MAX) {
         // few candidates, one per thread: every warp sorts its 32 keys with shuffles, then a key's rank is its
         // place in its own run plus, for every other run, the number of keys there above it (a binary search
@@ -674,13 +633,7 @@ __device__ void merge_finish(const KParams &P, const RowCfg &c, int row, unsigne
         csync();
         for (int i = tid; i < n; i += THREADS) buf[i] = dst[i];       // only the n best are used from here on
         csync();
-    } else {
-        const int m = next_pow2(Pn);
-        for (int i = Pn + tid; i < m; i += THREADS) buf[i] = 0ull;
-        csync();
-        bitonic_sort_desc_cta<THREADS>(buf, m, tid);
-    }
-#undef Pn
+    } else merge_bucket_sort<THREADS>(buf, bins, Pn, n, sh, tid);
 
     if (P.op == OP_TOPK) {
         for (int j = tid; j < n; j += THREADS) {
@@ -1736,7 +1689,7 @@ sonic_merge_kernel(const KParams P, const int tiles) {
         }
         return;
     }
-    const bool ok = merge_topk_row<MERGE_THREADS, BlockSync>(P, c, row, tiles, reinterpret_cast<unsigned long long *>(smem_raw), s_merge, tid, cells);
+    const bool ok = merge_topk_row<MERGE_THREADS, BlockSync>(P, c, row, tiles, reinterpret_cast<unsigned long long *>(smem_raw), reinterpret_cast<unsigned int *>(smem_raw + MERGE_CAP * 8), s_merge, tid, cells);
     if (tid == 0 && !ok) { rs->status = ST_FAILED; atomicAdd(&P.error[WS_FAILED_ROWS], 1u); }
     KERNEL_T1(1);
 }

@@ -1,0 +1,119 @@
+"""GPU parity tests of the row kernel (calls whose rows are resident at once: one cluster per row) and of the bucket sort of
+large candidate sets, at the sizes where they can go wrong: vocabularies at the edges of a CTA's part, every cluster size,
+supports at the limits of the short finish, ties, outliers that squash the bins, crowded buckets."""
+import numpy as np
+import pytest
+
+from paper_2607_20475_b200 import workloads as wl
+from tests.helpers import make_sample, pack_bits
+from tests.parity import compare_sample, compare_topk, compare_verify
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sonic():
+    from paper_2607_20475_b200 import harness
+    harness.lib()
+    return harness
+
+
+@pytest.fixture(scope="module")
+def oracle():
+    from oracle import oracle as o
+    return o
+
+
+def rows_of_every_class(rng, B, V, dtype):
+    """Greedy, small and large top-k, top-k beyond the gather, top-p, min-p, both, neither; lists and a mask on some."""
+    x = rng.standard_normal((B, V)).astype(np.float32) * 1.5
+    x[1::4] = (-1.1 * np.log(rng.permuted(np.tile(np.arange(1, V + 1), (len(x[1::4]), 1)), axis=1))).astype(np.float32)
+    x[2::4, :1] += 9.0
+    T = wl.TEMPERATURE
+    kinds = [(wl.GREEDY, 0), (wl.TOP_K | T, 20), (wl.TOP_K | T | wl.TOP_P, 100), (wl.TOP_K | T, 1000), (wl.TOP_P | T, 0),
+             (wl.MIN_P | T, 0), (wl.TOP_P | wl.MIN_P | T, 0), (T, 0), (wl.TOP_K | T | wl.TOP_P, 3000), (wl.TOP_K | wl.MIN_P, 128)]
+    mode = np.array([kinds[r % len(kinds)][0] for r in range(B)], np.uint32)
+    k = np.array([min(kinds[r % len(kinds)][1], V) for r in range(B)])
+    allowed = rng.random((B, V)) < 0.3
+    allowed[:, -1] = True
+    mode[3::7] |= wl.GRAMMAR
+    mode[::2] |= wl.REPETITION | wl.FREQUENCY | wl.PRESENCE | wl.BIAS
+    n = min(V, 40)
+    hist = [{int(i): int(c) for i, c in zip(rng.choice(V, n, replace=False), rng.integers(1, 5, n))} for _ in range(B)]
+    bias = [{int(i): float(v) for i, v in zip(rng.choice(V, min(V, 6), replace=False), rng.uniform(-5, 5, 6))} for _ in range(B)]
+    return make_sample(x, mode, dtype=dtype, temperature=rng.uniform(0.6, 1.4, B), top_k=k, top_p=np.full(B, 0.93),
+                       min_p=np.full(B, 0.03), rep=np.full(B, 1.2), freq=np.full(B, 0.2), pres=np.full(B, 0.3),
+                       bitmask=pack_bits(allowed), hist=hist, bias=bias, seed=np.arange(B) + V, offset=np.arange(B) * 3)
+
+
+@pytest.mark.parametrize("B,V", [(10, 1), (10, 5), (10, 2047), (10, 2048), (10, 2049), (10, 8192), (10, 8193), (12, 32767), (11, 32769),
+                                 (30, 65537), (40, 40960), (3, 262144), (11, 262143), (18, 200003), (74, 9000)])
+@pytest.mark.parametrize("dtype", [wl.DTYPE_F32, wl.DTYPE_BF16])
+def test_rows_of_every_class(sonic, oracle, B, V, dtype):
+    w = rows_of_every_class(np.random.default_rng(B * 1000003 + V), B, V, dtype)
+    dev = sonic.DeviceSample(w)
+    dev.run()
+    got = dev.results()
+    compare_sample(got, oracle.sample(w), w, max_near=B)         # (each near-margin row is held to an admissible outcome)
+    dev.run()
+    again = dev.results()
+    for key in got:
+        assert np.array_equal(got[key], again[key]), key
+
+
+@pytest.mark.parametrize("dtype", [wl.DTYPE_F32, wl.DTYPE_BF16])
+def test_ties_outliers_and_empty_parts(sonic, oracle, dtype):
+    # one value, two values, a single finite entry in the last CTA's part, a huge outlier, -1e9 in place of a mask
+    V = 50021
+    rng = np.random.default_rng(31)
+    base = rng.standard_normal(V).astype(np.float32)
+    rows = [np.zeros(V, np.float32), np.where(rng.random(V) < 0.4, 1.0, 0.0).astype(np.float32), np.full(V, -np.inf, np.float32),
+            base.copy(), np.where(rng.random(V) < 0.01, base, np.float32(-1e9)).astype(np.float32), base * 40, np.round(base * 4) / 4]
+    rows[2][V - 1] = 3.0
+    rows[3][77] = 1000.0
+    for mode, kw in ((wl.TOP_K, dict(top_k=50)), (wl.TOP_K | wl.TEMPERATURE, dict(top_k=700, temperature=1.7)),
+                     (wl.TOP_P | wl.TEMPERATURE, dict(top_p=0.9, temperature=1.3)), (wl.TOP_P | wl.MIN_P, dict(top_p=0.97, min_p=0.2)),
+                     (wl.TOP_K | wl.TOP_P, dict(top_k=5000, top_p=0.6)), (wl.GREEDY, {})):
+        B = len(rows)
+        w = make_sample(np.stack(rows), np.full(B, mode), dtype=dtype, seed=np.arange(B) + mode, offset=np.arange(B),
+                        **{n: np.full(B, v) for n, v in kw.items()})
+        dev = sonic.DeviceSample(w)
+        dev.run()
+        compare_sample(dev.results(), oracle.sample(w), w, max_near=B)
+
+
+@pytest.mark.parametrize("B,K,V", [(1, 0, 3000), (3, 2, 32003), (9, 3, 17000), (2, 7, 131072)])
+def test_verification_of_few_requests(sonic, oracle, B, K, V):
+    vw = wl.config4(B=B, K=K, V=V) if K else None
+    if vw is None:
+        full = wl.config4(B=B, K=1, V=V)
+        full.sample.logits = np.ascontiguousarray(full.sample.logits[::2])
+        vw = wl.VerifyWorkload(name="k0", B=B, K=0, V=V, sample=full.sample, draft_tokens=np.zeros((B, 0), np.int32),
+                               draft_probs=np.zeros((B, 0, V), np.float32))
+    else:
+        vw.draft_tokens[0, 0] = int(np.argmin(vw.sample.logits_f32()[0]))        # rejected
+    dev = sonic.DeviceVerify(vw)
+    dev.run()
+    got = dev.results()
+    compare_verify(got, oracle.verify(vw), vw, max_near=B)
+    dev.run()
+    again = dev.results()
+    for key in got:
+        assert np.array_equal(got[key], again[key]), key
+
+
+@pytest.mark.parametrize("B", [3, 80])                             # row kernel (k up to 2048), streaming chain
+@pytest.mark.parametrize("k", [100, 101, 129, 513, 1024, 2048, 2049, 4096])
+def test_large_top_k_sorts(sonic, oracle, B, k):
+    # smooth values, low-precision ties (crowded buckets), an outlier that squashes the buckets, few distinct values
+    V = 20001
+    rng = np.random.default_rng(k)
+    x = rng.standard_normal((B, V)).astype(np.float32)
+    x[1] = np.round(x[1] * 8) / 8
+    x[2] = np.where(rng.random(V) < 0.5, x[2], np.round(x[2]))
+    x[0, 5] = 1e30
+    tw = wl.TopKWorkload(name="t", B=B, V=V, dtype=wl.DTYPE_F32, logits=x)
+    dev = sonic.DeviceTopK(tw, k)
+    dev.run()
+    gv, gi = dev.results()
+    compare_topk(gv, gi, *oracle.topk(x, k))
