@@ -27,7 +27,6 @@
 #pragma once
 #include <cooperative_groups.h>
 #include "sonic_common.cuh"
-#include "sonic_dense.cuh"
 #include "sonic_stream.cuh"
 
 namespace sonic {
@@ -52,23 +51,24 @@ static_assert(ROW_KMAX <= KFAST_SAMPLE, "the epilogue's layout");
 static_assert(ROW_THREADS == MERGE_THREADS, "the merge epilogue runs on the row kernel's CTAs");
 static_assert(ROW_WARPS == ROW_CMAX, "half a warp: a lane per warp of the CTA, and per CTA of the cluster");
 
-// CTA 0 -> all.  again: 0 finished, 1 split the part [lo, hi] (need: what it has to bring), 2 the ties of one value (lo: its
-// key, need: how many of them are in), 3 masses at or above cutc.
-constexpr int RB_DONE = 0, RB_SPLIT = 1, RB_TIES = 2, RB_MASS = 3;
+// CTA 0 -> all.  again: 0 finished, 1 split the part [lo, hi] (need: what it has to bring), 2 masses at or above cutc.
+// tie_cta >= 0: the cut falls among the ties of the value with key cutc >> 32 (row_tie_cut).
+constexpr int RB_DONE = 0, RB_SPLIT = 1, RB_MASS = 2;
 constexpr unsigned int RB_ACCEPT = 1u, RB_REJECT = 2u;
 struct RowBcast {
     unsigned long long cutc, W, rest, need, lo, hi;
     unsigned int owner, support, flags;
     int again;
     float p_draft;
-    unsigned int pad;
+    int tie_cta;
+    unsigned int tie_in, pad;
 };
 
 struct RowShared {
     unsigned long long full;                      // mbarrier of the bulk copy
     unsigned int late[ROW_CMAX];                  // per CTA: its copy never came
     ulonglong2 ex1[ROW_CMAX];                     // per CTA: {max key << 32 | ~min finite key, best element or draft key}
-    ulonglong2 above[ROW_CMAX];                   // CTA 0: per CTA {mass, number} of what lies above the gathered part
+    ulonglong2 above[ROW_CMAX];                   // CTA 0: per CTA {mass, number | members << 32}: what lies above the gathered part; its members
     unsigned long long sum[2][ROW_CMAX];          // per CTA: exact masses that go with a level (total; above the first level's bin)
     ulonglong2 span[ROW_CMAX];                    // splits: per CTA {smallest, largest} element of the part
     double resid[ROW_CMAX][3];
@@ -76,9 +76,9 @@ struct RowShared {
     unsigned int land_n, land_min, land_max;      // CTA 0: elements received, their smallest and largest key
     unsigned int cross_bin;
     double cross_before, cross_in;
-    unsigned long long red64[ROW_WARPS], warp2[ROW_WARPS];
+    unsigned long long red64[ROW_WARPS], warp2[ROW_WARPS];       // (a search's scratch: both)
     unsigned int red32[ROW_WARPS];
-    double redd[3][ROW_WARPS];
+    double redd[3][ROW_WARPS];                    // (a search's scratch: two rows)
     unsigned long long cta_mass[ROW_CMAX];
     union {
         unsigned int gmax[ROW_GMAX];              // group maxima of all CTAs (keys)
@@ -132,6 +132,74 @@ __device__ __forceinline__ void row_each(const RowCtx &x, F f) {
         f(v.x, x.base + i); f(v.y, x.base + i + 1); f(v.z, x.base + i + 2); f(v.w, x.base + i + 3);
     }
 }
+
+// ---------------------------------------------------------------- block-level helpers
+__device__ __forceinline__ unsigned long long row_warp_sum(unsigned long long v) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
+    return v;
+}
+
+// Inclusive scan over the lanes of a warp.
+__device__ __forceinline__ unsigned long long row_warp_scan(unsigned long long v, int lane) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long up = __shfl_up_sync(0xFFFFFFFFu, v, o);
+        if (lane >= o) v += up;
+    }
+    return v;
+}
+
+// Exclusive prefix over the threads of the block (thread order) of one value per thread; `total` in every thread.
+template <typename T>
+__device__ __forceinline__ T row_block_scan(T v, T *wtot, int tid, T &total) {
+    const int lane = tid & 31, warp = tid >> 5;
+    T incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const T up = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += up;
+    }
+    __syncthreads();
+    if (lane == 31) wtot[warp] = incl;
+    __syncthreads();
+    T off = T(0), tot = T(0);
+#pragma unroll
+    for (int w = 0; w < ROW_WARPS; ++w) {
+        const T t = wtot[w];
+        if (w < warp) off += t;
+        tot += t;
+    }
+    total = tot;
+    return off + incl - v;
+}
+
+// 64-bit add to a shared-memory word as two native 32-bit atomics (low word first: the value it returns tells whether
+// the sum carried).  A 64-bit shared-memory atomic is a compare-and-swap loop, which crawls when many lanes add to a
+// handful of words (the per-tile masses of a row: 16 words, hundreds of listed elements).
+__device__ __forceinline__ void smem_add_u64(unsigned long long *p, unsigned long long w) {
+    unsigned int *q = reinterpret_cast<unsigned int *>(p);
+    const unsigned int lo = (unsigned int)w, hi = (unsigned int)(w >> 32);
+    unsigned int carry = 0u;
+    if (lo) { const unsigned int old = atomicAdd(q, lo); carry = (old + lo < old) ? 1u : 0u; }
+    if (hi + carry) atomicAdd(q + 1, hi + carry);
+}
+
+// Weight of an element in a residual.  The support's total weight W is known in fixed point first (from exp2 with a relative
+// error of up to 2e-7, too coarse where p - q cancels), so a part accumulates, in fp64, the residual sum R~ taken with
+// that W~, the sum Pp of the weights whose residual is positive, and the plain sum S of the weights; with W = sum of S the
+// residual is R~ - (1/W~ - 1/W) * Pp (exact up to the elements whose residual changes sign between W~ and W, each of which
+// contributes less than 1e-7 of its own probability).
+// An element that carries more than 2^-7 of the support's mass (at most 128 per row, usually a handful) is weighed with the
+// fp64 exponential: its residual is a difference of two numbers of that size.  The others use an fp32 exponential of
+// relative error below 1e-7 with no bias; independent errors of that size on probabilities below 2^-7 add up to less
+// than 1e-8 in the cumulative sums.
+__device__ __forceinline__ double resid_weight(uint32_t key, float Mf, double Md, float big) {
+    const float y = unkey(key);
+    const float w32 = exp_accurate(__fsub_rn(y, Mf));
+    return (w32 > big) ? exp((double)y - Md) : (double)w32;
+}
+
 
 // ---------------------------------------------------------------- weights
 // An element's weight exp(y - M) as qweight has it (the same operations, before the conversion).
@@ -232,7 +300,7 @@ __device__ __forceinline__ bool row_cross(const RowCtx &x, bool next, double wan
 __device__ __forceinline__ unsigned long long row_sum_bins(const RowCtx &x, int n) {
     RowShared &sh = row_sh();
     if (x.tid < ROW_BINS) {
-        const unsigned long long t = dense_warp_sum(x.tid < n ? sh.bins[x.tid] : 0ull);
+        const unsigned long long t = row_warp_sum(x.tid < n ? sh.bins[x.tid] : 0ull);
         if (x.lane == 0) sh.red64[x.warp] = t;
     }
     __syncthreads();
@@ -299,7 +367,7 @@ __device__ __noinline__ void row_split(const RowCtx &ctx, RowSel &sel, bool by_m
         for (int r = 0; r < x.ncta; ++r) v[u] += reinterpret_cast<const unsigned long long *>(row_rx())[r * ROW_XBINS + x.lane * 4 + u];
         run += v[u];
     }
-    const unsigned long long incl = dense_warp_scan(run, x.lane), all = __shfl_sync(0xFFFFFFFFu, incl, 31), want = max(1ull, min(need, all));
+    const unsigned long long incl = row_warp_scan(run, x.lane), all = __shfl_sync(0xFFFFFFFFu, incl, 31), want = max(1ull, min(need, all));
     const unsigned int hit = __ballot_sync(0xFFFFFFFFu, incl >= want);
     const int l = hit ? __ffs(hit) - 1 : 31;
     unsigned long long before = incl - run, in = 0ull;
@@ -334,54 +402,57 @@ __device__ __forceinline__ unsigned int row_room(const RowCtx &x, unsigned int m
     }
     return pos;
 }
-// The warps' sums of a mass and a number -> this CTA's entry of CTA 0's sh.above (block barrier inside).
-__device__ __forceinline__ void row_send_above(const RowCtx &x, unsigned long long m, unsigned int n, unsigned long long more) {
+// The warps' sums of a mass, a number and a number of members -> this CTA's entry of CTA 0's sh.above (block barrier inside).
+__device__ __forceinline__ void row_send_above(const RowCtx &x, unsigned long long m, unsigned int n, unsigned int members, unsigned long long more) {
     RowShared &sh = row_sh();
-    m = dense_warp_sum(m);
-    n = __reduce_add_sync(0xFFFFFFFFu, n);
-    if (x.lane == 0) { sh.warp2[x.warp] = m; sh.red32[x.warp] = n; }
+    m = row_warp_sum(m);
+    const unsigned int both = __reduce_add_sync(0xFFFFFFFFu, n | (members << 16));      // (a warp has at most 1024 elements)
+    if (x.lane == 0) { sh.warp2[x.warp] = m; sh.red32[x.warp] = both; }
     __syncthreads();
     if (x.warp == 0) {
-        m = dense_warp_sum(x.lane < ROW_WARPS ? sh.warp2[x.lane] : 0ull);
-        n = __reduce_add_sync(0xFFFFFFFFu, x.lane < ROW_WARPS ? sh.red32[x.lane] : 0u);
-        if (x.lane == 0) *cl_map(&sh.above[x.rank], 0) = make_ulonglong2(m + more, (unsigned long long)n);
+        m = row_warp_sum(x.lane < ROW_WARPS ? sh.warp2[x.lane] : 0ull);
+        const unsigned int t = x.lane < ROW_WARPS ? sh.red32[x.lane] : 0u;
+        n = __reduce_add_sync(0xFFFFFFFFu, t & 0xFFFFu);
+        members = __reduce_add_sync(0xFFFFFFFFu, t >> 16);
+        if (x.lane == 0) *cl_map(&sh.above[x.rank], 0) = make_ulonglong2(m + more, (unsigned long long)n | ((unsigned long long)members << 32));
     }
 }
-// Elements of a level's bin (their weights' bits, shifted, equal `code`) to CTA 0, and the number of those above it; `more`:
-// the exact mass above it (warp 0).  The caller's cluster barrier completes it.
+// Elements of a level's bin (their weights' bits, shifted, equal `code`) to CTA 0, and their number and that of the elements
+// above; `more`: the exact mass above (warp 0).  One pass marks the bin's elements in a bit per element of the lane, the few
+// that are marked are then fetched again.  The caller's cluster barrier completes it.
 __device__ __forceinline__ void row_gather_bin(const RowCtx &x, const RowSel &s, int shift, int code, unsigned long long more) {
     RowShared &sh = row_sh();
     const float Mf = x.Mf;
-    unsigned int an = 0u, mine = 0u;
+    unsigned int an = 0u, hits = 0u;
+    int bit = 0;
+    static_assert(ROW_SLICE_MAX / ROW_THREADS <= 32, "a bit per element of a lane");
     row_each(x, [&](float y, int idx) {
-        const uint32_t bits = __float_as_uint(row_w(y, Mf));
-        const int d = (int)((0x3FFFFFFFu - bits) >> shift);
+        const int d = (int)((0x3FFFFFFFu - __float_as_uint(row_w(y, Mf))) >> shift);
         const bool in = y >= s.vmin && d <= code && (!s.cut || row_elem(y, idx) >= s.base);
         an += (in && d < code) ? 1u : 0u;
-        mine += (in && d == code) ? 1u : 0u;
+        hits |= (in && d == code) ? (1u << bit) : 0u;
+        ++bit;
     });
+    const unsigned int mine = (unsigned int)__popc(hits);
     bool any;
     unsigned int pos = row_room(x, mine, any);
     if (any) {
         uint32_t mn = 0xFFFFFFFFu, mx = 0u;
-        if (mine) {
-            unsigned long long *land = cl_map(row_land(), 0);
-            row_each(x, [&](float y, int idx) {
-                const int d = (int)((0x3FFFFFFFu - __float_as_uint(row_w(y, Mf))) >> shift);
-                if (d == code && row_in(s, y, idx)) {
-                    const unsigned long long c = row_elem(y, idx);
-                    mn = min(mn, (uint32_t)(c >> 32)); mx = max(mx, (uint32_t)(c >> 32));
-                    if (pos < (unsigned int)ROW_MEMBERS) land[pos] = c;
-                    ++pos;
-                }
-            });
+        unsigned long long *land = cl_map(row_land(), 0);
+        while (hits) {
+            const int b = __ffs(hits) - 1, li = x.wlo + (b >> 2) * 128 + x.lane * 4 + (b & 3);
+            hits &= hits - 1u;
+            const unsigned long long c = row_elem(row_y()[li], x.base + li);
+            mn = min(mn, (uint32_t)(c >> 32)); mx = max(mx, (uint32_t)(c >> 32));
+            if (pos < (unsigned int)ROW_MEMBERS) land[pos] = c;
+            ++pos;
         }
         __syncwarp();
         mn = __reduce_min_sync(0xFFFFFFFFu, mn);
         mx = __reduce_max_sync(0xFFFFFFFFu, mx);
         if (x.lane == 0) { atomicMin(cl_map(&sh.land_min, 0), mn); atomicMax(cl_map(&sh.land_max, 0), mx); }
     }
-    row_send_above(x, 0ull, an, more);
+    row_send_above(x, 0ull, an, mine, more);
 }
 // Elements of the part [s.lo, s.hi] to CTA 0; mass and number of those above it.  MASS: also when the part is empty.
 __device__ __noinline__ void row_gather_part(const RowCtx &ctx, const RowSel &sel) {
@@ -415,7 +486,7 @@ __device__ __noinline__ void row_gather_part(const RowCtx &ctx, const RowSel &se
         mx = __reduce_max_sync(0xFFFFFFFFu, mx);
         if (x.lane == 0) { atomicMin(cl_map(&sh.land_min, 0), mn); atomicMax(cl_map(&sh.land_max, 0), mx); }
     }
-    row_send_above(x, am, an, 0ull);
+    row_send_above(x, am, an, mine, 0ull);
 }
 // Mass and number of the elements at or above cutc.
 __device__ __noinline__ void row_mass_above(const RowCtx &ctx, float vmin, unsigned long long cutc) {
@@ -433,11 +504,8 @@ __device__ __noinline__ void row_mass_above(const RowCtx &ctx, float vmin, unsig
         am += in ? q : 0ull;
         an += in ? 1u : 0u;
     });
-    row_send_above(x, am, an, 0ull);
+    row_send_above(x, am, an, 0u, 0ull);
 }
-// The `m` ties of key v that are in, by index: the last one's element, sent to all CTAs (in sh.span[0].x).  Two cluster barriers.
-__device__ __noinline__ unsigned long long row_ties(const RowCtx &ctx, const RowSel &sel, uint32_t v, unsigned long long m);
-
 // CTA 0's word to all, then a cluster barrier (bc: the same in every thread of CTA 0).
 __device__ __forceinline__ void row_broadcast(const RowCtx &x, const RowBcast &bc) {
     RowShared &sh = row_sh();
@@ -669,12 +737,18 @@ __device__ __forceinline__ void row_finish_small(const RowCtx &x, const KParams 
     }
 }
 
-// The element, in index order, at which the running weight of the CTA's part first exceeds `rest`: the warp, then its
-// 128-element groups, then the lane, then the element.  wf(value, index) -> weight, T integer or fp64.  f(index, weight)
-// is called by one thread of the CTA (the last element of positive weight if rounding keeps the sum below `rest`; not at
-// all if there is none).
+template <typename T>
+__device__ __forceinline__ T row_lane_scan(T v, int lane) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const T up = __shfl_up_sync(0xFFFFFFFFu, v, o); if (lane >= o) v += up; }
+    return v;
+}
+// The element, in index order, at which the running weight of the CTA's part first exceeds `rest`: the warp whose part it
+// is, then that part spread over the whole CTA (one or two consecutive elements per thread).  wf(value, index) -> weight,
+// T integer or fp64; wtot: 2 * ROW_WARPS words.  f(index, weight) is called by one thread of the CTA (for the last element of
+// positive weight if rounding keeps the sum below `rest`; not at all if there is none).  Three block barriers.
 template <typename T, typename WF, typename F>
-__device__ void row_find(const RowCtx &x, T rest, T *wtot, WF wf, F f) {
+__device__ __forceinline__ void row_find(const RowCtx &x, T rest, T *wtot, WF wf, F f) {
     T s = T(0);
     row_each(x, [&](float y, int idx) { s += wf(y, idx); });
 #pragma unroll
@@ -682,54 +756,28 @@ __device__ void row_find(const RowCtx &x, T rest, T *wtot, WF wf, F f) {
     __syncthreads();
     if (x.lane == 0) wtot[x.warp] = s;
     __syncthreads();
-    int w = -1, last = -1;
-    for (int v = 0; v < ROW_WARPS; ++v) {
-        const T t = wtot[v];
-        if (t > T(0)) last = v;
-        if (w < 0 && t > T(0)) { if (rest < t) w = v; else rest -= t; }
+    const T tw = (x.lane < ROW_WARPS) ? wtot[x.lane] : T(0);
+    T incl = row_lane_scan<T>(tw, x.lane);
+    const unsigned int pos = __ballot_sync(0xFFFFFFFFu, tw > T(0)), hit = __ballot_sync(0xFFFFFFFFu, tw > T(0) && incl > rest);
+    if (!pos) return;
+    const int w = hit ? __ffs(hit) - 1 : 31 - __clz(pos);           // (no hit: floating-point sums, past the end by rounding)
+    rest -= __shfl_sync(0xFFFFFFFFu, incl - tw, w);
+    const int per = (x.wn > ROW_THREADS) ? 2 : 1, li = w * x.wn + x.tid * per;
+    const bool mine = x.tid * per < x.wn;
+    const T a = mine ? wf(row_y()[li], x.base + li) : T(0), b = (mine && per == 2) ? wf(row_y()[li + 1], x.base + li + 1) : T(0);
+    incl = row_lane_scan<T>(a + b, x.lane);
+    if (x.lane == 31) wtot[ROW_WARPS + x.warp] = incl;
+    __syncthreads();
+    const T t2 = (x.lane < ROW_WARPS) ? wtot[ROW_WARPS + x.lane] : T(0), i2 = row_lane_scan<T>(t2, x.lane);
+    const T hi = incl + __shfl_sync(0xFFFFFFFFu, i2 - t2, x.warp), lo = hi - (a + b);
+    // the first element in index order that takes the sum beyond `rest`, else the last of positive weight
+    const unsigned int over = __ballot_sync(0xFFFFFFFFu, t2 > T(0) && i2 > rest), some = __ballot_sync(0xFFFFFFFFu, t2 > T(0));
+    const unsigned int mh = __ballot_sync(0xFFFFFFFFu, a + b > T(0) && hi > rest), mp = __ballot_sync(0xFFFFFFFFu, a + b > T(0));
+    if (x.warp != (over ? __ffs(over) - 1 : 31 - __clz(some))) return;
+    if (x.lane == (mh ? __ffs(mh) - 1 : 31 - __clz(mp))) {
+        const bool first = a > T(0) && (lo + a > rest || !(b > T(0)));
+        f(x.base + li + (first ? 0 : 1), first ? a : b);
     }
-    const bool over = w < 0;                                        // (floating-point sums: past the end by rounding)
-    if (over) w = last;
-    if (x.warp != w) return;
-    int fi = -1;
-    T fw = T(0);
-    bool hit_any = false;
-    for (int i = x.wlo; i < x.wlo + x.wn && !hit_any; i += 128) {
-        const int li = i + x.lane * 4;
-        const float4 v = *reinterpret_cast<const float4 *>(row_y() + li);
-        const float y4[4] = {v.x, v.y, v.z, v.w};
-        T w4[4], t = T(0);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) { w4[u] = wf(y4[u], x.base + li + u); t += w4[u]; }
-        T incl = t;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const T up = __shfl_up_sync(0xFFFFFFFFu, incl, o); if (x.lane >= o) incl += up; }
-        const T tot = __shfl_sync(0xFFFFFFFFu, incl, 31);
-        const unsigned int pos = __ballot_sync(0xFFFFFFFFu, t > T(0));
-        if (!pos) continue;
-        const unsigned int hit = over ? 0u : __ballot_sync(0xFFFFFFFFu, t > T(0) && incl > rest);
-        const int l = hit ? __ffs(hit) - 1 : 31 - __clz(pos);       // (no hit: remembered as the last positive one so far)
-        if (x.lane == l) {
-            T cum = incl - t;
-            int at = -1, lp = -1;
-            T aw = T(0), lw = T(0);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                cum += w4[u];
-                if (w4[u] > T(0)) {
-                    lp = u; lw = w4[u];
-                    if (hit && at < 0 && cum > rest) { at = u; aw = w4[u]; }
-                }
-            }
-            if (at < 0) { at = lp; aw = lw; }
-            fi = x.base + li + at; fw = aw;
-        }
-        fi = __shfl_sync(0xFFFFFFFFu, fi, l);
-        fw = __shfl_sync(0xFFFFFFFFu, fw, l);
-        hit_any = hit != 0u;
-        rest -= tot;
-    }
-    if (x.lane == 0 && fi >= 0) f(fi, fw);
 }
 
 // Ranks the n <= ROW_THREADS elements CTA 0 has received: the thread's element and its weight in descending order (0 past
@@ -747,33 +795,17 @@ __device__ __forceinline__ void row_rank(const RowCtx &x, int n, unsigned long l
     w = c ? row_q(row_w(unkey((uint32_t)(c >> 32)), x.Mf)) : 0ull;
 }
 
-__device__ __noinline__ unsigned long long row_ties(const RowCtx &ctx, const RowSel &sel, uint32_t v, unsigned long long m) {
-    const RowCtx x = ctx;
-    const RowSel s = sel;
+// The cut of this CTA's part when the cut falls among the ties of one value, by index: all of them are in before CTA
+// `tie_cta`, none behind it, its own first `tie_in` there.  (Called by the whole CTA; block barriers in that CTA alone.)
+__device__ __forceinline__ unsigned long long row_tie_cut(const RowCtx &x, const RowSel &s, uint32_t v, int tie_cta, unsigned int tie_in) {
+    if (x.rank != tie_cta) return ((unsigned long long)v + (x.rank > tie_cta ? 1ull : 0ull)) << 32;
     RowShared &sh = row_sh();
     const float vy = unkey(v);
-    unsigned int n = 0u;
-    row_each(x, [&](float y, int idx) { n += (y == vy && row_in(s, y, idx)) ? 1u : 0u; });
-    n = __reduce_add_sync(0xFFFFFFFFu, n);
-    if (x.lane == 0) sh.red32[x.warp] = n;
+    row_find<unsigned int>(x, tie_in - 1u, reinterpret_cast<unsigned int *>(sh.red64),
+                           [&](float y, int idx) -> unsigned int { return (y == vy && row_in(s, y, idx)) ? 1u : 0u; },
+                           [&](int idx, unsigned int) { sh.span[0].x = row_comp(v, idx); });
     __syncthreads();
-    if (x.tid < x.ncta) {
-        unsigned long long t = 0ull;
-        for (int w = 0; w < ROW_WARPS; ++w) t += sh.red32[w];
-        *cl_map(&sh.sum[0][x.rank], x.tid) = t;
-    }
-    cl_sync();
-    unsigned long long rest = m - 1ull;
-    int owner = -1;
-    for (int r = 0; r < x.ncta; ++r) {
-        const unsigned long long t = sh.sum[0][r];
-        if (owner < 0) { if (rest < t) owner = r; else rest -= t; }
-    }
-    if (owner == x.rank)
-        row_find<unsigned long long>(x, rest, sh.red64, [&](float y, int idx) -> unsigned long long { return (y == vy && row_in(s, y, idx)) ? 1ull : 0ull; },
-                                     [&](int idx, unsigned long long) { for (int r = 0; r < x.ncta; ++r) cl_map(&sh.span[0], r)->x = row_comp(v, idx); });
-    cl_sync();
-    return owner < 0 ? (unsigned long long)v << 32 : sh.span[0].x;
+    return sh.span[0].x;
 }
 
 // Whether some CTA's copy never came (checked after the first exchange).
@@ -830,6 +862,8 @@ __device__ __noinline__ bool row_residual(const RowCtx &ctx, const KParams &P, c
         to[0] = R; to[1] = Pp; to[2] = S;
     }
     cl_sync();
+    KERNEL_T1(4);
+    KERNEL_T0(9);
     double W = 0.0;
     for (int r = 0; r < x.ncta; ++r) W += sh.resid[r][2];
     const double corr = inv_Wt - 1.0 / W;
@@ -862,35 +896,33 @@ __device__ __noinline__ bool row_residual(const RowCtx &ctx, const KParams &P, c
 }
 
 
-// Grid: rows x CTAs of a cluster.  slice: elements per CTA (a multiple of ROW_UNIT, slice * cluster >= V).
-template <int DT>
-__global__ void __launch_bounds__(ROW_THREADS, 2)
-sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
+// One row by the CTAs of a cluster.  LISTED: the cluster takes row after row of those the streaming kernel leaves to it
+// (sampling rows with top-k off, or with a top-k beyond what it handles), beside that kernel; every path then ends with
+// the cluster barrier's phases complete, and a verification call's scan has a kernel of its own.  parity: of the row's copy.
+template <int DT, bool LISTED>
+__device__ __forceinline__ void row_body(const KParams &P, RowCtx &x, const int row, const unsigned int parity) {
     constexpr int VEC = VecTraits<DT>::VEC, ELT = VecTraits<DT>::ELT;
     RowShared &sh = row_sh();
-    RowCtx x;
-    x.rank = (int)cgr::this_cluster().block_rank();
-    x.ncta = (int)cgr::this_cluster().num_blocks();
-    x.slice = slice;
-    x.base = x.rank * slice;
-    x.tid = threadIdx.x; x.lane = x.tid & 31; x.warp = x.tid >> 5;
-    x.wn = slice / ROW_WARPS; x.wlo = x.warp * x.wn;
+    const int slice = x.slice;
     uint32_t *mask = row_mask();
     unsigned char *raw = row_smem + (DT == 0 ? 0 : ROW_OFF_RX);
-    const int row = (int)blockIdx.x / x.ncta;
     const int tid = x.tid, lane = x.lane;
     const bool lead = x.rank == 0 && tid == 0;
 
+    if (LISTED) KERNEL_T0(6);
     const CfgRaw cfg_raw = fetch_cfg(P, row);
     const int req = (P.op == OP_VERIFY) ? row / (P.K + 1) : row;
     // Everything the row needs from global memory is asked for at once: its logits by one bulk copy, mask words,
     // parameters and the first entries of its lists (none of the addresses depends on a loaded value).
     if (tid == 0) {
-        mbar_init(&sh.full, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         const int elems = min(slice, (P.V - x.base + VEC - 1) / VEC * VEC);
         if (elems > 0) {
             mbar_arrive_expect_tx(&sh.full, (unsigned int)elems * ELT);
+#ifdef SONIC_TEST_WITHHOLD
+            // test-only build: the copy of the part that holds one chosen tile is announced but never issued
+            const unsigned int held = __ldcg(&P.error[WS_TEST_WITHHOLD]), htiles = (unsigned int)(P.V + CTA_TILE - 1) / CTA_TILE;
+            if (held == 0u || (int)((held - 1u) / htiles) != row || (int)((held - 1u) % htiles) * CTA_TILE / slice != x.rank)
+#endif
             bulk_load(raw, reinterpret_cast<const unsigned char *>(P.logits) + ((size_t)row * (size_t)P.row_stride + (size_t)x.base) * ELT,
                       (unsigned int)elems * ELT, &sh.full, l2_evict_first_policy());
         } else mbar_arrive(&sh.full);
@@ -925,20 +957,22 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
     __syncthreads();
     cl_arrive();                                                    // (matched by the wait before the first remote write)
     const RowCfg c = resolve_cfg(P, row, cfg_raw);
-    const bool finish_request = P.op == OP_VERIFY;
-    const bool dense = c.cls == CLS_DENSE || c.cls == CLS_EXACT, greedy = c.cls == CLS_GREEDY;
+    const bool finish_request = !LISTED && P.op == OP_VERIFY;
+    const bool dense = LISTED || c.cls == CLS_DENSE || c.cls == CLS_EXACT, greedy = !LISTED && c.cls == CLS_GREEDY;
     auto emit = [&](int token, float prob, uint32_t flags, int support, float p_draft) {
         emit_row(P, c, row, token, prob, flags, support, p_draft);
         if (finish_request) row_ticket(P, c.b);
     };
-    auto emit_late = [&]() {                                        // (a wait for a copy ran out, in this call or an earlier one on this workspace)
+    auto emit_late = [&]() {
+        if (LISTED) return;                                         // (the chain's last kernel reports it for every row)
+                                            // (a wait for a copy ran out, in this call or an earlier one on this workspace)
         if (P.op == OP_TOPK) { for (int j = 0; j < P.ktop; ++j) { P.out_vals[(size_t)row * P.ktop + j] = -CUDART_INF_F; P.out_idx[(size_t)row * P.ktop + j] = -1; } }
         else emit(-1, 0.0f, F_TIMEOUT, 0, 0.0f);
     };
     // A copy that never comes, or the workspace's sticky error: every CTA of the cluster learns of it with the first
     // exchange, and all of them leave behind it (the values computed up to there are not used).
     bool late = (err & ERR_TIMEOUT) != 0u;
-    if (!mbar_wait(&sh.full, 0)) {
+    if (!mbar_wait(&sh.full, parity)) {
         if (tid == 0) atomicOr(P.error, ERR_TIMEOUT);
         late = true;
     }
@@ -975,6 +1009,10 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
         bad = __syncthreads_or(bad ? 1 : 0) != 0;                   // (every CTA reads the whole lists: all take the exit below or none)
     }
     if (bad) {
+        if (LISTED) {
+            cl_wait();
+            if (late && tid < x.ncta) *cl_map(&sh.late[x.rank], tid) = 1u;
+        }
         if (lead && late) emit_late();
         else if (lead) emit(-1, 0.0f, F_BADPARAM | (c.cls == CLS_DENSE ? F_DENSE : 0u), 0, 0.0f);
         return;
@@ -1030,7 +1068,7 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
         return make_uint2(r4[0] >> 8, r4[1] >> 8);
     };
 
-    if (direct) {
+    if (!LISTED && direct) {
         // ------------------------------------------------------------ top-k, small k
         float g = lmax;
         for (int off = 16 / gpw; off > 0; off >>= 1) g = fmaxf(g, __shfl_xor_sync(0xFFFFFFFFu, g, off));
@@ -1180,7 +1218,7 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
         return;
     }
 
-    if (!dense) {
+    if (!LISTED && !dense) {
         // ------------------------------------------------------------ top-k, larger k
         bool by_lanes = !direct && 4 * c.k <= x.ncta * ROW_THREADS;
         int n = 0;
@@ -1267,7 +1305,7 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
         unsigned long long t = row_sum_bins(x, ROW_BINS);
         if (tid < x.ncta) *cl_map(&sh.sum[0][x.rank], tid) = t;
         cl_sync();
-        for (int r = 0; r < x.ncta; ++r) Z += sh.sum[0][r];
+        Z = row_warp_sum(lane < x.ncta ? sh.sum[0][lane] : 0ull);
         goal = max(1ull, min((unsigned long long)ceil((double)c.p * (double)Z), Z));
         int bin_a, bin_b;
         double before, in_bin;
@@ -1282,49 +1320,89 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
         __syncthreads();
         row_fold<true>(x, true, [=](int) { return bin_a >> m; });
         cl_sync();
-        unsigned long long above_a = 0ull;
-        for (int r = 0; r < x.ncta; ++r) above_a += sh.sum[1][r];
+        const unsigned long long above_a = row_warp_sum(lane < x.ncta ? sh.sum[1][lane] : 0ull);
         row_cross(x, false, (double)(goal > above_a ? goal - above_a : 1ull), bin_b, before, in_bin);
         const unsigned long long own_b = row_sum_bins(x, bin_b);
+        if (LISTED) { KERNEL_T1(6); KERNEL_T0(3); }
         row_gather_bin(x, s, shift_b, (bin_a << 8) | bin_b, t + own_b);
     } else row_mass_above(x, s.vmin, floorc);
     cl_sync();
+    if (LISTED) { KERNEL_T1(3); KERNEL_T0(8); }
     bool exact = !top_p;                                            // the gathered part is the right one by construction
     bool masses = !top_p;                                           // sh.above: the whole support, nothing gathered
     unsigned long long cutc = floorc;
     for (int guard = 0; guard < 40; ++guard) {
         RowBcast bc;
         bc.cutc = cutc; bc.W = 0ull; bc.rest = 0ull; bc.need = 0ull; bc.lo = 0ull; bc.hi = 0ull;
-        bc.owner = 0u; bc.support = 0u; bc.flags = 0u; bc.again = RB_DONE; bc.p_draft = 0.0f; bc.pad = 0u;
+        bc.owner = 0u; bc.support = 0u; bc.flags = 0u; bc.again = RB_DONE; bc.p_draft = 0.0f; bc.tie_cta = -1; bc.tie_in = 0u; bc.pad = 0u;
         if (x.rank == 0) {
-            const int nm = (int)sh.land_n;
+            const int nm = masses ? 0 : (int)sh.land_n;
             const uint32_t kmn = sh.land_min, kmx = sh.land_max;
-            if (tid < x.ncta) sh.cta_mass[tid] = sh.above[tid].x;
-            unsigned long long n = 0ull;
-            for (int r = 0; r < x.ncta; ++r) { bc.W += sh.above[r].x; n += sh.above[r].y; }
+            const ulonglong2 ab = (lane < x.ncta) ? sh.above[lane] : make_ulonglong2(0ull, 0ull);      // (lane r: CTA r)
+            unsigned long long mass = ab.x;                         // CTA r's part of the support
+            const unsigned int members = (unsigned int)(ab.y >> 32);
+            bc.W = row_warp_sum(ab.x);
+            unsigned int n = __reduce_add_sync(0xFFFFFFFFu, (unsigned int)ab.y);
+            if (tid < x.ncta) sh.cta_mass[tid] = ab.x;
+            const uint32_t kd = (draft >= 0) ? (uint32_t)sh.ex1[draft / slice].y : 0u;
+            bool draft_tie_in = false;
             __syncthreads();                                        // (land_n is reset by the broadcast)
             if (!masses) {
                 // what is missing inside the part, exactly
                 bc.need = goal > bc.W ? goal - bc.W : 0ull;
                 bool lost = bc.need == 0ull || nm == 0;             // the float bins named a neighbour of the right bin
-                if (!lost && nm > ROW_MEMBERS) {
-                    if (kmn == kmx) {
-                        const unsigned long long wv = max(1ull, row_q(row_w(unkey(kmn), x.Mf)));
-                        bc.again = RB_TIES; bc.lo = kmn;
-                        bc.need = (bc.need + wv - 1ull) / wv;
-                        if (bc.need > (unsigned long long)nm) bc.need = (unsigned long long)nm;
-                    } else { bc.again = RB_SPLIT; bc.lo = (unsigned long long)kmn << 32; bc.hi = ((unsigned long long)kmx << 32) | 0xFFFFFFFFull; }
+                if (!lost && kmn == kmx && !(kd == kmn && nm > ROW_MEMBERS)) {
+                    // the ties of one value (low-precision logits: nearly always): as many as are missing, by index
+                    const unsigned long long wv = max(1ull, row_q(row_w(unkey(kmn), x.Mf)));
+                    unsigned long long m = (unsigned long long)((double)bc.need / (double)wv);
+                    while (m * wv < bc.need) ++m;
+                    while (m > 1ull && (m - 1ull) * wv >= bc.need) --m;
+                    // (the sums of single weights and of bins round differently below 2^-44)
+                    lost = m > (unsigned long long)nm && !exact && (m - (unsigned long long)nm) * wv > 65536ull;
+                    m = min(m, (unsigned long long)nm);
+                    if (lost) {
+                    } else if ((uint32_t)(floorc >> 32) > kmn) { bc.again = RB_MASS; bc.cutc = floorc; }       // min-p decides
+                    else {
+                        const unsigned int pre = row_lane_scan<unsigned int>(members, lane) - members;
+                        const unsigned int in = (unsigned int)min((unsigned long long)members, m > pre ? m - pre : 0ull);
+                        const unsigned int at = __ballot_sync(0xFFFFFFFFu, members > 0u && pre < m && m <= (unsigned long long)pre + members);
+                        mass += in * wv;
+                        bc.W += m * wv;
+                        n += (unsigned int)m;
+                        bc.tie_cta = __ffs(at) - 1;
+                        bc.tie_in = __shfl_sync(0xFFFFFFFFu, in, bc.tie_cta);
+                        bc.cutc = (unsigned long long)kmn << 32;
+                        if (kd == kmn) draft_tie_in = __syncthreads_count(tid < nm && row_land()[tid] > row_comp(kd, draft)) < (int)m;
+                    }
+                } else if (!lost && nm > ROW_MEMBERS) {
+                    bc.again = RB_SPLIT; bc.lo = (unsigned long long)kmn << 32; bc.hi = ((unsigned long long)kmx << 32) | 0xFFFFFFFFull;
                 } else if (!lost) {
+                    // a short list: the mass ranked above every member, by counting (at most 64) or by sorting
+                    unsigned long long mc = 0ull, mq = 0ull, pre = 0ull, tot;
                     if (tid == 0) sh.warp2[0] = 0ull;
-                    unsigned long long mc, mq;
-                    row_rank(x, nm, mc, mq);
-                    unsigned long long tot;
-                    const unsigned long long pre = dense_block_scan<unsigned long long>(mq, sh.red64, tid, tot);
+                    if (nm <= 64) {
+                        if (tid < 64) {
+                            const unsigned long long c0 = (tid < nm) ? row_land()[tid] : 0ull;
+                            sh.list[tid] = c0;
+                            sh.list[64 + tid] = c0 ? row_q(row_w(unkey((uint32_t)(c0 >> 32)), x.Mf)) : 0ull;
+                        }
+                        __syncthreads();
+                        const int j = tid >> 3;                     // eight threads per member
+                        const unsigned long long c0 = sh.list[j], q0 = sh.list[64 + j];
+                        for (int u = tid & 7; u < nm; u += 8) pre += (sh.list[u] > c0) ? sh.list[64 + u] : 0ull;
+#pragma unroll
+                        for (int off = 1; off < 8; off <<= 1) pre += __shfl_xor_sync(0xFFFFFFFFu, pre, off);
+                        tot = row_warp_sum(sh.list[64 + lane] + sh.list[96 + lane]);
+                        if ((tid & 7) == 0) { mc = c0; mq = q0; }
+                    } else {
+                        row_rank(x, nm, mc, mq);
+                        pre = row_block_scan<unsigned long long>(mq, sh.red64, tid, tot);
+                    }
                     // (the sums of single weights and of bins round differently below 2^-44)
                     if (bc.need > tot && (exact || bc.need - tot <= 65536ull)) bc.need = max(tot, 1ull);
                     lost = bc.need > tot && tot > 0ull;
                     // the element at which the running mass first reaches what is missing
-                    if (mq > 0ull && pre < bc.need && bc.need <= pre + mq) sh.warp2[0] = mc;
+                    if (mq > 0ull && pre < bc.need && bc.need <= pre + mq) { sh.warp2[0] = mc; sh.warp2[1] = pre + mq; }
                     __syncthreads();
                     const unsigned long long cut_p = sh.warp2[0];
                     bc.cutc = max(floorc, cut_p);
@@ -1333,34 +1411,32 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
                         else {
                             const bool in = mc != 0ull && mc >= cut_p;
                             if (in && mq) smem_add_u64(&sh.cta_mass[(int)(~(uint32_t)mc) / slice], mq);
-                            const int n_in = __syncthreads_count(in ? 1 : 0);
-                            if (in && tid + 1 == n_in) sh.warp2[1] = pre + mq;
-                            __syncthreads();
-                            if (n_in) { bc.W += sh.warp2[1]; n += (unsigned long long)n_in; }
+                            n += (unsigned int)__syncthreads_count(in ? 1 : 0);
+                            bc.W += cut_p ? sh.warp2[1] : 0ull;
+                            mass = (lane < x.ncta) ? sh.cta_mass[lane] : 0ull;
                         }
                     }
                 }
-                if (lost) { bc.again = RB_SPLIT; bc.lo = 0ull; bc.hi = ~0ull; bc.need = goal; }
+                if (lost) { bc.again = RB_SPLIT; bc.lo = 0ull; bc.hi = ~0ull; bc.need = goal; bc.cutc = cutc; }
             }
             if (bc.again == RB_DONE) {
-                bc.support = (unsigned int)n;
+                bc.support = n;
                 if (P.op == OP_VERIFY && c.l < P.K) {
                     unsigned long long qd = 0ull;
                     if (draft >= 0) {
-                        const uint32_t kd = (uint32_t)sh.ex1[draft / slice].y;
-                        if (row_comp(kd, draft) >= bc.cutc) qd = row_q(row_w(unkey(kd), x.Mf));
+                        const bool in = (bc.tie_cta >= 0 && kd == (uint32_t)(bc.cutc >> 32)) ? draft_tie_in : row_comp(kd, draft) >= bc.cutc;
+                        if (in) qd = row_q(row_w(unkey(kd), x.Mf));
                     }
                     const double Pd = (double)qd / (double)bc.W;
                     bc.flags = ((Pd > 0.0) && (cell_to_u(cells.x) * (double)q_draft <= Pd)) ? RB_ACCEPT : RB_REJECT;
                     bc.p_draft = (float)Pd;
                 }
                 bc.rest = draw_target(bc.W, cells.y);
-                int owner = -1;
-                for (int r = 0; r < x.ncta; ++r) {
-                    const unsigned long long t = sh.cta_mass[r];
-                    if (owner < 0) { if (bc.rest < t) owner = r; else bc.rest -= t; }
-                }
-                bc.owner = (unsigned int)max(owner, 0);
+                const unsigned long long incl = row_lane_scan<unsigned long long>(mass, lane);
+                const unsigned int hit = __ballot_sync(0xFFFFFFFFu, incl > bc.rest);
+                const int owner = hit ? __ffs(hit) - 1 : 0;
+                bc.rest -= __shfl_sync(0xFFFFFFFFu, incl - mass, owner);
+                bc.owner = (unsigned int)owner;
             }
         }
         row_broadcast(x, bc);
@@ -1373,20 +1449,24 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
             row_gather_part(x, s);
             exact = true;
         } else {
-            cutc = again == RB_TIES ? max(floorc, row_ties(x, s, (uint32_t)sh.bc.lo, sh.bc.need)) : sh.bc.cutc;
+            cutc = sh.bc.cutc;
             row_mass_above(x, s.vmin, cutc);
             masses = true;
         }
         cl_sync();
     }
-    const RowBcast bc = sh.bc;
+    RowBcast bc = sh.bc;
+    if (LISTED) { KERNEL_T1(8); if (bc.flags & RB_REJECT) KERNEL_T0(4); }
     if (bc.flags & RB_ACCEPT) {                                     // the request moves on with the draft token
         if (lead) emit(P.draft_tokens[(size_t)c.b * P.K + c.l], 0.0f, cls_flag | F_ACCEPT, (int)bc.support, bc.p_draft);
         return;
     }
+    if (bc.tie_cta >= 0 && ((bc.flags & RB_REJECT) || x.rank == (int)bc.owner))
+        bc.cutc = max(floorc, row_tie_cut(x, s, (uint32_t)(bc.cutc >> 32), bc.tie_cta, bc.tie_in));
     if (bc.flags & RB_REJECT) {
         int token = -1;
         if (row_residual(x, P, c, bc.cutc, bc.W, cells.y, token)) {
+            if (LISTED) { KERNEL_T1(9); }
             if (token >= 0) emit(token, 0.0f, cls_flag, (int)bc.support, bc.p_draft);
             return;
         }
@@ -1400,6 +1480,70 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
         }, [&](int idx, unsigned long long q) {
             emit(idx, (bc.flags & RB_REJECT) ? 0.0f : (float)((double)q / (double)bc.W), cls_flag, (int)bc.support, bc.p_draft);
         });
+    }
+}
+
+// The ord-th row of the call that the streaming kernel leaves to the row kernel, -1 if there are fewer.  Two block barriers
+// per 512 requests.
+__device__ int row_pick(const KParams &P, int ord, int tid) {
+    RowShared &sh = row_sh();
+    const int per = (P.op == OP_VERIFY) ? P.K + 1 : 1, requests = P.rows / per;
+    int seen = 0;
+    for (int base = 0; base < requests; base += ROW_THREADS) {
+        const int b = base + tid;
+        bool mine = false;
+        if (b < requests) {
+            const uint32_t z = P.mode[b];
+            const int k = P.top_k ? P.top_k[b] : 0;
+            mine = class_is_listed(class_of(P, (z & M_GREEDY) != 0, (P.top_k && (z & M_TOP_K)) ? max(k, 0) : 0));
+        }
+        const unsigned int m = __ballot_sync(0xFFFFFFFFu, mine);
+        __syncthreads();
+        if ((tid & 31) == 0) sh.red32[tid >> 5] = m;
+        __syncthreads();
+        for (int w = 0; w < ROW_WARPS; ++w) {
+            const unsigned int v = sh.red32[w];
+            const int n = __popc(v) * per;
+            if (ord < seen + n) return (base + w * 32 + (int)__fns(v, 0, (ord - seen) / per + 1)) * per + (ord - seen) % per;
+            seen += n;
+        }
+    }
+    return -1;
+}
+
+// Grid: clusters.  Every row of the call (a cluster per row), or LISTED rows.  slice: elements per CTA (a multiple of
+// ROW_UNIT, slice * cluster >= V).
+template <int DT, bool LISTED>
+__global__ void __launch_bounds__(ROW_THREADS, 2)
+sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
+    RowCtx x;
+    x.rank = (int)cgr::this_cluster().block_rank();
+    x.ncta = (int)cgr::this_cluster().num_blocks();
+    x.slice = slice;
+    x.base = x.rank * slice;
+    x.tid = threadIdx.x; x.lane = x.tid & 31; x.warp = x.tid >> 5;
+    x.wn = slice / ROW_WARPS; x.wlo = x.warp * x.wn;
+    if (x.tid == 0) {
+        mbar_init(&row_sh().full, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    const int first = (int)blockIdx.x / x.ncta;
+    if (!LISTED) {
+        row_body<DT, false>(P, x, first, 0u);
+        return;
+    }
+    pdl_launch_dependents();                                        // (the streaming kernel runs beside this one)
+    const int clusters = (int)gridDim.x / x.ncta;
+    unsigned int parity = 0u;
+    for (int ord = first;; ord += clusters) {
+        const int row = row_pick(P, ord, x.tid);
+        if (row < 0) return;
+        __syncthreads();
+        if (x.tid == 0) fence_async_proxy();                        // (the last row's reads and writes precede this row's copy)
+        row_body<DT, true>(P, x, row, parity);
+        parity ^= 1u;
+        cl_sync();
+        if (row_late(x)) return;                                    // (a copy is missing: its barrier's phase never ends)
     }
 }
 

@@ -27,7 +27,6 @@
 // is handed to the exact kernel.
 #pragma once
 #include "sonic_common.cuh"
-#include "sonic_dense.cuh"
 
 namespace sonic {
 
@@ -1061,7 +1060,6 @@ struct StreamShared {
     alignas(16) float tw[NSTAGE][STREAM_WARPS];
     unsigned int ncand[NSTAGE];
     unsigned long long best[NSTAGE][STREAM_WARPS];
-    unsigned int kmin[NSTAGE][STREAM_WARPS], nfin[NSTAGE][STREAM_WARPS];     // dense rows
     // hit lists: one buffer more than stages, so that the producer fills the next tile's while both stages are busy
     Hit pen[NSTAGE + 1][HIT_PEN_CAP];
     Hit bias[NSTAGE + 1][HIT_BIAS_CAP];
@@ -1103,7 +1101,6 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         static_assert(SONIC_MAX_VOCAB <= (1 << 18), "packed history entries hold an 18-bit id");
         constexpr int HPL = FILTER_HIST / 32;      // packed history entries per lane
         struct Prep { int patch, npen, nbias; };
-        int memo_k = -1, memo_G = -1;
         RowCfg c_next;
         uint32_t packed[HPL];                      // id | count << 18; 0 = no entry
         int b_id = -1;
@@ -1128,7 +1125,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             }
             int b0 = -1; float v0 = 0.0f;
             if (bid && bvl && lane < P.bias_stride) { b0 = __ldg(bid + lane); v0 = __ldg(bvl + lane); }
-            c_next = resolve_cfg(P, row, raw, &memo_k, &memo_G);
+            c_next = resolve_cfg(P, row, raw);
             cached_row = row;
             row_patch = 0;
             row_bad = 0;
@@ -1165,8 +1162,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             if (__any_sync(0xFFFFFFFFu, big)) return;          // a count too large to pack: consumers scan
             row_patch = 1;
         };
-        auto prepare = [&](int row, int tile, int hb) -> Prep {
-            if (row != cached_row) load_row(row);
+        auto prepare = [&](int tile, int hb) -> Prep {
             Prep r{row_patch, 0, 0};
             if (row_patch != 1) return r;
             const int first = tile * CTA_TILE;
@@ -1214,10 +1210,21 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 if (lane == 0 && run_lo < nitems) nxt_raw = (int)atomicAdd(queue, 1u);
             }
         };
-        int n = 0;
+        // Rows that the row kernel takes (sampling calls) are passed over, a whole row at a time; on return the row's
+        // parameters and lists are loaded (pass == false: of the current item, whatever its row is).
+        auto find_item = [&](bool pass) -> int {
+            for (;;) {
+                const int it = current_item();
+                if (it < 0) return -1;
+                const int row = it / tiles;
+                if (row != cached_row) load_row(row);
+                if (!pass || P.op == OP_TOPK || !class_is_listed(c_next.cls)) return it;
+                run_lo = min(run_hi, (row + 1) * tiles) - 1;
+                advance();
+            }
+        };
         Prep p_next{0, 0, 0};
         int item = current_item();
-        bool prepared = false;
         // lane 0: the tile's bulk copy, with the arrival on full[s] (arrive == true) or with the bytes announced only
         // (the arrival then follows once the stage's description is written)
         auto issue_copy = [&](int row, int tile, int s, bool arrive) {
@@ -1238,45 +1245,41 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         // rounds of global loads): the copy's latency hides behind them.  (A row of the cluster kernel's class gets
         // a copy nobody reads: such rows are rare.)
         if (item >= 0 && lane == 0) issue_copy(item / tiles, item % tiles, 0, false);
-        for (;; ++n) {
-            const int s = n % NSTAGE;
-            if (n >= NSTAGE) {
-                // the consumers have left tile n - NSTAGE: its stage and its hit buffer are free
-                if (!mbar_wait(&sh.empty[s], ((n / NSTAGE) - 1) & 1)) {
-                    if (lane == 0) atomicOr(P.error, ERR_TIMEOUT);
-                    return;
+        for (int n = -1;; ++n) {                       // (round -1 only prepares the first tile)
+            if (n >= 0) {
+                const int s = n % NSTAGE;
+                if (n >= NSTAGE) {
+                    // the consumers have left tile n - NSTAGE: its stage and its hit buffer are free
+                    if (!mbar_wait(&sh.empty[s], ((n / NSTAGE) - 1) & 1)) {
+                        if (lane == 0) atomicOr(P.error, ERR_TIMEOUT);
+                        return;
+                    }
                 }
+                if (item < 0) {                            // out of work: tell the consumers
+                    if (lane == 0) { sh.meta[s].stop = 1; mbar_arrive(&sh.full[s]); }
+                    break;
+                }
+                const int row = item / tiles, tile = item - row * tiles;
+                advance();
+                const int hint = current_item();           // (the tile that follows, unless its row is passed over)
+                __syncwarp();                              // the hit buffer's entries, written by all lanes, precede the arrival
+                if (lane == 0) {
+                    StageMeta &m = sh.meta[s];
+                    m.cfg = c_next; m.row = row; m.tile = tile; m.skip = class_is_listed(c_next.cls) ? 1 : 0;
+                    m.patch = p_next.patch; m.npen = p_next.npen; m.nbias = p_next.nbias; m.hb = n % (NSTAGE + 1);
+                    m.stop = 0;
+                    m.bad = row_bad;
+                    m.next_row = (hint >= 0) ? hint / tiles : -1;
+                    m.next_tile = (hint >= 0) ? hint % tiles : -1;
+                    // the first tile's copy is under way; nothing is copied for rows of the cluster kernel's class
+                    if (n == 0 || m.skip) mbar_arrive(&sh.full[s]);
+                    else issue_copy(row, tile, s, true);
+                }
+                __syncwarp();
             }
-            if (item < 0) {                            // out of work: tell the consumers
-                if (lane == 0) { sh.meta[s].stop = 1; mbar_arrive(&sh.full[s]); }
-                break;
-            }
-            const int row = item / tiles, tile = item - row * tiles;
-            if (!prepared) {                           // the CTA's first tile: nothing was prepared ahead
-                p_next = prepare(row, tile, n % (NSTAGE + 1));
-                prepared = true;
-            }
-            const RowCfg c = c_next;
-            const Prep pr = p_next;
-            const int bad_now = row_bad;
-            advance();
-            const int nxt = current_item();
-            __syncwarp();                              // the hit buffer's entries, written by all lanes, precede the arrival
-            if (lane == 0) {
-                StageMeta &m = sh.meta[s];
-                m.cfg = c; m.row = row; m.tile = tile; m.skip = (c.cls == CLS_EXACT) ? 1 : 0;
-                m.patch = pr.patch; m.npen = pr.npen; m.nbias = pr.nbias; m.hb = n % (NSTAGE + 1);
-                m.stop = 0;
-                m.bad = bad_now;
-                m.next_row = (nxt >= 0) ? nxt / tiles : -1;
-                m.next_tile = (nxt >= 0) ? nxt % tiles : -1;
-                if (n == 0 || c.cls == CLS_EXACT) mbar_arrive(&sh.full[s]);     // (the first tile's copy is under way; nothing is copied for rows of the cluster kernel's class)
-                else issue_copy(row, tile, s, true);
-            }
-            __syncwarp();
             // hit buffer (n + 1) % (NSTAGE + 1) was last used by tile n - NSTAGE, which the consumers have left
-            if (nxt >= 0) p_next = prepare(nxt / tiles, nxt % tiles, (n + 1) % (NSTAGE + 1));
-            item = nxt;
+            item = find_item(n >= 0);
+            if (item >= 0) p_next = prepare(item % tiles, (n + 1) % (NSTAGE + 1));
         }
         return;
     }
@@ -1308,28 +1311,17 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         }
         const StageMeta &meta = sh.meta[s];
         if (meta.skip) {
-            // a row of the cluster kernel: counted, its status word initialised
-            if (tile == 0 && tid == 0) { P.rs[row].status = 0u; atomicAdd(&P.error[WS_NEXACT], 1u); }
+            // a row of the cluster kernel (sonic_topk): counted, its status word initialised
+            if (tile == 0 && tid == 0 && P.op == OP_TOPK) { P.rs[row].status = 0u; atomicAdd(&P.error[WS_NEXACT], 1u); }
         } else {
             const RowCfg c = meta.cfg;
             RowState *rs = P.rs + row;
             TileRec *rec = P.tiles + (size_t)row * MAX_TILES + tile;
             // Every per-row word of the workspace is initialised by the call that reads it: the tile's flags here
-            // (before any barrier of this tile), the row's status word and, for rows of the histogram path, the
-            // row's control block and its histogram by the CTA of the row's first tile.
+            // (before any barrier of this tile), the row's status word by the CTA of the row's first tile.
             if (tid == 0) {
                 rec->flags = meta.bad ? TILE_BADID : 0u;
                 if (tile == 0) rs->status = 0u;
-            }
-            if (c.cls == CLS_DENSE && tile == 0) {
-                uint4 *h = reinterpret_cast<uint4 *>(P.hist + (size_t)row * DBINS);
-                for (int i = tid; i < DBINS / 2; i += STREAM_THREADS) h[i] = make_uint4(0u, 0u, 0u, 0u);
-                if (tid == 0) {
-                    DenseRow *dr = P.drow + row;
-                    dr->ticket_h = 0u; dr->ticket_c = 0u; dr->ticket_r = 0u; dr->nmembers = 0u;
-                    dr->kmin = 0xFFFFFFFFu; dr->kmax = 0u; dr->overflow = 0u; dr->state = 0u;
-                    P.dlist[atomicAdd(&P.error[WS_NDENSE], 1u)] = row;
-                }
             }
             unsigned char *stage = stages + (size_t)s * STAGE_BYTES;
             const bool masked = (c.z & M_GRAMMAR) != 0;
@@ -1459,32 +1451,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             const float h0 = fmaxf(qm[0], qm[1]), h1 = fmaxf(qm[2], qm[3]);
             const float lm = fmaxf(h0, h1);
 
-            if (c.cls == CLS_GREEDY || c.cls == CLS_DENSE) {
-                if (c.cls == CLS_DENSE) {
-                    // histogram path: the processed logits (already divided by the temperature) are kept as ordered
-                    // keys for the later passes; per tile the smallest finite key and the number of finite elements
-                    uint32_t kmn = 0xFFFFFFFFu;
-                    unsigned int nf = 0u;
-                    unsigned int *yk = P.ykeys + (size_t)row * ((size_t)P.ytiles * CTA_TILE) + tile_base + warp * WARP_TILE;
-#pragma unroll
-                    for (int j = 0; j < NV; ++j) {
-#pragma unroll
-                        for (int q4 = 0; q4 < VEC; q4 += 4) {
-                            uint32_t kk[4];
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                kk[u] = okey(e[j * VEC + q4 + u]);
-                                const bool fin = kk[u] > KEY_NEG_INF;
-                                nf += fin ? 1u : 0u;
-                                kmn = fin ? min(kmn, kk[u]) : kmn;
-                            }
-                            *reinterpret_cast<uint4 *>(yk + j * 32 * VEC + lane * VEC + q4) = make_uint4(kk[0], kk[1], kk[2], kk[3]);
-                        }
-                    }
-                    kmn = __reduce_min_sync(0xFFFFFFFFu, kmn);
-                    nf = __reduce_add_sync(0xFFFFFFFFu, nf);
-                    if (lane == 0) { sh.kmin[s][warp] = kmn; sh.nfin[s][warp] = nf; }
-                }
+            if (c.cls == CLS_GREEDY) {
                 float wm = lm;
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xFFFFFFFFu, wm, off));
@@ -1515,12 +1482,6 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
 #pragma unroll
                     for (int w = 1; w < STREAM_WARPS; ++w) b = max(b, sh.best[s][w]);
                     rec->best = b;
-                    if (c.cls == CLS_DENSE) {
-                        unsigned int kmn = sh.kmin[s][0], nf = sh.nfin[s][0];
-#pragma unroll
-                        for (int w = 1; w < STREAM_WARPS; ++w) { kmn = min(kmn, sh.kmin[s][w]); nf += sh.nfin[s][w]; }
-                        rec->minkey = kmn; rec->nfin = nf;
-                    }
                 }
             } else {
                 // warp cutoff: minimum over G groups of the group maximum.  Tile cutoff: the largest of the eight
@@ -1640,10 +1601,6 @@ sonic_merge_kernel(const KParams P, const int tiles) {
     uint2 cells = make_uint2(0u, 0u);
     if (P.op != OP_TOPK && c.cls == CLS_TOPK) draw_cells(P, c, cells.x, cells.y);
     pdl_wait_primary();                        // tile records and candidates of the streaming kernel
-    // The next kernel of the call (stage 2 of the histogram path) does not wait for this grid: it needs the
-    // streaming kernel's results only, and those are complete once every CTA here is past its wait (the first
-    // row's CTA never leaves before it).  So it is let go after the wait, and runs beside the merges.
-    pdl_launch_dependents();
     if (row == 0 && tid == 0) P.error[WS_QUEUE] = 0u;    // the streaming kernel is done with its work counter
     if (other) return;
     if (__ldcg(&P.error[WS_ERROR]) & ERR_TIMEOUT) {
