@@ -84,13 +84,6 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, unsigned i
 }
 __device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// Element index of register slot s of a lane.
-template <int DT>
-__device__ __forceinline__ int slot_index(int wbase, int lane, int s) {
-    constexpr int VEC = VecTraits<DT>::VEC;
-    return wbase + (s / VEC) * 32 * VEC + lane * VEC + (s % VEC);
-}
-
 template <int THREADS>
 struct MergeShared {
     int count;
@@ -1056,10 +1049,11 @@ struct StreamShared {
     unsigned long long full[NSTAGE];           // producer -> consumers: stage described and copy issued (one arrival + the copy's bytes)
     unsigned long long empty[NSTAGE];          // consumers -> producer: stage free (one arrival per consumer warp)
     StageMeta meta[NSTAGE];
-    // per-stage scratch of the consumer warps (a fast warp may already be on the next tile, in the other stage)
+    // per-stage results of the consumer warps, which the producer turns into the tile's record once all of them are done
     alignas(16) float tw[NSTAGE][STREAM_WARPS];
-    unsigned int ncand[NSTAGE];
+    unsigned int ncand[NSTAGE], tkey[NSTAGE], badid[NSTAGE];
     unsigned long long best[NSTAGE][STREAM_WARPS];
+    uint32_t list[FILTER_HIST];                // the producer's: the row's history, id | count << 18 (0: no entry)
     // hit lists: one buffer more than stages, so that the producer fills the next tile's while both stages are busy
     Hit pen[NSTAGE + 1][HIT_PEN_CAP];
     Hit bias[NSTAGE + 1][HIT_BIAS_CAP];
@@ -1099,10 +1093,9 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         // entries that fall into it and writing them to a hit buffer, so that the consumers patch only what is
         // there, each warp only its own part of the tile.
         static_assert(SONIC_MAX_VOCAB <= (1 << 18), "packed history entries hold an 18-bit id");
-        constexpr int HPL = FILTER_HIST / 32;      // packed history entries per lane
+        constexpr int HALF = FILTER_HIST / 64;     // history entries per lane and round of loads
         struct Prep { int patch, npen, nbias; };
         RowCfg c_next;
-        uint32_t packed[HPL];                      // id | count << 18; 0 = no entry
         int b_id = -1;
         float b_val = 0.0f;
         int row_patch = 0, cached_row = -1, row_bad = 0;
@@ -1114,7 +1107,6 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             const float *bvl = P.bias_vals ? P.bias_vals + (size_t)req * P.bias_stride : nullptr;
             // the first round of loads goes out before the first use (the lengths arrive with the parameters:
             // bound by the strides); the second half of a long history follows in a round of its own
-            constexpr int HALF = HPL / 2;
             const CfgRaw raw = fetch_cfg(P, row);
             int id[HALF], ct[HALF];
 #pragma unroll
@@ -1140,9 +1132,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 return (cnt > 0) ? ((uint32_t)i | ((uint32_t)cnt << 18)) : 0u;
             };
 #pragma unroll
-            for (int u = 0; u < HALF; ++u) packed[u] = pack(lane + 32 * u, id[u], ct[u]);
-#pragma unroll
-            for (int u = 0; u < HALF; ++u) packed[HALF + u] = 0u;
+            for (int u = 0; u < HALF; ++u) sh.list[lane + 32 * u] = pack(lane + 32 * u, id[u], ct[u]);
             if (c_next.hist_len > 32 * HALF) {
 #pragma unroll
                 for (int u = 0; u < HALF; ++u) {
@@ -1151,7 +1141,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                     if (t < c_next.hist_len) { id[u] = __ldg(hid + t); ct[u] = __ldg(hct + t); }
                 }
 #pragma unroll
-                for (int u = 0; u < HALF; ++u) packed[HALF + u] = pack(lane + 32 * (HALF + u), id[u], ct[u]);
+                for (int u = 0; u < HALF; ++u) sh.list[lane + 32 * (HALF + u)] = pack(lane + 32 * (HALF + u), id[u], ct[u]);
             }
             b_id = -1; b_val = 0.0f;
             if (lane < c_next.bias_len) {
@@ -1166,14 +1156,15 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             Prep r{row_patch, 0, 0};
             if (row_patch != 1) return r;
             const int first = tile * CTA_TILE;
-#pragma unroll
-            for (int u = 0; u < HPL; ++u) {
-                const unsigned int li = (packed[u] & 0x3FFFFu) - (unsigned int)first;
-                const bool hit = packed[u] != 0u && li < (unsigned int)CTA_TILE;
+#pragma unroll 4
+            for (int t = lane; t < ((c_next.hist_len + 31) & ~31); t += 32) {      // (a lane reads the entries it wrote)
+                const uint32_t e = sh.list[t];
+                const unsigned int li = (e & 0x3FFFFu) - (unsigned int)first;
+                const bool hit = e != 0u && li < (unsigned int)CTA_TILE;
                 const unsigned int hm = __ballot_sync(0xFFFFFFFFu, hit);
                 if (hit) {
                     const int pos = r.npen + __popc(hm & ((1u << lane) - 1u));
-                    if (pos < HIT_PEN_CAP) { sh.pen[hb][pos].li = (int)li; sh.pen[hb][pos].payload = (int)(packed[u] >> 18); }
+                    if (pos < HIT_PEN_CAP) { sh.pen[hb][pos].li = (int)li; sh.pen[hb][pos].payload = (int)(e >> 18); }
                 }
                 r.npen += __popc(hm);
             }
@@ -1245,7 +1236,29 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         // rounds of global loads): the copy's latency hides behind them.  (A row of the cluster kernel's class gets
         // a copy nobody reads: such rows are rare.)
         if (item >= 0 && lane == 0) issue_copy(item / tiles, item % tiles, 0, false);
-        for (int n = -1;; ++n) {                       // (round -1 only prepares the first tile)
+        // The record of a tile that every consumer warp has left: candidates, cutoff, argmax, bad list ids.
+        auto retire = [&](int s) {
+            const int row = sh.meta[s].row, tile = sh.meta[s].tile;
+            if (sh.meta[s].skip) {
+                // a row of the cluster kernel (sonic_topk): counted, its status word initialised
+                if (tile == 0 && lane == 0 && P.op == OP_TOPK) { P.rs[row].status = 0u; atomicAdd(&P.error[WS_NEXACT], 1u); }
+                return;
+            }
+            unsigned long long b = (lane < STREAM_WARPS) ? sh.best[s][lane] : 0ull;
+#pragma unroll
+            for (int off = STREAM_WARPS / 2; off > 0; off >>= 1) b = max(b, __shfl_xor_sync(0xFFFFFFFFu, b, off));
+            if (lane == 0) {
+                TileRec r;
+                r.best = b; r.cnt = sh.ncand[s]; r.tkey = sh.tkey[s];
+                r.flags = (sh.meta[s].bad || sh.badid[s]) ? TILE_BADID : 0u;
+                r.pad[0] = r.pad[1] = r.pad[2] = 0u;
+                P.tiles[(size_t)row * MAX_TILES + tile] = r;
+                if (tile == 0) P.rs[row].status = 0u;
+            }
+            __syncwarp();
+        };
+        int n = -1;
+        for (;; ++n) {                                 // (round -1 only prepares the first tile)
             if (n >= 0) {
                 const int s = n % NSTAGE;
                 if (n >= NSTAGE) {
@@ -1254,6 +1267,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                         if (lane == 0) atomicOr(P.error, ERR_TIMEOUT);
                         return;
                     }
+                    retire(s);
                 }
                 if (item < 0) {                            // out of work: tell the consumers
                     if (lane == 0) { sh.meta[s].stop = 1; mbar_arrive(&sh.full[s]); }
@@ -1269,6 +1283,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                     m.patch = p_next.patch; m.npen = p_next.npen; m.nbias = p_next.nbias; m.hb = n % (NSTAGE + 1);
                     m.stop = 0;
                     m.bad = row_bad;
+                    sh.ncand[s] = 0u; sh.tkey[s] = 0u; sh.badid[s] = 0u;
                     m.next_row = (hint >= 0) ? hint / tiles : -1;
                     m.next_tile = (hint >= 0) ? hint % tiles : -1;
                     // the first tile's copy is under way; nothing is copied for rows of the cluster kernel's class
@@ -1280,6 +1295,13 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             // hit buffer (n + 1) % (NSTAGE + 1) was last used by tile n - NSTAGE, which the consumers have left
             item = find_item(n >= 0);
             if (item >= 0) p_next = prepare(item % tiles, (n + 1) % (NSTAGE + 1));
+        }
+        for (int i = max(0, n - NSTAGE + 1); i < n; ++i) {     // the last tiles
+            if (!mbar_wait(&sh.empty[i % NSTAGE], (i / NSTAGE) & 1)) {
+                if (lane == 0) atomicOr(P.error, ERR_TIMEOUT);
+                return;
+            }
+            retire(i % NSTAGE);
         }
         return;
     }
@@ -1293,97 +1315,73 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         const int w = ((tile * CTA_TILE + warp * WARP_TILE) >> 5) + lane;
         return (w < ((P.V + 31) >> 5)) ? __ldg(P.bitmask + (size_t)row * P.bitmask_stride + w) : 0u;
     };
+    // What a warp carries from tile to tile of a row.  Top-k rows: the cutoff, taken from the CTA's first tile of the row
+    // and kept for the tiles that follow (any cutoff is good as long as the tile's record names it; a tile then costs its
+    // maxima and one vote, without a block barrier).  Greedy rows: what an element must reach to matter.
+    int cut_row = -1, g_row = -1;
+    float cut = 0.0f, g_thr = 0.0f;
     for (int n = 0;; ++n) {
         const int s = n % NSTAGE;
         if (!mbar_wait(&sh.full[s], (n / NSTAGE) & 1)) {
             if (lane == 0) atomicOr(P.error, ERR_TIMEOUT);
             return;
         }
-        if (sh.meta[s].stop) { KERNEL_T1(0); break; }
-        const int row = sh.meta[s].row, tile = sh.meta[s].tile;
+        const StageMeta &meta = sh.meta[s];
+        if (meta.stop) { KERNEL_T1(0); break; }
+        const int row = meta.row, tile = meta.tile;
         const int tile_base = tile * CTA_TILE;
         const int wbase = tile_base + warp * WARP_TILE;
         uint32_t mword = 0xFFFFFFFFu;
         if (P.bitmask) {
             mword = (row == pre_row && tile == pre_tile) ? mword_pre : load_mask_words(row, tile);
-            pre_row = sh.meta[s].next_row; pre_tile = sh.meta[s].next_tile;
+            pre_row = meta.next_row; pre_tile = meta.next_tile;
             if (pre_row >= 0) mword_pre = load_mask_words(pre_row, pre_tile);
         }
-        const StageMeta &meta = sh.meta[s];
-        if (meta.skip) {
-            // a row of the cluster kernel (sonic_topk): counted, its status word initialised
-            if (tile == 0 && tid == 0 && P.op == OP_TOPK) { P.rs[row].status = 0u; atomicAdd(&P.error[WS_NEXACT], 1u); }
-        } else {
-            const RowCfg c = meta.cfg;
-            RowState *rs = P.rs + row;
-            TileRec *rec = P.tiles + (size_t)row * MAX_TILES + tile;
-            // Every per-row word of the workspace is initialised by the call that reads it: the tile's flags here
-            // (before any barrier of this tile), the row's status word by the CTA of the row's first tile.
-            if (tid == 0) {
-                rec->flags = meta.bad ? TILE_BADID : 0u;
-                if (tile == 0) rs->status = 0u;
-            }
-            unsigned char *stage = stages + (size_t)s * STAGE_BYTES;
-            const bool masked = (c.z & M_GRAMMAR) != 0;
+        if (!meta.skip) {
+            const unsigned char *stage = stages + (size_t)s * STAGE_BYTES;
+            const bool masked = (meta.cfg.z & M_GRAMMAR) != 0;
             const bool tail = tile_base + CTA_TILE > P.V;
             const int patch = meta.patch;
-            const bool patched = patch != 0;
-            float *ptile = (DT == 0) ? reinterpret_cast<float *>(stage) : conv;    // fp32 view the sparse lists patch
-
-            float e[EPL];
-            auto read_raw = [&]() {
+            float *ptile = (DT == 0) ? reinterpret_cast<float *>(stages + (size_t)s * STAGE_BYTES) : conv;    // fp32 view the sparse lists patch
+            bool wide = DT == 0;                               // the warp's part is fp32 in ptile (else bf16 in the stage)
+            const int lane0 = warp * WARP_TILE + lane * VEC;   // the lane's first element within the tile
+            auto widen = [&]() {                               // bf16 only: the warp's part as fp32
 #pragma unroll
                 for (int j = 0; j < NV; ++j) {
-                    const int li = warp * WARP_TILE + j * 32 * VEC + lane * VEC;
-                    const uint4 raw = *reinterpret_cast<const uint4 *>(stage + (size_t)li * ELT);
-                    const uint32_t r[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-                    for (int q = 0; q < VEC; ++q) {
-                        if (DT == 0) e[j * VEC + q] = __uint_as_float(r[q]);
-                        else e[j * VEC + q] = __uint_as_float((q & 1) ? (r[q >> 1] & 0xFFFF0000u) : (r[q >> 1] << 16));
-                    }
+                    const uint4 raw = *reinterpret_cast<const uint4 *>(stage + (size_t)(lane0 + j * 32 * VEC) * ELT);
+                    float *p = conv + lane0 + j * 32 * VEC;
+                    *reinterpret_cast<float4 *>(p) = make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xFFFF0000u),
+                                                                 __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xFFFF0000u));
+                    *reinterpret_cast<float4 *>(p + 4) = make_float4(__uint_as_float(raw.z << 16), __uint_as_float(raw.z & 0xFFFF0000u),
+                                                                     __uint_as_float(raw.w << 16), __uint_as_float(raw.w & 0xFFFF0000u));
                 }
             };
-            auto read_f32 = [&](const float *src) {
-#pragma unroll
-                for (int j = 0; j < NV; ++j) {
-                    const float *p = src + warp * WARP_TILE + j * 32 * VEC + lane * VEC;
-#pragma unroll
-                    for (int q = 0; q < VEC; q += 4) {
-                        const float4 v = *reinterpret_cast<const float4 *>(p + q);
-                        e[j * VEC + q] = v.x; e[j * VEC + q + 1] = v.y; e[j * VEC + q + 2] = v.z; e[j * VEC + q + 3] = v.w;
-                    }
-                }
-            };
-            auto widen = [&]() {                      // bf16 only: the warp's part of the tile as fp32 in shared memory
-#pragma unroll
-                for (int j = 0; j < NV; ++j) {
-                    float *p = conv + warp * WARP_TILE + j * 32 * VEC + lane * VEC;
-#pragma unroll
-                    for (int q = 0; q < VEC; q += 4)
-                        *reinterpret_cast<float4 *>(p + q) = make_float4(e[j * VEC + q], e[j * VEC + q + 1], e[j * VEC + q + 2], e[j * VEC + q + 3]);
-                }
-            };
-            // penalties and biases commute with the mask (a masked logit stays -inf), so they are applied to
-            // the unmasked tile and the mask is applied when the lanes read their elements
+            // penalties and biases commute with the mask (a masked logit stays -inf), so they are applied to the unmasked tile
             if (patch == 1) {
-                // the producer listed this tile's entries: every warp patches its own part, no block-wide barrier
-                if (DT == 1) { read_raw(); widen(); }
-                __syncwarp();
-                for (int h = lane; h < meta.npen; h += 32) {
-                    const Hit x = sh.pen[meta.hb][h];
-                    if (x.li / WARP_TILE == warp) ptile[x.li] = apply_penalties(ptile[x.li], x.payload, c);
+                // the producer listed this tile's entries: every warp patches its own part, if there are any in it
+                const int npen = meta.npen, nbias = meta.nbias;
+                bool any = false;
+                for (int h = lane; h < npen; h += 32) any = any || (sh.pen[meta.hb][h].li / WARP_TILE == warp);
+                for (int h = lane; h < nbias; h += 32) any = any || (sh.bias[meta.hb][h].li / WARP_TILE == warp);
+                if (__any_sync(0xFFFFFFFFu, any)) {
+                    const RowCfg c = meta.cfg;
+                    if (DT == 1) { widen(); wide = true; }
+                    __syncwarp();
+                    for (int h = lane; h < npen; h += 32) {
+                        const Hit x = sh.pen[meta.hb][h];
+                        if (x.li / WARP_TILE == warp) ptile[x.li] = apply_penalties(ptile[x.li], x.payload, c);
+                    }
+                    __syncwarp();
+                    for (int h = lane; h < nbias; h += 32) {
+                        const Hit x = sh.bias[meta.hb][h];
+                        if (x.li / WARP_TILE == warp) ptile[x.li] = __fadd_rn(ptile[x.li], __int_as_float(x.payload));
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
-                for (int h = lane; h < meta.nbias; h += 32) {
-                    const Hit x = sh.bias[meta.hb][h];
-                    if (x.li / WARP_TILE == warp) ptile[x.li] = __fadd_rn(ptile[x.li], __int_as_float(x.payload));
-                }
-                __syncwarp();
-                read_f32(ptile);
             } else if (patch == 2) {
                 // long or crowded lists: all consumer threads scan them together
-                if (DT == 1) { read_raw(); widen(); csync(); }
+                const RowCfg c = meta.cfg;
+                if (DT == 1) { widen(); wide = true; csync(); }
                 const int req = (P.op == OP_VERIFY) ? row / (P.K + 1) : row;
                 const int *hid = P.hist_ids + (size_t)req * P.hist_stride;
                 const int *hct = P.hist_counts + (size_t)req * P.hist_stride;
@@ -1401,182 +1399,172 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                     const int li = id - tile_base;
                     if (li >= 0 && li < CTA_TILE) ptile[li] = __fadd_rn(ptile[li], __ldg(P.bias_vals + (size_t)req * P.bias_stride + t));
                 }
-                if (bad) atomicOr(&rec->flags, TILE_BADID);          // (ordered after the first thread's store by the barriers above)
+                if (bad) sh.badid[s] = 1u;
                 csync();
-                read_f32(ptile);
-            } else {
-                read_raw();
-            }
-            if (masked && !tail) {
-                // the common masked case: one select per element, no bounds test
-#pragma unroll
-                for (int j = 0; j < NV; ++j) {
-                    const uint32_t bits = __shfl_sync(0xFFFFFFFFu, mword, (j * 32 * VEC + lane * VEC) >> 5) >> ((lane * VEC) & 31);
-#pragma unroll
-                    for (int q = 0; q < VEC; ++q) e[j * VEC + q] = (bits & (1u << q)) ? e[j * VEC + q] : -CUDART_INF_F;
-                }
-            } else if (tail) {
-#pragma unroll
-                for (int j = 0; j < NV; ++j) {
-                    const int first = wbase + j * 32 * VEC + lane * VEC;
-                    const uint32_t bits = __shfl_sync(0xFFFFFFFFu, mword, (j * 32 * VEC + lane * VEC) >> 5) >> (first & 31);
-#pragma unroll
-                    for (int q = 0; q < VEC; ++q) {
-                        const bool dead = (first + q >= P.V) || (masked && !((bits >> q) & 1u));
-                        if (dead) e[j * VEC + q] = -CUDART_INF_F;
-                    }
-                }
-            }
-            if (c.div_all) {
-#pragma unroll
-                for (int q = 0; q < EPL; ++q) e[q] = div_tau(e[q], c.tau);
             }
 
-            // per-vector maxima, half maxima, lane maximum
+            // Maxima of the lane's vectors.  ebits: which of its 32 elements count (allowed by the mask, inside the row).
             float mv[NV];
+            uint32_t ebits = 0xFFFFFFFFu;
+            if (!masked && !tail) {
 #pragma unroll
-            for (int j = 0; j < NV; ++j) {
-                float m = e[j * VEC];
-#pragma unroll
-                for (int q = 1; q < VEC; ++q) m = fmaxf(m, e[j * VEC + q]);
-                mv[j] = m;
-            }
-            float qm[4];                               // maxima of the lane's four quarters (8 elements each)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                qm[i] = mv[i * (NV / 4)];
-#pragma unroll
-                for (int j = 1; j < NV / 4; ++j) qm[i] = fmaxf(qm[i], mv[i * (NV / 4) + j]);
-            }
-            const float h0 = fmaxf(qm[0], qm[1]), h1 = fmaxf(qm[2], qm[3]);
-            const float lm = fmaxf(h0, h1);
-
-            if (c.cls == CLS_GREEDY) {
-                float wm = lm;
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xFFFFFFFFu, wm, off));
-                unsigned long long key = 0ull;
-                if (wm > -CUDART_INF_F) {
-                    int best = 0x7FFFFFFF;
-                    if (lm == wm) {
-                        // slots ascend: the last write is the lowest; only the first quarter that holds the maximum is searched
-                        bool found = false;
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            if (!found && qm[i] == wm) {
-                                found = true;
-#pragma unroll
-                                for (int q = (i + 1) * (EPL / 4) - 1; q >= i * (EPL / 4); --q)
-                                    if (e[q] == wm) best = slot_index<DT>(wbase, lane, q);
-                            }
+                for (int j = 0; j < NV; ++j) {
+                    const int li = lane0 + j * 32 * VEC;
+                    if (DT == 1 && !wide) {
+                        // bf16 pairs: half an instruction per element
+                        const uint4 raw = *reinterpret_cast<const uint4 *>(stage + (size_t)li * ELT);
+                        const __nv_bfloat162 m = __hmax2(__hmax2(*reinterpret_cast<const __nv_bfloat162 *>(&raw.x), *reinterpret_cast<const __nv_bfloat162 *>(&raw.y)),
+                                                         __hmax2(*reinterpret_cast<const __nv_bfloat162 *>(&raw.z), *reinterpret_cast<const __nv_bfloat162 *>(&raw.w)));
+                        const uint32_t u = *reinterpret_cast<const uint32_t *>(&m);
+                        mv[j] = fmaxf(__uint_as_float(u << 16), __uint_as_float(u & 0xFFFF0000u));
+                    } else {
+                        const float4 a = *reinterpret_cast<const float4 *>(ptile + li);
+                        mv[j] = fmaxf(fmaxf(a.x, a.y), fmaxf(a.z, a.w));
+                        if (VEC == 8) {
+                            const float4 b = *reinterpret_cast<const float4 *>(ptile + li + 4);
+                            mv[j] = fmaxf(mv[j], fmaxf(fmaxf(b.x, b.y), fmaxf(b.z, b.w)));
                         }
                     }
-#pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) best = min(best, __shfl_xor_sync(0xFFFFFFFFu, best, off));
-                    key = ((unsigned long long)okey(wm) << 32) | (uint32_t)(~(uint32_t)best);
-                }
-                if (lane == 0) sh.best[s][warp] = key;
-                csync();
-                if (tid == 0) {
-                    unsigned long long b = sh.best[s][0];
-#pragma unroll
-                    for (int w = 1; w < STREAM_WARPS; ++w) b = max(b, sh.best[s][w]);
-                    rec->best = b;
                 }
             } else {
-                // warp cutoff: minimum over G groups of the group maximum.  Tile cutoff: the largest of the eight
-                // warp cutoffs (warp mode) or the smallest (tile mode: a minimum over all 8 G groups of the tile).
-                // In tile mode a group without a finite element (masked, or past the row's end) does not take
-                // part: it would drag the cutoff to -inf and the tile would emit everything it has.
-                float g;
-                const int G = c.G;
-                const bool tmin = c.tile_min;
-                switch (G) {                                   // (one straight-line butterfly per group count)
-                case 0: g = -CUDART_INF_F; break;
-                case 1: g = warp_cutoff<32>(lm, tmin); break;
-                case 2: g = warp_cutoff<16>(lm, tmin); break;
-                case 4: g = warp_cutoff<8>(lm, tmin); break;
-                case 8: g = warp_cutoff<4>(lm, tmin); break;
-                case 16: g = warp_cutoff<2>(lm, tmin); break;
-                case 32: g = warp_cutoff<1>(lm, tmin); break;
-                default: {                                     // 64: half-lane groups
-                    const float a0 = (tmin && h0 == -CUDART_INF_F) ? CUDART_INF_F : h0;
-                    const float a1 = (tmin && h1 == -CUDART_INF_F) ? CUDART_INF_F : h1;
-                    g = warp_cutoff<1>(fminf(a0, a1), false);
-                    break;
-                }
-                }
-                if (lane == 0) sh.tw[s][warp] = g;
-                if (tid == 0) { sh.ncand[s] = 0; rec->cnt = 0u; }          // (the warps add to the record after the barrier)
-                csync();
-                static_assert(STREAM_WARPS == 8, "the eight warp cutoffs are read as two 128-bit words");
-                const float4 ta = *reinterpret_cast<const float4 *>(&sh.tw[s][0]);
-                const float4 tb = *reinterpret_cast<const float4 *>(&sh.tw[s][4]);
-                float t;
-                if (tmin) {
-                    t = fminf(fminf(fminf(ta.x, ta.y), fminf(ta.z, ta.w)), fminf(fminf(tb.x, tb.y), fminf(tb.z, tb.w)));
-                    if (t == CUDART_INF_F) t = -CUDART_INF_F;          // no finite element in the tile: nothing to emit
-                } else {
-                    t = fmaxf(fmaxf(fmaxf(ta.x, ta.y), fmaxf(ta.z, ta.w)), fmaxf(fmaxf(tb.x, tb.y), fmaxf(tb.z, tb.w)));
-                }
-                // every finite element >= t goes to the tile's candidate slot; a warp reserves its share of the
-                // slot with one shared-memory atomic and adds it to the tile record (no second barrier).
-                // Most warps hold no candidate at all and leave after one vote.  The others mark their
-                // candidates in a bit mask and fetch the values again from the tile in shared memory (a
-                // candidate is neither masked nor past the row's end, so the tile holds its value).
-                const float t2 = fmaxf(t, -CUDART_MAX_NORMAL_F);           // e >= t2  <=>  e >= t and e is not -inf
-                if (__any_sync(0xFFFFFFFFu, lm >= t2)) {
-                    // a quarter of the lanes' elements without a candidate anywhere in the warp is skipped by one vote
-                    unsigned int cm = 0;
+                ebits = 0u;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        if (__any_sync(0xFFFFFFFFu, qm[i] >= t2)) {
+                for (int j = 0; j < NV; ++j) {
+                    const int li = lane0 + j * 32 * VEC;
+                    uint32_t bits = __shfl_sync(0xFFFFFFFFu, mword, (j * 32 * VEC + lane * VEC) >> 5) >> ((lane * VEC) & 31);
+                    if (!masked) bits = 0xFFFFFFFFu;
+                    if (tail) { const int left = P.V - tile_base - li; if (left < VEC) bits &= left > 0 ? (1u << left) - 1u : 0u; }
+                    bits &= (1u << VEC) - 1u;
+                    ebits |= bits << (j * VEC);
+                    float v[VEC];
+                    if (DT == 1 && !wide) {
+                        const uint4 raw = *reinterpret_cast<const uint4 *>(stage + (size_t)li * ELT);
+                        const uint32_t r[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
-                            for (int q = i * (EPL / 4); q < (i + 1) * (EPL / 4); ++q) cm |= (e[q] >= t2) ? (1u << q) : 0u;
-                        }
-                    }
-                    const int cnt = __popc(cm);
-                    int incl, total;
-                    if (!__any_sync(0xFFFFFFFFu, cnt > 1)) {
-                        // the usual case, at most one candidate per lane: positions from one vote
-                        const unsigned int has = __ballot_sync(0xFFFFFFFFu, cnt > 0);
-                        incl = __popc(has & (0xFFFFFFFFu >> (31 - lane)));
-                        total = __popc(has);
+                        for (int q = 0; q < VEC; ++q) v[q] = __uint_as_float((q & 1) ? (r[(q >> 1) & 3] & 0xFFFF0000u) : (r[(q >> 1) & 3] << 16));
                     } else {
-                        incl = cnt;
 #pragma unroll
-                        for (int off = 1; off < 32; off <<= 1) {
-                            const int o = __shfl_up_sync(0xFFFFFFFFu, incl, off);
-                            if (lane >= off) incl += o;
+                        for (int q = 0; q < VEC; q += 4) {
+                            const float4 a = *reinterpret_cast<const float4 *>(ptile + li + q);
+                            v[q] = a.x; v[q + 1] = a.y; v[q + 2] = a.z; v[q + 3] = a.w;
                         }
-                        total = __shfl_sync(0xFFFFFFFFu, incl, 31);
                     }
-                    unsigned int base = 0;
-                    if (lane == 0) {
-                        base = atomicAdd(&sh.ncand[s], (unsigned int)total);
-                        atomicAdd(&rec->cnt, (unsigned int)total);      // zero before the call; the merge kernel clears it
-                    }
-                    base = __shfl_sync(0xFFFFFFFFu, base, 0);
-                    if ((int)base + total <= cap_t) {
-                        unsigned long long *dst = P.cand + (size_t)row * P.cand_stride + (size_t)tile * cap_t + base + (incl - cnt);
-                        const int lbase = warp * WARP_TILE + lane * VEC;
-                        while (cm) {
-                            const int q = __ffs(cm) - 1;
-                            cm &= cm - 1;
-                            const int li = lbase + (q / VEC) * (32 * VEC) + (q % VEC);
-                            float v;
-                            if (DT == 0 || patched) v = ptile[li];
-                            else v = __uint_as_float((uint32_t)reinterpret_cast<const unsigned short *>(stage)[li] << 16);
-                            if (c.div_all) v = div_tau(v, c.tau);
-                            *dst++ = ((unsigned long long)okey(v) << 32) | (uint32_t)(~(uint32_t)(tile_base + li));
-                        }
+                    mv[j] = -CUDART_INF_F;
+#pragma unroll
+                    for (int q = 0; q < VEC; ++q) mv[j] = ((bits >> q) & 1u) ? fmaxf(mv[j], v[q]) : mv[j];
+                }
+            }
+            float h0 = mv[0], h1 = mv[NV / 2];
+#pragma unroll
+            for (int j = 1; j < NV / 2; ++j) { h0 = fmaxf(h0, mv[j]); h1 = fmaxf(h1, mv[NV / 2 + j]); }
+            const float lm = fmaxf(h0, h1);
+            // The elements of the lane's vectors whose maximum reaches t, one vector after the other (rare: read again):
+            // f(value, index within the tile) for those that reach t.
+            auto visit = [&](float t, auto f) {
+                unsigned int vm = 0u;
+#pragma unroll
+                for (int j = 0; j < NV; ++j) vm |= (mv[j] >= t) ? (1u << j) : 0u;
+#pragma unroll 1
+                while (vm) {
+                    const int j = __ffs(vm) - 1, li = lane0 + j * 32 * VEC;
+                    vm &= vm - 1u;
+                    const uint32_t bits = ebits >> (j * VEC);
+#pragma unroll
+                    for (int q = 0; q < VEC; q += 4) {
+                        float4 a;
+                        if (DT == 1 && !wide) {
+                            const uint2 r = *reinterpret_cast<const uint2 *>(stage + (size_t)(li + q) * ELT);
+                            a = make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xFFFF0000u), __uint_as_float(r.y << 16), __uint_as_float(r.y & 0xFFFF0000u));
+                        } else a = *reinterpret_cast<const float4 *>(ptile + li + q);
+                        if (a.x >= t && ((bits >> q) & 1u)) f(a.x, li + q);
+                        if (a.y >= t && ((bits >> (q + 1)) & 1u)) f(a.y, li + q + 1);
+                        if (a.z >= t && ((bits >> (q + 2)) & 1u)) f(a.z, li + q + 2);
+                        if (a.w >= t && ((bits >> (q + 3)) & 1u)) f(a.w, li + q + 3);
                     }
                 }
-                if (tid == 0) rec->tkey = okey(t);
+            };
+
+            if (meta.cfg.cls == CLS_GREEDY) {
+                // The argmax of the processed logits, lowest index first.  Only elements at or above the largest so far can
+                // matter (with a temperature: above a hair less, since the division may make them equal).
+                if (row != g_row) { g_row = row; g_thr = -CUDART_MAX_NORMAL_F; }
+                unsigned long long best = 0ull;
+                if (__any_sync(0xFFFFFFFFu, lm >= g_thr)) {
+                    const bool temp = meta.cfg.temp;
+                    const float tau = meta.cfg.tau;
+                    if (lm >= g_thr) visit(g_thr, [&](float z, int li) {
+                        const uint32_t key = okey(temp ? div_tau(z, tau) : z);
+                        best = max(best, ((unsigned long long)key << 32) | (uint32_t)(~(uint32_t)(tile_base + li)));
+                    });
+                    __syncwarp();
+                    const uint32_t hi = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(best >> 32));
+                    const uint32_t lo = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(best >> 32) == hi ? (uint32_t)best : 0u);
+                    best = ((unsigned long long)hi << 32) | lo;
+                    const float z = unkey(__reduce_max_sync(0xFFFFFFFFu, okey(lm)));
+                    g_thr = fmaxf(g_thr, temp ? z - fmaxf(fabsf(z) * 4.76837158203125e-07f, 1e-37f) : z);
+                }
+                if (lane == 0) sh.best[s][warp] = best;
+            } else {
+                const int G = meta.cfg.G;
+                const bool tmin = meta.cfg.tile_min;
+                // warp cutoff: minimum over G groups of the group maximum.  Tile cutoff: the largest of the eight warp cutoffs
+                // (warp mode) or the smallest (tile mode: a minimum over all 8 G groups of the tile).  In tile mode a group
+                // without a finite element (masked, or past the row's end) does not take part: it would drag the cutoff
+                // to -inf and the tile would emit everything it has.
+                auto group_cutoff = [&]() -> float {
+                    switch (G) {                               // (one straight-line butterfly per group count)
+                    case 0: return -CUDART_INF_F;
+                    case 1: return warp_cutoff<32>(lm, tmin);
+                    case 2: return warp_cutoff<16>(lm, tmin);
+                    case 4: return warp_cutoff<8>(lm, tmin);
+                    case 8: return warp_cutoff<4>(lm, tmin);
+                    case 16: return warp_cutoff<2>(lm, tmin);
+                    case 32: return warp_cutoff<1>(lm, tmin);
+                    default: {                                 // 64: half-lane groups
+                        const float a0 = (tmin && h0 == -CUDART_INF_F) ? CUDART_INF_F : h0;
+                        const float a1 = (tmin && h1 == -CUDART_INF_F) ? CUDART_INF_F : h1;
+                        return warp_cutoff<1>(fminf(a0, a1), false);
+                    }
+                    }
+                };
+                float t = cut;
+                if (row != cut_row) {
+                    const float g = group_cutoff();
+                    if (lane == 0) sh.tw[s][warp] = g;
+                    csync();
+                    static_assert(STREAM_WARPS == 8, "the eight warp cutoffs are read as two 128-bit words");
+                    const float4 ta = *reinterpret_cast<const float4 *>(&sh.tw[s][0]);
+                    const float4 tb = *reinterpret_cast<const float4 *>(&sh.tw[s][4]);
+                    if (tmin) {
+                        t = fminf(fminf(fminf(ta.x, ta.y), fminf(ta.z, ta.w)), fminf(fminf(tb.x, tb.y), fminf(tb.z, tb.w)));
+                        if (t == CUDART_INF_F) t = -CUDART_INF_F;          // no finite element in the tile: nothing to emit
+                    } else {
+                        t = fmaxf(fmaxf(fmaxf(ta.x, ta.y), fmaxf(ta.z, ta.w)), fmaxf(fmaxf(tb.x, tb.y), fmaxf(tb.z, tb.w)));
+                    }
+                    // (a tile that bounds nothing leaves the cutoff to the next one)
+                    cut = t;
+                    cut_row = (t > -CUDART_INF_F) ? row : -1;
+                } else if (G <= 8 && __popc(__ballot_sync(0xFFFFFFFFu, lm >= t)) > 28) {
+                    // far more candidates than the cutoff was meant for (values that depend on the position): the warp takes
+                    // a cutoff of its own for this tile
+                    t = fmaxf(t, group_cutoff());
+                    if (t == CUDART_INF_F) t = cut;
+                }
+                if (lane == 0) atomicMax(&sh.tkey[s], okey(t));
+                // every finite element >= t goes to the tile's candidate slot
+                const float t2 = fmaxf(t, -CUDART_MAX_NORMAL_F);           // e >= t2  <=>  e >= t and e is not -inf
+                if (lm >= t2) {
+                    unsigned long long *dst = P.cand + (size_t)row * P.cand_stride + (size_t)tile * cap_t;
+                    visit(t2, [&](float z, int li) {
+                        const unsigned int pos = atomicAdd(&sh.ncand[s], 1u);
+                        if ((int)pos < cap_t) dst[pos] = ((unsigned long long)okey(z) << 32) | (uint32_t)(~(uint32_t)(tile_base + li));
+                    });
+                }
+                __syncwarp();
             }
 
             // generic-proxy writes into the stage (in-place patches) precede the next bulk copy into it
-            if (DT == 0 && patched) fence_async_proxy();
+            if (DT == 0 && patch != 0) fence_async_proxy();
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&sh.empty[s]);
