@@ -74,7 +74,7 @@ static int fail_cuda(cudaError_t e, const char *what) {
 // Workspace layout.  Only the header (WS_HEADER bytes at offset 0) is shared by all calls and must be zero between
 // them; everything behind it is laid out for the shape of the call at hand (rows, V, operation) and initialised by the call's own kernels, so one workspace serves calls of any shape that fits.
 struct Layout {
-    size_t rs, pr, tiles, cand, total;
+    size_t rs, pr, tiles, wmax, cand, total;
     unsigned int cand_stride;
 };
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -95,6 +95,7 @@ static Layout layout_for(long long rows, int V, size_t cap) {
     L.rs = off;    off = align256(off + (size_t)rows * sizeof(RowState));
     L.pr = off;    off = align256(off + (size_t)rows * sizeof(PosResult));
     L.tiles = off; off = align256(off + (size_t)rows * sizeof(TileRec) * MAX_TILES);
+    L.wmax = off;  off = align256(off + (size_t)rows * MAX_TILES * STREAM_WARPS * 4);
     L.cand = off;  off = align256(off + (size_t)rows * slots * 8);
     L.total = off;
     return L;
@@ -270,6 +271,7 @@ static int launch_all(KParams &P, void *ws, size_t ws_bytes, cudaStream_t st, in
     P.rs = reinterpret_cast<RowState *>(base + L.rs);
     P.pr = reinterpret_cast<PosResult *>(base + L.pr);
     P.tiles = reinterpret_cast<TileRec *>(base + L.tiles);
+    P.wmax = reinterpret_cast<unsigned int *>(base + L.wmax);
     P.cand = reinterpret_cast<unsigned long long *>(base + L.cand);
     P.cand_stride = L.cand_stride;
     P.tickets = P.error + WS_TICKETS;
@@ -472,8 +474,8 @@ int sonic_topk(const void *logits, int dtype, int B, int V, int64_t row_stride, 
 // Scratch of sonic_topk_static: a workspace for SONIC_STATIC_MAX_ROWS rows of the largest vocabulary that lives in
 // the library image.  In host code this name is only a stand-in for the symbol; the device
 // address the kernels need comes from cudaGetSymbolAddress (below), never from `&`.
-constexpr size_t STATIC_WS_BYTES = WS_HEADER + 256 * 4 +
-    (size_t)SONIC_STATIC_MAX_ROWS * (sizeof(RowState) + sizeof(PosResult) + sizeof(TileRec) * MAX_TILES + 2 * (size_t)CAND_CAP * 8);
+constexpr size_t STATIC_WS_BYTES = WS_HEADER + 256 * 5 +
+    (size_t)SONIC_STATIC_MAX_ROWS * (sizeof(RowState) + sizeof(PosResult) + (sizeof(TileRec) + STREAM_WARPS * 4) * MAX_TILES + 2 * (size_t)CAND_CAP * 8);
 static __device__ __align__(256) unsigned char g_static_workspace[STATIC_WS_BYTES];
 
 static int static_workspace_address(void **out) {

@@ -45,7 +45,6 @@ constexpr int ROW_LAND = 2944;                    // elements CTA 0 can receive
 constexpr int ROW_MEMBERS = ROW_THREADS;          // ... of a top-p row's crossing bin (one per thread)
 constexpr int ROW_GMAX = 512;                     // group maxima that are exchanged directly (one per thread)
 constexpr int ROW_KMAX = 2048;                    // largest top-k finished from gathered elements
-constexpr int ROW_SMALL = 128;                    // candidates the short finish takes
 static_assert(ROW_SLICE_MAX * 4 >= MERGE_CAP * 8, "the epilogue's buffers take the values' place in CTA 0");
 static_assert(ROW_KMAX <= KFAST_SAMPLE, "the epilogue's layout");
 static_assert(ROW_THREADS == MERGE_THREADS, "the merge epilogue runs on the row kernel's CTAs");
@@ -567,176 +566,6 @@ __device__ __forceinline__ void row_gather_count(const RowCtx &x, const RowSel &
     __syncwarp();
 }
 
-// The k-th largest of the n group maxima in sh.gmax (32-bit keys, n <= ROW_GMAX, zeros behind them): every maximum counts
-// those above it (up to four threads share one), the smallest with fewer than k above is the answer.  Whole CTA, one
-// block barrier.
-__device__ __forceinline__ uint32_t row_kth_max(RowShared &sh, int n, int k, int tid) {
-    const int lg = n <= ROW_GMAX / 4 ? 2 : (n <= ROW_GMAX / 2 ? 1 : 0), part = tid & ((1 << lg) - 1);
-    const uint32_t mine = sh.gmax[tid >> lg];
-    int above = 0;
-#pragma unroll 4
-    for (int i = part; i < (n + 3) / 4; i += 1 << lg) {
-        const uint4 o = reinterpret_cast<const uint4 *>(sh.gmax)[i];
-        above += (o.x > mine ? 1 : 0) + (o.y > mine ? 1 : 0) + (o.z > mine ? 1 : 0) + (o.w > mine ? 1 : 0);
-    }
-    if (lg > 0) above += __shfl_xor_sync(0xFFFFFFFFu, above, 1);
-    if (lg > 1) above += __shfl_xor_sync(0xFFFFFFFFu, above, 2);
-    const uint32_t t = __reduce_min_sync(0xFFFFFFFFu, above < k ? mine : 0xFFFFFFFFu);
-    if ((tid & 31) == 0) sh.red32[tid >> 5] = t;
-    __syncthreads();
-    return __reduce_min_sync(0xFFFFFFFFu, sh.red32[tid & (ROW_WARPS - 1)]);
-}
-
-// A top-k row whose at most ROW_SMALL candidates (before the temperature) are in the landing zone: everything that is left of it,
-// with three block barriers.  Four threads per candidate count how many rank above it and how many have a smaller index;
-// the weights (fp64) go to both orders; one warp does the cuts and the draw.
-__device__ __forceinline__ void row_finish_small(const RowCtx &x, const KParams &P, const RowCfg &c, int row, int n, uint2 cells, int draft, float q_draft) {
-    RowShared &sh = row_sh();
-    unsigned long long *cand = &sh.list[0];                         // [ROW_SMALL] (value key after the temperature, ~index)
-    unsigned long long *byrank = cand + ROW_SMALL;                  // [ROW_SMALL] the same in ranking order
-    double *wr = reinterpret_cast<double *>(cand + 2 * ROW_SMALL);   // weights in ranking order
-    unsigned long long *byidx = cand + 3 * ROW_SMALL;               // rank of the j-th candidate in index order
-    const int tid = x.tid, lane = x.lane;
-    if (tid < ROW_SMALL) {
-        unsigned long long v = (tid < n) ? row_land()[tid] : 0ull;
-        if (v && c.temp) v = ((unsigned long long)okey(div_tau(unkey((uint32_t)(v >> 32)), c.tau)) << 32) | (uint32_t)v;
-        cand[tid] = v;
-        byrank[tid] = 0ull; wr[tid] = 0.0; byidx[tid] = 0xFFFFull;
-    }
-    __syncthreads();
-    {
-        const int j = tid >> 2, part = tid & 3;
-        const unsigned long long mine = cand[j];
-        int rv = 0, ri = 0;
-        uint32_t top = 0u;
-#pragma unroll 4
-        for (int u = part; u < (n + 1) / 2; u += 4) {              // (the four parts read 64 consecutive bytes)
-            const ulonglong2 o = reinterpret_cast<const ulonglong2 *>(cand)[u];
-            rv += (o.x > mine ? 1 : 0) + (o.y > mine ? 1 : 0);
-            ri += ((uint32_t)o.x > (uint32_t)mine ? 1 : 0) + ((uint32_t)o.y > (uint32_t)mine ? 1 : 0);
-            top = max(top, max((uint32_t)(o.x >> 32), (uint32_t)(o.y >> 32)));
-        }
-#pragma unroll
-        for (int off = 1; off < 4; off <<= 1) {
-            rv += __shfl_xor_sync(0xFFFFFFFFu, rv, off);
-            ri += __shfl_xor_sync(0xFFFFFFFFu, ri, off);
-            top = max(top, __shfl_xor_sync(0xFFFFFFFFu, top, off));
-        }
-        if (mine && part == 0) {
-            byrank[rv] = mine;
-            if (P.op == OP_TOPK) {
-                if (rv < P.ktop) {
-                    P.out_vals[(size_t)row * P.ktop + rv] = unkey((uint32_t)(mine >> 32));
-                    P.out_idx[(size_t)row * P.ktop + rv] = (int)(~(uint32_t)mine);
-                }
-            } else {
-                wr[rv] = exp((double)unkey((uint32_t)(mine >> 32)) - (double)unkey(top));
-                byidx[ri] = (unsigned long long)rv;
-            }
-        }
-    }
-    if (P.op == OP_TOPK) return;
-    __syncthreads();
-    if (tid >= 32) return;
-    // the ranking: four consecutive positions per lane
-    const double M = (double)unkey((uint32_t)(byrank[0] >> 32));
-    const int m = min(n, c.k);
-    double cs[4], run = 0.0;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) { const int j = lane * 4 + u; run += (j < m) ? wr[j] : 0.0; cs[u] = run; }
-    double incl = run;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) { const double up = __shfl_up_sync(0xFFFFFFFFu, incl, o); if (lane >= o) incl += up; }
-    const double Z = __shfl_sync(0xFFFFFFFFu, incl, 31), excl = incl - run;
-    auto first_hit = [&](int at) -> int {                           // first position from every lane's first hit among its four (4: none)
-        const unsigned int b = __ballot_sync(0xFFFFFFFFu, at < 4);
-        if (!b) return -1;
-        const int l = __ffs(b) - 1;
-        return l * 4 + __shfl_sync(0xFFFFFFFFu, at, l);
-    };
-    int keep = m;
-    if (c.z & M_TOP_P) {
-        const double target = (double)c.p * Z;
-        int at = 4;
-#pragma unroll
-        for (int u = 3; u >= 0; --u) if (lane * 4 + u < m && cs[u] + excl >= target) at = u;
-        const int j = first_hit(at);
-        if (j >= 0) keep = min(keep, j + 1);
-    }
-    if (c.z & M_MIN_P) {
-        const double thr = M + log((double)c.theta);
-        int at = 4;
-#pragma unroll
-        for (int u = 3; u >= 0; --u) { const int j = lane * 4 + u; if (j < m && !((double)unkey((uint32_t)(byrank[j] >> 32)) >= thr)) at = u; }
-        const int j = first_hit(at);
-        if (j >= 0) keep = min(keep, j);
-    }
-    double W = 0.0;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) if (((keep - 1) & 3) == u) W = cs[u] + excl;
-    W = __shfl_sync(0xFFFFFFFFu, W, (keep - 1) >> 2);
-    // index order: what is cut off weighs nothing
-    int rk[4];
-    double r4[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) { rk[u] = (int)byidx[lane * 4 + u]; r4[u] = (rk[u] < keep) ? wr[rk[u] & (ROW_SMALL - 1)] : 0.0; }
-    uint32_t flags = 0u;
-    float p_draft = 0.0f;
-    auto scan4 = [&]() -> double {                                  // cs: inclusive sums in index order; the total
-        double r = 0.0;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) { r += r4[u]; cs[u] = r; }
-        double in = r;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const double up = __shfl_up_sync(0xFFFFFFFFu, in, o); if (lane >= o) in += up; }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) cs[u] += in - r;
-        return __shfl_sync(0xFFFFFFFFu, in, 31);
-    };
-    double total = -1.0;
-    if (P.op == OP_VERIFY && c.l < P.K) {
-        double pd = 0.0;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) if (rk[u] < keep && draft >= 0 && (int)(~(uint32_t)byrank[rk[u] & (ROW_SMALL - 1)]) == draft) pd = r4[u];
-        const unsigned int b = __ballot_sync(0xFFFFFFFFu, pd > 0.0);
-        const double Pd = b ? __shfl_sync(0xFFFFFFFFu, pd, __ffs(b) - 1) / W : 0.0;
-        p_draft = (float)Pd;
-        if (Pd > 0.0 && cell_to_u(cells.x) * (double)q_draft <= Pd) flags |= F_ACCEPT;
-        else {                                                      // residual max(0, p - q) over the support
-            const float *q = P.draft_probs + ((size_t)c.b * P.K + c.l) * (size_t)P.V;
-            float q4[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) q4[u] = (rk[u] < keep) ? __ldg(q + (int)(~(uint32_t)byrank[rk[u] & (ROW_SMALL - 1)])) : 0.0f;
-            double keep4[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) { keep4[u] = r4[u]; const double r = (rk[u] < keep) ? r4[u] / W - (double)q4[u] : 0.0; r4[u] = r > 0.0 ? r : 0.0; }
-            total = scan4();
-            if (!(total > 0.0)) {
-#pragma unroll
-                for (int u = 0; u < 4; ++u) r4[u] = keep4[u];
-                total = -1.0;
-            }
-        }
-    }
-    if (total < 0.0) total = scan4();
-    const double target = cell_to_u(cells.y) * total;
-    int at = 4, lastpos = -1;
-#pragma unroll
-    for (int u = 3; u >= 0; --u) if (rk[u] < keep && cs[u] > target && r4[u] > 0.0) at = u;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) if (rk[u] < keep) lastpos = u;
-    int j = first_hit(at);
-    if (j < 0) {                                                    // (rounding: the last survivor in index order)
-        const unsigned int b = __ballot_sync(0xFFFFFFFFu, lastpos >= 0);
-        const int l = 31 - __clz(b);
-        j = l * 4 + __shfl_sync(0xFFFFFFFFu, lastpos, l);
-    }
-    if (lane == 0) {
-        const int r = (int)byidx[j];
-        emit_row(P, c, row, (int)(~(uint32_t)byrank[r]), (float)(wr[r] / W), flags, keep, p_draft);
-    }
-}
-
 template <typename T>
 __device__ __forceinline__ T row_lane_scan(T v, int lane) {
 #pragma unroll
@@ -1081,7 +910,7 @@ __device__ __forceinline__ void row_body(const KParams &P, RowCtx &x, const int 
         }
         cl_sync();
         if (row_late(x)) { if (lead) emit_late(); return; }
-        const uint32_t tk = row_kth_max(sh, ngroups, c.k, tid);
+        const uint32_t tk = kth_max<ROW_THREADS>(sh.gmax, sh.red32, ngroups, c.k, tid);
         // Everything that reaches the bound goes to CTA 0.  With a temperature a value a hair below the bound may become
         // equal to it when divided, and then the index decides: the bound is lowered by 2^-21 of itself.
         float t = max(unkey(tk), s.vmin);
@@ -1124,7 +953,7 @@ __device__ __forceinline__ void row_body(const KParams &P, RowCtx &x, const int 
             if (x.rank != 0) return;
             const uint2 cells = draw();
             if (n == 0) { if (tid == 0) emit_row(P, c, row, -1, 0.0f, F_NO_TOKEN, 0, 0.0f); }
-            else if (n <= ROW_SMALL) row_finish_small(x, P, c, row, n, cells, draft, q_draft);
+            else if (n <= SMALL_MAX) finish_small(P, c, row, row_land(), divide, n, sh.list, tid, cells, draft, q_draft);
             else {
                 unsigned long long *buf = reinterpret_cast<unsigned long long *>(row_smem);
                 for (int i = tid; i < n; i += ROW_THREADS) {

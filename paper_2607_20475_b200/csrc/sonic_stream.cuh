@@ -303,6 +303,179 @@ template <int THREADS, typename Sync>
 __device__ void merge_finish(const KParams &P, const RowCfg &c, int row, unsigned long long *buf, unsigned int *bins, const int Pn, const int n,
                              MergeShared<THREADS> &sh, int tid, uint2 cells);
 
+constexpr int SMALL_MAX = 128;                // candidates the short finish takes
+// A top-k row whose at most SMALL_MAX candidates are in src (divide: before the temperature): everything that is left of it,
+// with three block barriers.  Four threads per candidate count how many rank above it and how many have a smaller index;
+// the weights (fp64) go to both orders; one warp does the cuts and the draw.
+// list: 4 * SMALL_MAX words.
+__device__ __forceinline__ void finish_small(const KParams &P, const RowCfg &c, int row, const unsigned long long *src, bool divide, int n,
+                                             unsigned long long *list, int tid, uint2 cells, int draft, float q_draft) {
+    unsigned long long *cand = list;                                // [SMALL_MAX] (value key after the temperature, ~index)
+    unsigned long long *byrank = cand + SMALL_MAX;                  // [SMALL_MAX] the same in ranking order
+    double *wr = reinterpret_cast<double *>(cand + 2 * SMALL_MAX);   // weights in ranking order
+    unsigned long long *byidx = cand + 3 * SMALL_MAX;               // rank of the j-th candidate in index order
+    const int lane = tid & 31;
+    if (tid < SMALL_MAX) {
+        unsigned long long v = (tid < n) ? src[tid] : 0ull;
+        if (v && divide) v = ((unsigned long long)okey(div_tau(unkey((uint32_t)(v >> 32)), c.tau)) << 32) | (uint32_t)v;
+        cand[tid] = v;
+        byrank[tid] = 0ull; wr[tid] = 0.0; byidx[tid] = 0xFFFFull;
+    }
+    __syncthreads();
+    {
+        const int j = tid >> 2, part = tid & 3;
+        const unsigned long long mine = cand[j];
+        int rv = 0, ri = 0;
+        uint32_t top = 0u;
+#pragma unroll 4
+        for (int u = part; u < (n + 1) / 2; u += 4) {              // (the four parts read 64 consecutive bytes)
+            const ulonglong2 o = reinterpret_cast<const ulonglong2 *>(cand)[u];
+            rv += (o.x > mine ? 1 : 0) + (o.y > mine ? 1 : 0);
+            ri += ((uint32_t)o.x > (uint32_t)mine ? 1 : 0) + ((uint32_t)o.y > (uint32_t)mine ? 1 : 0);
+            top = max(top, max((uint32_t)(o.x >> 32), (uint32_t)(o.y >> 32)));
+        }
+#pragma unroll
+        for (int off = 1; off < 4; off <<= 1) {
+            rv += __shfl_xor_sync(0xFFFFFFFFu, rv, off);
+            ri += __shfl_xor_sync(0xFFFFFFFFu, ri, off);
+            top = max(top, __shfl_xor_sync(0xFFFFFFFFu, top, off));
+        }
+        if (mine && part == 0) {
+            byrank[rv] = mine;
+            if (P.op == OP_TOPK) {
+                if (rv < P.ktop) {
+                    P.out_vals[(size_t)row * P.ktop + rv] = unkey((uint32_t)(mine >> 32));
+                    P.out_idx[(size_t)row * P.ktop + rv] = (int)(~(uint32_t)mine);
+                }
+            } else {
+                wr[rv] = exp((double)unkey((uint32_t)(mine >> 32)) - (double)unkey(top));
+                byidx[ri] = (unsigned long long)rv;
+            }
+        }
+    }
+    if (P.op == OP_TOPK) return;
+    __syncthreads();
+    if (tid >= 32) return;
+    // the ranking: four consecutive positions per lane
+    const double M = (double)unkey((uint32_t)(byrank[0] >> 32));
+    const int m = min(n, c.k);
+    double cs[4], run = 0.0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) { const int j = lane * 4 + u; run += (j < m) ? wr[j] : 0.0; cs[u] = run; }
+    double incl = run;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const double up = __shfl_up_sync(0xFFFFFFFFu, incl, o); if (lane >= o) incl += up; }
+    const double Z = __shfl_sync(0xFFFFFFFFu, incl, 31), excl = incl - run;
+    auto first_hit = [&](int at) -> int {                           // first position from every lane's first hit among its four (4: none)
+        const unsigned int b = __ballot_sync(0xFFFFFFFFu, at < 4);
+        if (!b) return -1;
+        const int l = __ffs(b) - 1;
+        return l * 4 + __shfl_sync(0xFFFFFFFFu, at, l);
+    };
+    int keep = m;
+    if (c.z & M_TOP_P) {
+        const double target = (double)c.p * Z;
+        int at = 4;
+#pragma unroll
+        for (int u = 3; u >= 0; --u) if (lane * 4 + u < m && cs[u] + excl >= target) at = u;
+        const int j = first_hit(at);
+        if (j >= 0) keep = min(keep, j + 1);
+    }
+    if (c.z & M_MIN_P) {
+        const double thr = M + log((double)c.theta);
+        int at = 4;
+#pragma unroll
+        for (int u = 3; u >= 0; --u) { const int j = lane * 4 + u; if (j < m && !((double)unkey((uint32_t)(byrank[j] >> 32)) >= thr)) at = u; }
+        const int j = first_hit(at);
+        if (j >= 0) keep = min(keep, j);
+    }
+    double W = 0.0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) if (((keep - 1) & 3) == u) W = cs[u] + excl;
+    W = __shfl_sync(0xFFFFFFFFu, W, (keep - 1) >> 2);
+    // index order: what is cut off weighs nothing
+    int rk[4];
+    double r4[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) { rk[u] = (int)byidx[lane * 4 + u]; r4[u] = (rk[u] < keep) ? wr[rk[u] & (SMALL_MAX - 1)] : 0.0; }
+    uint32_t flags = 0u;
+    float p_draft = 0.0f;
+    auto scan4 = [&]() -> double {                                  // cs: inclusive sums in index order; the total
+        double r = 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { r += r4[u]; cs[u] = r; }
+        double in = r;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const double up = __shfl_up_sync(0xFFFFFFFFu, in, o); if (lane >= o) in += up; }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) cs[u] += in - r;
+        return __shfl_sync(0xFFFFFFFFu, in, 31);
+    };
+    double total = -1.0;
+    if (P.op == OP_VERIFY && c.l < P.K) {
+        double pd = 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) if (rk[u] < keep && draft >= 0 && (int)(~(uint32_t)byrank[rk[u] & (SMALL_MAX - 1)]) == draft) pd = r4[u];
+        const unsigned int b = __ballot_sync(0xFFFFFFFFu, pd > 0.0);
+        const double Pd = b ? __shfl_sync(0xFFFFFFFFu, pd, __ffs(b) - 1) / W : 0.0;
+        p_draft = (float)Pd;
+        if (Pd > 0.0 && cell_to_u(cells.x) * (double)q_draft <= Pd) flags |= F_ACCEPT;
+        else {                                                      // residual max(0, p - q) over the support
+            const float *q = P.draft_probs + ((size_t)c.b * P.K + c.l) * (size_t)P.V;
+            float q4[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) q4[u] = (rk[u] < keep) ? __ldg(q + (int)(~(uint32_t)byrank[rk[u] & (SMALL_MAX - 1)])) : 0.0f;
+            double keep4[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) { keep4[u] = r4[u]; const double r = (rk[u] < keep) ? r4[u] / W - (double)q4[u] : 0.0; r4[u] = r > 0.0 ? r : 0.0; }
+            total = scan4();
+            if (!(total > 0.0)) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) r4[u] = keep4[u];
+                total = -1.0;
+            }
+        }
+    }
+    if (total < 0.0) total = scan4();
+    const double target = cell_to_u(cells.y) * total;
+    int at = 4, lastpos = -1;
+#pragma unroll
+    for (int u = 3; u >= 0; --u) if (rk[u] < keep && cs[u] > target && r4[u] > 0.0) at = u;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) if (rk[u] < keep) lastpos = u;
+    int j = first_hit(at);
+    if (j < 0) {                                                    // (rounding: the last survivor in index order)
+        const unsigned int b = __ballot_sync(0xFFFFFFFFu, lastpos >= 0);
+        const int l = 31 - __clz(b);
+        j = l * 4 + __shfl_sync(0xFFFFFFFFu, lastpos, l);
+    }
+    if (lane == 0) {
+        const int r = (int)byidx[j];
+        emit_row(P, c, row, (int)(~(uint32_t)byrank[r]), (float)(wr[r] / W), flags, keep, p_draft);
+    }
+}
+
+// The k-th largest of the n maxima in gmax (32-bit keys, n <= THREADS, zeros behind them up to the next multiple of four):
+// every maximum counts those above it (up to four threads share one), the smallest with fewer than k above is the answer.
+// red: THREADS / 32 words.  Whole CTA, one block barrier.
+template <int THREADS>
+__device__ __forceinline__ uint32_t kth_max(const unsigned int *gmax, unsigned int *red, int n, int k, int tid) {
+    const int lg = n <= THREADS / 4 ? 2 : (n <= THREADS / 2 ? 1 : 0), part = tid & ((1 << lg) - 1);
+    const uint32_t mine = ((tid >> lg) < n) ? gmax[tid >> lg] : 0u;
+    int above = 0;
+#pragma unroll 4
+    for (int i = part; i < (n + 3) / 4; i += 1 << lg) {
+        const uint4 o = reinterpret_cast<const uint4 *>(gmax)[i];
+        above += (o.x > mine ? 1 : 0) + (o.y > mine ? 1 : 0) + (o.z > mine ? 1 : 0) + (o.w > mine ? 1 : 0);
+    }
+    if (lg > 0) above += __shfl_xor_sync(0xFFFFFFFFu, above, 1);
+    if (lg > 1) above += __shfl_xor_sync(0xFFFFFFFFu, above, 2);
+    const uint32_t t = __reduce_min_sync(0xFFFFFFFFu, (above < k && (tid >> lg) < n) ? mine : 0xFFFFFFFFu);
+    if ((tid & 31) == 0) red[tid >> 5] = t;
+    __syncthreads();
+    return __reduce_min_sync(0xFFFFFFFFu, red[tid & (THREADS / 32 - 1)]);
+}
+
 // Row merge for top-k class rows (one CTA per row).  buf is MERGE_CAP 64-bit
 // words of shared memory.  Returns false if the candidates cannot prove the
 // row's answer.
@@ -331,9 +504,22 @@ __device__ bool merge_topk_row(const KParams &P, const RowCfg &c, int row, int t
         sh.tcnt[tid + 1] = incl;                                   // lanes past the last tile repeat the total
         if (tid == 0) { sh.tcnt[0] = 0; sh.count = 0; sh.tkey = tk; sh.found = over ? 1 : 0; }
     }
+    // Small k: the k-th largest of the maxima of the row's warp tiles is a value that k elements reach and few more do (75
+    // of 2^18 for k = 64), all of them candidates.  bins: the maxima.
+    const int groups = tiles * STREAM_WARPS;
+    const bool tight = 2 * c.k <= groups && c.k <= 100;
+    static_assert(MAX_TILES * STREAM_WARPS * 2 == THREADS, "two threads per maximum at most");
+    if (tight && tid < MAX_TILES * STREAM_WARPS) bins[tid] = (tid < groups) ? __ldcg(&P.wmax[(size_t)row * MAX_TILES * STREAM_WARPS + tid]) : 0u;
     csync();
     if (sh.found) return false;
-    const unsigned int tkey = sh.tkey;
+    unsigned int tkey = sh.tkey;
+    if (tight && tkey != KEY_NEG_INF) {
+        const uint32_t kth = kth_max<THREADS>(bins, reinterpret_cast<unsigned int *>(sh.wsum), groups, c.k, tid);
+        // (with a temperature a hair less: a value just below the bound may become equal to it when divided)
+        float t = unkey(kth);
+        if (c.temp) t -= fmaxf(fabsf(t) * 4.76837158203125e-07f, 1e-37f);
+        if (kth > KEY_NEG_INF) tkey = max(tkey, okey(t));
+    }
     const bool complete = (tkey == KEY_NEG_INF);
     const bool strict = c.temp && !complete;            // keys are compared after the temperature division
     const uint32_t tykey = c.temp ? okey(div_tau(unkey(tkey), c.tau)) : tkey;
@@ -603,6 +789,17 @@ __device__ bool merge_topk_row(const KParams &P, const RowCfg &c, int row, int t
     if (Pn >= c.k) n = c.k;
     else if (complete && P.op != OP_TOPK) n = Pn;
     else return false;
+    if (Pn <= SMALL_MAX && n > 0) {
+        int draft = -1;
+        float q_draft = 0.0f;
+        if (P.op == OP_VERIFY && c.l < P.K) {
+            draft = __ldg(P.draft_tokens + (size_t)c.b * P.K + c.l);
+            if (draft < 0 || draft >= P.V) draft = -1;
+            if (draft >= 0) q_draft = __ldg(P.draft_probs + ((size_t)c.b * P.K + c.l) * (size_t)P.V + draft);
+        }
+        finish_small(P, c, row, buf, false, Pn, reinterpret_cast<unsigned long long *>(bins), tid, cells, draft, q_draft);
+        return true;
+    }
     merge_finish<THREADS, Sync>(P, c, row, buf, bins, Pn, n, sh, tid, cells);
     return true;
 }
@@ -1051,8 +1248,8 @@ struct StreamShared {
     StageMeta meta[NSTAGE];
     // per-stage results of the consumer warps, which the producer turns into the tile's record once all of them are done
     alignas(16) float tw[NSTAGE][STREAM_WARPS];
-    unsigned int ncand[NSTAGE], tkey[NSTAGE], badid[NSTAGE];
-    unsigned long long best[NSTAGE][STREAM_WARPS];
+    unsigned int ncand[NSTAGE], badid[NSTAGE];
+    unsigned long long best[NSTAGE][STREAM_WARPS];       // greedy rows: argmax; top-k rows: cutoff key << 32 | key of the warp's maximum
     uint32_t list[FILTER_HIST];                // the producer's: the row's history, id | count << 18 (0: no entry)
     // hit lists: one buffer more than stages, so that the producer fills the next tile's while both stages are busy
     Hit pen[NSTAGE + 1][HIT_PEN_CAP];
@@ -1245,11 +1442,12 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 return;
             }
             unsigned long long b = (lane < STREAM_WARPS) ? sh.best[s][lane] : 0ull;
+            if (lane < STREAM_WARPS && sh.meta[s].cfg.cls == CLS_TOPK) P.wmax[((size_t)row * MAX_TILES + tile) * STREAM_WARPS + lane] = (uint32_t)b;
 #pragma unroll
             for (int off = STREAM_WARPS / 2; off > 0; off >>= 1) b = max(b, __shfl_xor_sync(0xFFFFFFFFu, b, off));
             if (lane == 0) {
                 TileRec r;
-                r.best = b; r.cnt = sh.ncand[s]; r.tkey = sh.tkey[s];
+                r.best = b; r.cnt = sh.ncand[s]; r.tkey = (unsigned int)(b >> 32);
                 r.flags = (sh.meta[s].bad || sh.badid[s]) ? TILE_BADID : 0u;
                 r.pad[0] = r.pad[1] = r.pad[2] = 0u;
                 P.tiles[(size_t)row * MAX_TILES + tile] = r;
@@ -1283,7 +1481,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                     m.patch = p_next.patch; m.npen = p_next.npen; m.nbias = p_next.nbias; m.hb = n % (NSTAGE + 1);
                     m.stop = 0;
                     m.bad = row_bad;
-                    sh.ncand[s] = 0u; sh.tkey[s] = 0u; sh.badid[s] = 0u;
+                    sh.ncand[s] = 0u; sh.badid[s] = 0u;
                     m.next_row = (hint >= 0) ? hint / tiles : -1;
                     m.next_tile = (hint >= 0) ? hint % tiles : -1;
                     // the first tile's copy is under way; nothing is copied for rows of the cluster kernel's class
@@ -1330,7 +1528,6 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         if (meta.stop) { KERNEL_T1(0); break; }
         const int row = meta.row, tile = meta.tile;
         const int tile_base = tile * CTA_TILE;
-        const int wbase = tile_base + warp * WARP_TILE;
         uint32_t mword = 0xFFFFFFFFu;
         if (P.bitmask) {
             mword = (row == pre_row && tile == pre_tile) ? mword_pre : load_mask_words(row, tile);
@@ -1342,6 +1539,11 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             const bool masked = (meta.cfg.z & M_GRAMMAR) != 0;
             const bool tail = tile_base + CTA_TILE > P.V;
             const int patch = meta.patch;
+            // word: which of the 32 consecutive elements from lane * 32 count.  Under a sparse mask (a grammar allows a few per
+            // cent of the ids) a lane walks its word's few set bits instead of 32 elements.
+            uint32_t word = masked ? mword : 0xFFFFFFFFu;
+            if (tail) { const int left = P.V - tile_base - warp * WARP_TILE - lane * 32; if (left < 32) word &= left > 0 ? (1u << left) - 1u : 0u; }
+            const bool sparse = masked && __all_sync(0xFFFFFFFFu, __popc(word) <= 8);
             float *ptile = (DT == 0) ? reinterpret_cast<float *>(stages + (size_t)s * STAGE_BYTES) : conv;    // fp32 view the sparse lists patch
             bool wide = DT == 0;                               // the warp's part is fp32 in ptile (else bf16 in the stage)
             const int lane0 = warp * WARP_TILE + lane * VEC;   // the lane's first element within the tile
@@ -1359,10 +1561,18 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             // penalties and biases commute with the mask (a masked logit stays -inf), so they are applied to the unmasked tile
             if (patch == 1) {
                 // the producer listed this tile's entries: every warp patches its own part, if there are any in it
+                // (that the mask allows)
                 const int npen = meta.npen, nbias = meta.nbias;
                 bool any = false;
-                for (int h = lane; h < npen; h += 32) any = any || (sh.pen[meta.hb][h].li / WARP_TILE == warp);
-                for (int h = lane; h < nbias; h += 32) any = any || (sh.bias[meta.hb][h].li / WARP_TILE == warp);
+                auto look = [&](const Hit *hits, int count) {
+                    for (int h0 = 0; h0 < count; h0 += 32) {
+                        const int li = (h0 + lane < count) ? hits[h0 + lane].li : -1;
+                        const uint32_t w = __shfl_sync(0xFFFFFFFFu, word, (li >> 5) & 31);
+                        any = any || (li >= 0 && li / WARP_TILE == warp && ((w >> (li & 31)) & 1u));
+                    }
+                };
+                look(sh.pen[meta.hb], npen);
+                look(sh.bias[meta.hb], nbias);
                 if (__any_sync(0xFFFFFFFFu, any)) {
                     const RowCfg c = meta.cfg;
                     if (DT == 1) { widen(); wide = true; }
@@ -1406,7 +1616,17 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             // Maxima of the lane's vectors.  ebits: which of its 32 elements count (allowed by the mask, inside the row).
             float mv[NV];
             uint32_t ebits = 0xFFFFFFFFu;
-            if (!masked && !tail) {
+            auto value = [&](int li) -> float {                // one element of the tile
+                return (DT == 1 && !wide) ? __uint_as_float((uint32_t)reinterpret_cast<const unsigned short *>(stage)[li] << 16) : ptile[li];
+            };
+            float h0 = -CUDART_INF_F, h1 = -CUDART_INF_F;      // maxima of the lane's two halves
+            if (sparse) {
+                for (uint32_t w = word; w; w &= w - 1u) {
+                    const int b = __ffs(w) - 1;
+                    const float v = value(warp * WARP_TILE + lane * 32 + b);
+                    if (b < 16) h0 = fmaxf(h0, v); else h1 = fmaxf(h1, v);
+                }
+            } else if (!masked && !tail) {
 #pragma unroll
                 for (int j = 0; j < NV; ++j) {
                     const int li = lane0 + j * 32 * VEC;
@@ -1431,10 +1651,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
 #pragma unroll
                 for (int j = 0; j < NV; ++j) {
                     const int li = lane0 + j * 32 * VEC;
-                    uint32_t bits = __shfl_sync(0xFFFFFFFFu, mword, (j * 32 * VEC + lane * VEC) >> 5) >> ((lane * VEC) & 31);
-                    if (!masked) bits = 0xFFFFFFFFu;
-                    if (tail) { const int left = P.V - tile_base - li; if (left < VEC) bits &= left > 0 ? (1u << left) - 1u : 0u; }
-                    bits &= (1u << VEC) - 1u;
+                    const uint32_t bits = (__shfl_sync(0xFFFFFFFFu, word, (j * 32 * VEC + lane * VEC) >> 5) >> ((lane * VEC) & 31)) & ((1u << VEC) - 1u);
                     ebits |= bits << (j * VEC);
                     float v[VEC];
                     if (DT == 1 && !wide) {
@@ -1454,13 +1671,23 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                     for (int q = 0; q < VEC; ++q) mv[j] = ((bits >> q) & 1u) ? fmaxf(mv[j], v[q]) : mv[j];
                 }
             }
-            float h0 = mv[0], h1 = mv[NV / 2];
+            if (!sparse) {
 #pragma unroll
-            for (int j = 1; j < NV / 2; ++j) { h0 = fmaxf(h0, mv[j]); h1 = fmaxf(h1, mv[NV / 2 + j]); }
+                for (int j = 0; j < NV / 2; ++j) { h0 = fmaxf(h0, mv[j]); h1 = fmaxf(h1, mv[NV / 2 + j]); }
+            }
             const float lm = fmaxf(h0, h1);
             // The elements of the lane's vectors whose maximum reaches t, one vector after the other (rare: read again):
             // f(value, index within the tile) for those that reach t.
             auto visit = [&](float t, auto f) {
+                if (sparse) {
+#pragma unroll 1
+                    for (uint32_t w = word; w; w &= w - 1u) {
+                        const int li = warp * WARP_TILE + lane * 32 + __ffs(w) - 1;
+                        const float v = value(li);
+                        if (v >= t) f(v, li);
+                    }
+                    return;
+                }
                 unsigned int vm = 0u;
 #pragma unroll
                 for (int j = 0; j < NV; ++j) vm |= (mv[j] >= t) ? (1u << j) : 0u;
@@ -1527,8 +1754,9 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                     }
                     }
                 };
+                // (many groups, many candidates: a cutoff per tile keeps them down)
                 float t = cut;
-                if (row != cut_row) {
+                if (row != cut_row || G > 8) {
                     const float g = group_cutoff();
                     if (lane == 0) sh.tw[s][warp] = g;
                     csync();
@@ -1544,21 +1772,62 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                     // (a tile that bounds nothing leaves the cutoff to the next one)
                     cut = t;
                     cut_row = (t > -CUDART_INF_F) ? row : -1;
-                } else if (G <= 8 && __popc(__ballot_sync(0xFFFFFFFFu, lm >= t)) > 28) {
+                } else if (__popc(__ballot_sync(0xFFFFFFFFu, lm >= t)) > 28) {
                     // far more candidates than the cutoff was meant for (values that depend on the position): the warp takes
                     // a cutoff of its own for this tile
                     t = fmaxf(t, group_cutoff());
                     if (t == CUDART_INF_F) t = cut;
                 }
-                if (lane == 0) atomicMax(&sh.tkey[s], okey(t));
+                const uint32_t wk = __reduce_max_sync(0xFFFFFFFFu, okey(lm));
+                if (lane == 0) sh.best[s][warp] = ((unsigned long long)okey(t) << 32) | wk;
                 // every finite element >= t goes to the tile's candidate slot
                 const float t2 = fmaxf(t, -CUDART_MAX_NORMAL_F);           // e >= t2  <=>  e >= t and e is not -inf
-                if (lm >= t2) {
+                unsigned int cand = __ballot_sync(0xFFFFFFFFu, lm >= t2);
+                if (cand) {
                     unsigned long long *dst = P.cand + (size_t)row * P.cand_stride + (size_t)tile * cap_t;
-                    visit(t2, [&](float z, int li) {
-                        const unsigned int pos = atomicAdd(&sh.ncand[s], 1u);
+                    auto put = [&](unsigned int pos, float z, int li) {
                         if ((int)pos < cap_t) dst[pos] = ((unsigned long long)okey(z) << 32) | (uint32_t)(~(uint32_t)(tile_base + li));
-                    });
+                    };
+                    if (sparse) {
+                        visit(t2, [&](float z, int li) { put(atomicAdd(&sh.ncand[s], 1u), z, li); });
+                    } else if (__popc(cand) <= 8) {
+                        // few lanes hold candidates: one after the other, its 32 elements across the warp
+                        while (cand) {
+                            const int L = __ffs(cand) - 1;
+                            cand &= cand - 1u;
+                            const int li = warp * WARP_TILE + (lane / VEC) * (32 * VEC) + L * VEC + (lane % VEC);
+                            const float z = value(li);
+                            const bool in = z >= t2 && ((__shfl_sync(0xFFFFFFFFu, ebits, L) >> lane) & 1u);
+                            const unsigned int m = __ballot_sync(0xFFFFFFFFu, in);
+                            unsigned int base = 0u;
+                            if (lane == 0) base = atomicAdd(&sh.ncand[s], (unsigned int)__popc(m));
+                            base = __shfl_sync(0xFFFFFFFFu, base, 0);
+                            if (in) put(base + __popc(m & ((1u << lane) - 1u)), z, li);
+                        }
+                    } else {
+                        // many: every lane marks its own, one reservation for the warp
+                        unsigned int cm = 0u;
+#pragma unroll
+                        for (int j = 0; j < NV; ++j) {
+                            if (__any_sync(0xFFFFFFFFu, mv[j] >= t2)) {
+#pragma unroll
+                                for (int q = 0; q < VEC; ++q) cm |= (value(lane0 + j * 32 * VEC + q) >= t2) ? (1u << (j * VEC + q)) : 0u;
+                            }
+                        }
+                        cm &= ebits;
+                        const int cnt = __popc(cm);
+                        int incl = cnt;
+#pragma unroll
+                        for (int off = 1; off < 32; off <<= 1) { const int o = __shfl_up_sync(0xFFFFFFFFu, incl, off); if (lane >= off) incl += o; }
+                        unsigned int base = 0u;
+                        if (lane == 31) base = atomicAdd(&sh.ncand[s], (unsigned int)incl);
+                        base = __shfl_sync(0xFFFFFFFFu, base, 31) + (unsigned int)(incl - cnt);
+                        while (cm) {
+                            const int b = __ffs(cm) - 1, li = lane0 + (b / VEC) * (32 * VEC) + (b % VEC);
+                            cm &= cm - 1u;
+                            put(base++, value(li), li);
+                        }
+                    }
                 }
                 __syncwarp();
             }
