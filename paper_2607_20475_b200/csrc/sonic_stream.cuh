@@ -1797,7 +1797,8 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                             cand &= cand - 1u;
                             const int li = warp * WARP_TILE + (lane / VEC) * (32 * VEC) + L * VEC + (lane % VEC);
                             const float z = value(li);
-                            const bool in = z >= t2 && ((__shfl_sync(0xFFFFFFFFu, ebits, L) >> lane) & 1u);
+                            const uint32_t eb = __shfl_sync(0xFFFFFFFFu, ebits, L);
+                            const bool in = z >= t2 && ((eb >> lane) & 1u);
                             const unsigned int m = __ballot_sync(0xFFFFFFFFu, in);
                             unsigned int base = 0u;
                             if (lane == 0) base = atomicAdd(&sh.ncand[s], (unsigned int)__popc(m));
