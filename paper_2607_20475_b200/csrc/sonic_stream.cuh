@@ -1228,17 +1228,20 @@ __device__ __forceinline__ float warp_cutoff(float g, bool tile_mode) {
 
 // What the producer hands to the consumers with each stage.
 struct StageMeta {
-    RowCfg cfg;
-    int row, tile;
-    int skip;                                  // the row belongs to the exact kernel: nothing was loaded
-    int patch;                                 // 0 none, 1 the producer filtered the lists into hits[], 2 consumers scan the lists
-    int npen, nbias;                           // hits of this tile
-    int hb;                                    // which hit buffer holds them
+    int row, tile, slot;                       // slot: the row's parameters and lists
+    int skip;                                  // the row belongs to another kernel: nothing to do
     int stop;                                  // no more tiles for this CTA (nothing else in the entry is valid)
-    int bad;                                   // the producer met a list id outside [0, V)
-    int next_row, next_tile;                   // the tile that follows (-1: none, or not known yet)
+    int next_row, next_tile;                   // the tile that probably follows (-1: none, or not known yet)
 };
-struct Hit { int li; int payload; };           // element within the tile; history count, or the bias as float bits
+struct Hit { int id; int payload; };           // a bias entry: token, value bits
+struct RowSlot {                               // a row's parameters and lists
+    RowCfg cfg;
+    int patch;                                 // 0 no lists, 1 they are here, 2 consumers scan them in global memory
+    int bad;                                   // a list id outside [0, V)
+    int off[MAX_TILES + 1];                    // the history entries of tile t: list[off[t], off[t + 1])
+    uint32_t list[FILTER_HIST];                // id | count << 18
+    Hit bias[FILTER_BIAS];
+};
 
 template <int DT>
 struct StreamShared {
@@ -1250,10 +1253,7 @@ struct StreamShared {
     alignas(16) float tw[NSTAGE][STREAM_WARPS];
     unsigned int ncand[NSTAGE], badid[NSTAGE];
     unsigned long long best[NSTAGE][STREAM_WARPS];       // greedy rows: argmax; top-k rows: cutoff key << 32 | key of the warp's maximum
-    uint32_t list[FILTER_HIST];                // the producer's: the row's history, id | count << 18 (0: no entry)
-    // hit lists: one buffer more than stages, so that the producer fills the next tile's while both stages are busy
-    Hit pen[NSTAGE + 1][HIT_PEN_CAP];
-    Hit bias[NSTAGE + 1][HIT_BIAS_CAP];
+    RowSlot slot[NSTAGE + 1];                  // the rows of the tiles in the ring and of the one that is prepared
 };
 
 template <int DT>
@@ -1282,20 +1282,15 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
     if (warp == STREAM_WARPS) {
         // ------------------------------------------------------------ producer warp
         // The (row, tile) items are handed out through a counter in the workspace, so CTAs that become resident
-        // late (the SMs may be shared with the exact kernel) find less or no work instead of holding back a fixed
-        // share.  Per tile the
-        // producer (1) waits for a free stage, describes the tile and issues its bulk copy, then (2) prepares
-        // the NEXT tile while the ring is busy.  On a new row that means one round of global loads (parameters
-        // and sparse lists, kept in registers for the row's other tiles); on every tile, picking the list
-        // entries that fall into it and writing them to a hit buffer, so that the consumers patch only what is
-        // there, each warp only its own part of the tile.
+        // late (the row kernel's clusters hold part of the chip) find less or no work instead of holding back a fixed
+        // share.  Per tile the producer waits for a free stage, requests the next tile at once, and only then writes the
+        // record of the tile that left the stage and the description of the new one: what it does by itself is one warp's
+        // serial work of several hundred cycles, which would otherwise lie between a stage's release and its next request.
+        // On a new row one round of global loads brings the parameters and lists into a slot in shared memory.
         static_assert(SONIC_MAX_VOCAB <= (1 << 18), "packed history entries hold an 18-bit id");
+        static_assert(CTA_TILE == 1 << 13, "tile of a token");
         constexpr int HALF = FILTER_HIST / 64;     // history entries per lane and round of loads
-        struct Prep { int patch, npen, nbias; };
-        RowCfg c_next;
-        int b_id = -1;
-        float b_val = 0.0f;
-        int row_patch = 0, cached_row = -1, row_bad = 0;
+        int cached_row = -1, cur_slot = 0, used_slot = 0, cls_cur = CLS_GREEDY;      // used_slot: of the last tile handed over (a row that is passed over uses none)
         auto load_row = [&](int row) {
             const int req = (P.op == OP_VERIFY) ? row / (P.K + 1) : row;
             const int *hid = P.hist_ids ? P.hist_ids + (size_t)req * P.hist_stride : nullptr;
@@ -1314,69 +1309,66 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             }
             int b0 = -1; float v0 = 0.0f;
             if (bid && bvl && lane < P.bias_stride) { b0 = __ldg(bid + lane); v0 = __ldg(bvl + lane); }
-            c_next = resolve_cfg(P, row, raw);
+            const RowCfg c = resolve_cfg(P, row, raw);
             cached_row = row;
-            row_patch = 0;
-            row_bad = 0;
-            if (c_next.cls == CLS_EXACT || !(c_next.hist_len > 0 || c_next.bias_len > 0)) return;
-            row_patch = 2;
-            if (c_next.hist_len > FILTER_HIST || c_next.bias_len > FILTER_BIAS) return;
+            cls_cur = c.cls;
+            cur_slot = (used_slot + 1) % (NSTAGE + 1);
+            RowSlot &q = sh.slot[cur_slot];
+            int patch = (c.hist_len > 0 || c.bias_len > 0) ? 1 : 0;
+            if (c.hist_len > FILTER_HIST || c.bias_len > FILTER_BIAS) patch = 2;
             bool bad = false, big = false;
-            auto pack = [&](int t, int i, int cnt) -> uint32_t {
-                if (t >= c_next.hist_len) return 0u;
-                if (i < 0 || i >= P.V) { bad = true; return 0u; }
-                if (cnt > FILTER_COUNT_MAX) { big = true; return 0u; }
-                return (cnt > 0) ? ((uint32_t)i | ((uint32_t)cnt << 18)) : 0u;
-            };
+            if (patch == 1) {
+                // the history by tile: count, offsets, place
+                q.off[lane] = 0;
+                __syncwarp();
+                uint32_t e[2 * HALF];
+                int at[2 * HALF];
+                auto take = [&](int t, int i, int cnt, uint32_t &out, int &rank) {
+                    out = 0u; rank = 0;
+                    if (t >= c.hist_len) return;
+                    if (i < 0 || i >= P.V) { bad = true; return; }
+                    if (cnt > FILTER_COUNT_MAX) { big = true; return; }
+                    if (cnt <= 0) return;
+                    out = (uint32_t)i | ((uint32_t)cnt << 18);
+                    rank = atomicAdd(&q.off[i >> 13], 1);
+                };
 #pragma unroll
-            for (int u = 0; u < HALF; ++u) sh.list[lane + 32 * u] = pack(lane + 32 * u, id[u], ct[u]);
-            if (c_next.hist_len > 32 * HALF) {
+                for (int u = 0; u < HALF; ++u) take(lane + 32 * u, id[u], ct[u], e[u], at[u]);
 #pragma unroll
-                for (int u = 0; u < HALF; ++u) {
-                    const int t = lane + 32 * (HALF + u);
-                    id[u] = -1; ct[u] = 0;
-                    if (t < c_next.hist_len) { id[u] = __ldg(hid + t); ct[u] = __ldg(hct + t); }
-                }
+                for (int u = 0; u < HALF; ++u) { e[HALF + u] = 0u; at[HALF + u] = 0; }
+                if (c.hist_len > 32 * HALF) {
 #pragma unroll
-                for (int u = 0; u < HALF; ++u) sh.list[lane + 32 * (HALF + u)] = pack(lane + 32 * (HALF + u), id[u], ct[u]);
-            }
-            b_id = -1; b_val = 0.0f;
-            if (lane < c_next.bias_len) {
-                if (b0 < 0 || b0 >= P.V) bad = true;
-                else { b_id = b0; b_val = v0; }
-            }
-            row_bad = __any_sync(0xFFFFFFFFu, bad) ? 1 : 0;
-            if (__any_sync(0xFFFFFFFFu, big)) return;          // a count too large to pack: consumers scan
-            row_patch = 1;
-        };
-        auto prepare = [&](int tile, int hb) -> Prep {
-            Prep r{row_patch, 0, 0};
-            if (row_patch != 1) return r;
-            const int first = tile * CTA_TILE;
-#pragma unroll 4
-            for (int t = lane; t < ((c_next.hist_len + 31) & ~31); t += 32) {      // (a lane reads the entries it wrote)
-                const uint32_t e = sh.list[t];
-                const unsigned int li = (e & 0x3FFFFu) - (unsigned int)first;
-                const bool hit = e != 0u && li < (unsigned int)CTA_TILE;
-                const unsigned int hm = __ballot_sync(0xFFFFFFFFu, hit);
-                if (hit) {
-                    const int pos = r.npen + __popc(hm & ((1u << lane) - 1u));
-                    if (pos < HIT_PEN_CAP) { sh.pen[hb][pos].li = (int)li; sh.pen[hb][pos].payload = (int)(e >> 18); }
+                    for (int u = 0; u < HALF; ++u) {
+                        const int t = lane + 32 * (HALF + u);
+                        id[u] = -1; ct[u] = 0;
+                        if (t < c.hist_len) { id[u] = __ldg(hid + t); ct[u] = __ldg(hct + t); }
+                    }
+#pragma unroll
+                    for (int u = 0; u < HALF; ++u) take(lane + 32 * (HALF + u), id[u], ct[u], e[HALF + u], at[HALF + u]);
                 }
-                r.npen += __popc(hm);
-            }
-            {
-                const unsigned int li = (unsigned int)(b_id - first);
-                const bool hit = b_id >= 0 && li < (unsigned int)CTA_TILE;
-                const unsigned int hm = __ballot_sync(0xFFFFFFFFu, hit);
-                if (hit) {
-                    const int pos = __popc(hm & ((1u << lane) - 1u));
-                    sh.bias[hb][pos].li = (int)li; sh.bias[hb][pos].payload = __float_as_int(b_val);
+                __syncwarp();
+                const int cnt = q.off[lane];
+                int incl = cnt;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) { const int up = __shfl_up_sync(0xFFFFFFFFu, incl, o); if (lane >= o) incl += up; }
+                q.off[lane] = incl - cnt;
+                if (lane == 31) q.off[32] = incl;
+                __syncwarp();
+#pragma unroll
+                for (int u = 0; u < 2 * HALF; ++u)
+                    if (e[u]) q.list[q.off[(e[u] & 0x3FFFFu) >> 13] + at[u]] = e[u];
+                Hit h;
+                h.id = -1; h.payload = 0;
+                if (lane < c.bias_len) {
+                    if (b0 < 0 || b0 >= P.V) bad = true;
+                    else { h.id = b0; h.payload = __float_as_int(v0); }
                 }
-                r.nbias = __popc(hm);
+                q.bias[lane] = h;
+                bad = __any_sync(0xFFFFFFFFu, bad);
+                if (__any_sync(0xFFFFFFFFu, big)) patch = 2;       // a count too large to pack: consumers scan
             }
-            if (r.npen > HIT_PEN_CAP) r.patch = 2;             // crowded tile: the consumers scan the lists
-            return r;
+            if (lane == 0) { q.cfg = c; q.patch = patch; q.bad = bad ? 1 : 0; }
+            __syncwarp();
         };
         const unsigned long long l2_policy = l2_evict_first_policy();
         // Work queue: one counter of items.  A CTA first asks for `chunk` consecutive items (seven eighths of an
@@ -1406,12 +1398,11 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 if (it < 0) return -1;
                 const int row = it / tiles;
                 if (row != cached_row) load_row(row);
-                if (!pass || P.op == OP_TOPK || !class_is_listed(c_next.cls)) return it;
+                if (!pass || P.op == OP_TOPK || !class_is_listed(cls_cur)) return it;
                 run_lo = min(run_hi, (row + 1) * tiles) - 1;
                 advance();
             }
         };
-        Prep p_next{0, 0, 0};
         int item = current_item();
         // lane 0: the tile's bulk copy, with the arrival on full[s] (arrive == true) or with the bytes announced only
         // (the arrival then follows once the stage's description is written)
@@ -1441,14 +1432,15 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 if (tile == 0 && lane == 0 && P.op == OP_TOPK) { P.rs[row].status = 0u; atomicAdd(&P.error[WS_NEXACT], 1u); }
                 return;
             }
+            const RowSlot &q = sh.slot[sh.meta[s].slot];
             unsigned long long b = (lane < STREAM_WARPS) ? sh.best[s][lane] : 0ull;
-            if (lane < STREAM_WARPS && sh.meta[s].cfg.cls == CLS_TOPK) P.wmax[((size_t)row * MAX_TILES + tile) * STREAM_WARPS + lane] = (uint32_t)b;
+            if (lane < STREAM_WARPS && q.cfg.cls == CLS_TOPK) P.wmax[((size_t)row * MAX_TILES + tile) * STREAM_WARPS + lane] = (uint32_t)b;
 #pragma unroll
             for (int off = STREAM_WARPS / 2; off > 0; off >>= 1) b = max(b, __shfl_xor_sync(0xFFFFFFFFu, b, off));
             if (lane == 0) {
                 TileRec r;
                 r.best = b; r.cnt = sh.ncand[s]; r.tkey = (unsigned int)(b >> 32);
-                r.flags = (sh.meta[s].bad || sh.badid[s]) ? TILE_BADID : 0u;
+                r.flags = (q.bad || sh.badid[s]) ? TILE_BADID : 0u;
                 r.pad[0] = r.pad[1] = r.pad[2] = 0u;
                 P.tiles[(size_t)row * MAX_TILES + tile] = r;
                 if (tile == 0) P.rs[row].status = 0u;
@@ -1459,40 +1451,38 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         for (;; ++n) {                                 // (round -1 only prepares the first tile)
             if (n >= 0) {
                 const int s = n % NSTAGE;
+                const bool skip = item >= 0 && class_is_listed(cls_cur);
+                const int row = item / tiles, tile = item - row * tiles;
                 if (n >= NSTAGE) {
-                    // the consumers have left tile n - NSTAGE: its stage and its hit buffer are free
+                    // the consumers have left tile n - NSTAGE: its stage is free
                     if (!mbar_wait(&sh.empty[s], ((n / NSTAGE) - 1) & 1)) {
                         if (lane == 0) atomicOr(P.error, ERR_TIMEOUT);
                         return;
                     }
+                    // (the first tiles' copies are under way; nothing is copied for rows of the cluster kernel's class)
+                    if (item >= 0 && !skip && lane == 0) issue_copy(row, tile, s, false);
                     retire(s);
                 }
                 if (item < 0) {                            // out of work: tell the consumers
                     if (lane == 0) { sh.meta[s].stop = 1; mbar_arrive(&sh.full[s]); }
                     break;
                 }
-                const int row = item / tiles, tile = item - row * tiles;
+                used_slot = cur_slot;
                 advance();
                 const int hint = current_item();           // (the tile that follows, unless its row is passed over)
-                __syncwarp();                              // the hit buffer's entries, written by all lanes, precede the arrival
                 if (lane == 0) {
+                    if (n > 0 && n < NSTAGE && !skip) issue_copy(row, tile, s, false);
                     StageMeta &m = sh.meta[s];
-                    m.cfg = c_next; m.row = row; m.tile = tile; m.skip = class_is_listed(c_next.cls) ? 1 : 0;
-                    m.patch = p_next.patch; m.npen = p_next.npen; m.nbias = p_next.nbias; m.hb = n % (NSTAGE + 1);
+                    m.row = row; m.tile = tile; m.slot = cur_slot; m.skip = skip ? 1 : 0;
                     m.stop = 0;
-                    m.bad = row_bad;
-                    sh.ncand[s] = 0u; sh.badid[s] = 0u;
                     m.next_row = (hint >= 0) ? hint / tiles : -1;
-                    m.next_tile = (hint >= 0) ? hint % tiles : -1;
-                    // the first tile's copy is under way; nothing is copied for rows of the cluster kernel's class
-                    if (n == 0 || m.skip) mbar_arrive(&sh.full[s]);
-                    else issue_copy(row, tile, s, true);
+                    m.next_tile = (hint >= 0) ? hint - m.next_row * tiles : -1;
+                    sh.ncand[s] = 0u; sh.badid[s] = 0u;
+                    mbar_arrive(&sh.full[s]);
                 }
                 __syncwarp();
             }
-            // hit buffer (n + 1) % (NSTAGE + 1) was last used by tile n - NSTAGE, which the consumers have left
             item = find_item(n >= 0);
-            if (item >= 0) p_next = prepare(item % tiles, (n + 1) % (NSTAGE + 1));
         }
         for (int i = max(0, n - NSTAGE + 1); i < n; ++i) {     // the last tiles
             if (!mbar_wait(&sh.empty[i % NSTAGE], (i / NSTAGE) & 1)) {
@@ -1536,9 +1526,10 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         }
         if (!meta.skip) {
             const unsigned char *stage = stages + (size_t)s * STAGE_BYTES;
-            const bool masked = (meta.cfg.z & M_GRAMMAR) != 0;
+            const RowSlot &slot = sh.slot[meta.slot];
+            const bool masked = (slot.cfg.z & M_GRAMMAR) != 0;
             const bool tail = tile_base + CTA_TILE > P.V;
-            const int patch = meta.patch;
+            const int patch = slot.patch;
             // word: which of the 32 consecutive elements from lane * 32 count.  Under a sparse mask (a grammar allows a few per
             // cent of the ids) a lane walks its word's few set bits instead of 32 elements.
             uint32_t word = masked ? mword : 0xFFFFFFFFu;
@@ -1562,35 +1553,42 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             if (patch == 1) {
                 // the producer listed this tile's entries: every warp patches its own part, if there are any in it
                 // (that the mask allows)
-                const int npen = meta.npen, nbias = meta.nbias;
-                bool any = false;
-                auto look = [&](const Hit *hits, int count) {
-                    for (int h0 = 0; h0 < count; h0 += 32) {
-                        const int li = (h0 + lane < count) ? hits[h0 + lane].li : -1;
-                        const uint32_t w = __shfl_sync(0xFFFFFFFFu, word, (li >> 5) & 31);
-                        any = any || (li >= 0 && li / WARP_TILE == warp && ((w >> (li & 31)) & 1u));
-                    }
+                const int first = slot.off[tile], npen = slot.off[tile + 1] - first, nbias = slot.cfg.bias_len;
+                auto mine = [&](int li) -> bool {                // (every lane calls it; li: element of the tile, or anything outside)
+                    const uint32_t w = __shfl_sync(0xFFFFFFFFu, word, (li >> 5) & 31);
+                    return (li >> 10) == warp && ((w >> (li & 31)) & 1u);
                 };
-                look(sh.pen[meta.hb], npen);
-                look(sh.bias[meta.hb], nbias);
+                static_assert(WARP_TILE == 1024 && FILTER_BIAS == 32, "element -> warp; one bias entry per lane");
+                bool any = false;
+                for (int h0 = 0; h0 < npen; h0 += 32) {
+                    const bool m = mine((h0 + lane < npen) ? (int)(slot.list[first + h0 + lane] & 0x3FFFFu) - tile_base : -1);
+                    any = any || m;
+                }
+                int bli = -1;
+                float bval = 0.0f;
+                if (nbias > 0) {
+                    const Hit h = slot.bias[lane];
+                    bli = (h.id >= 0) ? h.id - tile_base : -1;
+                    bval = __int_as_float(h.payload);
+                    if (!mine(bli)) bli = -1;
+                    any = any || bli >= 0;
+                }
                 if (__any_sync(0xFFFFFFFFu, any)) {
-                    const RowCfg c = meta.cfg;
+                    const RowCfg c = slot.cfg;
                     if (DT == 1) { widen(); wide = true; }
                     __syncwarp();
                     for (int h = lane; h < npen; h += 32) {
-                        const Hit x = sh.pen[meta.hb][h];
-                        if (x.li / WARP_TILE == warp) ptile[x.li] = apply_penalties(ptile[x.li], x.payload, c);
+                        const uint32_t e = slot.list[first + h];
+                        const int li = (int)(e & 0x3FFFFu) - tile_base;
+                        if ((li >> 10) == warp) ptile[li] = apply_penalties(ptile[li], (int)(e >> 18), c);
                     }
                     __syncwarp();
-                    for (int h = lane; h < nbias; h += 32) {
-                        const Hit x = sh.bias[meta.hb][h];
-                        if (x.li / WARP_TILE == warp) ptile[x.li] = __fadd_rn(ptile[x.li], __int_as_float(x.payload));
-                    }
+                    if (bli >= 0) ptile[bli] = __fadd_rn(ptile[bli], bval);
                     __syncwarp();
                 }
             } else if (patch == 2) {
                 // long or crowded lists: all consumer threads scan them together
-                const RowCfg c = meta.cfg;
+                const RowCfg c = slot.cfg;
                 if (DT == 1) { widen(); wide = true; csync(); }
                 const int req = (P.op == OP_VERIFY) ? row / (P.K + 1) : row;
                 const int *hid = P.hist_ids + (size_t)req * P.hist_stride;
@@ -1711,14 +1709,14 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 }
             };
 
-            if (meta.cfg.cls == CLS_GREEDY) {
+            if (slot.cfg.cls == CLS_GREEDY) {
                 // The argmax of the processed logits, lowest index first.  Only elements at or above the largest so far can
                 // matter (with a temperature: above a hair less, since the division may make them equal).
                 if (row != g_row) { g_row = row; g_thr = -CUDART_MAX_NORMAL_F; }
                 unsigned long long best = 0ull;
                 if (__any_sync(0xFFFFFFFFu, lm >= g_thr)) {
-                    const bool temp = meta.cfg.temp;
-                    const float tau = meta.cfg.tau;
+                    const bool temp = slot.cfg.temp;
+                    const float tau = slot.cfg.tau;
                     if (lm >= g_thr) visit(g_thr, [&](float z, int li) {
                         const uint32_t key = okey(temp ? div_tau(z, tau) : z);
                         best = max(best, ((unsigned long long)key << 32) | (uint32_t)(~(uint32_t)(tile_base + li)));
@@ -1732,8 +1730,8 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 }
                 if (lane == 0) sh.best[s][warp] = best;
             } else {
-                const int G = meta.cfg.G;
-                const bool tmin = meta.cfg.tile_min;
+                const int G = slot.cfg.G;
+                const bool tmin = slot.cfg.tile_min;
                 // warp cutoff: minimum over G groups of the group maximum.  Tile cutoff: the largest of the eight warp cutoffs
                 // (warp mode) or the smallest (tile mode: a minimum over all 8 G groups of the tile).  In tile mode a group
                 // without a finite element (masked, or past the row's end) does not take part: it would drag the cutoff
