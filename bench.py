@@ -53,14 +53,16 @@ def profiled_traffic(name: str):
 
 
 def launches_per_call(name: str, w) -> int:
-    """Kernels one call enqueues.  A call whose rows fit the chip at once is one launch of the row kernel.  Larger sampling
-    calls: row kernel (rows with top-k off), streaming, merge, cluster kernel; verification adds the combine kernel;
-    sonic_topk has no rows with top-k off."""
+    """Kernels one call enqueues.  Sampling: streaming, merge, histogram pass, collect pass, row finish, cluster kernel.
+    Verification adds the residual pass, the residual draw and the combine kernel.  (sonic_topk: streaming, merge,
+    cluster kernel.)  A call whose rows fit the chip at once is one launch of the row kernel."""
     if name == "c1":
         return 1
     if name == "c4":
-        return 5
-    return 3 if name.startswith("c5") else 4
+        return 9 if w.K > 0 else 7
+    if name.startswith("c5"):
+        return 3
+    return 6
 
 
 def peaks():

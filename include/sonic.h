@@ -49,13 +49,14 @@ extern "C" {
 #define SONIC_FLAG_BADPARAM  0x2u   /* tau <= 0, p or theta outside (0,1], k < 0, list id out of range: token is -1 */
 #define SONIC_FLAG_FALLBACK  0x4u   /* diagnostic: the row was finished by the cluster kernel (top-k beyond the streaming
                                        path, or a row no other path could finish) */
-#define SONIC_FLAG_DENSE     0x8u   /* diagnostic: top-k off, the row was finished over the whole vocabulary */
+#define SONIC_FLAG_DENSE     0x8u   /* diagnostic: top-k off, the row was finished by the full-vocabulary histogram passes */
 #define SONIC_FLAG_TIMEOUT   0x10u  /* a bounded wait inside the streaming kernel expired: token is -1 (see sonic_workspace_init) */
 
 /* Bytes of workspace that serve every call over at most max_rows logit rows (B for sonic_sample / sonic_topk,
  * B*(K+1) for sonic_verify) of at most max_vocab entries each, and every sonic_topk call with k <= max_topk.  Pure
- * host arithmetic.  Per row: 1.1 KB of control words and 8 bytes per candidate slot (sampling and verification: min(131072, V
- * rounded up to 8192); sonic_topk needs a quarter of that, half with k > 2048). */
+ * host arithmetic.  Per row: 1.3 KB of control words, 8 bytes per candidate slot (min(32768, V rounded up to 8192);
+ * twice as many for sonic_topk with k > 2048), and for sampling and verification 4 bytes per vocabulary entry (the
+ * processed logits of rows with top-k off as ordered keys) plus 58 KB of histogram and lists. */
 size_t sonic_workspace_bytes(int max_rows, int max_vocab, int max_topk);
 
 /* Zeroes the workspace header (the first 17 KB: work counters, the sticky error word, a ticket per request) once after allocation
@@ -68,8 +69,17 @@ size_t sonic_workspace_bytes(int max_rows, int max_vocab, int max_topk);
  * (a tile copy that never completed) ran out.  Every row of such a call, and of later calls on that workspace,
  * reports SONIC_FLAG_TIMEOUT with token -1 until the workspace is initialised again with this function.
  *
- * Streams: all of a call's kernels go to the caller's `stream` (everything enqueued before the call precedes them,
- * everything after follows them). */
+ * Streams: a call's kernels are ordered on the caller's `stream` (everything enqueued before the call precedes
+ * them, everything after follows them).  A call of few rows is one kernel on that stream; the rest of this paragraph is
+ * about larger calls.  Per host thread and device the library keeps ONE internal non-blocking stream
+ * and two events, created by this function or by the thread's first sampling call outside a stream capture:
+ * sonic_sample / sonic_verify fork it from `stream` behind their first kernel and join it back before their last
+ * one, so that rows with and without top-k are finished side by side.  Under stream capture the fork is captured
+ * with the caller's stream (one graph, no dependency outside it).  Whenever the internal stream cannot be used -
+ * it does not exist yet and the caller is capturing, or it still belongs to another capture that is open - the
+ * call runs all of its kernels on `stream` alone: same results, about a third slower on mixed batches.  So: call
+ * this function (or one eager sampling call) on a thread before that thread captures, and do not keep two captures
+ * open on one thread at the same time if both should get the two-stream schedule.  sonic_topk uses no other stream. */
 int sonic_workspace_init(void *workspace, size_t bytes, void *stream);
 
 /*

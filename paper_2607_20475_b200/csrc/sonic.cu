@@ -8,6 +8,7 @@
 
 #include "../../include/sonic.h"
 #include "sonic_common.cuh"
+#include "sonic_dense.cuh"
 #include "sonic_stream.cuh"
 #include "sonic_exact.cuh"
 #include "sonic_row.cuh"
@@ -59,6 +60,8 @@ constexpr int STREAM_SMEM_F32 = VecTraits<0>::NSTAGE * CTA_TILE * 4 + (int)sizeo
 constexpr int STREAM_SMEM_BF16 = VecTraits<1>::NSTAGE * CTA_TILE * 2 + CTA_TILE * 4 + (int)sizeof(StreamShared<1>);
 constexpr int EXACT_CLUSTERS = 4;             // clusters of the cluster kernel (its rows are rare)
 constexpr int EXACT_SMEM = SLICE_MAX * 4 + HBINS * 16 + 8192 + MAX_TOPK * 8 + 8192;
+static_assert(MERGE_SMEM >= DENSE_DYN_SMEM, "stage 2 of the histogram path runs in the merge kernel's shared memory");
+static_assert(DENSE_THREADS == MERGE_THREADS, "stage 2 of the histogram path runs in the merge kernel's CTAs");
 
 static thread_local char g_err[256] = "";
 
@@ -72,31 +75,39 @@ static int fail_cuda(cudaError_t e, const char *what) {
 }
 
 // Workspace layout.  Only the header (WS_HEADER bytes at offset 0) is shared by all calls and must be zero between
-// them; everything behind it is laid out for the shape of the call at hand (rows, V, operation) and initialised by the call's own kernels, so one workspace serves calls of any shape that fits.
+// them; everything behind it is laid out for the shape of the call at hand (rows, V, whether the histogram path
+// can be taken) and initialised by the call's own kernels, so one workspace serves calls of any shape that fits.
 struct Layout {
-    size_t rs, pr, tiles, wmax, cand, total;
+    size_t rs, pr, tiles, wmax, cand, drow, dtile, dlist, rlist, hist, members, ykeys, total;
     unsigned int cand_stride;
+    int ytiles;
 };
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
-// Candidate slots per row: SAMPLE_CAP for sampling; for sonic_topk CAND_CAP, twice that with k beyond 2048 (its tiles bring
-// up to ~1100 candidates each at k = 4096, V = 2^18, where an even share of CAND_CAP is 1024); never more than the row has
-// elements.
-static size_t slot_cap(int op, int ktop) {
-    if (op != OP_TOPK) return (size_t)SAMPLE_CAP;
-    return ktop > 2048 ? 2 * (size_t)CAND_CAP : (size_t)CAND_CAP;
-}
-static Layout layout_for(long long rows, int V, size_t cap) {
+// Candidate slots per row: CAND_CAP, twice that for sonic_topk with k beyond 2048 (its tiles bring up to ~1100
+// candidates each at k = 4096, V = 2^18, where an even share of CAND_CAP is 1024), never more than the row has elements.
+static size_t slot_cap(int op, int ktop) { return (op == OP_TOPK && ktop > 2048) ? 2 * (size_t)CAND_CAP : (size_t)CAND_CAP; }
+static Layout layout_for(long long rows, int V, bool dense, size_t cap = CAND_CAP) {
     Layout L;
     memset(&L, 0, sizeof(L));
     const int tiles = (V + CTA_TILE - 1) / CTA_TILE;
     const size_t slots = (size_t)tiles * CTA_TILE < cap ? (size_t)tiles * CTA_TILE : cap;
     L.cand_stride = (unsigned int)slots;
+    L.ytiles = tiles;
     size_t off = WS_HEADER;
     L.rs = off;    off = align256(off + (size_t)rows * sizeof(RowState));
     L.pr = off;    off = align256(off + (size_t)rows * sizeof(PosResult));
     L.tiles = off; off = align256(off + (size_t)rows * sizeof(TileRec) * MAX_TILES);
     L.wmax = off;  off = align256(off + (size_t)rows * MAX_TILES * STREAM_WARPS * 4);
     L.cand = off;  off = align256(off + (size_t)rows * slots * 8);
+    if (dense) {
+        L.drow = off;    off = align256(off + (size_t)rows * sizeof(DenseRow));
+        L.dtile = off;   off = align256(off + (size_t)rows * sizeof(DenseTile) * MAX_TILES);
+        L.dlist = off;   off = align256(off + (size_t)rows * 4);
+        L.rlist = off;   off = align256(off + (size_t)rows * 4);
+        L.hist = off;    off = align256(off + (size_t)rows * DBINS * 8);
+        L.members = off; off = align256(off + (size_t)rows * MEMBER_CAP * 8);
+        L.ykeys = off;   off = align256(off + (size_t)rows * tiles * CTA_TILE * 4);
+    }
     L.total = off;
     return L;
 }
@@ -138,7 +149,6 @@ static const GroupTable &group_table(int V) {
 }
 
 static int g_sm_count[64];
-static int g_clusters[64][ROW_CMAX + 1];           // clusters of so many CTAs of the row kernel that are resident at once
 
 static int configure_once(int *sm_count, int *device) {
     static std::once_flag once[64];
@@ -154,27 +164,16 @@ static int configure_once(int *sm_count, int *device) {
             if (r == cudaSuccess) r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         };
         set((const void *)sonic_merge_kernel, MERGE_SMEM);
+        set((const void *)sonic_dense_collect_kernel, DENSE_DYN_SMEM);
+        set((const void *)sonic_dense_stage2_kernel, DENSE_DYN_SMEM);
+        set((const void *)sonic_dense_finish_kernel, DENSE_DYN_SMEM);
         set((const void *)sonic_stream_kernel<0>, STREAM_SMEM_F32);
         set((const void *)sonic_stream_kernel<1>, STREAM_SMEM_BF16);
         if (r == cudaSuccess) r = cudaDeviceGetAttribute(&g_sm_count[dev], cudaDevAttrMultiProcessorCount, dev);
-        for (const void *f : {(const void *)sonic_row_kernel<0, false>, (const void *)sonic_row_kernel<1, false>,
-                              (const void *)sonic_row_kernel<0, true>, (const void *)sonic_row_kernel<1, true>}) {
-            set(f, ROW_DYN_SMEM);
+        set((const void *)sonic_row_kernel<0>, ROW_DYN_SMEM);
+        set((const void *)sonic_row_kernel<1>, ROW_DYN_SMEM);
+        for (const void *f : {(const void *)sonic_row_kernel<0>, (const void *)sonic_row_kernel<1>})
             if (r == cudaSuccess) r = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);      // (clusters of up to 16)
-        }
-        for (int C = ROW_CMIN; C <= ROW_CMAX && r == cudaSuccess; ++C) {
-            cudaLaunchAttribute attr;
-            attr.id = cudaLaunchAttributeClusterDimension;
-            attr.val.clusterDim.x = C; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-            cudaLaunchConfig_t cfg;
-            memset(&cfg, 0, sizeof(cfg));
-            cfg.gridDim = dim3(C);
-            cfg.blockDim = dim3(ROW_THREADS);
-            cfg.dynamicSmemBytes = ROW_DYN_SMEM;
-            cfg.attrs = &attr;
-            cfg.numAttrs = 1;
-            r = cudaOccupancyMaxActiveClusters(&g_clusters[dev][C], (const void *)sonic_row_kernel<0, true>, &cfg);
-        }
         set((const void *)sonic_exact_kernel<0>, EXACT_SMEM);
         set((const void *)sonic_exact_kernel<1>, EXACT_SMEM);
         int n = 0;
@@ -201,6 +200,45 @@ static int configure_once(int *sm_count, int *device) {
     return SONIC_OK;
 }
 
+// Per host thread and device: one internal stream and two events, so that the histogram passes (rows with top-k off)
+// run beside the merges (rows with top-k) instead of behind them.  A call forks the stream from the caller's after
+// the streaming kernel and joins it before the call's last kernel; under stream capture it is captured with the
+// caller's stream.  Created by the thread's first call on a device outside a capture; whenever the stream cannot
+// be used safely (not created yet and the caller is capturing; still part of another, open capture) the call runs all
+// of its kernels on the caller's stream instead, with the same results.
+struct SideStream {
+    cudaStream_t s = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
+    bool tried = false, ok = false;
+    ~SideStream() {
+        if (join) cudaEventDestroy(join);
+        if (fork) cudaEventDestroy(fork);
+        if (s) cudaStreamDestroy(s);
+    }
+};
+static thread_local SideStream g_side[64];
+
+static SideStream *side_stream_for(int dev, cudaStream_t st) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone, ss = cudaStreamCaptureStatusNone;
+    unsigned long long cid = 0, sid = 0;
+    if (cudaStreamGetCaptureInfo(st, &cs, &cid) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    if (cs == cudaStreamCaptureStatusInvalidated) return nullptr;
+    SideStream &S = g_side[dev];
+    if (!S.tried) {
+        if (cs != cudaStreamCaptureStatusNone) return nullptr;          // (nothing is created while a capture is open)
+        S.tried = true;
+        S.ok = cudaStreamCreateWithFlags(&S.s, cudaStreamNonBlocking) == cudaSuccess &&
+               cudaEventCreateWithFlags(&S.fork, cudaEventDisableTiming) == cudaSuccess &&
+               cudaEventCreateWithFlags(&S.join, cudaEventDisableTiming) == cudaSuccess;
+        if (!S.ok) cudaGetLastError();
+    }
+    if (!S.ok) return nullptr;
+    if (cudaStreamGetCaptureInfo(S.s, &ss, &sid) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    if (ss == cudaStreamCaptureStatusInvalidated) return nullptr;
+    if (ss == cudaStreamCaptureStatusActive && !(cs == cudaStreamCaptureStatusActive && cid == sid)) return nullptr;   // busy in another capture
+    return &S;
+}
+
 // Whether a call goes to the row kernel as a whole: when all of its rows' clusters are resident at once (two CTAs per SM).
 // Measured (us per call, streaming chain against row kernel): one bf16 row of 131072 with top-k 25.7 -> 13.6; 3 x 3
 // verification rows of 32003 47 -> 27; 37 fp32 rows of 50021 of every kind 48.8 -> 40.7; 32 bf16 rows of 100003 without
@@ -216,52 +254,45 @@ static bool row_route(const KParams &P, int sm_count) {
 #endif
 }
 
-// The row kernel over every row of the call, or (listed) over the rows that the streaming kernel leaves to it.  The number
-// of those is not known here: a quarter of the rows is expected, the clusters share them out among themselves, and those
-// that find none leave after a look at the parameters.  CTAs of a row's cluster: as many as are resident for this number of
-// rows, so that every CTA has few elements (a step costs 64 cycles per instruction and 8192 elements), within what a slice
-// can be.
-static cudaError_t launch_rows(const KParams &P, cudaStream_t st, int dev, bool listed) {
-    const int sm_count = g_sm_count[dev];
+// CTAs of a row's cluster: as many as are resident for this number of rows, so that every CTA has few elements (a step
+// costs 64 cycles per instruction and 8192 elements), within what a slice can be.
+static cudaError_t launch_rows(const KParams &P, cudaStream_t st, int sm_count) {
     const int cmin = std::max(ROW_CMIN, (P.V + ROW_SLICE_MAX - 1) / ROW_SLICE_MAX);
     const int cmax = std::min(ROW_CMAX, std::max(cmin, (P.V + ROW_UNIT - 1) / ROW_UNIT));
-    const int fit = 2 * sm_count / (listed ? (P.rows + 3) / 4 : P.rows);
+    const int fit = (int)(2ll * sm_count / P.rows);
     int C = 1;
     while (C * 2 <= std::min(fit, cmax)) C *= 2;
     C = std::max(C, cmin);
     const int per = (P.V + C - 1) / C, slice = (per + ROW_UNIT - 1) / ROW_UNIT * ROW_UNIT;
-    const int clusters = listed ? std::max(1, std::min(P.rows, g_clusters[dev][C])) : P.rows;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = C; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.stream = st;
-    cfg.gridDim = dim3((unsigned)clusters * C);
+    cfg.gridDim = dim3((unsigned)P.rows * C);
     cfg.blockDim = dim3(ROW_THREADS);
     cfg.dynamicSmemBytes = ROW_DYN_SMEM;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    const bool f32 = P.dtype == SONIC_DTYPE_F32;
-    if (listed) return cudaLaunchKernelEx(&cfg, f32 ? sonic_row_kernel<0, true> : sonic_row_kernel<1, true>, P, slice);
-    return cudaLaunchKernelEx(&cfg, f32 ? sonic_row_kernel<0, false> : sonic_row_kernel<1, false>, P, slice);
+    return P.dtype == SONIC_DTYPE_F32 ? cudaLaunchKernelEx(&cfg, sonic_row_kernel<0>, P, slice)
+                                      : cudaLaunchKernelEx(&cfg, sonic_row_kernel<1>, P, slice);
 }
 
-// A call whose rows do not all fit the chip at once, on the caller's stream:
-//   row kernel (rows with top-k off or beyond the streaming path; not in sonic_topk)
-//   -> stream kernel -> merge kernel (the others) -> cluster kernel -> [verification scan]
-// The stream kernel is a programmatic dependent of the row kernel that never waits for it: it starts once the row kernel's
-// clusters (no more than are resident at once) have found their places, takes what they leave of the chip and shares the
-// tiles out through a queue, so both run side by side.  In the other order its persistent CTAs would fill every SM first
-// and the clusters would only start behind them.  The merge kernel is a programmatic dependent of the stream kernel and
-// waits for it; the cluster kernel is an ordinary launch behind everything (in a captured call the row kernel is added to
-// its dependencies, since the merge kernel does not stand for it).
+// One call = a chain of kernels on the caller's stream.  Up to the residual pass each is a programmatic dependent
+// of the one before (it may begin launching while its predecessor runs; the paper overlaps its two stages the
+// same way, Section 3.5):
+//   stream kernel -> merge kernel (rows with top-k)
+//                 \-> [histogram pass -> its row step -> collect pass -> its row step -> residual pass]   (rows with top-k off)
+//   -> cluster kernel (an ordinary launch after all of it: rows no other path finished; usually none) -> [verification scan]
+// The second line runs on the thread's internal stream beside the merges when that stream can be used, else behind
+// them on the caller's stream.
 // clear: the header may hold anything (sonic_topk_static's array keeps what the previous call left).
 static int launch_all(KParams &P, void *ws, size_t ws_bytes, cudaStream_t st, int B_requests, bool clear = false) {
     if (!ws) return fail(SONIC_EINVAL, "workspace is NULL");
     if (((uintptr_t)ws & 255) != 0) return fail(SONIC_EINVAL, "workspace must be 256-byte aligned");
-    const bool sampling = (P.op != OP_TOPK);
-    const Layout L = layout_for(P.rows, P.V, slot_cap(P.op, P.ktop));
+    const bool dense = (P.op != OP_TOPK);
+    const Layout L = layout_for(P.rows, P.V, dense, slot_cap(P.op, P.ktop));
     if (ws_bytes < L.total) return fail(SONIC_EWORKSPACE, "workspace too small for this many rows of this vocabulary size");
     int sm_count = 1, dev = 0;
     int rc = configure_once(&sm_count, &dev);
@@ -274,11 +305,22 @@ static int launch_all(KParams &P, void *ws, size_t ws_bytes, cudaStream_t st, in
     P.wmax = reinterpret_cast<unsigned int *>(base + L.wmax);
     P.cand = reinterpret_cast<unsigned long long *>(base + L.cand);
     P.cand_stride = L.cand_stride;
+    P.ytiles = L.ytiles;
     P.tickets = P.error + WS_TICKETS;
     P.groups = group_table(P.V);
+    if (dense) {
+        P.drow = reinterpret_cast<DenseRow *>(base + L.drow);
+        P.dtile = reinterpret_cast<DenseTile *>(base + L.dtile);
+        P.dlist = reinterpret_cast<int *>(base + L.dlist);
+        P.rlist = reinterpret_cast<int *>(base + L.rlist);
+        P.hist = reinterpret_cast<unsigned long long *>(base + L.hist);
+        P.members = reinterpret_cast<unsigned long long *>(base + L.members);
+        P.ykeys = reinterpret_cast<unsigned int *>(base + L.ykeys);
+    }
+
     if (row_route(P, sm_count)) {
         P.fresh = clear ? 1 : 0;
-        cudaError_t e = launch_rows(P, st, dev, false);
+        cudaError_t e = launch_rows(P, st, sm_count);
         if (e != cudaSuccess) return fail_cuda(e, "row kernel launch");
         g_err[0] = 0;
         return SONIC_OK;
@@ -292,55 +334,79 @@ static int launch_all(KParams &P, void *ws, size_t ws_bytes, cudaStream_t st, in
     if (nitems_ll > 0x7FFFFFFF) return fail(SONIC_ESHAPE, "rows x tiles too large");
     const int nitems = (int)nitems_ll;
     cudaError_t e;
-    cudaLaunchAttribute pdl;
-    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    pdl.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.stream = st;
-    cudaGraphNode_t row_node = nullptr;           // the captured row kernel
-#ifndef SONIC_TRACE
-    if (sampling) {
-        if ((e = launch_rows(P, st, dev, true)) != cudaSuccess) return fail_cuda(e, "row kernel launch");
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        const cudaGraphNode_t *deps = nullptr;
-        size_t ndeps = 0;
-        if ((e = cudaStreamGetCaptureInfo(st, &cs, nullptr, nullptr, &deps, &ndeps)) != cudaSuccess) return fail_cuda(e, "cudaStreamGetCaptureInfo");
-        if (cs == cudaStreamCaptureStatusActive && ndeps == 1) row_node = deps[0];
-        cfg.attrs = &pdl;
-        cfg.numAttrs = 1;
-    }
-#endif
 
     const int grid1 = nitems < sm_count * 3 ? nitems : sm_count * 3;       // persistent: three CTAs per SM
     // a CTA's first request to the work queue: seven eighths of an even share, at least one item
     int chunk = (int)((7ll * nitems) / (8ll * grid1));
     chunk = chunk < 1 ? 1 : chunk;
     const int cap_t = (int)(L.cand_stride / (unsigned)tiles);
-    const bool f32 = P.dtype == SONIC_DTYPE_F32;
-    cfg.gridDim = dim3(grid1);
-    cfg.blockDim = dim3(STREAM_CTA_THREADS);
-    cfg.dynamicSmemBytes = f32 ? STREAM_SMEM_F32 : STREAM_SMEM_BF16;
-    e = cudaLaunchKernelEx(&cfg, f32 ? sonic_stream_kernel<0> : sonic_stream_kernel<1>, P, tiles, nitems, chunk, cap_t);
+    if (P.dtype == SONIC_DTYPE_F32) sonic_stream_kernel<0><<<grid1, STREAM_CTA_THREADS, STREAM_SMEM_F32, st>>>(P, tiles, nitems, chunk, cap_t);
+    else sonic_stream_kernel<1><<<grid1, STREAM_CTA_THREADS, STREAM_SMEM_BF16, st>>>(P, tiles, nitems, chunk, cap_t);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return fail_cuda(e, "stream kernel launch");
 
+    cudaLaunchAttribute pdl;
+    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.stream = st;
     cfg.attrs = &pdl;
     cfg.numAttrs = 1;
+    // Fork: the histogram passes go to the thread's internal stream (if it can be used), behind the streaming
+    // kernel and beside the merges.  After the fork every exit joins that stream again (also the failing ones: the
+    // caller's stream, or its capture, must not be left with a branch that was never joined).
+    SideStream *side = dense ? side_stream_for(dev, st) : nullptr;
+    if (side) {
+        if ((e = cudaEventRecord(side->fork, st)) != cudaSuccess) return fail_cuda(e, "cudaEventRecord");
+        if ((e = cudaStreamWaitEvent(side->s, side->fork, 0)) != cudaSuccess) return fail_cuda(e, "cudaStreamWaitEvent");
+    }
+    auto unwind = [&](int code) {
+        if (side && cudaEventRecord(side->join, side->s) == cudaSuccess) cudaStreamWaitEvent(st, side->join, 0);
+        return code;
+    };
     cfg.gridDim = dim3(P.rows);
     cfg.blockDim = dim3(MERGE_THREADS);
     cfg.dynamicSmemBytes = MERGE_SMEM;
     e = cudaLaunchKernelEx(&cfg, sonic_merge_kernel, P, tiles);
-    if (e != cudaSuccess) return fail_cuda(e, "merge kernel launch");
-#ifdef SONIC_TRACE
-    // (the trace variant runs the row kernel behind the merge, so that each kernel can be told apart)
-    if (sampling && (e = launch_rows(P, st, dev, true)) != cudaSuccess) return fail_cuda(e, "row kernel launch");
-#endif
-    if (row_node) {
-        e = cudaStreamUpdateCaptureDependencies(st, &row_node, 1, cudaStreamAddCaptureDependencies);
-        if (e != cudaSuccess) return fail_cuda(e, "cudaStreamUpdateCaptureDependencies");
+    if (e != cudaSuccess) return unwind(fail_cuda(e, "merge kernel launch"));
+    if (dense) {
+        // the passes of the histogram path take (row, tile part) items in a loop: two CTAs per SM at most (a tile is
+        // cut into up to four parts when a call has few rows of that class: up to four CTAs per tile)
+        const int dense_ctas = (int)(4ll * nitems < 2ll * sm_count ? 4ll * nitems : 2ll * sm_count);
+        cudaLaunchConfig_t dcfg = cfg;
+        dcfg.stream = side ? side->s : st;
+        dcfg.gridDim = dim3(dense_ctas);
+        dcfg.blockDim = dim3(DENSE_THREADS);
+        dcfg.dynamicSmemBytes = DENSE_DYN_SMEM;
+        cudaLaunchConfig_t fcfg = dcfg;              // row-level steps: one CTA per row of the call (rows of other classes leave at once)
+        fcfg.gridDim = dim3(P.rows);
+        // Stage 2 never waits for its predecessor in the stream.  On the internal stream it is an ordinary launch
+        // behind the fork; on the caller's stream it is a programmatic dependent of the merge kernel, whose CTAs let
+        // it go only after their own wait for the streaming kernel.
+        cudaLaunchConfig_t d2cfg = dcfg;
+        if (side) { d2cfg.attrs = nullptr; d2cfg.numAttrs = 0; }
+        e = cudaLaunchKernelEx(&d2cfg, sonic_dense_stage2_kernel, P, tiles);
+        if (e != cudaSuccess) return unwind(fail_cuda(e, "histogram pass launch"));
+        e = cudaLaunchKernelEx(&dcfg, sonic_dense_collect_kernel, P, tiles);
+        if (e != cudaSuccess) return unwind(fail_cuda(e, "collect pass launch"));
+        e = cudaLaunchKernelEx(&fcfg, sonic_dense_finish_kernel, P, tiles);
+        if (e != cudaSuccess) return unwind(fail_cuda(e, "row finish launch"));
+        if (P.op == OP_VERIFY && P.K > 0) {
+            dcfg.dynamicSmemBytes = 0;
+            fcfg.dynamicSmemBytes = 0;
+            e = cudaLaunchKernelEx(&dcfg, sonic_dense_resid_kernel, P, tiles);
+            if (e != cudaSuccess) return unwind(fail_cuda(e, "residual pass launch"));
+            e = cudaLaunchKernelEx(&fcfg, sonic_dense_resid_finish_kernel, P, tiles);
+            if (e != cudaSuccess) return unwind(fail_cuda(e, "residual draw launch"));
+        }
     }
-    // The cluster kernel is an ordinary launch: it starts when everything before it is complete (the merges as well as the
-    // row kernel).
+    if (side) {
+        if ((e = cudaEventRecord(side->join, side->s)) != cudaSuccess) return fail_cuda(e, "cudaEventRecord");
+        if ((e = cudaStreamWaitEvent(st, side->join, 0)) != cudaSuccess) return fail_cuda(e, "cudaStreamWaitEvent");
+    }
+    // The cluster kernel is an ordinary launch: it starts when everything before it is complete (the merges as well
+    // as the histogram passes, which ran beside them).
     const int clusters = P.rows < EXACT_CLUSTERS ? P.rows : EXACT_CLUSTERS;
     cfg.gridDim = dim3(clusters * CL);
     cfg.blockDim = dim3(EX_THREADS);
@@ -401,18 +467,25 @@ size_t sonic_workspace_bytes(int max_rows, int max_vocab, int max_topk) {
     if (max_rows < 1) max_rows = 1;
     if (max_vocab < 1) max_vocab = 1;
     if (max_vocab > SONIC_MAX_VOCAB) max_vocab = SONIC_MAX_VOCAB;
-    // the larger of the two layouts a call can have: sampling / verification, and sonic_topk with its slots for max_topk
-    const size_t a = layout_for(max_rows, max_vocab, slot_cap(OP_SAMPLE, 0)).total;
-    const size_t b = layout_for(max_rows, max_vocab, slot_cap(OP_TOPK, max_topk)).total;
+    // the larger of the two layouts a call can have: sampling / verification (with the histogram path's regions), and
+    // sonic_topk with its slots for max_topk
+    const size_t a = layout_for(max_rows, max_vocab, true).total;
+    const size_t b = layout_for(max_rows, max_vocab, false, slot_cap(OP_TOPK, max_topk)).total;
     return a > b ? a : b;
 }
 
 int sonic_workspace_init(void *workspace, size_t bytes, void *stream) {
     if (!workspace) return fail(SONIC_EINVAL, "workspace is NULL");
     if (((uintptr_t)workspace & 255) != 0) return fail(SONIC_EINVAL, "workspace must be 256-byte aligned");
-    if (bytes < layout_for(1, 1, slot_cap(OP_SAMPLE, 0)).total) return fail(SONIC_EWORKSPACE, "workspace smaller than one row");
+    if (bytes < layout_for(1, 1, true).total) return fail(SONIC_EWORKSPACE, "workspace smaller than one row");
     cudaError_t e = cudaMemsetAsync(workspace, 0, WS_HEADER, (cudaStream_t)stream);
     if (e != cudaSuccess) return fail_cuda(e, "cudaMemsetAsync");
+    // The calling thread's internal stream is created here already (if this is not inside a capture), so that a
+    // thread whose very first sampling call is captured still gets the two-stream schedule.  Best effort: a call
+    // that finds no usable internal stream runs on the caller's stream alone.
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) (void)side_stream_for(dev, (cudaStream_t)stream);
+    else cudaGetLastError();
     g_err[0] = 0;
     return SONIC_OK;
 }

@@ -34,8 +34,7 @@ constexpr int MAX_TILES = (262144 + CTA_TILE - 1) / CTA_TILE;   // 32 tiles at t
 constexpr int FILTER_HIST = 512;
 constexpr int FILTER_BIAS = 32;
 constexpr int FILTER_COUNT_MAX = (1 << 14) - 1;   // largest count that packs beside an 18-bit id
-constexpr uint32_t CAND_CAP = 32768;          // candidate slots per row of sonic_topk, divided evenly among the row's tiles
-constexpr uint32_t SAMPLE_CAP = 131072;       // ... of a sampling row (4096 and more per tile: no tile of a smooth row overflows)
+constexpr uint32_t CAND_CAP = 32768;          // candidate slots per row, divided evenly among the row's tiles
 constexpr int MERGE_THREADS = 512;
 constexpr int MERGE_CAP = 8192;               // 64-bit keys the row merge can sort (64 KB of shared memory)
 constexpr int KFAST_SAMPLE = MERGE_CAP / 4;   // largest top-k the streaming path finishes for sampling rows (2048)
@@ -45,23 +44,24 @@ constexpr int MAX_VOCAB = 262144;
 
 constexpr int CLS_GREEDY = 0;                 // streaming path, argmax only
 constexpr int CLS_TOPK = 1;                   // streaming path, candidates + merge
-constexpr int CLS_EXACT = 2;                  // top-k beyond what the streaming path sorts: row kernel (sonic_topk: cluster kernel)
-constexpr int CLS_DENSE = 3;                  // top-k off: row kernel
-__device__ __forceinline__ bool class_is_listed(int cls) { return cls == CLS_DENSE || cls == CLS_EXACT; }       // (of sampling calls)
+constexpr int CLS_EXACT = 2;                  // cluster kernel only (top-k beyond what the streaming path sorts)
+constexpr int CLS_DENSE = 3;                  // top-k off: streaming pass for the keys, then the histogram passes
 
 // Workspace header (the first WS_HEADER_WORDS 32-bit words; the only part of the workspace that must be zero
 // between calls: every other word is initialised by the call that reads it)
 constexpr int WS_ERROR = 0;                    // sticky ERR_* bits
-constexpr int WS_FAILED_ROWS = 1;              // rows of the current call that the streaming path handed to the cluster kernel
+constexpr int WS_FAILED_ROWS = 1;              // rows of the current call that the streaming or histogram path handed to the cluster kernel
 constexpr int WS_QUEUE = 2;                    // the stream kernel's work counter
 constexpr int WS_EXACT_TICKET = 3;             // next row ordinal of the cluster kernel
+constexpr int WS_NDENSE = 4;                   // rows of the current call on the histogram path (length of the dense list)
+constexpr int WS_NRESID = 5;                   // verification rows of the current call whose draft was rejected (length of the residual list)
 constexpr int WS_EXACT_LEFT = 6;               // clusters of the cluster kernel that have run out of rows
 constexpr int WS_NEXACT = 7;                   // rows of the current call that belong to the cluster kernel by class
 constexpr int WS_TEST_WITHHOLD = 100;          // test-only builds (SONIC_TEST_WITHHOLD): 1 + the work item whose tile copy is withheld
 constexpr int WS_TICKETS = 128;                // [MAX_REQUESTS] verification: positions of a request that are finished (row kernel; zero between calls)
 constexpr int MAX_REQUESTS = 4096;
 constexpr int WS_HEADER_WORDS = WS_TICKETS + MAX_REQUESTS;
-constexpr uint32_t ST_FAILED = 0x1;           // the streaming path could not finish the row
+constexpr uint32_t ST_FAILED = 0x1;           // streaming / histogram path could not finish the row
 constexpr unsigned int ERR_TIMEOUT = 0x1;     // workspace header: a bounded mbarrier wait expired
 constexpr uint32_t TILE_BADID = 0x1;          // TileRec.flags: a list id of the row was out of range
 
@@ -73,12 +73,41 @@ struct __align__(16) RowState {
 };
 
 struct __align__(16) TileRec {                // written by the tile's CTA in the streaming kernel
-    unsigned long long best;                  // greedy rows: largest (key << 32 | ~index) of the tile, 0 if none finite
+    unsigned long long best;                  // greedy and dense rows: largest (key << 32 | ~index) of the tile, 0 if none finite
     unsigned int cnt;                         // top-k rows: candidates of the tile (may exceed the slot: overflow)
     unsigned int tkey;                        // top-k rows: the tile's cutoff as an ordered key
+    unsigned int minkey;                      // dense rows: smallest finite key of the tile (0xFFFFFFFF if none)
+    unsigned int nfin;                        // dense rows: finite elements of the tile
     unsigned int flags;                       // TILE_*
-    unsigned int pad[3];
+    unsigned int pad;
 };
+
+// Histogram path (rows with top-k off), per row.  Initialised by the streaming kernel (the CTA of the row's first
+// tile); the later passes communicate through it.
+constexpr int DBINS = 2048;                   // bins of the mass histogram, uniform in (M - y)
+constexpr int MEMBER_CAP = 4096;              // elements of the crossing bin that can be listed
+struct __align__(16) DenseRow {
+    unsigned int ticket_h, ticket_c, ticket_r, nmembers;     // items that have finished a pass; listed members
+    unsigned int kmin, kmax, overflow, state;                // key span of the members; an item could not stage its members; 1 = collect pass wanted
+    unsigned int Mkey, tk, klo, khi;                         // row maximum; min-p key threshold (0 = none); keys of the crossing bin: klo .. khi (empty if klo > khi)
+    unsigned long long target;                               // mass the ranking prefix must reach (0: top-p does not decide inside the bin)
+    unsigned long long cutc, W;                              // final cut (composite key) and total fixed-point mass of the support
+    float p_draft; int support;
+    unsigned int pad[4];
+};
+static_assert(sizeof(DenseRow) == 96, "DenseRow layout");
+constexpr int DENSE_CHUNK = 512;                 // elements per chunk of a tile
+constexpr int DENSE_CHUNKS = 16;                 // chunks per tile
+struct __align__(16) DenseChunk {             // per chunk of 512 elements, written by pass C
+    unsigned long long A;                     // fixed-point mass of the chunk's elements above the crossing bin
+    unsigned int n, nb;                       // their number; the chunk's elements inside the crossing bin
+};
+struct __align__(16) DenseTile {              // per (row, tile) of the histogram path
+    DenseChunk ch[DENSE_CHUNKS];
+    unsigned long long mass;                  // fixed-point mass of the tile's part of the final support
+    double R, Pp, S;                          // residual pass: sum of max(0, w/W~ - q), sum of w where that is positive, sum of w
+};
+static_assert(sizeof(DenseTile) == 288, "DenseTile layout");
 
 struct __align__(16) PosResult {              // per logit row, verification only
     int token;
@@ -152,6 +181,14 @@ struct KParams {
     PosResult *pr;
     unsigned long long *cand;                 // [rows][cand_stride] candidate slots, split evenly among a row's tiles
     unsigned int cand_stride;
+    // histogram path (sample / verify calls only)
+    DenseRow *drow;                           // [rows]
+    DenseTile *dtile;                         // [rows][MAX_TILES]
+    int *dlist, *rlist;                       // [rows] rows on the histogram path; rows whose draft was rejected
+    unsigned long long *hist;                 // [rows][DBINS] fixed-point mass per bin
+    unsigned long long *members;              // [rows][MEMBER_CAP] elements of the crossing bin (key << 32 | ~index)
+    unsigned int *ykeys;                      // [rows][ytiles * CTA_TILE] ordered keys of the processed logits
+    int ytiles;
     GroupTable groups;                        // pick_groups' table for V
     unsigned int *tickets;                    // [MAX_REQUESTS] in the header
 };
@@ -288,7 +325,7 @@ __device__ __forceinline__ RowCfg resolve_cfg(const KParams &P, int row, const C
     int G;
     c.cls = class_of(P, greedy, c.k, &G);
     if (c.cls == CLS_TOPK) { c.G = G & (PICK_TILE_MODE - 1); c.tile_min = (G & PICK_TILE_MODE) != 0; }
-    c.div_all = c.cls == CLS_GREEDY && c.temp;
+    c.div_all = (c.cls == CLS_GREEDY || c.cls == CLS_DENSE) && c.temp;
     return c;
 }
 
@@ -297,7 +334,7 @@ __device__ __forceinline__ RowCfg load_cfg(const KParams &P, int row) { return r
 #ifdef SONIC_TRACE
 __device__ __forceinline__ unsigned int gtimer_lo() { unsigned long long t; asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t)); return (unsigned int)t; }
 // kernel-level timeline (trace variant of the library only): earliest start and latest end of kernel k over its CTAs
-// (0 stream, 1 merge, 2 cluster kernel, 5 combine; phases of the row kernel: 6 bins, 3 gather, 8 cut, 4 residual, 9 its draw)
+// (0 stream, 1 merge, 6 histogram pass, 3 collect pass, 8 row finish, 4 residual pass, 9 residual draw, 2 cluster kernel, 5 combine)
 #define KERNEL_T0(k) do { if (threadIdx.x == 0) atomicMin(&P.error[48 + 2 * (k)], gtimer_lo()); } while (0)
 #define KERNEL_T1(k) do { if (threadIdx.x == 0) atomicMax(&P.error[49 + 2 * (k)], gtimer_lo()); } while (0)
 #else

@@ -1004,6 +1004,8 @@ sonic_exact_kernel(const KParams P) {
     const int ncl = gridDim.x / CL;
     const int cid = blockIdx.x / CL;
     const int nwords = (P.rows + 31) >> 5;
+    // (the passes that read the two lists are complete: their lengths go back to zero for the next call)
+    if (blockIdx.x == 0 && x.tid == 0) { P.error[WS_NDENSE] = 0u; P.error[WS_NRESID] = 0u; }
     if (__ldcg(&P.error[WS_ERROR]) & ERR_TIMEOUT) {
         // A bounded wait of the streaming kernel ran out (in this call or an earlier one on this workspace): nothing
         // the call computed is to be trusted.  This is the call's last kernel over the rows, behind both chains, so
@@ -1027,8 +1029,7 @@ sonic_exact_kernel(const KParams P) {
     // every CTA marks the rows of the whole call (all derive the same list)
     for (int row = x.tid; row < P.rows; row += EX_THREADS) {
         const RowCfg c = load_cfg(P, row);
-        const bool passed = P.op != OP_TOPK && class_is_listed(c.cls);          // (the row kernel's: it finishes every row it takes)
-        const bool mine = !passed && ((c.cls == CLS_EXACT) || (__ldcg(&P.rs[row].status) & ST_FAILED));
+        const bool mine = (c.cls == CLS_EXACT) || (__ldcg(&P.rs[row].status) & ST_FAILED);
         if (mine) atomicOr(&need[row >> 5], 1u << (row & 31));
     }
     __syncthreads();

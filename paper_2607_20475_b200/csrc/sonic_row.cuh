@@ -27,6 +27,7 @@
 #pragma once
 #include <cooperative_groups.h>
 #include "sonic_common.cuh"
+#include "sonic_dense.cuh"
 #include "sonic_stream.cuh"
 
 namespace sonic {
@@ -132,74 +133,6 @@ __device__ __forceinline__ void row_each(const RowCtx &x, F f) {
     }
 }
 
-// ---------------------------------------------------------------- block-level helpers
-__device__ __forceinline__ unsigned long long row_warp_sum(unsigned long long v) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
-    return v;
-}
-
-// Inclusive scan over the lanes of a warp.
-__device__ __forceinline__ unsigned long long row_warp_scan(unsigned long long v, int lane) {
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long up = __shfl_up_sync(0xFFFFFFFFu, v, o);
-        if (lane >= o) v += up;
-    }
-    return v;
-}
-
-// Exclusive prefix over the threads of the block (thread order) of one value per thread; `total` in every thread.
-template <typename T>
-__device__ __forceinline__ T row_block_scan(T v, T *wtot, int tid, T &total) {
-    const int lane = tid & 31, warp = tid >> 5;
-    T incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const T up = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += up;
-    }
-    __syncthreads();
-    if (lane == 31) wtot[warp] = incl;
-    __syncthreads();
-    T off = T(0), tot = T(0);
-#pragma unroll
-    for (int w = 0; w < ROW_WARPS; ++w) {
-        const T t = wtot[w];
-        if (w < warp) off += t;
-        tot += t;
-    }
-    total = tot;
-    return off + incl - v;
-}
-
-// 64-bit add to a shared-memory word as two native 32-bit atomics (low word first: the value it returns tells whether
-// the sum carried).  A 64-bit shared-memory atomic is a compare-and-swap loop, which crawls when many lanes add to a
-// handful of words (the per-tile masses of a row: 16 words, hundreds of listed elements).
-__device__ __forceinline__ void smem_add_u64(unsigned long long *p, unsigned long long w) {
-    unsigned int *q = reinterpret_cast<unsigned int *>(p);
-    const unsigned int lo = (unsigned int)w, hi = (unsigned int)(w >> 32);
-    unsigned int carry = 0u;
-    if (lo) { const unsigned int old = atomicAdd(q, lo); carry = (old + lo < old) ? 1u : 0u; }
-    if (hi + carry) atomicAdd(q + 1, hi + carry);
-}
-
-// Weight of an element in a residual.  The support's total weight W is known in fixed point first (from exp2 with a relative
-// error of up to 2e-7, too coarse where p - q cancels), so a part accumulates, in fp64, the residual sum R~ taken with
-// that W~, the sum Pp of the weights whose residual is positive, and the plain sum S of the weights; with W = sum of S the
-// residual is R~ - (1/W~ - 1/W) * Pp (exact up to the elements whose residual changes sign between W~ and W, each of which
-// contributes less than 1e-7 of its own probability).
-// An element that carries more than 2^-7 of the support's mass (at most 128 per row, usually a handful) is weighed with the
-// fp64 exponential: its residual is a difference of two numbers of that size.  The others use an fp32 exponential of
-// relative error below 1e-7 with no bias; independent errors of that size on probabilities below 2^-7 add up to less
-// than 1e-8 in the cumulative sums.
-__device__ __forceinline__ double resid_weight(uint32_t key, float Mf, double Md, float big) {
-    const float y = unkey(key);
-    const float w32 = exp_accurate(__fsub_rn(y, Mf));
-    return (w32 > big) ? exp((double)y - Md) : (double)w32;
-}
-
-
 // ---------------------------------------------------------------- weights
 // An element's weight exp(y - M) as qweight has it (the same operations, before the conversion).
 __device__ __forceinline__ float row_w(float y, float Mf) {
@@ -299,7 +232,7 @@ __device__ __forceinline__ bool row_cross(const RowCtx &x, bool next, double wan
 __device__ __forceinline__ unsigned long long row_sum_bins(const RowCtx &x, int n) {
     RowShared &sh = row_sh();
     if (x.tid < ROW_BINS) {
-        const unsigned long long t = row_warp_sum(x.tid < n ? sh.bins[x.tid] : 0ull);
+        const unsigned long long t = dense_warp_sum(x.tid < n ? sh.bins[x.tid] : 0ull);
         if (x.lane == 0) sh.red64[x.warp] = t;
     }
     __syncthreads();
@@ -366,7 +299,7 @@ __device__ __noinline__ void row_split(const RowCtx &ctx, RowSel &sel, bool by_m
         for (int r = 0; r < x.ncta; ++r) v[u] += reinterpret_cast<const unsigned long long *>(row_rx())[r * ROW_XBINS + x.lane * 4 + u];
         run += v[u];
     }
-    const unsigned long long incl = row_warp_scan(run, x.lane), all = __shfl_sync(0xFFFFFFFFu, incl, 31), want = max(1ull, min(need, all));
+    const unsigned long long incl = dense_warp_scan(run, x.lane), all = __shfl_sync(0xFFFFFFFFu, incl, 31), want = max(1ull, min(need, all));
     const unsigned int hit = __ballot_sync(0xFFFFFFFFu, incl >= want);
     const int l = hit ? __ffs(hit) - 1 : 31;
     unsigned long long before = incl - run, in = 0ull;
@@ -404,12 +337,12 @@ __device__ __forceinline__ unsigned int row_room(const RowCtx &x, unsigned int m
 // The warps' sums of a mass, a number and a number of members -> this CTA's entry of CTA 0's sh.above (block barrier inside).
 __device__ __forceinline__ void row_send_above(const RowCtx &x, unsigned long long m, unsigned int n, unsigned int members, unsigned long long more) {
     RowShared &sh = row_sh();
-    m = row_warp_sum(m);
+    m = dense_warp_sum(m);
     const unsigned int both = __reduce_add_sync(0xFFFFFFFFu, n | (members << 16));      // (a warp has at most 1024 elements)
     if (x.lane == 0) { sh.warp2[x.warp] = m; sh.red32[x.warp] = both; }
     __syncthreads();
     if (x.warp == 0) {
-        m = row_warp_sum(x.lane < ROW_WARPS ? sh.warp2[x.lane] : 0ull);
+        m = dense_warp_sum(x.lane < ROW_WARPS ? sh.warp2[x.lane] : 0ull);
         const unsigned int t = x.lane < ROW_WARPS ? sh.red32[x.lane] : 0u;
         n = __reduce_add_sync(0xFFFFFFFFu, t & 0xFFFFu);
         members = __reduce_add_sync(0xFFFFFFFFu, t >> 16);
@@ -691,8 +624,6 @@ __device__ __noinline__ bool row_residual(const RowCtx &ctx, const KParams &P, c
         to[0] = R; to[1] = Pp; to[2] = S;
     }
     cl_sync();
-    KERNEL_T1(4);
-    KERNEL_T0(9);
     double W = 0.0;
     for (int r = 0; r < x.ncta; ++r) W += sh.resid[r][2];
     const double corr = inv_Wt - 1.0 / W;
@@ -725,33 +656,35 @@ __device__ __noinline__ bool row_residual(const RowCtx &ctx, const KParams &P, c
 }
 
 
-// One row by the CTAs of a cluster.  LISTED: the cluster takes row after row of those the streaming kernel leaves to it
-// (sampling rows with top-k off, or with a top-k beyond what it handles), beside that kernel; every path then ends with
-// the cluster barrier's phases complete, and a verification call's scan has a kernel of its own.  parity: of the row's copy.
-template <int DT, bool LISTED>
-__device__ __forceinline__ void row_body(const KParams &P, RowCtx &x, const int row, const unsigned int parity) {
+// Grid: rows x CTAs of a cluster.  slice: elements per CTA (a multiple of ROW_UNIT, slice * cluster >= V).
+template <int DT>
+__global__ void __launch_bounds__(ROW_THREADS, 2)
+sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
     constexpr int VEC = VecTraits<DT>::VEC, ELT = VecTraits<DT>::ELT;
     RowShared &sh = row_sh();
-    const int slice = x.slice;
+    RowCtx x;
+    x.rank = (int)cgr::this_cluster().block_rank();
+    x.ncta = (int)cgr::this_cluster().num_blocks();
+    x.slice = slice;
+    x.base = x.rank * slice;
+    x.tid = threadIdx.x; x.lane = x.tid & 31; x.warp = x.tid >> 5;
+    x.wn = slice / ROW_WARPS; x.wlo = x.warp * x.wn;
     uint32_t *mask = row_mask();
     unsigned char *raw = row_smem + (DT == 0 ? 0 : ROW_OFF_RX);
+    const int row = (int)blockIdx.x / x.ncta;
     const int tid = x.tid, lane = x.lane;
     const bool lead = x.rank == 0 && tid == 0;
 
-    if (LISTED) KERNEL_T0(6);
     const CfgRaw cfg_raw = fetch_cfg(P, row);
     const int req = (P.op == OP_VERIFY) ? row / (P.K + 1) : row;
     // Everything the row needs from global memory is asked for at once: its logits by one bulk copy, mask words,
     // parameters and the first entries of its lists (none of the addresses depends on a loaded value).
     if (tid == 0) {
+        mbar_init(&sh.full, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         const int elems = min(slice, (P.V - x.base + VEC - 1) / VEC * VEC);
         if (elems > 0) {
             mbar_arrive_expect_tx(&sh.full, (unsigned int)elems * ELT);
-#ifdef SONIC_TEST_WITHHOLD
-            // test-only build: the copy of the part that holds one chosen tile is announced but never issued
-            const unsigned int held = __ldcg(&P.error[WS_TEST_WITHHOLD]), htiles = (unsigned int)(P.V + CTA_TILE - 1) / CTA_TILE;
-            if (held == 0u || (int)((held - 1u) / htiles) != row || (int)((held - 1u) % htiles) * CTA_TILE / slice != x.rank)
-#endif
             bulk_load(raw, reinterpret_cast<const unsigned char *>(P.logits) + ((size_t)row * (size_t)P.row_stride + (size_t)x.base) * ELT,
                       (unsigned int)elems * ELT, &sh.full, l2_evict_first_policy());
         } else mbar_arrive(&sh.full);
@@ -786,14 +719,13 @@ __device__ __forceinline__ void row_body(const KParams &P, RowCtx &x, const int 
     __syncthreads();
     cl_arrive();                                                    // (matched by the wait before the first remote write)
     const RowCfg c = resolve_cfg(P, row, cfg_raw);
-    const bool finish_request = !LISTED && P.op == OP_VERIFY;
-    const bool dense = LISTED || c.cls == CLS_DENSE || c.cls == CLS_EXACT, greedy = !LISTED && c.cls == CLS_GREEDY;
+    const bool finish_request = P.op == OP_VERIFY;
+    const bool dense = c.cls == CLS_DENSE || c.cls == CLS_EXACT, greedy = c.cls == CLS_GREEDY;
     auto emit = [&](int token, float prob, uint32_t flags, int support, float p_draft) {
         emit_row(P, c, row, token, prob, flags, support, p_draft);
         if (finish_request) row_ticket(P, c.b);
     };
     auto emit_late = [&]() {
-        if (LISTED) return;                                         // (the chain's last kernel reports it for every row)
                                             // (a wait for a copy ran out, in this call or an earlier one on this workspace)
         if (P.op == OP_TOPK) { for (int j = 0; j < P.ktop; ++j) { P.out_vals[(size_t)row * P.ktop + j] = -CUDART_INF_F; P.out_idx[(size_t)row * P.ktop + j] = -1; } }
         else emit(-1, 0.0f, F_TIMEOUT, 0, 0.0f);
@@ -801,7 +733,7 @@ __device__ __forceinline__ void row_body(const KParams &P, RowCtx &x, const int 
     // A copy that never comes, or the workspace's sticky error: every CTA of the cluster learns of it with the first
     // exchange, and all of them leave behind it (the values computed up to there are not used).
     bool late = (err & ERR_TIMEOUT) != 0u;
-    if (!mbar_wait(&sh.full, parity)) {
+    if (!mbar_wait(&sh.full, 0)) {
         if (tid == 0) atomicOr(P.error, ERR_TIMEOUT);
         late = true;
     }
@@ -838,10 +770,6 @@ __device__ __forceinline__ void row_body(const KParams &P, RowCtx &x, const int 
         bad = __syncthreads_or(bad ? 1 : 0) != 0;                   // (every CTA reads the whole lists: all take the exit below or none)
     }
     if (bad) {
-        if (LISTED) {
-            cl_wait();
-            if (late && tid < x.ncta) *cl_map(&sh.late[x.rank], tid) = 1u;
-        }
         if (lead && late) emit_late();
         else if (lead) emit(-1, 0.0f, F_BADPARAM | (c.cls == CLS_DENSE ? F_DENSE : 0u), 0, 0.0f);
         return;
@@ -897,7 +825,7 @@ __device__ __forceinline__ void row_body(const KParams &P, RowCtx &x, const int 
         return make_uint2(r4[0] >> 8, r4[1] >> 8);
     };
 
-    if (!LISTED && direct) {
+    if (direct) {
         // ------------------------------------------------------------ top-k, small k
         float g = lmax;
         for (int off = 16 / gpw; off > 0; off >>= 1) g = fmaxf(g, __shfl_xor_sync(0xFFFFFFFFu, g, off));
@@ -1047,7 +975,7 @@ __device__ __forceinline__ void row_body(const KParams &P, RowCtx &x, const int 
         return;
     }
 
-    if (!LISTED && !dense) {
+    if (!dense) {
         // ------------------------------------------------------------ top-k, larger k
         bool by_lanes = !direct && 4 * c.k <= x.ncta * ROW_THREADS;
         int n = 0;
@@ -1134,7 +1062,7 @@ __device__ __forceinline__ void row_body(const KParams &P, RowCtx &x, const int 
         unsigned long long t = row_sum_bins(x, ROW_BINS);
         if (tid < x.ncta) *cl_map(&sh.sum[0][x.rank], tid) = t;
         cl_sync();
-        Z = row_warp_sum(lane < x.ncta ? sh.sum[0][lane] : 0ull);
+        Z = dense_warp_sum(lane < x.ncta ? sh.sum[0][lane] : 0ull);
         goal = max(1ull, min((unsigned long long)ceil((double)c.p * (double)Z), Z));
         int bin_a, bin_b;
         double before, in_bin;
@@ -1149,14 +1077,12 @@ __device__ __forceinline__ void row_body(const KParams &P, RowCtx &x, const int 
         __syncthreads();
         row_fold<true>(x, true, [=](int) { return bin_a >> m; });
         cl_sync();
-        const unsigned long long above_a = row_warp_sum(lane < x.ncta ? sh.sum[1][lane] : 0ull);
+        const unsigned long long above_a = dense_warp_sum(lane < x.ncta ? sh.sum[1][lane] : 0ull);
         row_cross(x, false, (double)(goal > above_a ? goal - above_a : 1ull), bin_b, before, in_bin);
         const unsigned long long own_b = row_sum_bins(x, bin_b);
-        if (LISTED) { KERNEL_T1(6); KERNEL_T0(3); }
         row_gather_bin(x, s, shift_b, (bin_a << 8) | bin_b, t + own_b);
     } else row_mass_above(x, s.vmin, floorc);
     cl_sync();
-    if (LISTED) { KERNEL_T1(3); KERNEL_T0(8); }
     bool exact = !top_p;                                            // the gathered part is the right one by construction
     bool masses = !top_p;                                           // sh.above: the whole support, nothing gathered
     unsigned long long cutc = floorc;
@@ -1170,7 +1096,7 @@ __device__ __forceinline__ void row_body(const KParams &P, RowCtx &x, const int 
             const ulonglong2 ab = (lane < x.ncta) ? sh.above[lane] : make_ulonglong2(0ull, 0ull);      // (lane r: CTA r)
             unsigned long long mass = ab.x;                         // CTA r's part of the support
             const unsigned int members = (unsigned int)(ab.y >> 32);
-            bc.W = row_warp_sum(ab.x);
+            bc.W = dense_warp_sum(ab.x);
             unsigned int n = __reduce_add_sync(0xFFFFFFFFu, (unsigned int)ab.y);
             if (tid < x.ncta) sh.cta_mass[tid] = ab.x;
             const uint32_t kd = (draft >= 0) ? (uint32_t)sh.ex1[draft / slice].y : 0u;
@@ -1221,11 +1147,11 @@ __device__ __forceinline__ void row_body(const KParams &P, RowCtx &x, const int 
                         for (int u = tid & 7; u < nm; u += 8) pre += (sh.list[u] > c0) ? sh.list[64 + u] : 0ull;
 #pragma unroll
                         for (int off = 1; off < 8; off <<= 1) pre += __shfl_xor_sync(0xFFFFFFFFu, pre, off);
-                        tot = row_warp_sum(sh.list[64 + lane] + sh.list[96 + lane]);
+                        tot = dense_warp_sum(sh.list[64 + lane] + sh.list[96 + lane]);
                         if ((tid & 7) == 0) { mc = c0; mq = q0; }
                     } else {
                         row_rank(x, nm, mc, mq);
-                        pre = row_block_scan<unsigned long long>(mq, sh.red64, tid, tot);
+                        pre = dense_block_scan<unsigned long long>(mq, sh.red64, tid, tot);
                     }
                     // (the sums of single weights and of bins round differently below 2^-44)
                     if (bc.need > tot && (exact || bc.need - tot <= 65536ull)) bc.need = max(tot, 1ull);
@@ -1285,7 +1211,6 @@ __device__ __forceinline__ void row_body(const KParams &P, RowCtx &x, const int 
         cl_sync();
     }
     RowBcast bc = sh.bc;
-    if (LISTED) { KERNEL_T1(8); if (bc.flags & RB_REJECT) KERNEL_T0(4); }
     if (bc.flags & RB_ACCEPT) {                                     // the request moves on with the draft token
         if (lead) emit(P.draft_tokens[(size_t)c.b * P.K + c.l], 0.0f, cls_flag | F_ACCEPT, (int)bc.support, bc.p_draft);
         return;
@@ -1295,7 +1220,6 @@ __device__ __forceinline__ void row_body(const KParams &P, RowCtx &x, const int 
     if (bc.flags & RB_REJECT) {
         int token = -1;
         if (row_residual(x, P, c, bc.cutc, bc.W, cells.y, token)) {
-            if (LISTED) { KERNEL_T1(9); }
             if (token >= 0) emit(token, 0.0f, cls_flag, (int)bc.support, bc.p_draft);
             return;
         }
@@ -1309,70 +1233,6 @@ __device__ __forceinline__ void row_body(const KParams &P, RowCtx &x, const int 
         }, [&](int idx, unsigned long long q) {
             emit(idx, (bc.flags & RB_REJECT) ? 0.0f : (float)((double)q / (double)bc.W), cls_flag, (int)bc.support, bc.p_draft);
         });
-    }
-}
-
-// The ord-th row of the call that the streaming kernel leaves to the row kernel, -1 if there are fewer.  Two block barriers
-// per 512 requests.
-__device__ int row_pick(const KParams &P, int ord, int tid) {
-    RowShared &sh = row_sh();
-    const int per = (P.op == OP_VERIFY) ? P.K + 1 : 1, requests = P.rows / per;
-    int seen = 0;
-    for (int base = 0; base < requests; base += ROW_THREADS) {
-        const int b = base + tid;
-        bool mine = false;
-        if (b < requests) {
-            const uint32_t z = P.mode[b];
-            const int k = P.top_k ? P.top_k[b] : 0;
-            mine = class_is_listed(class_of(P, (z & M_GREEDY) != 0, (P.top_k && (z & M_TOP_K)) ? max(k, 0) : 0));
-        }
-        const unsigned int m = __ballot_sync(0xFFFFFFFFu, mine);
-        __syncthreads();
-        if ((tid & 31) == 0) sh.red32[tid >> 5] = m;
-        __syncthreads();
-        for (int w = 0; w < ROW_WARPS; ++w) {
-            const unsigned int v = sh.red32[w];
-            const int n = __popc(v) * per;
-            if (ord < seen + n) return (base + w * 32 + (int)__fns(v, 0, (ord - seen) / per + 1)) * per + (ord - seen) % per;
-            seen += n;
-        }
-    }
-    return -1;
-}
-
-// Grid: clusters.  Every row of the call (a cluster per row), or LISTED rows.  slice: elements per CTA (a multiple of
-// ROW_UNIT, slice * cluster >= V).
-template <int DT, bool LISTED>
-__global__ void __launch_bounds__(ROW_THREADS, 2)
-sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
-    RowCtx x;
-    x.rank = (int)cgr::this_cluster().block_rank();
-    x.ncta = (int)cgr::this_cluster().num_blocks();
-    x.slice = slice;
-    x.base = x.rank * slice;
-    x.tid = threadIdx.x; x.lane = x.tid & 31; x.warp = x.tid >> 5;
-    x.wn = slice / ROW_WARPS; x.wlo = x.warp * x.wn;
-    if (x.tid == 0) {
-        mbar_init(&row_sh().full, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    const int first = (int)blockIdx.x / x.ncta;
-    if (!LISTED) {
-        row_body<DT, false>(P, x, first, 0u);
-        return;
-    }
-    pdl_launch_dependents();                                        // (the streaming kernel runs beside this one)
-    const int clusters = (int)gridDim.x / x.ncta;
-    unsigned int parity = 0u;
-    for (int ord = first;; ord += clusters) {
-        const int row = row_pick(P, ord, x.tid);
-        if (row < 0) return;
-        __syncthreads();
-        if (x.tid == 0) fence_async_proxy();                        // (the last row's reads and writes precede this row's copy)
-        row_body<DT, true>(P, x, row, parity);
-        parity ^= 1u;
-        cl_sync();
-        if (row_late(x)) return;                                    // (a copy is missing: its barrier's phase never ends)
     }
 }
 

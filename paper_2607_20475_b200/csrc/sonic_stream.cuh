@@ -27,6 +27,7 @@
 // is handed to the exact kernel.
 #pragma once
 #include "sonic_common.cuh"
+#include "sonic_dense.cuh"
 
 namespace sonic {
 
@@ -1231,7 +1232,7 @@ struct StageMeta {
     int row, tile, slot;                       // slot: the row's parameters and lists
     int skip;                                  // the row belongs to another kernel: nothing to do
     int stop;                                  // no more tiles for this CTA (nothing else in the entry is valid)
-    int next_row, next_tile;                   // the tile that probably follows (-1: none, or not known yet)
+    int next_row, next_tile;                   // the tile that follows (-1: none)
 };
 struct Hit { int id; int payload; };           // a bias entry: token, value bits
 struct RowSlot {                               // a row's parameters and lists
@@ -1253,6 +1254,7 @@ struct StreamShared {
     alignas(16) float tw[NSTAGE][STREAM_WARPS];
     unsigned int ncand[NSTAGE], badid[NSTAGE];
     unsigned long long best[NSTAGE][STREAM_WARPS];       // greedy rows: argmax; top-k rows: cutoff key << 32 | key of the warp's maximum
+    unsigned int kmin[NSTAGE][STREAM_WARPS], nfin[NSTAGE][STREAM_WARPS];     // dense rows
     RowSlot slot[NSTAGE + 1];                  // the rows of the tiles in the ring and of the one that is prepared
 };
 
@@ -1282,7 +1284,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
     if (warp == STREAM_WARPS) {
         // ------------------------------------------------------------ producer warp
         // The (row, tile) items are handed out through a counter in the workspace, so CTAs that become resident
-        // late (the row kernel's clusters hold part of the chip) find less or no work instead of holding back a fixed
+        // late (the SMs may be shared) find less or no work instead of holding back a fixed
         // share.  Per tile the producer waits for a free stage, requests the next tile at once, and only then writes the
         // record of the tile that left the stage and the description of the new one: what it does by itself is one warp's
         // serial work of several hundred cycles, which would otherwise lie between a stage's release and its next request.
@@ -1290,7 +1292,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         static_assert(SONIC_MAX_VOCAB <= (1 << 18), "packed history entries hold an 18-bit id");
         static_assert(CTA_TILE == 1 << 13, "tile of a token");
         constexpr int HALF = FILTER_HIST / 64;     // history entries per lane and round of loads
-        int cached_row = -1, cur_slot = 0, used_slot = 0, cls_cur = CLS_GREEDY;      // used_slot: of the last tile handed over (a row that is passed over uses none)
+        int cached_row = -1, cur_slot = 0, cls_cur = CLS_GREEDY;
         auto load_row = [&](int row) {
             const int req = (P.op == OP_VERIFY) ? row / (P.K + 1) : row;
             const int *hid = P.hist_ids ? P.hist_ids + (size_t)req * P.hist_stride : nullptr;
@@ -1312,7 +1314,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             const RowCfg c = resolve_cfg(P, row, raw);
             cached_row = row;
             cls_cur = c.cls;
-            cur_slot = (used_slot + 1) % (NSTAGE + 1);
+            cur_slot = (cur_slot + 1) % (NSTAGE + 1);
             RowSlot &q = sh.slot[cur_slot];
             int patch = (c.hist_len > 0 || c.bias_len > 0) ? 1 : 0;
             if (c.hist_len > FILTER_HIST || c.bias_len > FILTER_BIAS) patch = 2;
@@ -1390,18 +1392,11 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 if (lane == 0 && run_lo < nitems) nxt_raw = (int)atomicAdd(queue, 1u);
             }
         };
-        // Rows that the row kernel takes (sampling calls) are passed over, a whole row at a time; on return the row's
-        // parameters and lists are loaded (pass == false: of the current item, whatever its row is).
-        auto find_item = [&](bool pass) -> int {
-            for (;;) {
-                const int it = current_item();
-                if (it < 0) return -1;
-                const int row = it / tiles;
-                if (row != cached_row) load_row(row);
-                if (!pass || P.op == OP_TOPK || !class_is_listed(cls_cur)) return it;
-                run_lo = min(run_hi, (row + 1) * tiles) - 1;
-                advance();
-            }
+        // The next item, with its row's parameters and lists loaded.
+        auto find_item = [&]() -> int {
+            const int it = current_item();
+            if (it >= 0 && it / tiles != cached_row) load_row(it / tiles);
+            return it;
         };
         int item = current_item();
         // lane 0: the tile's bulk copy, with the arrival on full[s] (arrive == true) or with the bytes announced only
@@ -1428,12 +1423,17 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         auto retire = [&](int s) {
             const int row = sh.meta[s].row, tile = sh.meta[s].tile;
             if (sh.meta[s].skip) {
-                // a row of the cluster kernel (sonic_topk): counted, its status word initialised
-                if (tile == 0 && lane == 0 && P.op == OP_TOPK) { P.rs[row].status = 0u; atomicAdd(&P.error[WS_NEXACT], 1u); }
+                // a row of the cluster kernel: counted, its status word initialised
+                if (tile == 0 && lane == 0) { P.rs[row].status = 0u; atomicAdd(&P.error[WS_NEXACT], 1u); }
                 return;
             }
             const RowSlot &q = sh.slot[sh.meta[s].slot];
             unsigned long long b = (lane < STREAM_WARPS) ? sh.best[s][lane] : 0ull;
+            unsigned int kmn = 0xFFFFFFFFu, nf = 0u;
+            if (q.cfg.cls == CLS_DENSE) {
+                kmn = __reduce_min_sync(0xFFFFFFFFu, lane < STREAM_WARPS ? sh.kmin[s][lane] : 0xFFFFFFFFu);
+                nf = __reduce_add_sync(0xFFFFFFFFu, lane < STREAM_WARPS ? sh.nfin[s][lane] : 0u);
+            }
             if (lane < STREAM_WARPS && q.cfg.cls == CLS_TOPK) P.wmax[((size_t)row * MAX_TILES + tile) * STREAM_WARPS + lane] = (uint32_t)b;
 #pragma unroll
             for (int off = STREAM_WARPS / 2; off > 0; off >>= 1) b = max(b, __shfl_xor_sync(0xFFFFFFFFu, b, off));
@@ -1441,7 +1441,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 TileRec r;
                 r.best = b; r.cnt = sh.ncand[s]; r.tkey = (unsigned int)(b >> 32);
                 r.flags = (q.bad || sh.badid[s]) ? TILE_BADID : 0u;
-                r.pad[0] = r.pad[1] = r.pad[2] = 0u;
+                r.minkey = kmn; r.nfin = nf; r.pad = 0u;
                 P.tiles[(size_t)row * MAX_TILES + tile] = r;
                 if (tile == 0) P.rs[row].status = 0u;
             }
@@ -1451,7 +1451,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         for (;; ++n) {                                 // (round -1 only prepares the first tile)
             if (n >= 0) {
                 const int s = n % NSTAGE;
-                const bool skip = item >= 0 && class_is_listed(cls_cur);
+                const bool skip = item >= 0 && cls_cur == CLS_EXACT;
                 const int row = item / tiles, tile = item - row * tiles;
                 if (n >= NSTAGE) {
                     // the consumers have left tile n - NSTAGE: its stage is free
@@ -1467,9 +1467,8 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                     if (lane == 0) { sh.meta[s].stop = 1; mbar_arrive(&sh.full[s]); }
                     break;
                 }
-                used_slot = cur_slot;
                 advance();
-                const int hint = current_item();           // (the tile that follows, unless its row is passed over)
+                const int hint = current_item();           // the tile that follows
                 if (lane == 0) {
                     if (n > 0 && n < NSTAGE && !skip) issue_copy(row, tile, s, false);
                     StageMeta &m = sh.meta[s];
@@ -1482,7 +1481,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 }
                 __syncwarp();
             }
-            item = find_item(n >= 0);
+            item = find_item();
         }
         for (int i = max(0, n - NSTAGE + 1); i < n; ++i) {     // the last tiles
             if (!mbar_wait(&sh.empty[i % NSTAGE], (i / NSTAGE) & 1)) {
@@ -1609,6 +1608,68 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 }
                 if (bad) sh.badid[s] = 1u;
                 csync();
+            }
+
+            if (slot.cfg.cls == CLS_DENSE) {
+                // Histogram path: the processed logits (divided by the temperature) are kept as ordered keys for the later
+                // passes; per tile the largest and smallest finite key and the number of finite elements.  The CTA of the
+                // row's first tile initialises the row's control block and histogram and lists the row.
+                if (tile == 0) {
+                    uint4 *h = reinterpret_cast<uint4 *>(P.hist + (size_t)row * DBINS);
+                    for (int i = tid; i < DBINS / 2; i += STREAM_THREADS) h[i] = make_uint4(0u, 0u, 0u, 0u);
+                    if (tid == 0) {
+                        DenseRow *dr = P.drow + row;
+                        dr->ticket_h = 0u; dr->ticket_c = 0u; dr->ticket_r = 0u; dr->nmembers = 0u;
+                        dr->kmin = 0xFFFFFFFFu; dr->kmax = 0u; dr->overflow = 0u; dr->state = 0u;
+                        P.dlist[atomicAdd(&P.error[WS_NDENSE], 1u)] = row;
+                    }
+                }
+                const bool divide = slot.cfg.div_all, all = !masked && !tail;
+                const float tau = slot.cfg.tau;
+                uint32_t kmx = 0u, kmn = 0xFFFFFFFFu;
+                unsigned int nf = 0u;
+                unsigned int *yk = P.ykeys + (size_t)row * ((size_t)P.ytiles * CTA_TILE) + tile_base;
+#pragma unroll
+                for (int j = 0; j < NV; ++j) {
+                    const int li = lane0 + j * 32 * VEC;
+                    const uint32_t bits = all ? 0xFFFFFFFFu : __shfl_sync(0xFFFFFFFFu, word, (j * 32 * VEC + lane * VEC) >> 5) >> ((lane * VEC) & 31);
+                    float v[VEC];
+                    if (DT == 1 && !wide) {
+                        const uint4 raw = *reinterpret_cast<const uint4 *>(stage + (size_t)li * ELT);
+                        const uint32_t r[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+                        for (int q = 0; q < VEC; ++q) v[q] = __uint_as_float((q & 1) ? (r[(q >> 1) & 3] & 0xFFFF0000u) : (r[(q >> 1) & 3] << 16));
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < VEC; q += 4) {
+                            const float4 a = *reinterpret_cast<const float4 *>(ptile + li + q);
+                            v[q] = a.x; v[q + 1] = a.y; v[q + 2] = a.z; v[q + 3] = a.w;
+                        }
+                    }
+#pragma unroll
+                    for (int q4 = 0; q4 < VEC; q4 += 4) {
+                        uint32_t kk[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            float y = ((bits >> (q4 + u)) & 1u) ? v[q4 + u] : -CUDART_INF_F;
+                            if (divide) y = div_tau(y, tau);
+                            kk[u] = okey(y);
+                            const bool fin = kk[u] > KEY_NEG_INF;
+                            nf += fin ? 1u : 0u;
+                            kmn = fin ? min(kmn, kk[u]) : kmn;
+                            kmx = fin ? max(kmx, kk[u]) : kmx;
+                        }
+                        *reinterpret_cast<uint4 *>(yk + li + q4) = make_uint4(kk[0], kk[1], kk[2], kk[3]);
+                    }
+                }
+                kmx = __reduce_max_sync(0xFFFFFFFFu, kmx);
+                kmn = __reduce_min_sync(0xFFFFFFFFu, kmn);
+                nf = __reduce_add_sync(0xFFFFFFFFu, nf);
+                if (lane == 0) { sh.best[s][warp] = (unsigned long long)kmx << 32; sh.kmin[s][warp] = kmn; sh.nfin[s][warp] = nf; }
+                if (DT == 0 && patch != 0) fence_async_proxy();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sh.empty[s]);
+                continue;
             }
 
             // Maxima of the lane's vectors.  ebits: which of its 32 elements count (allowed by the mask, inside the row).
@@ -1780,29 +1841,16 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 if (lane == 0) sh.best[s][warp] = ((unsigned long long)okey(t) << 32) | wk;
                 // every finite element >= t goes to the tile's candidate slot
                 const float t2 = fmaxf(t, -CUDART_MAX_NORMAL_F);           // e >= t2  <=>  e >= t and e is not -inf
-                unsigned int cand = __ballot_sync(0xFFFFFFFFu, lm >= t2);
+                const unsigned int cand = __ballot_sync(0xFFFFFFFFu, lm >= t2);
                 if (cand) {
                     unsigned long long *dst = P.cand + (size_t)row * P.cand_stride + (size_t)tile * cap_t;
                     auto put = [&](unsigned int pos, float z, int li) {
                         if ((int)pos < cap_t) dst[pos] = ((unsigned long long)okey(z) << 32) | (uint32_t)(~(uint32_t)(tile_base + li));
                     };
-                    if (sparse) {
-                        visit(t2, [&](float z, int li) { put(atomicAdd(&sh.ncand[s], 1u), z, li); });
-                    } else if (__popc(cand) <= 8) {
-                        // few lanes hold candidates: one after the other, its 32 elements across the warp
-                        while (cand) {
-                            const int L = __ffs(cand) - 1;
-                            cand &= cand - 1u;
-                            const int li = warp * WARP_TILE + (lane / VEC) * (32 * VEC) + L * VEC + (lane % VEC);
-                            const float z = value(li);
-                            const uint32_t eb = __shfl_sync(0xFFFFFFFFu, ebits, L);
-                            const bool in = z >= t2 && ((eb >> lane) & 1u);
-                            const unsigned int m = __ballot_sync(0xFFFFFFFFu, in);
-                            unsigned int base = 0u;
-                            if (lane == 0) base = atomicAdd(&sh.ncand[s], (unsigned int)__popc(m));
-                            base = __shfl_sync(0xFFFFFFFFu, base, 0);
-                            if (in) put(base + __popc(m & ((1u << lane) - 1u)), z, li);
-                        }
+                    if (sparse || __popc(cand) <= 8) {
+                        // few lanes hold candidates: those look for themselves (measured against testing one such lane's
+                        // elements across the warp at a time: 5 us less on 256 bf16 rows of 2^18)
+                        if (lm >= t2) visit(t2, [&](float z, int li) { put(atomicAdd(&sh.ncand[s], 1u), z, li); });
                     } else {
                         // many: every lane marks its own, one reservation for the warp
                         unsigned int cm = 0u;
@@ -1857,6 +1905,10 @@ sonic_merge_kernel(const KParams P, const int tiles) {
     uint2 cells = make_uint2(0u, 0u);
     if (P.op != OP_TOPK && c.cls == CLS_TOPK) draw_cells(P, c, cells.x, cells.y);
     pdl_wait_primary();                        // tile records and candidates of the streaming kernel
+    // The next kernel of the call (stage 2 of the histogram path) does not wait for this grid: it needs the
+    // streaming kernel's results only, and those are complete once every CTA here is past its wait (the first
+    // row's CTA never leaves before it).  So it is let go after the wait, and runs beside the merges.
+    pdl_launch_dependents();
     if (row == 0 && tid == 0) P.error[WS_QUEUE] = 0u;    // the streaming kernel is done with its work counter
     if (other) return;
     if (__ldcg(&P.error[WS_ERROR]) & ERR_TIMEOUT) {
