@@ -1673,7 +1673,9 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             }
 
             // Maxima of the lane's vectors.  ebits: which of its 32 elements count (allowed by the mask, inside the row).
+            // raw: the lane's elements as they lie in the stage (not of a widened part): what is looked at again stays in registers
             float mv[NV];
+            uint4 raw[NV];
             uint32_t ebits = 0xFFFFFFFFu;
             auto value = [&](int li) -> float {                // one element of the tile
                 return (DT == 1 && !wide) ? __uint_as_float((uint32_t)reinterpret_cast<const unsigned short *>(stage)[li] << 16) : ptile[li];
@@ -1691,13 +1693,14 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                     const int li = lane0 + j * 32 * VEC;
                     if (DT == 1 && !wide) {
                         // bf16 pairs: half an instruction per element
-                        const uint4 raw = *reinterpret_cast<const uint4 *>(stage + (size_t)li * ELT);
-                        const __nv_bfloat162 m = __hmax2(__hmax2(*reinterpret_cast<const __nv_bfloat162 *>(&raw.x), *reinterpret_cast<const __nv_bfloat162 *>(&raw.y)),
-                                                         __hmax2(*reinterpret_cast<const __nv_bfloat162 *>(&raw.z), *reinterpret_cast<const __nv_bfloat162 *>(&raw.w)));
+                        raw[j] = *reinterpret_cast<const uint4 *>(stage + (size_t)li * ELT);
+                        const __nv_bfloat162 m = __hmax2(__hmax2(*reinterpret_cast<const __nv_bfloat162 *>(&raw[j].x), *reinterpret_cast<const __nv_bfloat162 *>(&raw[j].y)),
+                                                         __hmax2(*reinterpret_cast<const __nv_bfloat162 *>(&raw[j].z), *reinterpret_cast<const __nv_bfloat162 *>(&raw[j].w)));
                         const uint32_t u = *reinterpret_cast<const uint32_t *>(&m);
                         mv[j] = fmaxf(__uint_as_float(u << 16), __uint_as_float(u & 0xFFFF0000u));
                     } else {
                         const float4 a = *reinterpret_cast<const float4 *>(ptile + li);
+                        if (DT == 0) raw[j] = make_uint4(__float_as_uint(a.x), __float_as_uint(a.y), __float_as_uint(a.z), __float_as_uint(a.w));
                         mv[j] = fmaxf(fmaxf(a.x, a.y), fmaxf(a.z, a.w));
                         if (VEC == 8) {
                             const float4 b = *reinterpret_cast<const float4 *>(ptile + li + 4);
@@ -1713,11 +1716,11 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                     const uint32_t bits = (__shfl_sync(0xFFFFFFFFu, word, (j * 32 * VEC + lane * VEC) >> 5) >> ((lane * VEC) & 31)) & ((1u << VEC) - 1u);
                     ebits |= bits << (j * VEC);
                     float v[VEC];
-                    if (DT == 1 && !wide) {
-                        const uint4 raw = *reinterpret_cast<const uint4 *>(stage + (size_t)li * ELT);
-                        const uint32_t r[4] = {raw.x, raw.y, raw.z, raw.w};
+                    if (DT == 0 || !wide) {
+                        raw[j] = *reinterpret_cast<const uint4 *>(stage + (size_t)li * ELT);
+                        const uint32_t r[4] = {raw[j].x, raw[j].y, raw[j].z, raw[j].w};
 #pragma unroll
-                        for (int q = 0; q < VEC; ++q) v[q] = __uint_as_float((q & 1) ? (r[(q >> 1) & 3] & 0xFFFF0000u) : (r[(q >> 1) & 3] << 16));
+                        for (int q = 0; q < VEC; ++q) v[q] = DT == 0 ? __uint_as_float(r[q & 3]) : __uint_as_float((q & 1) ? (r[(q >> 1) & 3] & 0xFFFF0000u) : (r[(q >> 1) & 3] << 16));
                     } else {
 #pragma unroll
                         for (int q = 0; q < VEC; q += 4) {
@@ -1847,28 +1850,53 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                     auto put = [&](unsigned int pos, float z, int li) {
                         if ((int)pos < cap_t) dst[pos] = ((unsigned long long)okey(z) << 32) | (uint32_t)(~(uint32_t)(tile_base + li));
                     };
-                    if (sparse || __popc(cand) <= 8) {
-                        // few lanes hold candidates: those look for themselves (measured against testing one such lane's
-                        // elements across the warp at a time: 5 us less on 256 bf16 rows of 2^18)
+                    if (sparse) {
                         if (lm >= t2) visit(t2, [&](float z, int li) { put(atomicAdd(&sh.ncand[s], 1u), z, li); });
                     } else {
-                        // many: every lane marks its own, one reservation for the warp
+                        // Every lane marks its candidates in a bit mask, a quarter of its elements at a time (a quarter without
+                        // one anywhere in the warp is skipped by a vote); one reservation for the warp.  The marked values are
+                        // fetched again from the tile.
                         unsigned int cm = 0u;
 #pragma unroll
-                        for (int j = 0; j < NV; ++j) {
-                            if (__any_sync(0xFFFFFFFFu, mv[j] >= t2)) {
+                        for (int i = 0; i < 4; ++i) {
+                            float qm = mv[i * NV / 4];
+                            if (NV == 8) qm = fmaxf(qm, mv[i * NV / 4 + 1]);
+                            if (__any_sync(0xFFFFFFFFu, qm >= t2)) {
 #pragma unroll
-                                for (int q = 0; q < VEC; ++q) cm |= (value(lane0 + j * 32 * VEC + q) >= t2) ? (1u << (j * VEC + q)) : 0u;
+                                for (int j = i * NV / 4; j < (i + 1) * NV / 4; ++j) {
+                                    const uint32_t r[4] = {raw[j].x, raw[j].y, raw[j].z, raw[j].w};
+                                    if (DT == 1 && wide) {
+                                        const float4 a = *reinterpret_cast<const float4 *>(ptile + lane0 + j * 32 * VEC);
+                                        const float4 b = *reinterpret_cast<const float4 *>(ptile + lane0 + j * 32 * VEC + (VEC == 8 ? 4 : 0));
+                                        cm |= ((a.x >= t2 ? 1u : 0u) | (a.y >= t2 ? 2u : 0u) | (a.z >= t2 ? 4u : 0u) | (a.w >= t2 ? 8u : 0u)) << (j * VEC);
+                                        cm |= ((b.x >= t2 ? 16u : 0u) | (b.y >= t2 ? 32u : 0u) | (b.z >= t2 ? 64u : 0u) | (b.w >= t2 ? 128u : 0u)) << (j * VEC);
+                                    } else {
+#pragma unroll
+                                        for (int q = 0; q < VEC; ++q) {
+                                            const float v = DT == 0 ? __uint_as_float(r[q & 3]) : __uint_as_float((q & 1) ? (r[(q >> 1) & 3] & 0xFFFF0000u) : (r[(q >> 1) & 3] << 16));
+                                            cm |= (v >= t2) ? (1u << (j * VEC + q)) : 0u;
+                                        }
+                                    }
+                                }
                             }
                         }
                         cm &= ebits;
                         const int cnt = __popc(cm);
-                        int incl = cnt;
+                        int incl, total;
+                        if (!__any_sync(0xFFFFFFFFu, cnt > 1)) {
+                            // the usual case, at most one candidate per lane: positions from one vote
+                            const unsigned int has = __ballot_sync(0xFFFFFFFFu, cnt > 0);
+                            incl = __popc(has & (0xFFFFFFFFu >> (31 - lane)));
+                            total = __popc(has);
+                        } else {
+                            incl = cnt;
 #pragma unroll
-                        for (int off = 1; off < 32; off <<= 1) { const int o = __shfl_up_sync(0xFFFFFFFFu, incl, off); if (lane >= off) incl += o; }
+                            for (int off = 1; off < 32; off <<= 1) { const int o = __shfl_up_sync(0xFFFFFFFFu, incl, off); if (lane >= off) incl += o; }
+                            total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+                        }
                         unsigned int base = 0u;
-                        if (lane == 31) base = atomicAdd(&sh.ncand[s], (unsigned int)incl);
-                        base = __shfl_sync(0xFFFFFFFFu, base, 31) + (unsigned int)(incl - cnt);
+                        if (lane == 0) base = atomicAdd(&sh.ncand[s], (unsigned int)total);
+                        base = __shfl_sync(0xFFFFFFFFu, base, 0) + (unsigned int)(incl - cnt);
                         while (cm) {
                             const int b = __ffs(cm) - 1, li = lane0 + (b / VEC) * (32 * VEC) + (b % VEC);
                             cm &= cm - 1u;
