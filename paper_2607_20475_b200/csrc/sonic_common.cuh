@@ -28,12 +28,14 @@ constexpr int STREAM_THREADS = 256;
 constexpr int STREAM_WARPS = STREAM_THREADS / 32;
 constexpr int CTA_TILE = WARP_TILE * STREAM_WARPS;   // 8192
 constexpr int MAX_TILES = (262144 + CTA_TILE - 1) / CTA_TILE;   // 32 tiles at the largest vocabulary
-// Sparse lists in the stream kernel: the producer warp brings a request's lists into shared memory once per row (up to
-// FILTER_HIST history entries, sorted by tile, id and count packed in one word, and FILTER_BIAS bias entries); longer lists
-// are scanned by the consumer threads.
+// Sparse lists in the stream kernel: the producer warp keeps a request's lists in registers (up to FILTER_HIST
+// history entries, id and count packed in one word, and FILTER_BIAS bias entries) and hands each tile the
+// entries that fall into it; longer lists are scanned by the consumer threads.
 constexpr int FILTER_HIST = 512;
 constexpr int FILTER_BIAS = 32;
 constexpr int FILTER_COUNT_MAX = (1 << 14) - 1;   // largest count that packs beside an 18-bit id
+constexpr int HIT_PEN_CAP = 320;              // history entries of one tile the producer can hand over
+constexpr int HIT_BIAS_CAP = FILTER_BIAS;
 constexpr uint32_t CAND_CAP = 32768;          // candidate slots per row, divided evenly among the row's tiles
 constexpr int MERGE_THREADS = 512;
 constexpr int MERGE_CAP = 8192;               // 64-bit keys the row merge can sort (64 KB of shared memory)

@@ -85,6 +85,13 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, unsigned i
 }
 __device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// Element index of register slot s of a lane.
+template <int DT>
+__device__ __forceinline__ int slot_index(int wbase, int lane, int s) {
+    constexpr int VEC = VecTraits<DT>::VEC;
+    return wbase + (s / VEC) * 32 * VEC + lane * VEC + (s % VEC);
+}
+
 template <int THREADS>
 struct MergeShared {
     int count;
@@ -506,9 +513,10 @@ __device__ bool merge_topk_row(const KParams &P, const RowCfg &c, int row, int t
         if (tid == 0) { sh.tcnt[0] = 0; sh.count = 0; sh.tkey = tk; sh.found = over ? 1 : 0; }
     }
     // Small k: the k-th largest of the maxima of the row's warp tiles is a value that k elements reach and few more do (75
-    // of 2^18 for k = 64), all of them candidates.  bins: the maxima.
+    // of 2^18 for k = 64), all of them candidates, so that the short finish takes them.  (sonic_topk only ranks: there the
+    // bound costs more than it saves, 15.0 against 13.0 us for k = 64.)  bins: the maxima.
     const int groups = tiles * STREAM_WARPS;
-    const bool tight = 2 * c.k <= groups && c.k <= 100;
+    const bool tight = P.op != OP_TOPK && 2 * c.k <= groups && c.k <= 100;
     static_assert(MAX_TILES * STREAM_WARPS * 2 == THREADS, "two threads per maximum at most");
     if (tight && tid < MAX_TILES * STREAM_WARPS) bins[tid] = (tid < groups) ? __ldcg(&P.wmax[(size_t)row * MAX_TILES * STREAM_WARPS + tid]) : 0u;
     csync();
@@ -1229,20 +1237,17 @@ __device__ __forceinline__ float warp_cutoff(float g, bool tile_mode) {
 
 // What the producer hands to the consumers with each stage.
 struct StageMeta {
-    int row, tile, slot;                       // slot: the row's parameters and lists
-    int skip;                                  // the row belongs to another kernel: nothing to do
-    int stop;                                  // no more tiles for this CTA (nothing else in the entry is valid)
-    int next_row, next_tile;                   // the tile that follows (-1: none)
-};
-struct Hit { int id; int payload; };           // a bias entry: token, value bits
-struct RowSlot {                               // a row's parameters and lists
     RowCfg cfg;
-    int patch;                                 // 0 no lists, 1 they are here, 2 consumers scan them in global memory
-    int bad;                                   // a list id outside [0, V)
-    int off[MAX_TILES + 1];                    // the history entries of tile t: list[off[t], off[t + 1])
-    uint32_t list[FILTER_HIST];                // id | count << 18
-    Hit bias[FILTER_BIAS];
+    int row, tile;
+    int skip;                                  // the row belongs to the exact kernel: nothing was loaded
+    int patch;                                 // 0 none, 1 the producer filtered the lists into hits[], 2 consumers scan the lists
+    int npen, nbias;                           // hits of this tile
+    int hb;                                    // which hit buffer holds them
+    int stop;                                  // no more tiles for this CTA (nothing else in the entry is valid)
+    int bad;                                   // the producer met a list id outside [0, V)
+    int next_row, next_tile;                   // the tile that follows (-1: none, or not known yet)
 };
+struct Hit { int li; int payload; };           // element within the tile; history count, or the bias as float bits
 
 template <int DT>
 struct StreamShared {
@@ -1250,12 +1255,14 @@ struct StreamShared {
     unsigned long long full[NSTAGE];           // producer -> consumers: stage described and copy issued (one arrival + the copy's bytes)
     unsigned long long empty[NSTAGE];          // consumers -> producer: stage free (one arrival per consumer warp)
     StageMeta meta[NSTAGE];
-    // per-stage results of the consumer warps, which the producer turns into the tile's record once all of them are done
+    // per-stage scratch of the consumer warps (a fast warp may already be on the next tile, in the other stage)
     alignas(16) float tw[NSTAGE][STREAM_WARPS];
-    unsigned int ncand[NSTAGE], badid[NSTAGE];
-    unsigned long long best[NSTAGE][STREAM_WARPS];       // greedy rows: argmax; top-k rows: cutoff key << 32 | key of the warp's maximum
+    unsigned int ncand[NSTAGE];
+    unsigned long long best[NSTAGE][STREAM_WARPS];
     unsigned int kmin[NSTAGE][STREAM_WARPS], nfin[NSTAGE][STREAM_WARPS];     // dense rows
-    RowSlot slot[NSTAGE + 1];                  // the rows of the tiles in the ring and of the one that is prepared
+    // hit lists: one buffer more than stages, so that the producer fills the next tile's while both stages are busy
+    Hit pen[NSTAGE + 1][HIT_PEN_CAP];
+    Hit bias[NSTAGE + 1][HIT_BIAS_CAP];
 };
 
 template <int DT>
@@ -1284,15 +1291,21 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
     if (warp == STREAM_WARPS) {
         // ------------------------------------------------------------ producer warp
         // The (row, tile) items are handed out through a counter in the workspace, so CTAs that become resident
-        // late (the SMs may be shared) find less or no work instead of holding back a fixed
-        // share.  Per tile the producer waits for a free stage, requests the next tile at once, and only then writes the
-        // record of the tile that left the stage and the description of the new one: what it does by itself is one warp's
-        // serial work of several hundred cycles, which would otherwise lie between a stage's release and its next request.
-        // On a new row one round of global loads brings the parameters and lists into a slot in shared memory.
+        // late (the SMs may be shared with the exact kernel) find less or no work instead of holding back a fixed
+        // share.  Per tile the
+        // producer (1) waits for a free stage, describes the tile and issues its bulk copy, then (2) prepares
+        // the NEXT tile while the ring is busy.  On a new row that means one round of global loads (parameters
+        // and sparse lists, kept in registers for the row's other tiles); on every tile, picking the list
+        // entries that fall into it and writing them to a hit buffer, so that the consumers patch only what is
+        // there, each warp only its own part of the tile.
         static_assert(SONIC_MAX_VOCAB <= (1 << 18), "packed history entries hold an 18-bit id");
-        static_assert(CTA_TILE == 1 << 13, "tile of a token");
-        constexpr int HALF = FILTER_HIST / 64;     // history entries per lane and round of loads
-        int cached_row = -1, cur_slot = 0, cls_cur = CLS_GREEDY;
+        constexpr int HPL = FILTER_HIST / 32;      // packed history entries per lane
+        struct Prep { int patch, npen, nbias; };
+        RowCfg c_next;
+        uint32_t packed[HPL];                      // id | count << 18; 0 = no entry
+        int b_id = -1;
+        float b_val = 0.0f;
+        int row_patch = 0, cached_row = -1, row_bad = 0;
         auto load_row = [&](int row) {
             const int req = (P.op == OP_VERIFY) ? row / (P.K + 1) : row;
             const int *hid = P.hist_ids ? P.hist_ids + (size_t)req * P.hist_stride : nullptr;
@@ -1301,6 +1314,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             const float *bvl = P.bias_vals ? P.bias_vals + (size_t)req * P.bias_stride : nullptr;
             // the first round of loads goes out before the first use (the lengths arrive with the parameters:
             // bound by the strides); the second half of a long history follows in a round of its own
+            constexpr int HALF = HPL / 2;
             const CfgRaw raw = fetch_cfg(P, row);
             int id[HALF], ct[HALF];
 #pragma unroll
@@ -1311,66 +1325,71 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             }
             int b0 = -1; float v0 = 0.0f;
             if (bid && bvl && lane < P.bias_stride) { b0 = __ldg(bid + lane); v0 = __ldg(bvl + lane); }
-            const RowCfg c = resolve_cfg(P, row, raw);
+            c_next = resolve_cfg(P, row, raw);
             cached_row = row;
-            cls_cur = c.cls;
-            cur_slot = (cur_slot + 1) % (NSTAGE + 1);
-            RowSlot &q = sh.slot[cur_slot];
-            int patch = (c.hist_len > 0 || c.bias_len > 0) ? 1 : 0;
-            if (c.hist_len > FILTER_HIST || c.bias_len > FILTER_BIAS) patch = 2;
+            row_patch = 0;
+            row_bad = 0;
+            if (c_next.cls == CLS_EXACT || !(c_next.hist_len > 0 || c_next.bias_len > 0)) return;
+            row_patch = 2;
+            if (c_next.hist_len > FILTER_HIST || c_next.bias_len > FILTER_BIAS) return;
             bool bad = false, big = false;
-            if (patch == 1) {
-                // the history by tile: count, offsets, place
-                q.off[lane] = 0;
-                __syncwarp();
-                uint32_t e[2 * HALF];
-                int at[2 * HALF];
-                auto take = [&](int t, int i, int cnt, uint32_t &out, int &rank) {
-                    out = 0u; rank = 0;
-                    if (t >= c.hist_len) return;
-                    if (i < 0 || i >= P.V) { bad = true; return; }
-                    if (cnt > FILTER_COUNT_MAX) { big = true; return; }
-                    if (cnt <= 0) return;
-                    out = (uint32_t)i | ((uint32_t)cnt << 18);
-                    rank = atomicAdd(&q.off[i >> 13], 1);
-                };
+            auto pack = [&](int t, int i, int cnt) -> uint32_t {
+                if (t >= c_next.hist_len) return 0u;
+                if (i < 0 || i >= P.V) { bad = true; return 0u; }
+                if (cnt > FILTER_COUNT_MAX) { big = true; return 0u; }
+                return (cnt > 0) ? ((uint32_t)i | ((uint32_t)cnt << 18)) : 0u;
+            };
 #pragma unroll
-                for (int u = 0; u < HALF; ++u) take(lane + 32 * u, id[u], ct[u], e[u], at[u]);
+            for (int u = 0; u < HALF; ++u) packed[u] = pack(lane + 32 * u, id[u], ct[u]);
 #pragma unroll
-                for (int u = 0; u < HALF; ++u) { e[HALF + u] = 0u; at[HALF + u] = 0; }
-                if (c.hist_len > 32 * HALF) {
+            for (int u = 0; u < HALF; ++u) packed[HALF + u] = 0u;
+            if (c_next.hist_len > 32 * HALF) {
 #pragma unroll
-                    for (int u = 0; u < HALF; ++u) {
-                        const int t = lane + 32 * (HALF + u);
-                        id[u] = -1; ct[u] = 0;
-                        if (t < c.hist_len) { id[u] = __ldg(hid + t); ct[u] = __ldg(hct + t); }
-                    }
-#pragma unroll
-                    for (int u = 0; u < HALF; ++u) take(lane + 32 * (HALF + u), id[u], ct[u], e[HALF + u], at[HALF + u]);
+                for (int u = 0; u < HALF; ++u) {
+                    const int t = lane + 32 * (HALF + u);
+                    id[u] = -1; ct[u] = 0;
+                    if (t < c_next.hist_len) { id[u] = __ldg(hid + t); ct[u] = __ldg(hct + t); }
                 }
-                __syncwarp();
-                const int cnt = q.off[lane];
-                int incl = cnt;
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) { const int up = __shfl_up_sync(0xFFFFFFFFu, incl, o); if (lane >= o) incl += up; }
-                q.off[lane] = incl - cnt;
-                if (lane == 31) q.off[32] = incl;
-                __syncwarp();
-#pragma unroll
-                for (int u = 0; u < 2 * HALF; ++u)
-                    if (e[u]) q.list[q.off[(e[u] & 0x3FFFFu) >> 13] + at[u]] = e[u];
-                Hit h;
-                h.id = -1; h.payload = 0;
-                if (lane < c.bias_len) {
-                    if (b0 < 0 || b0 >= P.V) bad = true;
-                    else { h.id = b0; h.payload = __float_as_int(v0); }
-                }
-                q.bias[lane] = h;
-                bad = __any_sync(0xFFFFFFFFu, bad);
-                if (__any_sync(0xFFFFFFFFu, big)) patch = 2;       // a count too large to pack: consumers scan
+                for (int u = 0; u < HALF; ++u) packed[HALF + u] = pack(lane + 32 * (HALF + u), id[u], ct[u]);
             }
-            if (lane == 0) { q.cfg = c; q.patch = patch; q.bad = bad ? 1 : 0; }
-            __syncwarp();
+            b_id = -1; b_val = 0.0f;
+            if (lane < c_next.bias_len) {
+                if (b0 < 0 || b0 >= P.V) bad = true;
+                else { b_id = b0; b_val = v0; }
+            }
+            row_bad = __any_sync(0xFFFFFFFFu, bad) ? 1 : 0;
+            if (__any_sync(0xFFFFFFFFu, big)) return;          // a count too large to pack: consumers scan
+            row_patch = 1;
+        };
+        auto prepare = [&](int row, int tile, int hb) -> Prep {
+            if (row != cached_row) load_row(row);
+            Prep r{row_patch, 0, 0};
+            if (row_patch != 1) return r;
+            const int first = tile * CTA_TILE;
+#pragma unroll
+            for (int u = 0; u < HPL; ++u) {
+                const unsigned int li = (packed[u] & 0x3FFFFu) - (unsigned int)first;
+                const bool hit = packed[u] != 0u && li < (unsigned int)CTA_TILE;
+                const unsigned int hm = __ballot_sync(0xFFFFFFFFu, hit);
+                if (hit) {
+                    const int pos = r.npen + __popc(hm & ((1u << lane) - 1u));
+                    if (pos < HIT_PEN_CAP) { sh.pen[hb][pos].li = (int)li; sh.pen[hb][pos].payload = (int)(packed[u] >> 18); }
+                }
+                r.npen += __popc(hm);
+            }
+            {
+                const unsigned int li = (unsigned int)(b_id - first);
+                const bool hit = b_id >= 0 && li < (unsigned int)CTA_TILE;
+                const unsigned int hm = __ballot_sync(0xFFFFFFFFu, hit);
+                if (hit) {
+                    const int pos = __popc(hm & ((1u << lane) - 1u));
+                    sh.bias[hb][pos].li = (int)li; sh.bias[hb][pos].payload = __float_as_int(b_val);
+                }
+                r.nbias = __popc(hm);
+            }
+            if (r.npen > HIT_PEN_CAP) r.patch = 2;             // crowded tile: the consumers scan the lists
+            return r;
         };
         const unsigned long long l2_policy = l2_evict_first_policy();
         // Work queue: one counter of items.  A CTA first asks for `chunk` consecutive items (seven eighths of an
@@ -1392,13 +1411,10 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 if (lane == 0 && run_lo < nitems) nxt_raw = (int)atomicAdd(queue, 1u);
             }
         };
-        // The next item, with its row's parameters and lists loaded.
-        auto find_item = [&]() -> int {
-            const int it = current_item();
-            if (it >= 0 && it / tiles != cached_row) load_row(it / tiles);
-            return it;
-        };
+        int n = 0;
+        Prep p_next{0, 0, 0};
         int item = current_item();
+        bool prepared = false;
         // lane 0: the tile's bulk copy, with the arrival on full[s] (arrive == true) or with the bytes announced only
         // (the arrival then follows once the stage's description is written)
         auto issue_copy = [&](int row, int tile, int s, bool arrive) {
@@ -1419,76 +1435,45 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         // rounds of global loads): the copy's latency hides behind them.  (A row of the cluster kernel's class gets
         // a copy nobody reads: such rows are rare.)
         if (item >= 0 && lane == 0) issue_copy(item / tiles, item % tiles, 0, false);
-        // The record of a tile that every consumer warp has left: candidates, cutoff, argmax, bad list ids.
-        auto retire = [&](int s) {
-            const int row = sh.meta[s].row, tile = sh.meta[s].tile;
-            if (sh.meta[s].skip) {
-                // a row of the cluster kernel: counted, its status word initialised
-                if (tile == 0 && lane == 0) { P.rs[row].status = 0u; atomicAdd(&P.error[WS_NEXACT], 1u); }
-                return;
+        for (;; ++n) {
+            const int s = n % NSTAGE;
+            if (n >= NSTAGE) {
+                // the consumers have left tile n - NSTAGE: its stage and its hit buffer are free
+                if (!mbar_wait(&sh.empty[s], ((n / NSTAGE) - 1) & 1)) {
+                    if (lane == 0) atomicOr(P.error, ERR_TIMEOUT);
+                    return;
+                }
             }
-            const RowSlot &q = sh.slot[sh.meta[s].slot];
-            unsigned long long b = (lane < STREAM_WARPS) ? sh.best[s][lane] : 0ull;
-            unsigned int kmn = 0xFFFFFFFFu, nf = 0u;
-            if (q.cfg.cls == CLS_DENSE) {
-                kmn = __reduce_min_sync(0xFFFFFFFFu, lane < STREAM_WARPS ? sh.kmin[s][lane] : 0xFFFFFFFFu);
-                nf = __reduce_add_sync(0xFFFFFFFFu, lane < STREAM_WARPS ? sh.nfin[s][lane] : 0u);
+            if (item < 0) {                            // out of work: tell the consumers
+                if (lane == 0) { sh.meta[s].stop = 1; mbar_arrive(&sh.full[s]); }
+                break;
             }
-            if (lane < STREAM_WARPS && q.cfg.cls == CLS_TOPK) P.wmax[((size_t)row * MAX_TILES + tile) * STREAM_WARPS + lane] = (uint32_t)b;
-#pragma unroll
-            for (int off = STREAM_WARPS / 2; off > 0; off >>= 1) b = max(b, __shfl_xor_sync(0xFFFFFFFFu, b, off));
+            const int row = item / tiles, tile = item - row * tiles;
+            if (!prepared) {                           // the CTA's first tile: nothing was prepared ahead
+                p_next = prepare(row, tile, n % (NSTAGE + 1));
+                prepared = true;
+            }
+            const RowCfg c = c_next;
+            const Prep pr = p_next;
+            const int bad_now = row_bad;
+            advance();
+            const int nxt = current_item();
+            __syncwarp();                              // the hit buffer's entries, written by all lanes, precede the arrival
             if (lane == 0) {
-                TileRec r;
-                r.best = b; r.cnt = sh.ncand[s]; r.tkey = (unsigned int)(b >> 32);
-                r.flags = (q.bad || sh.badid[s]) ? TILE_BADID : 0u;
-                r.minkey = kmn; r.nfin = nf; r.pad = 0u;
-                P.tiles[(size_t)row * MAX_TILES + tile] = r;
-                if (tile == 0) P.rs[row].status = 0u;
+                StageMeta &m = sh.meta[s];
+                m.cfg = c; m.row = row; m.tile = tile; m.skip = (c.cls == CLS_EXACT) ? 1 : 0;
+                m.patch = pr.patch; m.npen = pr.npen; m.nbias = pr.nbias; m.hb = n % (NSTAGE + 1);
+                m.stop = 0;
+                m.bad = bad_now;
+                m.next_row = (nxt >= 0) ? nxt / tiles : -1;
+                m.next_tile = (nxt >= 0) ? nxt % tiles : -1;
+                if (n == 0 || c.cls == CLS_EXACT) mbar_arrive(&sh.full[s]);     // (the first tile's copy is under way; nothing is copied for rows of the cluster kernel's class)
+                else issue_copy(row, tile, s, true);
             }
             __syncwarp();
-        };
-        int n = -1;
-        for (;; ++n) {                                 // (round -1 only prepares the first tile)
-            if (n >= 0) {
-                const int s = n % NSTAGE;
-                const bool skip = item >= 0 && cls_cur == CLS_EXACT;
-                const int row = item / tiles, tile = item - row * tiles;
-                if (n >= NSTAGE) {
-                    // the consumers have left tile n - NSTAGE: its stage is free
-                    if (!mbar_wait(&sh.empty[s], ((n / NSTAGE) - 1) & 1)) {
-                        if (lane == 0) atomicOr(P.error, ERR_TIMEOUT);
-                        return;
-                    }
-                    // (the first tiles' copies are under way; nothing is copied for rows of the cluster kernel's class)
-                    if (item >= 0 && !skip && lane == 0) issue_copy(row, tile, s, false);
-                    retire(s);
-                }
-                if (item < 0) {                            // out of work: tell the consumers
-                    if (lane == 0) { sh.meta[s].stop = 1; mbar_arrive(&sh.full[s]); }
-                    break;
-                }
-                advance();
-                const int hint = current_item();           // the tile that follows
-                if (lane == 0) {
-                    if (n > 0 && n < NSTAGE && !skip) issue_copy(row, tile, s, false);
-                    StageMeta &m = sh.meta[s];
-                    m.row = row; m.tile = tile; m.slot = cur_slot; m.skip = skip ? 1 : 0;
-                    m.stop = 0;
-                    m.next_row = (hint >= 0) ? hint / tiles : -1;
-                    m.next_tile = (hint >= 0) ? hint - m.next_row * tiles : -1;
-                    sh.ncand[s] = 0u; sh.badid[s] = 0u;
-                    mbar_arrive(&sh.full[s]);
-                }
-                __syncwarp();
-            }
-            item = find_item();
-        }
-        for (int i = max(0, n - NSTAGE + 1); i < n; ++i) {     // the last tiles
-            if (!mbar_wait(&sh.empty[i % NSTAGE], (i / NSTAGE) & 1)) {
-                if (lane == 0) atomicOr(P.error, ERR_TIMEOUT);
-                return;
-            }
-            retire(i % NSTAGE);
+            // hit buffer (n + 1) % (NSTAGE + 1) was last used by tile n - NSTAGE, which the consumers have left
+            if (nxt >= 0) p_next = prepare(nxt / tiles, nxt % tiles, (n + 1) % (NSTAGE + 1));
+            item = nxt;
         }
         return;
     }
@@ -1502,93 +1487,128 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         const int w = ((tile * CTA_TILE + warp * WARP_TILE) >> 5) + lane;
         return (w < ((P.V + 31) >> 5)) ? __ldg(P.bitmask + (size_t)row * P.bitmask_stride + w) : 0u;
     };
-    // What a warp carries from tile to tile of a row.  Top-k rows: the cutoff, taken from the CTA's first tile of the row
-    // and kept for the tiles that follow (any cutoff is good as long as the tile's record names it; a tile then costs its
-    // maxima and one vote, without a block barrier).  Greedy rows: what an element must reach to matter.
-    int cut_row = -1, g_row = -1;
-    float cut = 0.0f, g_thr = 0.0f;
     for (int n = 0;; ++n) {
         const int s = n % NSTAGE;
         if (!mbar_wait(&sh.full[s], (n / NSTAGE) & 1)) {
             if (lane == 0) atomicOr(P.error, ERR_TIMEOUT);
             return;
         }
-        const StageMeta &meta = sh.meta[s];
-        if (meta.stop) { KERNEL_T1(0); break; }
-        const int row = meta.row, tile = meta.tile;
+        if (sh.meta[s].stop) { KERNEL_T1(0); break; }
+        const int row = sh.meta[s].row, tile = sh.meta[s].tile;
         const int tile_base = tile * CTA_TILE;
+        const int wbase = tile_base + warp * WARP_TILE;
         uint32_t mword = 0xFFFFFFFFu;
         if (P.bitmask) {
             mword = (row == pre_row && tile == pre_tile) ? mword_pre : load_mask_words(row, tile);
-            pre_row = meta.next_row; pre_tile = meta.next_tile;
+            pre_row = sh.meta[s].next_row; pre_tile = sh.meta[s].next_tile;
             if (pre_row >= 0) mword_pre = load_mask_words(pre_row, pre_tile);
         }
-        if (!meta.skip) {
-            const unsigned char *stage = stages + (size_t)s * STAGE_BYTES;
-            const RowSlot &slot = sh.slot[meta.slot];
-            const bool masked = (slot.cfg.z & M_GRAMMAR) != 0;
+        const StageMeta &meta = sh.meta[s];
+        if (meta.skip) {
+            // a row of the cluster kernel: counted, its status word initialised
+            if (tile == 0 && tid == 0) { P.rs[row].status = 0u; atomicAdd(&P.error[WS_NEXACT], 1u); }
+        } else {
+            const RowCfg c = meta.cfg;
+            RowState *rs = P.rs + row;
+            TileRec *rec = P.tiles + (size_t)row * MAX_TILES + tile;
+            // Every per-row word of the workspace is initialised by the call that reads it: the tile's flags here
+            // (before any barrier of this tile), the row's status word and, for rows of the histogram path, the
+            // row's control block and its histogram by the CTA of the row's first tile.
+            if (tid == 0) {
+                rec->flags = meta.bad ? TILE_BADID : 0u;
+                if (tile == 0) rs->status = 0u;
+            }
+            if (c.cls == CLS_DENSE && tile == 0) {
+                uint4 *h = reinterpret_cast<uint4 *>(P.hist + (size_t)row * DBINS);
+                for (int i = tid; i < DBINS / 2; i += STREAM_THREADS) h[i] = make_uint4(0u, 0u, 0u, 0u);
+                if (tid == 0) {
+                    DenseRow *dr = P.drow + row;
+                    dr->ticket_h = 0u; dr->ticket_c = 0u; dr->ticket_r = 0u; dr->nmembers = 0u;
+                    dr->kmin = 0xFFFFFFFFu; dr->kmax = 0u; dr->overflow = 0u; dr->state = 0u;
+                    P.dlist[atomicAdd(&P.error[WS_NDENSE], 1u)] = row;
+                }
+            }
+            unsigned char *stage = stages + (size_t)s * STAGE_BYTES;
+            const bool masked = (c.z & M_GRAMMAR) != 0;
             const bool tail = tile_base + CTA_TILE > P.V;
-            const int patch = slot.patch;
-            // word: which of the 32 consecutive elements from lane * 32 count.  Under a sparse mask (a grammar allows a few per
-            // cent of the ids) a lane walks its word's few set bits instead of 32 elements.
-            uint32_t word = masked ? mword : 0xFFFFFFFFu;
-            if (tail) { const int left = P.V - tile_base - warp * WARP_TILE - lane * 32; if (left < 32) word &= left > 0 ? (1u << left) - 1u : 0u; }
-            const bool sparse = masked && __all_sync(0xFFFFFFFFu, __popc(word) <= 8);
-            float *ptile = (DT == 0) ? reinterpret_cast<float *>(stages + (size_t)s * STAGE_BYTES) : conv;    // fp32 view the sparse lists patch
-            bool wide = DT == 0;                               // the warp's part is fp32 in ptile (else bf16 in the stage)
-            const int lane0 = warp * WARP_TILE + lane * VEC;   // the lane's first element within the tile
-            auto widen = [&]() {                               // bf16 only: the warp's part as fp32
+            int patch = meta.patch;
+            // word: which of the warp tile's 32 consecutive elements from lane * 32 count.  Under a sparse mask (a grammar allows
+            // a few per cent of the ids) a lane walks its word's few set bits instead of 32 elements, and list entries that
+            // the mask forbids are not patched (they stay -inf).  2 % of 2^18 fp32 entries, 128 rows with 512 entries of
+            // history: the kernel's warp instructions from 19.6 to 14 million.
+            uint32_t word = mword;
+            if (masked && tail) { const int left = P.V - wbase - lane * 32; if (left < 32) word &= left > 0 ? (1u << left) - 1u : 0u; }
+            const bool sparse = masked && c.cls != CLS_DENSE && __all_sync(0xFFFFFFFFu, __popc(word) <= 8);
+            if (sparse && patch == 1) {
+                bool any = false;
+                auto look = [&](const Hit *hits, int count) {
+                    for (int h0 = 0; h0 < count; h0 += 32) {
+                        const int li = (h0 + lane < count) ? hits[h0 + lane].li : -1;
+                        const uint32_t w = __shfl_sync(0xFFFFFFFFu, word, (li >> 5) & 31);
+                        any = any || (li >= 0 && li / WARP_TILE == warp && ((w >> (li & 31)) & 1u));
+                    }
+                };
+                look(sh.pen[meta.hb], meta.npen);
+                look(sh.bias[meta.hb], meta.nbias);
+                if (!__any_sync(0xFFFFFFFFu, any)) patch = 0;
+            }
+            const bool patched = patch != 0;
+            float *ptile = (DT == 0) ? reinterpret_cast<float *>(stage) : conv;    // fp32 view the sparse lists patch
+
+            float e[EPL];
+            auto read_raw = [&]() {
 #pragma unroll
                 for (int j = 0; j < NV; ++j) {
-                    const uint4 raw = *reinterpret_cast<const uint4 *>(stage + (size_t)(lane0 + j * 32 * VEC) * ELT);
-                    float *p = conv + lane0 + j * 32 * VEC;
-                    *reinterpret_cast<float4 *>(p) = make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xFFFF0000u),
-                                                                 __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xFFFF0000u));
-                    *reinterpret_cast<float4 *>(p + 4) = make_float4(__uint_as_float(raw.z << 16), __uint_as_float(raw.z & 0xFFFF0000u),
-                                                                     __uint_as_float(raw.w << 16), __uint_as_float(raw.w & 0xFFFF0000u));
+                    const int li = warp * WARP_TILE + j * 32 * VEC + lane * VEC;
+                    const uint4 raw = *reinterpret_cast<const uint4 *>(stage + (size_t)li * ELT);
+                    const uint32_t r[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+                    for (int q = 0; q < VEC; ++q) {
+                        if (DT == 0) e[j * VEC + q] = __uint_as_float(r[q]);
+                        else e[j * VEC + q] = __uint_as_float((q & 1) ? (r[q >> 1] & 0xFFFF0000u) : (r[q >> 1] << 16));
+                    }
                 }
             };
-            // penalties and biases commute with the mask (a masked logit stays -inf), so they are applied to the unmasked tile
-            if (patch == 1) {
-                // the producer listed this tile's entries: every warp patches its own part, if there are any in it
-                // (that the mask allows)
-                const int first = slot.off[tile], npen = slot.off[tile + 1] - first, nbias = slot.cfg.bias_len;
-                auto mine = [&](int li) -> bool {                // (every lane calls it; li: element of the tile, or anything outside)
-                    const uint32_t w = __shfl_sync(0xFFFFFFFFu, word, (li >> 5) & 31);
-                    return (li >> 10) == warp && ((w >> (li & 31)) & 1u);
-                };
-                static_assert(WARP_TILE == 1024 && FILTER_BIAS == 32, "element -> warp; one bias entry per lane");
-                bool any = false;
-                for (int h0 = 0; h0 < npen; h0 += 32) {
-                    const bool m = mine((h0 + lane < npen) ? (int)(slot.list[first + h0 + lane] & 0x3FFFFu) - tile_base : -1);
-                    any = any || m;
-                }
-                int bli = -1;
-                float bval = 0.0f;
-                if (nbias > 0) {
-                    const Hit h = slot.bias[lane];
-                    bli = (h.id >= 0) ? h.id - tile_base : -1;
-                    bval = __int_as_float(h.payload);
-                    if (!mine(bli)) bli = -1;
-                    any = any || bli >= 0;
-                }
-                if (__any_sync(0xFFFFFFFFu, any)) {
-                    const RowCfg c = slot.cfg;
-                    if (DT == 1) { widen(); wide = true; }
-                    __syncwarp();
-                    for (int h = lane; h < npen; h += 32) {
-                        const uint32_t e = slot.list[first + h];
-                        const int li = (int)(e & 0x3FFFFu) - tile_base;
-                        if ((li >> 10) == warp) ptile[li] = apply_penalties(ptile[li], (int)(e >> 18), c);
+            auto read_f32 = [&](const float *src) {
+#pragma unroll
+                for (int j = 0; j < NV; ++j) {
+                    const float *p = src + warp * WARP_TILE + j * 32 * VEC + lane * VEC;
+#pragma unroll
+                    for (int q = 0; q < VEC; q += 4) {
+                        const float4 v = *reinterpret_cast<const float4 *>(p + q);
+                        e[j * VEC + q] = v.x; e[j * VEC + q + 1] = v.y; e[j * VEC + q + 2] = v.z; e[j * VEC + q + 3] = v.w;
                     }
-                    __syncwarp();
-                    if (bli >= 0) ptile[bli] = __fadd_rn(ptile[bli], bval);
-                    __syncwarp();
                 }
+            };
+            auto widen = [&]() {                      // bf16 only: the warp's part of the tile as fp32 in shared memory
+#pragma unroll
+                for (int j = 0; j < NV; ++j) {
+                    float *p = conv + warp * WARP_TILE + j * 32 * VEC + lane * VEC;
+#pragma unroll
+                    for (int q = 0; q < VEC; q += 4)
+                        *reinterpret_cast<float4 *>(p + q) = make_float4(e[j * VEC + q], e[j * VEC + q + 1], e[j * VEC + q + 2], e[j * VEC + q + 3]);
+                }
+            };
+            // penalties and biases commute with the mask (a masked logit stays -inf), so they are applied to
+            // the unmasked tile and the mask is applied when the lanes read their elements
+            if (patch == 1) {
+                // the producer listed this tile's entries: every warp patches its own part, no block-wide barrier
+                if (DT == 1) { read_raw(); widen(); }
+                __syncwarp();
+                for (int h = lane; h < meta.npen; h += 32) {
+                    const Hit x = sh.pen[meta.hb][h];
+                    if (x.li / WARP_TILE == warp) ptile[x.li] = apply_penalties(ptile[x.li], x.payload, c);
+                }
+                __syncwarp();
+                for (int h = lane; h < meta.nbias; h += 32) {
+                    const Hit x = sh.bias[meta.hb][h];
+                    if (x.li / WARP_TILE == warp) ptile[x.li] = __fadd_rn(ptile[x.li], __int_as_float(x.payload));
+                }
+                __syncwarp();
+                if (!sparse) read_f32(ptile);
             } else if (patch == 2) {
                 // long or crowded lists: all consumer threads scan them together
-                const RowCfg c = slot.cfg;
-                if (DT == 1) { widen(); wide = true; csync(); }
+                if (DT == 1) { read_raw(); widen(); csync(); }
                 const int req = (P.op == OP_VERIFY) ? row / (P.K + 1) : row;
                 const int *hid = P.hist_ids + (size_t)req * P.hist_stride;
                 const int *hct = P.hist_counts + (size_t)req * P.hist_stride;
@@ -1606,309 +1626,245 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                     const int li = id - tile_base;
                     if (li >= 0 && li < CTA_TILE) ptile[li] = __fadd_rn(ptile[li], __ldg(P.bias_vals + (size_t)req * P.bias_stride + t));
                 }
-                if (bad) sh.badid[s] = 1u;
+                if (bad) atomicOr(&rec->flags, TILE_BADID);          // (ordered after the first thread's store by the barriers above)
                 csync();
+                if (!sparse) read_f32(ptile);
+            } else if (!sparse) {
+                read_raw();
             }
-
-            if (slot.cfg.cls == CLS_DENSE) {
-                // Histogram path: the processed logits (divided by the temperature) are kept as ordered keys for the later
-                // passes; per tile the largest and smallest finite key and the number of finite elements.  The CTA of the
-                // row's first tile initialises the row's control block and histogram and lists the row.
-                if (tile == 0) {
-                    uint4 *h = reinterpret_cast<uint4 *>(P.hist + (size_t)row * DBINS);
-                    for (int i = tid; i < DBINS / 2; i += STREAM_THREADS) h[i] = make_uint4(0u, 0u, 0u, 0u);
-                    if (tid == 0) {
-                        DenseRow *dr = P.drow + row;
-                        dr->ticket_h = 0u; dr->ticket_c = 0u; dr->ticket_r = 0u; dr->nmembers = 0u;
-                        dr->kmin = 0xFFFFFFFFu; dr->kmax = 0u; dr->overflow = 0u; dr->state = 0u;
-                        P.dlist[atomicAdd(&P.error[WS_NDENSE], 1u)] = row;
-                    }
-                }
-                const bool divide = slot.cfg.div_all, all = !masked && !tail;
-                const float tau = slot.cfg.tau;
-                uint32_t kmx = 0u, kmn = 0xFFFFFFFFu;
-                unsigned int nf = 0u;
-                unsigned int *yk = P.ykeys + (size_t)row * ((size_t)P.ytiles * CTA_TILE) + tile_base;
+            if (sparse) {
+            } else if (masked && !tail) {
+                // the common masked case: one select per element, no bounds test
 #pragma unroll
                 for (int j = 0; j < NV; ++j) {
-                    const int li = lane0 + j * 32 * VEC;
-                    const uint32_t bits = all ? 0xFFFFFFFFu : __shfl_sync(0xFFFFFFFFu, word, (j * 32 * VEC + lane * VEC) >> 5) >> ((lane * VEC) & 31);
-                    float v[VEC];
-                    if (DT == 1 && !wide) {
-                        const uint4 raw = *reinterpret_cast<const uint4 *>(stage + (size_t)li * ELT);
-                        const uint32_t r[4] = {raw.x, raw.y, raw.z, raw.w};
+                    const uint32_t bits = __shfl_sync(0xFFFFFFFFu, mword, (j * 32 * VEC + lane * VEC) >> 5) >> ((lane * VEC) & 31);
 #pragma unroll
-                        for (int q = 0; q < VEC; ++q) v[q] = __uint_as_float((q & 1) ? (r[(q >> 1) & 3] & 0xFFFF0000u) : (r[(q >> 1) & 3] << 16));
-                    } else {
+                    for (int q = 0; q < VEC; ++q) e[j * VEC + q] = (bits & (1u << q)) ? e[j * VEC + q] : -CUDART_INF_F;
+                }
+            } else if (tail) {
 #pragma unroll
-                        for (int q = 0; q < VEC; q += 4) {
-                            const float4 a = *reinterpret_cast<const float4 *>(ptile + li + q);
-                            v[q] = a.x; v[q + 1] = a.y; v[q + 2] = a.z; v[q + 3] = a.w;
-                        }
-                    }
+                for (int j = 0; j < NV; ++j) {
+                    const int first = wbase + j * 32 * VEC + lane * VEC;
+                    const uint32_t bits = __shfl_sync(0xFFFFFFFFu, mword, (j * 32 * VEC + lane * VEC) >> 5) >> (first & 31);
 #pragma unroll
-                    for (int q4 = 0; q4 < VEC; q4 += 4) {
-                        uint32_t kk[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            float y = ((bits >> (q4 + u)) & 1u) ? v[q4 + u] : -CUDART_INF_F;
-                            if (divide) y = div_tau(y, tau);
-                            kk[u] = okey(y);
-                            const bool fin = kk[u] > KEY_NEG_INF;
-                            nf += fin ? 1u : 0u;
-                            kmn = fin ? min(kmn, kk[u]) : kmn;
-                            kmx = fin ? max(kmx, kk[u]) : kmx;
-                        }
-                        *reinterpret_cast<uint4 *>(yk + li + q4) = make_uint4(kk[0], kk[1], kk[2], kk[3]);
+                    for (int q = 0; q < VEC; ++q) {
+                        const bool dead = (first + q >= P.V) || (masked && !((bits >> q) & 1u));
+                        if (dead) e[j * VEC + q] = -CUDART_INF_F;
                     }
                 }
-                kmx = __reduce_max_sync(0xFFFFFFFFu, kmx);
-                kmn = __reduce_min_sync(0xFFFFFFFFu, kmn);
-                nf = __reduce_add_sync(0xFFFFFFFFu, nf);
-                if (lane == 0) { sh.best[s][warp] = (unsigned long long)kmx << 32; sh.kmin[s][warp] = kmn; sh.nfin[s][warp] = nf; }
-                if (DT == 0 && patch != 0) fence_async_proxy();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sh.empty[s]);
-                continue;
+            }
+            if (c.div_all && !sparse) {
+#pragma unroll
+                for (int q = 0; q < EPL; ++q) e[q] = div_tau(e[q], c.tau);
             }
 
-            // Maxima of the lane's vectors.  ebits: which of its 32 elements count (allowed by the mask, inside the row).
-            // raw: the lane's elements as they lie in the stage (not of a widened part): what is looked at again stays in registers
-            float mv[NV];
-            uint4 raw[NV];
-            uint32_t ebits = 0xFFFFFFFFu;
-            auto value = [&](int li) -> float {                // one element of the tile
-                return (DT == 1 && !wide) ? __uint_as_float((uint32_t)reinterpret_cast<const unsigned short *>(stage)[li] << 16) : ptile[li];
+            // one element of the tile, by its place in the lane's mask word
+            auto word_value = [&](int b) -> float {
+                const int li = warp * WARP_TILE + lane * 32 + b;
+                float v;
+                if (DT == 0 || patched) v = ptile[li];
+                else v = __uint_as_float((uint32_t)reinterpret_cast<const unsigned short *>(stage)[li] << 16);
+                return c.div_all ? div_tau(v, c.tau) : v;
             };
-            float h0 = -CUDART_INF_F, h1 = -CUDART_INF_F;      // maxima of the lane's two halves
+            // per-vector maxima, half maxima, lane maximum
+            float qm[4];                               // maxima of the lane's four quarters (8 elements each)
             if (sparse) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) qm[i] = -CUDART_INF_F;
                 for (uint32_t w = word; w; w &= w - 1u) {
                     const int b = __ffs(w) - 1;
-                    const float v = value(warp * WARP_TILE + lane * 32 + b);
-                    if (b < 16) h0 = fmaxf(h0, v); else h1 = fmaxf(h1, v);
-                }
-            } else if (!masked && !tail) {
-#pragma unroll
-                for (int j = 0; j < NV; ++j) {
-                    const int li = lane0 + j * 32 * VEC;
-                    if (DT == 1 && !wide) {
-                        // bf16 pairs: half an instruction per element
-                        raw[j] = *reinterpret_cast<const uint4 *>(stage + (size_t)li * ELT);
-                        const __nv_bfloat162 m = __hmax2(__hmax2(*reinterpret_cast<const __nv_bfloat162 *>(&raw[j].x), *reinterpret_cast<const __nv_bfloat162 *>(&raw[j].y)),
-                                                         __hmax2(*reinterpret_cast<const __nv_bfloat162 *>(&raw[j].z), *reinterpret_cast<const __nv_bfloat162 *>(&raw[j].w)));
-                        const uint32_t u = *reinterpret_cast<const uint32_t *>(&m);
-                        mv[j] = fmaxf(__uint_as_float(u << 16), __uint_as_float(u & 0xFFFF0000u));
-                    } else {
-                        const float4 a = *reinterpret_cast<const float4 *>(ptile + li);
-                        if (DT == 0) raw[j] = make_uint4(__float_as_uint(a.x), __float_as_uint(a.y), __float_as_uint(a.z), __float_as_uint(a.w));
-                        mv[j] = fmaxf(fmaxf(a.x, a.y), fmaxf(a.z, a.w));
-                        if (VEC == 8) {
-                            const float4 b = *reinterpret_cast<const float4 *>(ptile + li + 4);
-                            mv[j] = fmaxf(mv[j], fmaxf(fmaxf(b.x, b.y), fmaxf(b.z, b.w)));
-                        }
-                    }
+                    const float v = word_value(b);
+                    if (b < 16) qm[0] = fmaxf(qm[0], v); else qm[2] = fmaxf(qm[2], v);
                 }
             } else {
-                ebits = 0u;
+            float mv[NV];
 #pragma unroll
-                for (int j = 0; j < NV; ++j) {
-                    const int li = lane0 + j * 32 * VEC;
-                    const uint32_t bits = (__shfl_sync(0xFFFFFFFFu, word, (j * 32 * VEC + lane * VEC) >> 5) >> ((lane * VEC) & 31)) & ((1u << VEC) - 1u);
-                    ebits |= bits << (j * VEC);
-                    float v[VEC];
-                    if (DT == 0 || !wide) {
-                        raw[j] = *reinterpret_cast<const uint4 *>(stage + (size_t)li * ELT);
-                        const uint32_t r[4] = {raw[j].x, raw[j].y, raw[j].z, raw[j].w};
+            for (int j = 0; j < NV; ++j) {
+                float m = e[j * VEC];
 #pragma unroll
-                        for (int q = 0; q < VEC; ++q) v[q] = DT == 0 ? __uint_as_float(r[q & 3]) : __uint_as_float((q & 1) ? (r[(q >> 1) & 3] & 0xFFFF0000u) : (r[(q >> 1) & 3] << 16));
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < VEC; q += 4) {
-                            const float4 a = *reinterpret_cast<const float4 *>(ptile + li + q);
-                            v[q] = a.x; v[q + 1] = a.y; v[q + 2] = a.z; v[q + 3] = a.w;
-                        }
-                    }
-                    mv[j] = -CUDART_INF_F;
-#pragma unroll
-                    for (int q = 0; q < VEC; ++q) mv[j] = ((bits >> q) & 1u) ? fmaxf(mv[j], v[q]) : mv[j];
-                }
+                for (int q = 1; q < VEC; ++q) m = fmaxf(m, e[j * VEC + q]);
+                mv[j] = m;
             }
-            if (!sparse) {
 #pragma unroll
-                for (int j = 0; j < NV / 2; ++j) { h0 = fmaxf(h0, mv[j]); h1 = fmaxf(h1, mv[NV / 2 + j]); }
+            for (int i = 0; i < 4; ++i) {
+                qm[i] = mv[i * (NV / 4)];
+#pragma unroll
+                for (int j = 1; j < NV / 4; ++j) qm[i] = fmaxf(qm[i], mv[i * (NV / 4) + j]);
             }
+            }
+            const float h0 = fmaxf(qm[0], qm[1]), h1 = fmaxf(qm[2], qm[3]);
             const float lm = fmaxf(h0, h1);
-            // The elements of the lane's vectors whose maximum reaches t, one vector after the other (rare: read again):
-            // f(value, index within the tile) for those that reach t.
-            auto visit = [&](float t, auto f) {
-                if (sparse) {
-#pragma unroll 1
-                    for (uint32_t w = word; w; w &= w - 1u) {
-                        const int li = warp * WARP_TILE + lane * 32 + __ffs(w) - 1;
-                        const float v = value(li);
-                        if (v >= t) f(v, li);
-                    }
-                    return;
-                }
-                unsigned int vm = 0u;
-#pragma unroll
-                for (int j = 0; j < NV; ++j) vm |= (mv[j] >= t) ? (1u << j) : 0u;
-#pragma unroll 1
-                while (vm) {
-                    const int j = __ffs(vm) - 1, li = lane0 + j * 32 * VEC;
-                    vm &= vm - 1u;
-                    const uint32_t bits = ebits >> (j * VEC);
-#pragma unroll
-                    for (int q = 0; q < VEC; q += 4) {
-                        float4 a;
-                        if (DT == 1 && !wide) {
-                            const uint2 r = *reinterpret_cast<const uint2 *>(stage + (size_t)(li + q) * ELT);
-                            a = make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xFFFF0000u), __uint_as_float(r.y << 16), __uint_as_float(r.y & 0xFFFF0000u));
-                        } else a = *reinterpret_cast<const float4 *>(ptile + li + q);
-                        if (a.x >= t && ((bits >> q) & 1u)) f(a.x, li + q);
-                        if (a.y >= t && ((bits >> (q + 1)) & 1u)) f(a.y, li + q + 1);
-                        if (a.z >= t && ((bits >> (q + 2)) & 1u)) f(a.z, li + q + 2);
-                        if (a.w >= t && ((bits >> (q + 3)) & 1u)) f(a.w, li + q + 3);
-                    }
-                }
-            };
 
-            if (slot.cfg.cls == CLS_GREEDY) {
-                // The argmax of the processed logits, lowest index first.  Only elements at or above the largest so far can
-                // matter (with a temperature: above a hair less, since the division may make them equal).
-                if (row != g_row) { g_row = row; g_thr = -CUDART_MAX_NORMAL_F; }
-                unsigned long long best = 0ull;
-                if (__any_sync(0xFFFFFFFFu, lm >= g_thr)) {
-                    const bool temp = slot.cfg.temp;
-                    const float tau = slot.cfg.tau;
-                    if (lm >= g_thr) visit(g_thr, [&](float z, int li) {
-                        const uint32_t key = okey(temp ? div_tau(z, tau) : z);
-                        best = max(best, ((unsigned long long)key << 32) | (uint32_t)(~(uint32_t)(tile_base + li)));
-                    });
-                    __syncwarp();
-                    const uint32_t hi = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(best >> 32));
-                    const uint32_t lo = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(best >> 32) == hi ? (uint32_t)best : 0u);
-                    best = ((unsigned long long)hi << 32) | lo;
-                    const float z = unkey(__reduce_max_sync(0xFFFFFFFFu, okey(lm)));
-                    g_thr = fmaxf(g_thr, temp ? z - fmaxf(fabsf(z) * 4.76837158203125e-07f, 1e-37f) : z);
+            if (c.cls == CLS_GREEDY || c.cls == CLS_DENSE) {
+                if (c.cls == CLS_DENSE) {
+                    // histogram path: the processed logits (already divided by the temperature) are kept as ordered
+                    // keys for the later passes; per tile the smallest finite key and the number of finite elements
+                    uint32_t kmn = 0xFFFFFFFFu;
+                    unsigned int nf = 0u;
+                    unsigned int *yk = P.ykeys + (size_t)row * ((size_t)P.ytiles * CTA_TILE) + tile_base + warp * WARP_TILE;
+#pragma unroll
+                    for (int j = 0; j < NV; ++j) {
+#pragma unroll
+                        for (int q4 = 0; q4 < VEC; q4 += 4) {
+                            uint32_t kk[4];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                kk[u] = okey(e[j * VEC + q4 + u]);
+                                const bool fin = kk[u] > KEY_NEG_INF;
+                                nf += fin ? 1u : 0u;
+                                kmn = fin ? min(kmn, kk[u]) : kmn;
+                            }
+                            *reinterpret_cast<uint4 *>(yk + j * 32 * VEC + lane * VEC + q4) = make_uint4(kk[0], kk[1], kk[2], kk[3]);
+                        }
+                    }
+                    kmn = __reduce_min_sync(0xFFFFFFFFu, kmn);
+                    nf = __reduce_add_sync(0xFFFFFFFFu, nf);
+                    if (lane == 0) { sh.kmin[s][warp] = kmn; sh.nfin[s][warp] = nf; }
                 }
-                if (lane == 0) sh.best[s][warp] = best;
-            } else {
-                const int G = slot.cfg.G;
-                const bool tmin = slot.cfg.tile_min;
-                // warp cutoff: minimum over G groups of the group maximum.  Tile cutoff: the largest of the eight warp cutoffs
-                // (warp mode) or the smallest (tile mode: a minimum over all 8 G groups of the tile).  In tile mode a group
-                // without a finite element (masked, or past the row's end) does not take part: it would drag the cutoff
-                // to -inf and the tile would emit everything it has.
-                auto group_cutoff = [&]() -> float {
-                    switch (G) {                               // (one straight-line butterfly per group count)
-                    case 0: return -CUDART_INF_F;
-                    case 1: return warp_cutoff<32>(lm, tmin);
-                    case 2: return warp_cutoff<16>(lm, tmin);
-                    case 4: return warp_cutoff<8>(lm, tmin);
-                    case 8: return warp_cutoff<4>(lm, tmin);
-                    case 16: return warp_cutoff<2>(lm, tmin);
-                    case 32: return warp_cutoff<1>(lm, tmin);
-                    default: {                                 // 64: half-lane groups
-                        const float a0 = (tmin && h0 == -CUDART_INF_F) ? CUDART_INF_F : h0;
-                        const float a1 = (tmin && h1 == -CUDART_INF_F) ? CUDART_INF_F : h1;
-                        return warp_cutoff<1>(fminf(a0, a1), false);
-                    }
-                    }
-                };
-                // (many groups, many candidates: a cutoff per tile keeps them down)
-                float t = cut;
-                if (row != cut_row || G > 8) {
-                    const float g = group_cutoff();
-                    if (lane == 0) sh.tw[s][warp] = g;
-                    csync();
-                    static_assert(STREAM_WARPS == 8, "the eight warp cutoffs are read as two 128-bit words");
-                    const float4 ta = *reinterpret_cast<const float4 *>(&sh.tw[s][0]);
-                    const float4 tb = *reinterpret_cast<const float4 *>(&sh.tw[s][4]);
-                    if (tmin) {
-                        t = fminf(fminf(fminf(ta.x, ta.y), fminf(ta.z, ta.w)), fminf(fminf(tb.x, tb.y), fminf(tb.z, tb.w)));
-                        if (t == CUDART_INF_F) t = -CUDART_INF_F;          // no finite element in the tile: nothing to emit
-                    } else {
-                        t = fmaxf(fmaxf(fmaxf(ta.x, ta.y), fmaxf(ta.z, ta.w)), fmaxf(fmaxf(tb.x, tb.y), fmaxf(tb.z, tb.w)));
-                    }
-                    // (a tile that bounds nothing leaves the cutoff to the next one)
-                    cut = t;
-                    cut_row = (t > -CUDART_INF_F) ? row : -1;
-                } else if (__popc(__ballot_sync(0xFFFFFFFFu, lm >= t)) > 28) {
-                    // far more candidates than the cutoff was meant for (values that depend on the position): the warp takes
-                    // a cutoff of its own for this tile
-                    t = fmaxf(t, group_cutoff());
-                    if (t == CUDART_INF_F) t = cut;
-                }
-                const uint32_t wk = __reduce_max_sync(0xFFFFFFFFu, okey(lm));
-                if (lane == 0) sh.best[s][warp] = ((unsigned long long)okey(t) << 32) | wk;
-                // every finite element >= t goes to the tile's candidate slot
-                const float t2 = fmaxf(t, -CUDART_MAX_NORMAL_F);           // e >= t2  <=>  e >= t and e is not -inf
-                const unsigned int cand = __ballot_sync(0xFFFFFFFFu, lm >= t2);
-                if (cand) {
-                    unsigned long long *dst = P.cand + (size_t)row * P.cand_stride + (size_t)tile * cap_t;
-                    auto put = [&](unsigned int pos, float z, int li) {
-                        if ((int)pos < cap_t) dst[pos] = ((unsigned long long)okey(z) << 32) | (uint32_t)(~(uint32_t)(tile_base + li));
-                    };
-                    if (sparse) {
-                        if (lm >= t2) visit(t2, [&](float z, int li) { put(atomicAdd(&sh.ncand[s], 1u), z, li); });
-                    } else {
-                        // Every lane marks its candidates in a bit mask, a quarter of its elements at a time (a quarter without
-                        // one anywhere in the warp is skipped by a vote); one reservation for the warp.  The marked values are
-                        // fetched again from the tile.
-                        unsigned int cm = 0u;
+                float wm = lm;
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xFFFFFFFFu, wm, off));
+                unsigned long long key = 0ull;
+                if (wm > -CUDART_INF_F) {
+                    int best = 0x7FFFFFFF;
+                    if (sparse && lm == wm) {
+                        for (uint32_t w = word; w; w &= w - 1u) {
+                            const int b = __ffs(w) - 1;
+                            if (best == 0x7FFFFFFF && word_value(b) == wm) best = wbase + lane * 32 + b;
+                        }
+                    } else if (lm == wm) {
+                        // slots ascend: the last write is the lowest; only the first quarter that holds the maximum is searched
+                        bool found = false;
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            float qm = mv[i * NV / 4];
-                            if (NV == 8) qm = fmaxf(qm, mv[i * NV / 4 + 1]);
-                            if (__any_sync(0xFFFFFFFFu, qm >= t2)) {
+                            if (!found && qm[i] == wm) {
+                                found = true;
 #pragma unroll
-                                for (int j = i * NV / 4; j < (i + 1) * NV / 4; ++j) {
-                                    const uint32_t r[4] = {raw[j].x, raw[j].y, raw[j].z, raw[j].w};
-                                    if (DT == 1 && wide) {
-                                        const float4 a = *reinterpret_cast<const float4 *>(ptile + lane0 + j * 32 * VEC);
-                                        const float4 b = *reinterpret_cast<const float4 *>(ptile + lane0 + j * 32 * VEC + (VEC == 8 ? 4 : 0));
-                                        cm |= ((a.x >= t2 ? 1u : 0u) | (a.y >= t2 ? 2u : 0u) | (a.z >= t2 ? 4u : 0u) | (a.w >= t2 ? 8u : 0u)) << (j * VEC);
-                                        cm |= ((b.x >= t2 ? 16u : 0u) | (b.y >= t2 ? 32u : 0u) | (b.z >= t2 ? 64u : 0u) | (b.w >= t2 ? 128u : 0u)) << (j * VEC);
-                                    } else {
-#pragma unroll
-                                        for (int q = 0; q < VEC; ++q) {
-                                            const float v = DT == 0 ? __uint_as_float(r[q & 3]) : __uint_as_float((q & 1) ? (r[(q >> 1) & 3] & 0xFFFF0000u) : (r[(q >> 1) & 3] << 16));
-                                            cm |= (v >= t2) ? (1u << (j * VEC + q)) : 0u;
-                                        }
-                                    }
-                                }
+                                for (int q = (i + 1) * (EPL / 4) - 1; q >= i * (EPL / 4); --q)
+                                    if (e[q] == wm) best = slot_index<DT>(wbase, lane, q);
                             }
                         }
-                        cm &= ebits;
-                        const int cnt = __popc(cm);
-                        int incl, total;
-                        if (!__any_sync(0xFFFFFFFFu, cnt > 1)) {
-                            // the usual case, at most one candidate per lane: positions from one vote
-                            const unsigned int has = __ballot_sync(0xFFFFFFFFu, cnt > 0);
-                            incl = __popc(has & (0xFFFFFFFFu >> (31 - lane)));
-                            total = __popc(has);
-                        } else {
-                            incl = cnt;
+                    }
 #pragma unroll
-                            for (int off = 1; off < 32; off <<= 1) { const int o = __shfl_up_sync(0xFFFFFFFFu, incl, off); if (lane >= off) incl += o; }
-                            total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+                    for (int off = 16; off > 0; off >>= 1) best = min(best, __shfl_xor_sync(0xFFFFFFFFu, best, off));
+                    key = ((unsigned long long)okey(wm) << 32) | (uint32_t)(~(uint32_t)best);
+                }
+                if (lane == 0) sh.best[s][warp] = key;
+                csync();
+                if (tid == 0) {
+                    unsigned long long b = sh.best[s][0];
+#pragma unroll
+                    for (int w = 1; w < STREAM_WARPS; ++w) b = max(b, sh.best[s][w]);
+                    rec->best = b;
+                    if (c.cls == CLS_DENSE) {
+                        unsigned int kmn = sh.kmin[s][0], nf = sh.nfin[s][0];
+#pragma unroll
+                        for (int w = 1; w < STREAM_WARPS; ++w) { kmn = min(kmn, sh.kmin[s][w]); nf += sh.nfin[s][w]; }
+                        rec->minkey = kmn; rec->nfin = nf;
+                    }
+                }
+            } else {
+                // warp cutoff: minimum over G groups of the group maximum.  Tile cutoff: the largest of the eight
+                // warp cutoffs (warp mode) or the smallest (tile mode: a minimum over all 8 G groups of the tile).
+                // In tile mode a group without a finite element (masked, or past the row's end) does not take
+                // part: it would drag the cutoff to -inf and the tile would emit everything it has.
+                float g;
+                const int G = c.G;
+                const bool tmin = c.tile_min;
+                switch (G) {                                   // (one straight-line butterfly per group count)
+                case 0: g = -CUDART_INF_F; break;
+                case 1: g = warp_cutoff<32>(lm, tmin); break;
+                case 2: g = warp_cutoff<16>(lm, tmin); break;
+                case 4: g = warp_cutoff<8>(lm, tmin); break;
+                case 8: g = warp_cutoff<4>(lm, tmin); break;
+                case 16: g = warp_cutoff<2>(lm, tmin); break;
+                case 32: g = warp_cutoff<1>(lm, tmin); break;
+                default: {                                     // 64: half-lane groups
+                    const float a0 = (tmin && h0 == -CUDART_INF_F) ? CUDART_INF_F : h0;
+                    const float a1 = (tmin && h1 == -CUDART_INF_F) ? CUDART_INF_F : h1;
+                    g = warp_cutoff<1>(fminf(a0, a1), false);
+                    break;
+                }
+                }
+                if (lane == 0) sh.tw[s][warp] = g;
+                if (P.op != OP_TOPK) {
+                    // (the merge bounds rows of small k by the warp tiles' maxima)
+                    const uint32_t wk = __reduce_max_sync(0xFFFFFFFFu, okey(lm));
+                    if (lane == 0) P.wmax[((size_t)row * MAX_TILES + tile) * STREAM_WARPS + warp] = wk;
+                }
+                if (tid == 0) { sh.ncand[s] = 0; rec->cnt = 0u; }          // (the warps add to the record after the barrier)
+                csync();
+                static_assert(STREAM_WARPS == 8, "the eight warp cutoffs are read as two 128-bit words");
+                const float4 ta = *reinterpret_cast<const float4 *>(&sh.tw[s][0]);
+                const float4 tb = *reinterpret_cast<const float4 *>(&sh.tw[s][4]);
+                float t;
+                if (tmin) {
+                    t = fminf(fminf(fminf(ta.x, ta.y), fminf(ta.z, ta.w)), fminf(fminf(tb.x, tb.y), fminf(tb.z, tb.w)));
+                    if (t == CUDART_INF_F) t = -CUDART_INF_F;          // no finite element in the tile: nothing to emit
+                } else {
+                    t = fmaxf(fmaxf(fmaxf(ta.x, ta.y), fmaxf(ta.z, ta.w)), fmaxf(fmaxf(tb.x, tb.y), fmaxf(tb.z, tb.w)));
+                }
+                // every finite element >= t goes to the tile's candidate slot; a warp reserves its share of the
+                // slot with one shared-memory atomic and adds it to the tile record (no second barrier).
+                // Most warps hold no candidate at all and leave after one vote.  The others mark their
+                // candidates in a bit mask and fetch the values again from the tile in shared memory (a
+                // candidate is neither masked nor past the row's end, so the tile holds its value).
+                const float t2 = fmaxf(t, -CUDART_MAX_NORMAL_F);           // e >= t2  <=>  e >= t and e is not -inf
+                if (__any_sync(0xFFFFFFFFu, lm >= t2)) {
+                    // a quarter of the lanes' elements without a candidate anywhere in the warp is skipped by one vote
+                    unsigned int cm = 0;
+                    if (sparse) {
+                        for (uint32_t w = word; w; w &= w - 1u) { const int b = __ffs(w) - 1; cm |= (word_value(b) >= t2) ? (1u << b) : 0u; }
+                    } else
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        if (__any_sync(0xFFFFFFFFu, qm[i] >= t2)) {
+#pragma unroll
+                            for (int q = i * (EPL / 4); q < (i + 1) * (EPL / 4); ++q) cm |= (e[q] >= t2) ? (1u << q) : 0u;
                         }
-                        unsigned int base = 0u;
-                        if (lane == 0) base = atomicAdd(&sh.ncand[s], (unsigned int)total);
-                        base = __shfl_sync(0xFFFFFFFFu, base, 0) + (unsigned int)(incl - cnt);
+                    }
+                    const int cnt = __popc(cm);
+                    int incl, total;
+                    if (!__any_sync(0xFFFFFFFFu, cnt > 1)) {
+                        // the usual case, at most one candidate per lane: positions from one vote
+                        const unsigned int has = __ballot_sync(0xFFFFFFFFu, cnt > 0);
+                        incl = __popc(has & (0xFFFFFFFFu >> (31 - lane)));
+                        total = __popc(has);
+                    } else {
+                        incl = cnt;
+#pragma unroll
+                        for (int off = 1; off < 32; off <<= 1) {
+                            const int o = __shfl_up_sync(0xFFFFFFFFu, incl, off);
+                            if (lane >= off) incl += o;
+                        }
+                        total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+                    }
+                    unsigned int base = 0;
+                    if (lane == 0) {
+                        base = atomicAdd(&sh.ncand[s], (unsigned int)total);
+                        atomicAdd(&rec->cnt, (unsigned int)total);      // zero before the call; the merge kernel clears it
+                    }
+                    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+                    if ((int)base + total <= cap_t) {
+                        unsigned long long *dst = P.cand + (size_t)row * P.cand_stride + (size_t)tile * cap_t + base + (incl - cnt);
+                        const int lbase = warp * WARP_TILE + lane * VEC;
                         while (cm) {
-                            const int b = __ffs(cm) - 1, li = lane0 + (b / VEC) * (32 * VEC) + (b % VEC);
-                            cm &= cm - 1u;
-                            put(base++, value(li), li);
+                            const int q = __ffs(cm) - 1;
+                            cm &= cm - 1;
+                            const int li = sparse ? warp * WARP_TILE + lane * 32 + q : lbase + (q / VEC) * (32 * VEC) + (q % VEC);
+                            float v;
+                            if (DT == 0 || patched) v = ptile[li];
+                            else v = __uint_as_float((uint32_t)reinterpret_cast<const unsigned short *>(stage)[li] << 16);
+                            if (c.div_all) v = div_tau(v, c.tau);
+                            *dst++ = ((unsigned long long)okey(v) << 32) | (uint32_t)(~(uint32_t)(tile_base + li));
                         }
                     }
                 }
-                __syncwarp();
+                if (tid == 0) rec->tkey = okey(t);
             }
 
             // generic-proxy writes into the stage (in-place patches) precede the next bulk copy into it
-            if (DT == 0 && patch != 0) fence_async_proxy();
+            if (DT == 0 && patched) fence_async_proxy();
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&sh.empty[s]);
