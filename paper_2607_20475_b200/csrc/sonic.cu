@@ -10,6 +10,7 @@
 #include "sonic_common.cuh"
 #include "sonic_dense.cuh"
 #include "sonic_stream.cuh"
+#include "sonic_mask.cuh"
 #include "sonic_exact.cuh"
 #include "sonic_row.cuh"
 
@@ -58,6 +59,8 @@ constexpr size_t WS_CLEAR = WS_TICKETS * 4;       // the part of it that the str
 constexpr int MERGE_SMEM = MERGE_CAP * 8 + MERGE_BUCKETS * 4;
 constexpr int STREAM_SMEM_F32 = VecTraits<0>::NSTAGE * CTA_TILE * 4 + (int)sizeof(StreamShared<0>);
 constexpr int STREAM_SMEM_BF16 = VecTraits<1>::NSTAGE * CTA_TILE * 2 + CTA_TILE * 4 + (int)sizeof(StreamShared<1>);
+constexpr int MASK_SMEM_F32 = VecTraits<0>::NSTAGE * CTA_TILE * 4 + (int)sizeof(masked_stream::StreamShared<0>);
+constexpr int MASK_SMEM_BF16 = VecTraits<1>::NSTAGE * CTA_TILE * 2 + CTA_TILE * 4 + (int)sizeof(masked_stream::StreamShared<1>);
 constexpr int EXACT_CLUSTERS = 4;             // clusters of the cluster kernel (its rows are rare)
 constexpr int EXACT_SMEM = SLICE_MAX * 4 + HBINS * 16 + 8192 + MAX_TOPK * 8 + 8192;
 static_assert(MERGE_SMEM >= DENSE_DYN_SMEM, "stage 2 of the histogram path runs in the merge kernel's shared memory");
@@ -78,7 +81,7 @@ static int fail_cuda(cudaError_t e, const char *what) {
 // them; everything behind it is laid out for the shape of the call at hand (rows, V, whether the histogram path
 // can be taken) and initialised by the call's own kernels, so one workspace serves calls of any shape that fits.
 struct Layout {
-    size_t rs, pr, tiles, wmax, cand, drow, dtile, dlist, rlist, hist, members, ykeys, total;
+    size_t rs, pr, tiles, cand, drow, dtile, dlist, rlist, hist, members, ykeys, total;
     unsigned int cand_stride;
     int ytiles;
 };
@@ -97,7 +100,6 @@ static Layout layout_for(long long rows, int V, bool dense, size_t cap = CAND_CA
     L.rs = off;    off = align256(off + (size_t)rows * sizeof(RowState));
     L.pr = off;    off = align256(off + (size_t)rows * sizeof(PosResult));
     L.tiles = off; off = align256(off + (size_t)rows * sizeof(TileRec) * MAX_TILES);
-    L.wmax = off;  off = align256(off + (size_t)rows * MAX_TILES * STREAM_WARPS * 4);
     L.cand = off;  off = align256(off + (size_t)rows * slots * 8);
     if (dense) {
         L.drow = off;    off = align256(off + (size_t)rows * sizeof(DenseRow));
@@ -169,6 +171,8 @@ static int configure_once(int *sm_count, int *device) {
         set((const void *)sonic_dense_finish_kernel, DENSE_DYN_SMEM);
         set((const void *)sonic_stream_kernel<0>, STREAM_SMEM_F32);
         set((const void *)sonic_stream_kernel<1>, STREAM_SMEM_BF16);
+        set((const void *)sonic_mask_kernel<0>, MASK_SMEM_F32);
+        set((const void *)sonic_mask_kernel<1>, MASK_SMEM_BF16);
         if (r == cudaSuccess) r = cudaDeviceGetAttribute(&g_sm_count[dev], cudaDevAttrMultiProcessorCount, dev);
         set((const void *)sonic_row_kernel<0>, ROW_DYN_SMEM);
         set((const void *)sonic_row_kernel<1>, ROW_DYN_SMEM);
@@ -302,7 +306,6 @@ static int launch_all(KParams &P, void *ws, size_t ws_bytes, cudaStream_t st, in
     P.rs = reinterpret_cast<RowState *>(base + L.rs);
     P.pr = reinterpret_cast<PosResult *>(base + L.pr);
     P.tiles = reinterpret_cast<TileRec *>(base + L.tiles);
-    P.wmax = reinterpret_cast<unsigned int *>(base + L.wmax);
     P.cand = reinterpret_cast<unsigned long long *>(base + L.cand);
     P.cand_stride = L.cand_stride;
     P.ytiles = L.ytiles;
@@ -340,8 +343,14 @@ static int launch_all(KParams &P, void *ws, size_t ws_bytes, cudaStream_t st, in
     int chunk = (int)((7ll * nitems) / (8ll * grid1));
     chunk = chunk < 1 ? 1 : chunk;
     const int cap_t = (int)(L.cand_stride / (unsigned)tiles);
-    if (P.dtype == SONIC_DTYPE_F32) sonic_stream_kernel<0><<<grid1, STREAM_CTA_THREADS, STREAM_SMEM_F32, st>>>(P, tiles, nitems, chunk, cap_t);
-    else sonic_stream_kernel<1><<<grid1, STREAM_CTA_THREADS, STREAM_SMEM_BF16, st>>>(P, tiles, nitems, chunk, cap_t);
+    const bool f32 = P.dtype == SONIC_DTYPE_F32;
+    if (P.bitmask) {
+        if (f32) sonic_mask_kernel<0><<<grid1, STREAM_CTA_THREADS, MASK_SMEM_F32, st>>>(P, tiles, nitems, chunk, cap_t);
+        else sonic_mask_kernel<1><<<grid1, STREAM_CTA_THREADS, MASK_SMEM_BF16, st>>>(P, tiles, nitems, chunk, cap_t);
+    } else {
+        if (f32) sonic_stream_kernel<0><<<grid1, STREAM_CTA_THREADS, STREAM_SMEM_F32, st>>>(P, tiles, nitems, chunk, cap_t);
+        else sonic_stream_kernel<1><<<grid1, STREAM_CTA_THREADS, STREAM_SMEM_BF16, st>>>(P, tiles, nitems, chunk, cap_t);
+    }
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail_cuda(e, "stream kernel launch");
 
@@ -547,8 +556,8 @@ int sonic_topk(const void *logits, int dtype, int B, int V, int64_t row_stride, 
 // Scratch of sonic_topk_static: a workspace for SONIC_STATIC_MAX_ROWS rows of the largest vocabulary that lives in
 // the library image.  In host code this name is only a stand-in for the symbol; the device
 // address the kernels need comes from cudaGetSymbolAddress (below), never from `&`.
-constexpr size_t STATIC_WS_BYTES = WS_HEADER + 256 * 5 +
-    (size_t)SONIC_STATIC_MAX_ROWS * (sizeof(RowState) + sizeof(PosResult) + (sizeof(TileRec) + STREAM_WARPS * 4) * MAX_TILES + 2 * (size_t)CAND_CAP * 8);
+constexpr size_t STATIC_WS_BYTES = WS_HEADER + 256 * 4 +
+    (size_t)SONIC_STATIC_MAX_ROWS * (sizeof(RowState) + sizeof(PosResult) + sizeof(TileRec) * MAX_TILES + 2 * (size_t)CAND_CAP * 8);
 static __device__ __align__(256) unsigned char g_static_workspace[STATIC_WS_BYTES];
 
 static int static_workspace_address(void **out) {

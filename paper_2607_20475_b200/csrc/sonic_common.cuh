@@ -179,7 +179,6 @@ struct KParams {
     unsigned int *error;                      // workspace header (WS_* words); word 0: ERR_* (sticky)
     RowState *rs;
     TileRec *tiles;
-    unsigned int *wmax;                       // [rows][MAX_TILES][STREAM_WARPS] top-k rows: key of the largest element of every warp tile
     PosResult *pr;
     unsigned long long *cand;                 // [rows][cand_stride] candidate slots, split evenly among a row's tiles
     unsigned int cand_stride;

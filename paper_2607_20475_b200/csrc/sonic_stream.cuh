@@ -11,7 +11,7 @@
 // Kernel" and "Stage 2: Cross-Tile Merge and Selection Kernel"; the selection
 // itself is ours.
 //
-// Structure of the streaming kernel: persistent CTAs (three per SM), each a
+// (Calls with a grammar bitmask: sonic_mask.cuh.)  Structure of the streaming kernel: persistent CTAs (three per SM), each a
 // producer warp plus eight consumer warps.  The producer takes tiles from a work
 // queue, resolves each tile's row configuration and issues one bulk-TMA copy
 // (cp.async.bulk, completion on an mbarrier) of the tile's logits into a ring of
@@ -512,23 +512,9 @@ __device__ bool merge_topk_row(const KParams &P, const RowCfg &c, int row, int t
         sh.tcnt[tid + 1] = incl;                                   // lanes past the last tile repeat the total
         if (tid == 0) { sh.tcnt[0] = 0; sh.count = 0; sh.tkey = tk; sh.found = over ? 1 : 0; }
     }
-    // Small k: the k-th largest of the maxima of the row's warp tiles is a value that k elements reach and few more do (75
-    // of 2^18 for k = 64), all of them candidates, so that the short finish takes them.  (sonic_topk only ranks: there the
-    // bound costs more than it saves, 15.0 against 13.0 us for k = 64.)  bins: the maxima.
-    const int groups = tiles * STREAM_WARPS;
-    const bool tight = P.op != OP_TOPK && 2 * c.k <= groups && c.k <= 100;
-    static_assert(MAX_TILES * STREAM_WARPS * 2 == THREADS, "two threads per maximum at most");
-    if (tight && tid < MAX_TILES * STREAM_WARPS) bins[tid] = (tid < groups) ? __ldcg(&P.wmax[(size_t)row * MAX_TILES * STREAM_WARPS + tid]) : 0u;
     csync();
     if (sh.found) return false;
-    unsigned int tkey = sh.tkey;
-    if (tight && tkey != KEY_NEG_INF) {
-        const uint32_t kth = kth_max<THREADS>(bins, reinterpret_cast<unsigned int *>(sh.wsum), groups, c.k, tid);
-        // (with a temperature a hair less: a value just below the bound may become equal to it when divided)
-        float t = unkey(kth);
-        if (c.temp) t -= fmaxf(fabsf(t) * 4.76837158203125e-07f, 1e-37f);
-        if (kth > KEY_NEG_INF) tkey = max(tkey, okey(t));
-    }
+    const unsigned int tkey = sh.tkey;
     const bool complete = (tkey == KEY_NEG_INF);
     const bool strict = c.temp && !complete;            // keys are compared after the temperature division
     const uint32_t tykey = c.temp ? okey(div_tau(unkey(tkey), c.tau)) : tkey;
@@ -798,17 +784,6 @@ __device__ bool merge_topk_row(const KParams &P, const RowCfg &c, int row, int t
     if (Pn >= c.k) n = c.k;
     else if (complete && P.op != OP_TOPK) n = Pn;
     else return false;
-    if (Pn <= SMALL_MAX && n > 0) {
-        int draft = -1;
-        float q_draft = 0.0f;
-        if (P.op == OP_VERIFY && c.l < P.K) {
-            draft = __ldg(P.draft_tokens + (size_t)c.b * P.K + c.l);
-            if (draft < 0 || draft >= P.V) draft = -1;
-            if (draft >= 0) q_draft = __ldg(P.draft_probs + ((size_t)c.b * P.K + c.l) * (size_t)P.V + draft);
-        }
-        finish_small(P, c, row, buf, false, Pn, reinterpret_cast<unsigned long long *>(bins), tid, cells, draft, q_draft);
-        return true;
-    }
     merge_finish<THREADS, Sync>(P, c, row, buf, bins, Pn, n, sh, tid, cells);
     return true;
 }
@@ -1245,7 +1220,6 @@ struct StageMeta {
     int hb;                                    // which hit buffer holds them
     int stop;                                  // no more tiles for this CTA (nothing else in the entry is valid)
     int bad;                                   // the producer met a list id outside [0, V)
-    int next_row, next_tile;                   // the tile that follows (-1: none, or not known yet)
 };
 struct Hit { int li; int payload; };           // element within the tile; history count, or the bias as float bits
 
@@ -1465,8 +1439,6 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 m.patch = pr.patch; m.npen = pr.npen; m.nbias = pr.nbias; m.hb = n % (NSTAGE + 1);
                 m.stop = 0;
                 m.bad = bad_now;
-                m.next_row = (nxt >= 0) ? nxt / tiles : -1;
-                m.next_tile = (nxt >= 0) ? nxt % tiles : -1;
                 if (n == 0 || c.cls == CLS_EXACT) mbar_arrive(&sh.full[s]);     // (the first tile's copy is under way; nothing is copied for rows of the cluster kernel's class)
                 else issue_copy(row, tile, s, true);
             }
@@ -1479,14 +1451,6 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
     }
 
     // ---------------------------------------------------------------- consumer warps
-    // The grammar words of a warp tile (32 words, one coalesced load, handed to the lanes that need them by
-    // shuffles later) are requested one tile ahead: each stage names the tile that follows it.
-    uint32_t mword_pre = 0u;
-    int pre_row = -1, pre_tile = -1;
-    auto load_mask_words = [&](int row, int tile) -> uint32_t {
-        const int w = ((tile * CTA_TILE + warp * WARP_TILE) >> 5) + lane;
-        return (w < ((P.V + 31) >> 5)) ? __ldg(P.bitmask + (size_t)row * P.bitmask_stride + w) : 0u;
-    };
     for (int n = 0;; ++n) {
         const int s = n % NSTAGE;
         if (!mbar_wait(&sh.full[s], (n / NSTAGE) & 1)) {
@@ -1497,12 +1461,6 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         const int row = sh.meta[s].row, tile = sh.meta[s].tile;
         const int tile_base = tile * CTA_TILE;
         const int wbase = tile_base + warp * WARP_TILE;
-        uint32_t mword = 0xFFFFFFFFu;
-        if (P.bitmask) {
-            mword = (row == pre_row && tile == pre_tile) ? mword_pre : load_mask_words(row, tile);
-            pre_row = sh.meta[s].next_row; pre_tile = sh.meta[s].next_tile;
-            if (pre_row >= 0) mword_pre = load_mask_words(pre_row, pre_tile);
-        }
         const StageMeta &meta = sh.meta[s];
         if (meta.skip) {
             // a row of the cluster kernel: counted, its status word initialised
@@ -1529,29 +1487,8 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 }
             }
             unsigned char *stage = stages + (size_t)s * STAGE_BYTES;
-            const bool masked = (c.z & M_GRAMMAR) != 0;
             const bool tail = tile_base + CTA_TILE > P.V;
-            int patch = meta.patch;
-            // word: which of the warp tile's 32 consecutive elements from lane * 32 count.  Under a sparse mask (a grammar allows
-            // a few per cent of the ids) a lane walks its word's few set bits instead of 32 elements, and list entries that
-            // the mask forbids are not patched (they stay -inf).  2 % of 2^18 fp32 entries, 128 rows with 512 entries of
-            // history: the kernel's warp instructions from 19.6 to 14 million.
-            uint32_t word = mword;
-            if (masked && tail) { const int left = P.V - wbase - lane * 32; if (left < 32) word &= left > 0 ? (1u << left) - 1u : 0u; }
-            const bool sparse = masked && c.cls != CLS_DENSE && __all_sync(0xFFFFFFFFu, __popc(word) <= 8);
-            if (sparse && patch == 1) {
-                bool any = false;
-                auto look = [&](const Hit *hits, int count) {
-                    for (int h0 = 0; h0 < count; h0 += 32) {
-                        const int li = (h0 + lane < count) ? hits[h0 + lane].li : -1;
-                        const uint32_t w = __shfl_sync(0xFFFFFFFFu, word, (li >> 5) & 31);
-                        any = any || (li >= 0 && li / WARP_TILE == warp && ((w >> (li & 31)) & 1u));
-                    }
-                };
-                look(sh.pen[meta.hb], meta.npen);
-                look(sh.bias[meta.hb], meta.nbias);
-                if (!__any_sync(0xFFFFFFFFu, any)) patch = 0;
-            }
+            const int patch = meta.patch;
             const bool patched = patch != 0;
             float *ptile = (DT == 0) ? reinterpret_cast<float *>(stage) : conv;    // fp32 view the sparse lists patch
 
@@ -1589,8 +1526,6 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                         *reinterpret_cast<float4 *>(p + q) = make_float4(e[j * VEC + q], e[j * VEC + q + 1], e[j * VEC + q + 2], e[j * VEC + q + 3]);
                 }
             };
-            // penalties and biases commute with the mask (a masked logit stays -inf), so they are applied to
-            // the unmasked tile and the mask is applied when the lanes read their elements
             if (patch == 1) {
                 // the producer listed this tile's entries: every warp patches its own part, no block-wide barrier
                 if (DT == 1) { read_raw(); widen(); }
@@ -1605,7 +1540,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                     if (x.li / WARP_TILE == warp) ptile[x.li] = __fadd_rn(ptile[x.li], __int_as_float(x.payload));
                 }
                 __syncwarp();
-                if (!sparse) read_f32(ptile);
+                read_f32(ptile);
             } else if (patch == 2) {
                 // long or crowded lists: all consumer threads scan them together
                 if (DT == 1) { read_raw(); widen(); csync(); }
@@ -1628,55 +1563,24 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 }
                 if (bad) atomicOr(&rec->flags, TILE_BADID);          // (ordered after the first thread's store by the barriers above)
                 csync();
-                if (!sparse) read_f32(ptile);
-            } else if (!sparse) {
+                read_f32(ptile);
+            } else {
                 read_raw();
             }
-            if (sparse) {
-            } else if (masked && !tail) {
-                // the common masked case: one select per element, no bounds test
-#pragma unroll
-                for (int j = 0; j < NV; ++j) {
-                    const uint32_t bits = __shfl_sync(0xFFFFFFFFu, mword, (j * 32 * VEC + lane * VEC) >> 5) >> ((lane * VEC) & 31);
-#pragma unroll
-                    for (int q = 0; q < VEC; ++q) e[j * VEC + q] = (bits & (1u << q)) ? e[j * VEC + q] : -CUDART_INF_F;
-                }
-            } else if (tail) {
+            if (tail) {
 #pragma unroll
                 for (int j = 0; j < NV; ++j) {
                     const int first = wbase + j * 32 * VEC + lane * VEC;
-                    const uint32_t bits = __shfl_sync(0xFFFFFFFFu, mword, (j * 32 * VEC + lane * VEC) >> 5) >> (first & 31);
 #pragma unroll
-                    for (int q = 0; q < VEC; ++q) {
-                        const bool dead = (first + q >= P.V) || (masked && !((bits >> q) & 1u));
-                        if (dead) e[j * VEC + q] = -CUDART_INF_F;
-                    }
+                    for (int q = 0; q < VEC; ++q) if (first + q >= P.V) e[j * VEC + q] = -CUDART_INF_F;
                 }
             }
-            if (c.div_all && !sparse) {
+            if (c.div_all) {
 #pragma unroll
                 for (int q = 0; q < EPL; ++q) e[q] = div_tau(e[q], c.tau);
             }
 
-            // one element of the tile, by its place in the lane's mask word
-            auto word_value = [&](int b) -> float {
-                const int li = warp * WARP_TILE + lane * 32 + b;
-                float v;
-                if (DT == 0 || patched) v = ptile[li];
-                else v = __uint_as_float((uint32_t)reinterpret_cast<const unsigned short *>(stage)[li] << 16);
-                return c.div_all ? div_tau(v, c.tau) : v;
-            };
             // per-vector maxima, half maxima, lane maximum
-            float qm[4];                               // maxima of the lane's four quarters (8 elements each)
-            if (sparse) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) qm[i] = -CUDART_INF_F;
-                for (uint32_t w = word; w; w &= w - 1u) {
-                    const int b = __ffs(w) - 1;
-                    const float v = word_value(b);
-                    if (b < 16) qm[0] = fmaxf(qm[0], v); else qm[2] = fmaxf(qm[2], v);
-                }
-            } else {
             float mv[NV];
 #pragma unroll
             for (int j = 0; j < NV; ++j) {
@@ -1685,12 +1589,12 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 for (int q = 1; q < VEC; ++q) m = fmaxf(m, e[j * VEC + q]);
                 mv[j] = m;
             }
+            float qm[4];                               // maxima of the lane's four quarters (8 elements each)
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 qm[i] = mv[i * (NV / 4)];
 #pragma unroll
                 for (int j = 1; j < NV / 4; ++j) qm[i] = fmaxf(qm[i], mv[i * (NV / 4) + j]);
-            }
             }
             const float h0 = fmaxf(qm[0], qm[1]), h1 = fmaxf(qm[2], qm[3]);
             const float lm = fmaxf(h0, h1);
@@ -1727,12 +1631,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 unsigned long long key = 0ull;
                 if (wm > -CUDART_INF_F) {
                     int best = 0x7FFFFFFF;
-                    if (sparse && lm == wm) {
-                        for (uint32_t w = word; w; w &= w - 1u) {
-                            const int b = __ffs(w) - 1;
-                            if (best == 0x7FFFFFFF && word_value(b) == wm) best = wbase + lane * 32 + b;
-                        }
-                    } else if (lm == wm) {
+                    if (lm == wm) {
                         // slots ascend: the last write is the lowest; only the first quarter that holds the maximum is searched
                         bool found = false;
 #pragma unroll
@@ -1787,11 +1686,6 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 }
                 }
                 if (lane == 0) sh.tw[s][warp] = g;
-                if (P.op != OP_TOPK) {
-                    // (the merge bounds rows of small k by the warp tiles' maxima)
-                    const uint32_t wk = __reduce_max_sync(0xFFFFFFFFu, okey(lm));
-                    if (lane == 0) P.wmax[((size_t)row * MAX_TILES + tile) * STREAM_WARPS + warp] = wk;
-                }
                 if (tid == 0) { sh.ncand[s] = 0; rec->cnt = 0u; }          // (the warps add to the record after the barrier)
                 csync();
                 static_assert(STREAM_WARPS == 8, "the eight warp cutoffs are read as two 128-bit words");
@@ -1813,9 +1707,6 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 if (__any_sync(0xFFFFFFFFu, lm >= t2)) {
                     // a quarter of the lanes' elements without a candidate anywhere in the warp is skipped by one vote
                     unsigned int cm = 0;
-                    if (sparse) {
-                        for (uint32_t w = word; w; w &= w - 1u) { const int b = __ffs(w) - 1; cm |= (word_value(b) >= t2) ? (1u << b) : 0u; }
-                    } else
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         if (__any_sync(0xFFFFFFFFu, qm[i] >= t2)) {
@@ -1851,7 +1742,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                         while (cm) {
                             const int q = __ffs(cm) - 1;
                             cm &= cm - 1;
-                            const int li = sparse ? warp * WARP_TILE + lane * 32 + q : lbase + (q / VEC) * (32 * VEC) + (q % VEC);
+                            const int li = lbase + (q / VEC) * (32 * VEC) + (q % VEC);
                             float v;
                             if (DT == 0 || patched) v = ptile[li];
                             else v = __uint_as_float((uint32_t)reinterpret_cast<const unsigned short *>(stage)[li] << 16);
