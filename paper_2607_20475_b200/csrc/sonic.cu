@@ -171,8 +171,8 @@ static int configure_once(int *sm_count, int *device) {
         set((const void *)sonic_dense_finish_kernel, DENSE_DYN_SMEM);
         set((const void *)sonic_stream_kernel<0>, STREAM_SMEM_F32);
         set((const void *)sonic_stream_kernel<1>, STREAM_SMEM_BF16);
-        set((const void *)sonic_mask_kernel<0>, MASK_SMEM_F32);
-        set((const void *)sonic_mask_kernel<1>, MASK_SMEM_BF16);
+        set((const void *)masked_stream::sonic_stream_kernel<0>, MASK_SMEM_F32);
+        set((const void *)masked_stream::sonic_stream_kernel<1>, MASK_SMEM_BF16);
         if (r == cudaSuccess) r = cudaDeviceGetAttribute(&g_sm_count[dev], cudaDevAttrMultiProcessorCount, dev);
         set((const void *)sonic_row_kernel<0>, ROW_DYN_SMEM);
         set((const void *)sonic_row_kernel<1>, ROW_DYN_SMEM);
@@ -345,8 +345,8 @@ static int launch_all(KParams &P, void *ws, size_t ws_bytes, cudaStream_t st, in
     const int cap_t = (int)(L.cand_stride / (unsigned)tiles);
     const bool f32 = P.dtype == SONIC_DTYPE_F32;
     if (P.bitmask) {
-        if (f32) sonic_mask_kernel<0><<<grid1, STREAM_CTA_THREADS, MASK_SMEM_F32, st>>>(P, tiles, nitems, chunk, cap_t);
-        else sonic_mask_kernel<1><<<grid1, STREAM_CTA_THREADS, MASK_SMEM_BF16, st>>>(P, tiles, nitems, chunk, cap_t);
+        if (f32) masked_stream::sonic_stream_kernel<0><<<grid1, STREAM_CTA_THREADS, MASK_SMEM_F32, st>>>(P, tiles, nitems, chunk, cap_t);
+        else masked_stream::sonic_stream_kernel<1><<<grid1, STREAM_CTA_THREADS, MASK_SMEM_BF16, st>>>(P, tiles, nitems, chunk, cap_t);
     } else {
         if (f32) sonic_stream_kernel<0><<<grid1, STREAM_CTA_THREADS, STREAM_SMEM_F32, st>>>(P, tiles, nitems, chunk, cap_t);
         else sonic_stream_kernel<1><<<grid1, STREAM_CTA_THREADS, STREAM_SMEM_BF16, st>>>(P, tiles, nitems, chunk, cap_t);

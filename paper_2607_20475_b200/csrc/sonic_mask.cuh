@@ -1,6 +1,6 @@
 // Streaming kernel of calls that carry a grammar bitmask (rows without the mode bit among them).
 //
-// The same work as sonic_stream_kernel (tiles through a bulk-copy ring, one record per tile), built the other way round:
+// The same work as the kernel of that name in sonic_stream.cuh (tiles through a bulk-copy ring, one record per tile), built the other way round:
 // nothing of a tile stays in registers.  Under a sparse mask (a grammar allows a few per cent of the ids) a lane walks its
 // mask word's few set bits instead of its 32 elements, and list entries that the mask forbids are not patched.  The CTA
 // takes a top-k row's cutoff from its first tile of the row and keeps it, so that a tile needs no block barrier; the
@@ -47,7 +47,7 @@ struct StreamShared {
 
 template <int DT>
 __global__ void __launch_bounds__(STREAM_CTA_THREADS, 3)
-sonic_mask_kernel(const KParams P, const int tiles, const int nitems, const int chunk, const int cap_t) {     // cap_t: candidate slots per tile, CAND_CAP / tiles
+sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const int chunk, const int cap_t) {     // cap_t: candidate slots per tile, CAND_CAP / tiles
     constexpr int VEC = VecTraits<DT>::VEC, NV = VecTraits<DT>::NV, NSTAGE = VecTraits<DT>::NSTAGE;
     constexpr int ELT = VecTraits<DT>::ELT;
     constexpr int STAGE_BYTES = CTA_TILE * ELT;
@@ -672,5 +672,4 @@ sonic_mask_kernel(const KParams P, const int tiles, const int nitems, const int 
 }
 
 }  // namespace masked_stream
-using masked_stream::sonic_mask_kernel;
 }  // namespace sonic
