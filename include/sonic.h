@@ -50,7 +50,7 @@ extern "C" {
 #define SONIC_FLAG_FALLBACK  0x4u   /* diagnostic: the row was finished by the cluster kernel (top-k beyond the streaming
                                        path, or a row no other path could finish) */
 #define SONIC_FLAG_DENSE     0x8u   /* diagnostic: top-k off, the row was finished by the full-vocabulary histogram passes */
-#define SONIC_FLAG_TIMEOUT   0x10u  /* a bounded wait inside the streaming kernel expired: token is -1 (see sonic_workspace_init) */
+#define SONIC_FLAG_TIMEOUT   0x10u  /* a bounded wait for a copy expired: token is -1 (see sonic_workspace_init) */
 
 /* Bytes of workspace that serve every call over at most max_rows logit rows (B for sonic_sample / sonic_topk,
  * B*(K+1) for sonic_verify) of at most max_vocab entries each, and every sonic_topk call with k <= max_topk.  Pure
@@ -67,7 +67,8 @@ size_t sonic_workspace_bytes(int max_rows, int max_vocab, int max_topk);
  *
  * Error word: 32-bit word 0 of the workspace is sticky; bit 0 is set when a bounded wait of the streaming kernel
  * (a tile copy that never completed) ran out.  Every row of such a call, and of later calls on that workspace,
- * reports SONIC_FLAG_TIMEOUT with token -1 until the workspace is initialised again with this function.
+ * reports SONIC_FLAG_TIMEOUT with token -1 until the workspace is initialised again with this function.  (A call of
+ * few rows runs each row on its own: there the rows whose copy failed report it, and all rows of later calls.)
  *
  * Streams: a call's kernels are ordered on the caller's `stream` (everything enqueued before the call precedes
  * them, everything after follows them).  A call of few rows is one kernel on that stream; the rest of this paragraph is

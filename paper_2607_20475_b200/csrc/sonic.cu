@@ -244,10 +244,11 @@ static SideStream *side_stream_for(int dev, cudaStream_t st) {
 }
 
 // Whether a call goes to the row kernel as a whole: when all of its rows' clusters are resident at once (two CTAs per SM).
-// Measured (us per call, streaming chain against row kernel): one bf16 row of 131072 with top-k 25.7 -> 13.6; 3 x 3
-// verification rows of 32003 47 -> 27; 37 fp32 rows of 50021 of every kind 48.8 -> 40.7; 32 bf16 rows of 100003 without
-// top-k 73.8 -> 63.7.  With 64 rows of 131072 (1.7 times what is resident) the chain is ahead again, 58 against 64.5: its
-// persistent CTAs keep loading while the rows' selections wait for one another.  sonic_topk beyond ROW_KMAX: the chain.
+// Measured (us per call, streaming chain against row kernel): one bf16 row of 131072 with top-k 25.5 -> 13.6; 4 fp32 rows
+// of 32768, one of each kind, 29.9 -> 23.2; 3 x 3 verification rows of 32003 50.4 -> 25.7; 37 fp32 rows of 50021 of every
+// kind 64.3 -> 36.4; 32 bf16 rows of 100003 without top-k 73.9 -> 49.3; 8 bf16 rows of 65536 with k = 50 22.7 -> 14.4.
+// With 64 rows of 131072 (1.7 times what is resident) the chain is ahead, 58 against 64: its persistent CTAs keep loading
+// while the rows' selections wait for one another.  sonic_topk beyond ROW_KMAX: the chain.
 static bool row_route(const KParams &P, int sm_count) {
 #if defined(SONIC_TRACE) || defined(SONIC_TEST_WITHHOLD)
     return false;                                 // (these variants exist to look into the streaming chain)
