@@ -57,8 +57,8 @@ __global__ void sonic_verify_combine_kernel(const KParams P, int B) {
 constexpr size_t WS_HEADER = WS_HEADER_WORDS * 4;
 constexpr size_t WS_CLEAR = WS_TICKETS * 4;       // the part of it that the streaming chain uses
 constexpr int MERGE_SMEM = MERGE_CAP * 8 + MERGE_BUCKETS * 4;
-constexpr int STREAM_SMEM_F32 = VecTraits<0>::NSTAGE * CTA_TILE * 4 + (int)sizeof(StreamShared<0>);
-constexpr int STREAM_SMEM_BF16 = VecTraits<1>::NSTAGE * CTA_TILE * 2 + CTA_TILE * 4 + (int)sizeof(StreamShared<1>);
+template <int DT, bool LISTS>
+constexpr int STREAM_SMEM = STREAM_STAGES<DT, LISTS> * CTA_TILE * VecTraits<DT>::ELT + (DT == 1 && LISTS ? CTA_TILE * 4 : 0) + (int)sizeof(StreamShared<DT, LISTS>);
 constexpr int MASK_SMEM_F32 = VecTraits<0>::NSTAGE * CTA_TILE * 4 + (int)sizeof(masked_stream::StreamShared<0>);
 constexpr int MASK_SMEM_BF16 = VecTraits<1>::NSTAGE * CTA_TILE * 2 + CTA_TILE * 4 + (int)sizeof(masked_stream::StreamShared<1>);
 constexpr int EXACT_CLUSTERS = 4;             // clusters of the cluster kernel (its rows are rare)
@@ -169,8 +169,10 @@ static int configure_once(int *sm_count, int *device) {
         set((const void *)sonic_dense_collect_kernel, DENSE_DYN_SMEM);
         set((const void *)sonic_dense_stage2_kernel, DENSE_DYN_SMEM);
         set((const void *)sonic_dense_finish_kernel, DENSE_DYN_SMEM);
-        set((const void *)sonic_stream_kernel<0>, STREAM_SMEM_F32);
-        set((const void *)sonic_stream_kernel<1>, STREAM_SMEM_BF16);
+        set((const void *)sonic_stream_kernel<0, false>, STREAM_SMEM<0, false>);
+        set((const void *)sonic_stream_kernel<0, true>, STREAM_SMEM<0, true>);
+        set((const void *)sonic_stream_kernel<1, false>, STREAM_SMEM<1, false>);
+        set((const void *)sonic_stream_kernel<1, true>, STREAM_SMEM<1, true>);
         set((const void *)masked_stream::sonic_stream_kernel<0>, MASK_SMEM_F32);
         set((const void *)masked_stream::sonic_stream_kernel<1>, MASK_SMEM_BF16);
         if (r == cudaSuccess) r = cudaDeviceGetAttribute(&g_sm_count[dev], cudaDevAttrMultiProcessorCount, dev);
@@ -349,8 +351,12 @@ static int launch_all(KParams &P, void *ws, size_t ws_bytes, cudaStream_t st, in
         if (f32) masked_stream::sonic_stream_kernel<0><<<grid1, STREAM_CTA_THREADS, MASK_SMEM_F32, st>>>(P, tiles, nitems, chunk, cap_t);
         else masked_stream::sonic_stream_kernel<1><<<grid1, STREAM_CTA_THREADS, MASK_SMEM_BF16, st>>>(P, tiles, nitems, chunk, cap_t);
     } else {
-        if (f32) sonic_stream_kernel<0><<<grid1, STREAM_CTA_THREADS, STREAM_SMEM_F32, st>>>(P, tiles, nitems, chunk, cap_t);
-        else sonic_stream_kernel<1><<<grid1, STREAM_CTA_THREADS, STREAM_SMEM_BF16, st>>>(P, tiles, nitems, chunk, cap_t);
+        // (a row has entries only where all arrays of a kind are given: anything less makes the row a bad one)
+        const bool lists = (P.hist_ids && P.hist_counts && P.hist_len && P.hist_stride > 0) || (P.bias_ids && P.bias_vals && P.bias_len && P.bias_stride > 0);
+        if (f32 && lists) sonic_stream_kernel<0, true><<<grid1, STREAM_CTA_THREADS, STREAM_SMEM<0, true>, st>>>(P, tiles, nitems, chunk, cap_t);
+        else if (f32) sonic_stream_kernel<0, false><<<grid1, STREAM_CTA_THREADS, STREAM_SMEM<0, false>, st>>>(P, tiles, nitems, chunk, cap_t);
+        else if (lists) sonic_stream_kernel<1, true><<<grid1, STREAM_CTA_THREADS, STREAM_SMEM<1, true>, st>>>(P, tiles, nitems, chunk, cap_t);
+        else sonic_stream_kernel<1, false><<<grid1, STREAM_CTA_THREADS, STREAM_SMEM<1, false>, st>>>(P, tiles, nitems, chunk, cap_t);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail_cuda(e, "stream kernel launch");

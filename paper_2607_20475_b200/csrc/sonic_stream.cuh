@@ -1223,9 +1223,12 @@ struct StageMeta {
 };
 struct Hit { int li; int payload; };           // element within the tile; history count, or the bias as float bits
 
-template <int DT>
+// Stages of the ring: two tiles of fp32 take 64 KB, and so do four of bf16, or two and the fp32 tile that sparse lists patch.
+template <int DT, bool LISTS> constexpr int STREAM_STAGES = (DT == 1 && !LISTS) ? 4 : 2;
+
+template <int DT, bool LISTS>
 struct StreamShared {
-    static constexpr int NSTAGE = VecTraits<DT>::NSTAGE;
+    static constexpr int NSTAGE = STREAM_STAGES<DT, LISTS>;
     unsigned long long full[NSTAGE];           // producer -> consumers: stage described and copy issued (one arrival + the copy's bytes)
     unsigned long long empty[NSTAGE];          // consumers -> producer: stage free (one arrival per consumer warp)
     StageMeta meta[NSTAGE];
@@ -1235,21 +1238,21 @@ struct StreamShared {
     unsigned long long best[NSTAGE][STREAM_WARPS];
     unsigned int kmin[NSTAGE][STREAM_WARPS], nfin[NSTAGE][STREAM_WARPS];     // dense rows
     // hit lists: one buffer more than stages, so that the producer fills the next tile's while both stages are busy
-    Hit pen[NSTAGE + 1][HIT_PEN_CAP];
-    Hit bias[NSTAGE + 1][HIT_BIAS_CAP];
+    Hit pen[LISTS ? NSTAGE + 1 : 1][LISTS ? HIT_PEN_CAP : 1];
+    Hit bias[LISTS ? NSTAGE + 1 : 1][LISTS ? HIT_BIAS_CAP : 1];
 };
 
-template <int DT>
+template <int DT, bool LISTS>
 __global__ void __launch_bounds__(STREAM_CTA_THREADS, 3)
 sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const int chunk, const int cap_t) {     // cap_t: candidate slots per tile, CAND_CAP / tiles
-    constexpr int VEC = VecTraits<DT>::VEC, NV = VecTraits<DT>::NV, NSTAGE = VecTraits<DT>::NSTAGE;
+    constexpr int VEC = VecTraits<DT>::VEC, NV = VecTraits<DT>::NV, NSTAGE = STREAM_STAGES<DT, LISTS>;
     constexpr int ELT = VecTraits<DT>::ELT;
     constexpr int STAGE_BYTES = CTA_TILE * ELT;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    // layout: NSTAGE raw stages | fp32 conversion tile (bf16 only) | control
+    // layout: NSTAGE raw stages | fp32 conversion tile (bf16 with lists only) | control
     unsigned char *stages = smem_raw;
-    float *conv = reinterpret_cast<float *>(smem_raw + NSTAGE * STAGE_BYTES);      // bf16 only
-    StreamShared<DT> &sh = *reinterpret_cast<StreamShared<DT> *>(smem_raw + NSTAGE * STAGE_BYTES + (DT == 1 ? CTA_TILE * 4 : 0));
+    float *conv = reinterpret_cast<float *>(smem_raw + NSTAGE * STAGE_BYTES);      // bf16 with lists only
+    StreamShared<DT, LISTS> &sh = *reinterpret_cast<StreamShared<DT, LISTS> *>(smem_raw + NSTAGE * STAGE_BYTES + (DT == 1 && LISTS ? CTA_TILE * 4 : 0));
     ConsumerSync csync;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1281,6 +1284,11 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         float b_val = 0.0f;
         int row_patch = 0, cached_row = -1, row_bad = 0;
         auto load_row = [&](int row) {
+            if (!LISTS) {
+                c_next = resolve_cfg(P, row, fetch_cfg(P, row));
+                cached_row = row;
+                return;
+            }
             const int req = (P.op == OP_VERIFY) ? row / (P.K + 1) : row;
             const int *hid = P.hist_ids ? P.hist_ids + (size_t)req * P.hist_stride : nullptr;
             const int *hct = P.hist_counts ? P.hist_counts + (size_t)req * P.hist_stride : nullptr;
@@ -1339,7 +1347,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         auto prepare = [&](int row, int tile, int hb) -> Prep {
             if (row != cached_row) load_row(row);
             Prep r{row_patch, 0, 0};
-            if (row_patch != 1) return r;
+            if (!LISTS || row_patch != 1) return r;
             const int first = tile * CTA_TILE;
 #pragma unroll
             for (int u = 0; u < HPL; ++u) {
@@ -1488,7 +1496,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             }
             unsigned char *stage = stages + (size_t)s * STAGE_BYTES;
             const bool tail = tile_base + CTA_TILE > P.V;
-            const int patch = meta.patch;
+            const int patch = LISTS ? meta.patch : 0;
             const bool patched = patch != 0;
             float *ptile = (DT == 0) ? reinterpret_cast<float *>(stage) : conv;    // fp32 view the sparse lists patch
 
