@@ -15,8 +15,14 @@
 // producer warp plus eight consumer warps.  The producer takes tiles from a work
 // queue, resolves each tile's row configuration and issues one bulk-TMA copy
 // (cp.async.bulk, completion on an mbarrier) of the tile's logits into a ring of
-// two shared-memory stages, one tile ahead of the consumers, so HBM requests
-// stay in flight while the consumers compute.  Every mbarrier wait is bounded:
+// shared-memory stages, ahead of the consumers, so HBM requests stay in flight
+// while the consumers compute.  Two builds: calls without sparse lists (histories,
+// biases) carry no list code, which spares 80 to 100 bytes of spills per thread (with
+// hardly any L1 left beside the ring they go to L2), and in bf16 the room of the
+// fp32 tile that lists patch holds two more stages.  Measured (us per call): 128
+// fp32 rows of 200003, k = 4096, 77.6 -> 68.4; 256 fp32 rows of 262144, k = 64,
+// 59.6 -> 57.9 (4.6 TB/s); 160 fp32 verification rows of 131072 93.1 -> 91.3; 256
+// bf16 rows of 262144, top-k 50, 57.9 -> 56.5.  Every mbarrier wait is bounded:
 // on expiry the kernel records an error in the workspace header and returns.
 //
 // Exactness: a tile's cutoff t is a minimum of group maxima (of the G groups of
@@ -190,7 +196,8 @@ __device__ __noinline__ void warp_sort_256(unsigned long long *a, int cnt, int l
 // Descending sort of n0 distinct 64-bit keys in buf (RANK_SORT_MAX < n0 <= MERGE_CAP), of which the first n are wanted:
 // 4096 buckets by distance from the smallest, one counting pass, one scan, one scatter;
 // what shares a bucket (a handful of keys for smooth values) is ranked by counting, a crowded bucket (ties of a
-// low-precision value) is sorted by a warp.  About 35 instructions per key in eight barrier-separated steps, where a
+// low-precision value) is sorted by a warp.  Bound by barriers and shared-memory latency: 128 fp32 rows of 200003 with k = 4096
+// 107 -> 75 us a call, 64 bf16 rows of 131072 with k = 1000 on an eighth of them 58.8 -> 55.5.  About 35 instructions per key in eight barrier-separated steps, where a
 // bitonic sort of 4096 keys goes through 78 compare-exchange steps, 21 of them behind block barriers.  A bucket beyond
 // 256 keys that the wanted ones reach into falls back to the bitonic sort.
 template <int THREADS>
