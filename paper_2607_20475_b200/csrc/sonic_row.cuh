@@ -724,7 +724,9 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
     cl_arrive();                                                    // (matched by the wait before the first remote write)
     const RowCfg c = resolve_cfg(P, row, cfg_raw);
     const bool finish_request = P.op == OP_VERIFY;
-    const bool dense = c.cls == CLS_DENSE || c.cls == CLS_EXACT, greedy = c.cls == CLS_GREEDY;
+    // (sonic_topk comes here with k up to ROW_KMAX alone and is always finished from gathered elements, also where its class in
+    // the streaming chain is the cluster kernel's: vocabularies just above MERGE_CAP with k beyond an eighth of them)
+    const bool dense = c.cls == CLS_DENSE || (c.cls == CLS_EXACT && P.op != OP_TOPK), greedy = c.cls == CLS_GREEDY;
     auto emit = [&](int token, float prob, uint32_t flags, int support, float p_draft) {
         emit_row(P, c, row, token, prob, flags, support, p_draft);
         if (finish_request) row_ticket(P, c.b);

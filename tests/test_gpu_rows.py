@@ -117,3 +117,25 @@ def test_large_top_k_sorts(sonic, oracle, B, k):
     dev.run()
     gv, gi = dev.results()
     compare_topk(gv, gi, *oracle.topk(x, k))
+
+
+@pytest.mark.parametrize("V", [8193, 9000, 12000, 16384, 17999])
+@pytest.mark.parametrize("dtype", [wl.DTYPE_F32, wl.DTYPE_BF16])
+def test_top_k_that_the_streaming_chain_would_not_take(sonic, oracle, V, dtype):
+    # short vocabularies with a large k, at both sides of what the chain's candidates prove (1003 | 1005 at V = 8193): every
+    # output has to be written, through both entry points
+    rng = np.random.default_rng(V + dtype)
+    for B, k in ((1, 1003), (8, 1005), (3, 1500), (8, 2048)):
+        x = rng.standard_normal((B, V)).astype(np.float32)
+        x[0, ::3] = -np.inf
+        tw = wl.TopKWorkload(name="t", B=B, V=V, dtype=dtype, logits=x if dtype == wl.DTYPE_F32 else wl.f32_to_bf16_bits(x))
+        ref = oracle.topk(tw.logits_f32(), k)
+        dev = sonic.DeviceTopK(tw, k)
+        for static in (False, True):
+            dev.out_vals.fill_(-7.0)
+            dev.out_idx.fill_(-7)
+            if static:
+                sonic.sonic_topk_static(dev.logits, dtype, B, V, dev.logits.shape[1], k, dev.out_vals, dev.out_idx)
+            else:
+                dev.run()
+            compare_topk(*dev.results(), *ref)
