@@ -68,6 +68,7 @@ constexpr unsigned int ERR_TIMEOUT = 0x1;     // workspace header: a bounded mba
 constexpr uint32_t TILE_BADID = 0x1;          // TileRec.flags: a list id of the row was out of range
 
 constexpr uint32_t KEY_NEG_INF = 0x007FFFFFu; // okey(-inf)
+constexpr uint32_t KEY_MAX_NORMAL = 0xFF7FFFFFu;      // okey(largest finite value)
 
 struct __align__(16) RowState {
     unsigned int status;                      // ST_*; set to zero by the streaming kernel, ST_FAILED by a row's finisher

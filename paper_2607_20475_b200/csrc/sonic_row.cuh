@@ -147,7 +147,8 @@ __device__ __forceinline__ float row_w(float y, float Mf) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(fmaf(d, L1, d * L2)));
     return w;
 }
-// ... as an integer, 2^-44 of the largest.  (NaN - past the row's end - gives 0.)
+// ... as an integer, 2^-44 of the largest.  The weight of a NaN (past the row's end) converts to 2^63: every sum takes elements
+// of at least vmin alone, which a NaN is not.
 constexpr double ROW_Q1 = 17592186044416.0;              // 2^44
 __device__ __forceinline__ unsigned long long row_q(float w) { return __float2ull_rz(w * 17592186044416.0f); }
 // Weights below 2^-41 count as nothing (their fixed-point value was 0 before it was refined to 2^-44).
@@ -1032,6 +1033,15 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
     // ---------------------------------------------------------------- top-k off, or a top-k beyond the gather
     const uint2 cells = draw();
     const uint32_t cls_flag = c.cls == CLS_DENSE ? F_DENSE : F_FALLBACK;
+    // A finite logit over a small temperature can be +inf, whose weight relative to itself would be NaN: the largest finite value
+    // stands for it (weight 1 for all such elements, 0 for the others: the limit), so that weights stay within [0, 1] and bins
+    // and masses within their range.
+    if (kmax > KEY_MAX_NORMAL) {
+        for (int i = x.wlo + lane; i < x.wlo + x.wn; i += 32) if (row_y()[i] > CUDART_MAX_NORMAL_F) row_y()[i] = CUDART_MAX_NORMAL_F;
+        __syncwarp();
+        kmax = KEY_MAX_NORMAL; kmin = min(kmin, KEY_MAX_NORMAL);
+        x.Mf = CUDART_MAX_NORMAL_F;
+    }
     if (c.cls == CLS_EXACT) {
         // the k-th largest element by count: the row is split until that element is alone
         s.lo = 0ull; s.hi = ~0ull;
@@ -1053,8 +1063,10 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
     unsigned long long Z = 0ull, goal = 0ull;
     if (top_p) {
         // Bins by the weight's bits: 2^m per octave, so that the row's finite range (41 octaves carry mass at all) takes 256.
-        const float w_min = row_w(unkey(kmin), x.Mf);
-        const int octaves = 128 - min(127, max(86, (int)(__float_as_uint(w_min) >> 23)));
+        // (the smallest weight's octave is taken a hair lower: the approximate exponential is not promised to be monotone, and a
+        // larger value's weight must not fall below the last bin)
+        const uint32_t w_min = __float_as_uint(row_w(unkey(kmin), x.Mf));
+        const int octaves = 128 - min(127, max(86, (int)((max(w_min, 16u) - 16u) >> 23)));
         const int m = octaves <= 4 ? 6 : octaves <= 8 ? 5 : octaves <= 16 ? 4 : octaves <= 32 ? 3 : 2, shift_a = 23 - m, shift_b = 15 - m;
         const float Mf = x.Mf;
         row_zero_bins(x);
@@ -1105,7 +1117,7 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
             bc.W = dense_warp_sum(ab.x);
             unsigned int n = __reduce_add_sync(0xFFFFFFFFu, (unsigned int)ab.y);
             if (tid < x.ncta) sh.cta_mass[tid] = ab.x;
-            const uint32_t kd = (draft >= 0) ? (uint32_t)sh.ex1[draft / slice].y : 0u;
+            const uint32_t kd = (draft >= 0) ? min((uint32_t)sh.ex1[draft / slice].y, KEY_MAX_NORMAL) : 0u;
             bool draft_tie_in = false;
             __syncthreads();                                        // (land_n is reset by the broadcast)
             if (!masses) {

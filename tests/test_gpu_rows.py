@@ -139,3 +139,59 @@ def test_top_k_that_the_streaming_chain_would_not_take(sonic, oracle, V, dtype):
             else:
                 dev.run()
             compare_topk(*dev.results(), *ref)
+
+
+@pytest.mark.parametrize("dtype", [wl.DTYPE_F32, wl.DTYPE_BF16])
+def test_processed_logits_that_overflow(sonic, oracle, dtype):
+    # finite logits over a temperature of 0.5: ten ids become +inf and share the whole mass (the limit of the softmax); no
+    # truncation, top-p, min-p, a top-k beyond the gather; then the same as verification rows, whose requests must be finished
+    import torch
+    V, n = 20001, 10
+    rng = np.random.default_rng(5 + dtype)
+    ids = np.sort(rng.choice(V, n, replace=False))
+    x = rng.standard_normal((4, V)).astype(np.float32)
+    x[:, ids] = 3e38
+    T = wl.TEMPERATURE
+    w = make_sample(x, [T, T | wl.TOP_P, T | wl.MIN_P, T | wl.TOP_K], dtype=dtype, temperature=np.full(4, 0.5), top_p=np.full(4, 0.85),
+                    min_p=np.full(4, 0.1), top_k=np.full(4, 3000), seed=np.arange(4) + 11, offset=np.arange(4))
+    dev = sonic.DeviceSample(w)
+    dev.run()
+    got = dev.results()
+    assert np.isin(got["token"], ids).all() and not (got["flags"] & 0x13).any()
+    assert got["support"].tolist() == [V, 9, n, 3000]                # (elements without weight count where nothing cuts them off)
+    assert np.allclose(got["prob"], [1 / n, 1 / 9, 1 / n, 1 / n], rtol=1e-5)
+    B, K = 2, 1
+    vw = wl.VerifyWorkload(name="v", B=B, K=K, V=V, sample=make_sample(x[:B], [T | wl.TOP_P, T | wl.MIN_P], dtype=dtype,
+                           temperature=np.full(B, 0.5), top_p=np.full(B, 0.85), min_p=np.full(B, 0.1), seed=np.arange(B), offset=np.arange(B)),
+                           draft_tokens=np.array([[ids[-1]], [ids[0]]], np.int32), draft_probs=np.zeros((B, K, V), np.float32))
+    vw.draft_probs[0, 0, ids[:5]] = 0.2                           # (the first draft lies outside the top-p support: rejected)
+    vw.draft_probs[1, 0, ids[0]] = 0.05
+    vw.sample.logits = w.logits
+    dv = sonic.DeviceVerify(vw)
+    for _ in range(3):
+        dv.run()
+        got = dv.results()
+        assert got["accept_len"].tolist() == [0, 1] and got["tokens"][1, 0] == ids[0]
+        assert got["tokens"][0, 0] in ids[5:9] and got["tokens"][0, 1] == -1 and got["tokens"][1, 1] in ids
+        assert not dv.ws[512:512 + 4 * 4096].view(torch.int32).any()                # the requests' tickets
+
+
+@pytest.mark.parametrize("octaves", [1, 4, 8, 16, 32, 41])
+def test_smallest_weight_at_the_edge_of_an_octave(sonic, oracle, octaves):
+    # the row's smallest value a whole number of halvings below its largest, give or take a unit in the last place: every
+    # weight must stay within the bins that this number is given
+    V = 30011
+    rng = np.random.default_rng(octaves)
+    x = (rng.random((12, V)) * -(octaves * np.log(2.0))).astype(np.float32)
+    low = np.float32(-octaves * np.log(2.0))
+    for r in range(12):
+        edge = low
+        for _ in range(abs(r - 6)):
+            edge = np.nextafter(edge, np.float32(-np.inf if r < 6 else np.inf))
+        x[r] = np.maximum(x[r], edge)
+        x[r, rng.choice(V, V // 3, replace=False)] = edge
+        x[r, r * 100] = 0.0
+    w = make_sample(x, np.full(12, wl.TOP_P), top_p=np.where(np.arange(12) % 2, 0.9999, 0.6), seed=np.arange(12) + 3, offset=np.arange(12))
+    dev = sonic.DeviceSample(w)
+    dev.run()
+    compare_sample(dev.results(), oracle.sample(w), w, max_near=12)
