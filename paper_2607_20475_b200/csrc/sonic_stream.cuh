@@ -217,8 +217,8 @@ __device__ __forceinline__ void merge_bucket_sort(unsigned long long *buf, unsig
     mx = __reduce_max_sync(0xFFFFFFFFu, mx);
     mn = __reduce_min_sync(0xFFFFFFFFu, mn);
     if (lane == 0) { sh.wsum[warp] = (int)mx; sh.wsum2[warp] = (int)mn; }
-    if (tid == 0) { sh.count = 0; sh.found = 0; }
     __syncthreads();
+    if (tid == 0) { sh.count = 0; sh.found = 0; }                  // (behind the barrier: until then a warp may still be reading the caller's count)
     mx = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)sh.wsum[lane & (THREADS / 32 - 1)]);
     mn = __reduce_min_sync(0xFFFFFFFFu, (uint32_t)sh.wsum2[lane & (THREADS / 32 - 1)]);
     // Bucket: 256 per octave of the distance above the smallest key.  The upper tail of a smooth distribution is dense at

@@ -195,3 +195,21 @@ def test_smallest_weight_at_the_edge_of_an_octave(sonic, oracle, octaves):
     dev = sonic.DeviceSample(w)
     dev.run()
     compare_sample(dev.results(), oracle.sample(w), w, max_near=12)
+
+
+@pytest.mark.parametrize("B,k", [(8, 1500), (80, 1500), (148, 3000)])
+def test_repeated_sorts_of_large_candidate_sets(sonic, oracle, B, k):
+    # many sorts of thousands of candidates under load, in the row kernel and in the merge: the same rows every time
+    import torch
+    V = 20001
+    x = np.random.default_rng(k).standard_normal((B, V)).astype(np.float32)
+    dev = sonic.DeviceTopK(wl.TopKWorkload(name="t", B=B, V=V, dtype=wl.DTYPE_F32, logits=x), k)
+    dev.run()
+    vals, idx = dev.results()
+    compare_topk(vals, idx, *oracle.topk(x, k))
+    vals, idx = torch.from_numpy(vals).cuda(), torch.from_numpy(idx).cuda()
+    for _ in range(300):
+        dev.out_vals.fill_(-7.0)
+        dev.out_idx.fill_(-7)
+        dev.run()
+        assert torch.equal(dev.out_vals, vals) and torch.equal(dev.out_idx, idx)
