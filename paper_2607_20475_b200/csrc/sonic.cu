@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <mutex>
 
@@ -252,9 +253,12 @@ static SideStream *side_stream_for(int dev, cudaStream_t st) {
 // With 64 rows of 131072 (1.7 times what is resident) the chain is ahead, 58 against 64: its persistent CTAs keep loading
 // while the rows' selections wait for one another.  sonic_topk beyond ROW_KMAX: the chain.
 static bool row_route(const KParams &P, int sm_count) {
-#if defined(SONIC_TRACE) || defined(SONIC_TEST_WITHHOLD)
-    return false;                                 // (these variants exist to look into the streaming chain)
+#ifdef SONIC_TRACE
+    return false;                                 // (this variant exists to look into the streaming chain)
 #else
+#ifdef SONIC_TEST_WITHHOLD
+    if (!getenv("SONIC_TEST_ROW")) return false;  // (this one into the waits of both)
+#endif
     if (P.op == OP_TOPK && P.ktop > ROW_KMAX) return false;
     const int c = std::max(ROW_CMIN, (P.V + ROW_SLICE_MAX - 1) / ROW_SLICE_MAX);
     return (long long)P.rows * c <= 2ll * sm_count;

@@ -243,6 +243,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                     // the consumers have left tile n - NSTAGE: its stage is free
                     if (!mbar_wait(&sh.empty[s], ((n / NSTAGE) - 1) & 1)) {
                         if (lane == 0) atomicOr(P.error, ERR_TIMEOUT);
+                        for (int i = n - NSTAGE; i < n; ++i) (void)mbar_wait(&sh.full[i % NSTAGE], (i / NSTAGE) & 1);       // copies under way
                         return;
                     }
                     // (the first tiles' copies are under way; nothing is copied for rows of the cluster kernel's class)
@@ -272,6 +273,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         for (int i = max(0, n - NSTAGE + 1); i < n; ++i) {     // the last tiles
             if (!mbar_wait(&sh.empty[i % NSTAGE], (i / NSTAGE) & 1)) {
                 if (lane == 0) atomicOr(P.error, ERR_TIMEOUT);
+                for (; i < n; ++i) (void)mbar_wait(&sh.full[i % NSTAGE], (i / NSTAGE) & 1);
                 return;
             }
             retire(i % NSTAGE);

@@ -690,6 +690,10 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
         const int elems = min(slice, (P.V - x.base + VEC - 1) / VEC * VEC);
         if (elems > 0) {
             mbar_arrive_expect_tx(&sh.full, (unsigned int)elems * ELT);
+#ifdef SONIC_TEST_WITHHOLD
+            // test-only build: the bytes of one chosen part of a row are announced but its copy is never issued
+            if (__ldcg(&P.error[WS_TEST_WITHHOLD]) != (unsigned int)(row * ROW_CMAX + x.rank) + 1u)
+#endif
             bulk_load(raw, reinterpret_cast<const unsigned char *>(P.logits) + ((size_t)row * (size_t)P.row_stride + (size_t)x.base) * ELT,
                       (unsigned int)elems * ELT, &sh.full, l2_evict_first_policy());
         } else mbar_arrive(&sh.full);
@@ -738,11 +742,13 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
         else emit(-1, 0.0f, F_TIMEOUT, 0, 0.0f);
     };
     // A copy that never comes, or the workspace's sticky error: every CTA of the cluster learns of it with the first
-    // exchange, and all of them leave behind it (the values computed up to there are not used).
+    // exchange, and all of them leave behind it (the values computed up to there are not used).  Every thread waits and reads
+    // the error word for itself, and any of them may be the only one that is late: each tells all CTAs.
     bool late = (err & ERR_TIMEOUT) != 0u;
     if (!mbar_wait(&sh.full, 0)) {
-        if (tid == 0) atomicOr(P.error, ERR_TIMEOUT);
+        atomicOr(P.error, ERR_TIMEOUT);
         late = true;
+        (void)mbar_wait(&sh.full, 0);                               // (once more: a copy under way must not land in the shared memory of what runs here next)
     }
 
     // ---------------------------------------------------------------- logit processing
@@ -820,7 +826,7 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
     const bool divide = c.temp && c.tau != 1.0f;
     process(divide && !direct, true);
     cl_wait();                                                      // every CTA of the cluster is running
-    if (late && tid < (greedy ? 1 : x.ncta)) *cl_map(&sh.late[x.rank], tid) = 1u;        // (a greedy row's other CTAs wait for nobody)
+    if (late) for (int r = 0; r < (greedy ? 1 : x.ncta); ++r) *cl_map(&sh.late[x.rank], r) = 1u;        // (a greedy row's other CTAs wait for nobody)
 
     RowSel s;
     s.vmin = P.op == OP_TOPK ? -CUDART_INF_F : -CUDART_MAX_NORMAL_F;

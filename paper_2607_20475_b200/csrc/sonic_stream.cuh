@@ -1430,6 +1430,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 // the consumers have left tile n - NSTAGE: its stage and its hit buffer are free
                 if (!mbar_wait(&sh.empty[s], ((n / NSTAGE) - 1) & 1)) {
                     if (lane == 0) atomicOr(P.error, ERR_TIMEOUT);
+                    for (int i = n - NSTAGE; i < n; ++i) (void)mbar_wait(&sh.full[i % NSTAGE], (i / NSTAGE) & 1);       // copies under way
                     return;
                 }
             }
