@@ -227,6 +227,19 @@ __device__ __forceinline__ float div_tau(float z, float tau) {
     return special ? z : q;
 }
 
+// A bound on undivided values: whatever lies below it divides to less than t does.  (With q' the float below t / tau as
+// rounded: z < q' * tau gives z / tau < q', which rounds to q' at most.  The product of two floats is exact in double.  A margin
+// relative to t would do for normal quotients alone: subnormal ones repeat over wider ranges, overflowing ones are all equal.)
+__device__ __forceinline__ float bound_before_div(float t, float tau) {
+    return __double2float_rd((double)nextafterf(div_tau(t, tau), -CUDART_INF_F) * (double)tau);
+}
+
+// The smallest value whose quotient by tau is finite.  (z / tau rounds to -inf from the middle between the largest finite value
+// and 2^128 on, the middle included.)
+__device__ __forceinline__ float first_finite_quotient(float tau) {
+    return nextafterf(__double2float_rd(-3.4028235677973366e38 * (double)tau), CUDART_INF_F);
+}
+
 // Returns G, plus PICK_TILE_MODE in tile mode; 0 means "keep every finite element" (vocabularies the merge can sort
 // whole); -1 hands the row to the exact kernel.
 __device__ __forceinline__ int pick_groups(const GroupTable &t, int k, int V) {

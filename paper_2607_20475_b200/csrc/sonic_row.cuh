@@ -852,10 +852,12 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
         cl_sync();
         if (row_late(x)) { if (lead) emit_late(); return; }
         const uint32_t tk = kth_max<ROW_THREADS>(sh.gmax, sh.red32, ngroups, c.k, tid);
-        // Everything that reaches the bound goes to CTA 0.  With a temperature a value a hair below the bound may become
-        // equal to it when divided, and then the index decides: the bound is lowered by 2^-21 of itself.
-        float t = max(unkey(tk), s.vmin);
-        if (divide && t > s.vmin) t = fmaxf(t - fmaxf(fabsf(t) * 4.76837158203125e-07f, 1e-37f), s.vmin);
+        // Everything that reaches the bound goes to CTA 0.  With a temperature a value a little below the bound may become
+        // equal to it when divided, and then the index decides: the bound is what can divide to as much as it does.  (What
+        // divides to -inf is masked by that.)
+        const float low = divide ? first_finite_quotient(c.tau) : s.vmin;
+        float t = max(unkey(tk), low);
+        if (divide && t > low) t = fmaxf(bound_before_div(t, c.tau), low);
         if (__any_sync(0xFFFFFFFFu, lmax >= t)) {
             unsigned long long *land = cl_map(row_land(), 0);
             unsigned int mine = 0u;

@@ -213,3 +213,25 @@ def test_repeated_sorts_of_large_candidate_sets(sonic, oracle, B, k):
         dev.out_idx.fill_(-7)
         dev.run()
         assert torch.equal(dev.out_vals, vals) and torch.equal(dev.out_idx, idx)
+
+
+@pytest.mark.parametrize("temperature", [3e38, 1e38, 1e-39, 1e-40, 0.3])
+@pytest.mark.parametrize("dtype", [wl.DTYPE_F32, wl.DTYPE_BF16])
+def test_values_that_become_equal_under_the_temperature(sonic, oracle, temperature, dtype):
+    # quotients that are subnormal (steps of 1e-6 of the value) or overflow: ascending logits a few units in the last place
+    # apart, so that the largest index holds the largest logit but the lowest index among its equals wins
+    V = 9000
+    rng = np.random.default_rng(8)
+    x = np.full((6, V), -1.0, np.float32)
+    for r in range(6):
+        ids = np.sort(rng.choice(V, 400, replace=False))
+        x[r, ids] = np.float32(0.1) * (1 + np.arange(400) * np.float32(2.0 ** -22 if dtype == wl.DTYPE_F32 else 2.0 ** -8) * (r + 1))
+    if temperature < 1e-30:
+        x = np.where(x < 0, x, -x * 3)                            # (below 1e-38 most quotients are -inf)
+        x[:, 5] = -temperature
+    mode = np.full(6, wl.TOP_K | wl.TEMPERATURE, np.uint32)
+    mode[5] = wl.GREEDY | wl.TEMPERATURE
+    w = make_sample(x, mode, dtype=dtype, temperature=np.full(6, temperature), top_k=[1, 2, 20, 50, 90, 0], seed=np.arange(6) + 7, offset=np.arange(6))
+    dev = sonic.DeviceSample(w)
+    dev.run()
+    compare_sample(dev.results(), oracle.sample(w), w, max_near=6)
