@@ -560,22 +560,22 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
 
             if (slot.cfg.cls == CLS_GREEDY) {
                 // The argmax of the processed logits, lowest index first.  Only elements at or above the largest so far can
-                // matter (with a temperature: above a hair less, since the division may make them equal).
+                // matter, this tile's included (with a temperature: above what can divide to as much): a dense tile's lanes look
+                // at a vector or two instead of all of theirs.
                 if (row != g_row) { g_row = row; g_thr = -CUDART_MAX_NORMAL_F; }
                 unsigned long long best = 0ull;
                 if (__any_sync(0xFFFFFFFFu, lm >= g_thr)) {
                     const bool temp = slot.cfg.temp;
-                    const float tau = slot.cfg.tau;
+                    const float tau = slot.cfg.tau, z = unkey(__reduce_max_sync(0xFFFFFFFFu, okey(lm)));
+                    g_thr = fmaxf(g_thr, temp ? bound_before_div(z, tau) : z);
                     if (lm >= g_thr) visit(g_thr, [&](float z, int li) {
                         const uint32_t key = okey(temp ? div_tau(z, tau) : z);
-                        best = max(best, ((unsigned long long)key << 32) | (uint32_t)(~(uint32_t)(tile_base + li)));
+                        if (key > KEY_NEG_INF) best = max(best, ((unsigned long long)key << 32) | (uint32_t)(~(uint32_t)(tile_base + li)));
                     });
                     __syncwarp();
                     const uint32_t hi = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(best >> 32));
                     const uint32_t lo = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(best >> 32) == hi ? (uint32_t)best : 0u);
                     best = ((unsigned long long)hi << 32) | lo;
-                    const float z = unkey(__reduce_max_sync(0xFFFFFFFFu, okey(lm)));
-                    g_thr = fmaxf(g_thr, temp ? z - fmaxf(fabsf(z) * 4.76837158203125e-07f, 1e-37f) : z);
                 }
                 if (lane == 0) sh.best[s][warp] = best;
             } else {

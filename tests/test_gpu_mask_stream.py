@@ -49,3 +49,28 @@ def test_masked_batches(V, dtype):
     again = dev.results()
     for key in got:
         assert np.array_equal(got[key], again[key]), key
+
+
+@pytest.mark.parametrize("temperature", [1.0, 0.7, 1e38, 1e-39, 1e-40])
+@pytest.mark.parametrize("dtype", [wl.DTYPE_F32, wl.DTYPE_BF16])
+def test_masked_greedy_rows(dtype, temperature):
+    # dense, sparse and missing masks; logits a few units in the last place apart, which an extreme temperature makes equal (the
+    # lowest index wins) or sends to -inf (no token)
+    from oracle import oracle
+    from paper_2607_20475_b200 import harness
+    B, V = 80, 20001
+    rng = np.random.default_rng(9)
+    x = rng.standard_normal((B, V)).astype(np.float32)
+    step = 2.0 ** -22 if dtype == wl.DTYPE_F32 else 2.0 ** -8
+    x[::4] = np.float32(0.1) * (1 + np.arange(V) * np.float32(step) / 64)
+    x[1::4] = -np.float32(0.3) * (1 + np.arange(V)[::-1] * np.float32(step) / 64)
+    if temperature < 1e-30:
+        x = -np.abs(x)
+        x[::8, 777] = -2 * temperature
+    allowed = rng.random((B, V)) < np.array([0.02, 0.3, 0.9, 1.0])[rng.integers(0, 4, B)][:, None]
+    mode = np.full(B, wl.GREEDY | wl.TEMPERATURE, np.uint32)
+    mode[rng.random(B) < 0.7] |= wl.GRAMMAR
+    w = make_sample(x, mode, dtype=dtype, temperature=np.full(B, temperature), bitmask=pack_bits(allowed))
+    dev = harness.DeviceSample(w)
+    dev.run()
+    compare_sample(dev.results(), oracle.sample(w), w)
