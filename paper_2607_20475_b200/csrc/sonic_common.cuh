@@ -252,6 +252,14 @@ __device__ __forceinline__ int pick_groups(const GroupTable &t, int k, int V) {
     return -1;
 }
 
+// Groups of the smallest warp-mode step that serves k (0: none): what one warp can bound by itself, without the tile's others.
+__device__ __forceinline__ int pick_warp_groups(const GroupTable &t, int k) {
+#pragma unroll
+    for (int step = 0; step < GK_STEPS; step += 2)
+        if (k <= t.k[step]) return ((t.over >> step) & 1u) ? 0 : (2 << (step >> 1));
+    return 0;
+}
+
 // The per-request parameters as read from global memory.  Every array that exists is read at once (one
 // global-memory latency, not a chain behind the mode word); values whose mode bit is clear are dropped by
 // resolve_cfg.

@@ -25,11 +25,16 @@ struct Hit { int id; int payload; };           // a bias entry: token, value bit
 struct RowSlot {                               // a row's parameters and lists
     RowCfg cfg;
     int patch;                                 // 0 no lists, 1 they are here, 2 consumers scan them in global memory
+    int wgroups;                               // top-k rows: groups by which a warp bounds its part alone (0: none serves the row's k)
     int bad;                                   // a list id outside [0, V)
     int off[MAX_TILES + 1];                    // the history entries of tile t: list[off[t], off[t + 1])
     uint32_t list[FILTER_HIST];                // id | count << 18
     Hit bias[FILTER_BIAS];
 };
+
+// A kept cutoff is taken for stale where more lanes of a warp than this hold a candidate.  The fullest steps it is kept for bring
+// one to 22 of 32 lanes (8 groups per warp tile, the smallest of 64 maxima as the cutoff: 38 of 1024 elements), the usual ones to 4.
+constexpr int CROWDED = 28;
 
 template <int DT>
 struct StreamShared {
@@ -156,7 +161,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 bad = __any_sync(0xFFFFFFFFu, bad);
                 if (__any_sync(0xFFFFFFFFu, big)) patch = 2;       // a count too large to pack: consumers scan
             }
-            if (lane == 0) { q.cfg = c; q.patch = patch; q.bad = bad ? 1 : 0; }
+            if (lane == 0) { q.cfg = c; q.patch = patch; q.bad = bad ? 1 : 0; q.wgroups = (c.cls == CLS_TOPK) ? pick_warp_groups(P.groups, c.k) : 0; }
             __syncwarp();
         };
         const unsigned long long l2_policy = l2_evict_first_policy();
@@ -581,22 +586,22 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             } else {
                 const int G = slot.cfg.G;
                 const bool tmin = slot.cfg.tile_min;
-                // warp cutoff: minimum over G groups of the group maximum.  Tile cutoff: the largest of the eight warp cutoffs
-                // (warp mode) or the smallest (tile mode: a minimum over all 8 G groups of the tile).  In tile mode a group
+                // warp cutoff: minimum over g groups of the group maximum.  Tile cutoff: the largest of the eight warp cutoffs
+                // (warp mode) or the smallest (tile mode: a minimum over all 8 g groups of the tile).  In tile mode a group
                 // without a finite element (masked, or past the row's end) does not take part: it would drag the cutoff
                 // to -inf and the tile would emit everything it has.
-                auto group_cutoff = [&]() -> float {
-                    switch (G) {                               // (one straight-line butterfly per group count)
+                auto group_cutoff = [&](int g, bool tile_mode) -> float {
+                    switch (g) {                               // (one straight-line butterfly per group count)
                     case 0: return -CUDART_INF_F;
-                    case 1: return warp_cutoff<32>(lm, tmin);
-                    case 2: return warp_cutoff<16>(lm, tmin);
-                    case 4: return warp_cutoff<8>(lm, tmin);
-                    case 8: return warp_cutoff<4>(lm, tmin);
-                    case 16: return warp_cutoff<2>(lm, tmin);
-                    case 32: return warp_cutoff<1>(lm, tmin);
+                    case 1: return warp_cutoff<32>(lm, tile_mode);
+                    case 2: return warp_cutoff<16>(lm, tile_mode);
+                    case 4: return warp_cutoff<8>(lm, tile_mode);
+                    case 8: return warp_cutoff<4>(lm, tile_mode);
+                    case 16: return warp_cutoff<2>(lm, tile_mode);
+                    case 32: return warp_cutoff<1>(lm, tile_mode);
                     default: {                                 // 64: half-lane groups
-                        const float a0 = (tmin && h0 == -CUDART_INF_F) ? CUDART_INF_F : h0;
-                        const float a1 = (tmin && h1 == -CUDART_INF_F) ? CUDART_INF_F : h1;
+                        const float a0 = (tile_mode && h0 == -CUDART_INF_F) ? CUDART_INF_F : h0;
+                        const float a1 = (tile_mode && h1 == -CUDART_INF_F) ? CUDART_INF_F : h1;
                         return warp_cutoff<1>(fminf(a0, a1), false);
                     }
                     }
@@ -604,7 +609,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 // (many groups, many candidates: a cutoff per tile keeps them down)
                 float t = cut;
                 if (row != cut_row || G > 8) {
-                    const float g = group_cutoff();
+                    const float g = group_cutoff(G, tmin);
                     if (lane == 0) sh.tw[s][warp] = g;
                     csync();
                     static_assert(STREAM_WARPS == 8, "the eight warp cutoffs are read as two 128-bit words");
@@ -619,11 +624,11 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                     // (a tile that bounds nothing leaves the cutoff to the next one)
                     cut = t;
                     cut_row = (t > -CUDART_INF_F) ? row : -1;
-                } else if (__popc(__ballot_sync(0xFFFFFFFFu, lm >= t)) > 28) {
-                    // far more candidates than the cutoff was meant for (values that depend on the position): the warp takes
-                    // a cutoff of its own for this tile
-                    t = fmaxf(t, group_cutoff());
-                    if (t == CUDART_INF_F) t = cut;
+                } else if (__popc(__ballot_sync(0xFFFFFFFFu, lm >= t)) > CROWDED) {
+                    // Far more candidates than the cutoff was meant for (values that depend on the position): the warp bounds its
+                    // own part, by the warp-mode step for the row's k.  (Not by the row's own step: a warp's share of a tile-mode
+                    // cutoff lies so high that the row could no longer be proven, and the cluster kernel would have to finish it.)
+                    t = fmaxf(t, group_cutoff(slot.wgroups, false));
                 }
                 if (lane == 0) sh.best[s][warp] = (unsigned long long)okey(t) << 32;
                 // every finite element >= t goes to the tile's candidate slot

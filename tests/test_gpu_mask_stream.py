@@ -74,3 +74,26 @@ def test_masked_greedy_rows(dtype, temperature):
     dev = harness.DeviceSample(w)
     dev.run()
     compare_sample(dev.results(), oracle.sample(w), w)
+
+
+@pytest.mark.parametrize("share", [0.3, 1.0])
+@pytest.mark.parametrize("dtype", [wl.DTYPE_F32, wl.DTYPE_BF16])
+def test_masked_rows_whose_values_depend_on_the_position(dtype, share):
+    # the cutoff that a CTA keeps from its first tile of a row lies far below a later tile's values: the rows have to be right, and
+    # but for the few that miss their proof (half the row is as good as not there) the merge has to finish them
+    from oracle import oracle
+    from paper_2607_20475_b200 import harness
+    B, V = 128, 131072                                             # (several tiles of a row in a CTA)
+    rng = np.random.default_rng(17)
+    x = rng.standard_normal((B, V)).astype(np.float32)
+    x[0::2, V // 2:] += 6                                          # the second half
+    x[1::2] += 6 * (np.arange(V) // 8192 % 2)                      # every other tile
+    allowed = rng.random((B, V)) < share
+    w = make_sample(x, np.full(B, wl.TOP_K | wl.TEMPERATURE | wl.TOP_P | wl.GRAMMAR), dtype=dtype, temperature=np.full(B, 0.8),
+                    top_k=np.array([8, 20, 64, 100])[np.arange(B) // 4 % 4], top_p=np.full(B, 0.95), bitmask=pack_bits(allowed),
+                    seed=np.arange(B), offset=np.arange(B))
+    dev = harness.DeviceSample(w)
+    dev.run()
+    got = dev.results()
+    compare_sample(got, oracle.sample(w), w, max_near=B)
+    assert ((got["flags"] & 4) != 0).sum() <= B // 8, np.nonzero(got["flags"] & 4)[0]
