@@ -260,25 +260,26 @@ __device__ __forceinline__ void merge_bucket_sort(unsigned long long *buf, unsig
                     reinterpret_cast<unsigned int *>(sh.scratch)[at] = run | (v[j] << 16);       // (more than MERGE_CAP / FEW never exist)
                 }
             }
+            if (run < (unsigned int)n && (unsigned int)n <= run + v[j]) sh.bracket[0] = (int)(run + v[j]);      // where the last wanted bucket ends
             const unsigned int t = v[j]; v[j] = run; run += t;
         }
 #pragma unroll
         for (int j = 0; j < BPT; j += 4) *reinterpret_cast<uint4 *>(bins + tid * BPT + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
     }
     __syncthreads();
-    if (sh.found) {
-        const int m = next_pow2(n0);
-        for (int i = n0 + tid; i < m; i += THREADS) buf[i] = 0ull;
-        __syncthreads();
-        bitonic_sort_desc_cta<THREADS>(buf, m, tid);
-        return;
-    }
 #pragma unroll
     for (int u = 0; u < ITEMS; ++u) {
         if (u * THREADS >= n0) break;
         if (u * THREADS + tid < n0) buf[atomicAdd(&bins[bucket(key[u])], 1u)] = key[u];
     }
     __syncthreads();
+    if (sh.found) {                                                 // the wanted buckets are in front now: the others are left out
+        const int nw = sh.bracket[0], m = next_pow2(nw);
+        for (int i = nw + tid; i < m; i += THREADS) buf[i] = 0ull;
+        __syncthreads();
+        bitonic_sort_desc_cta<THREADS>(buf, m, tid);
+        return;
+    }
     // bins[b] is now where bucket b ends: rank inside the bucket, for the wanted ones
     int to[ITEMS];
 #pragma unroll

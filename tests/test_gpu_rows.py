@@ -235,3 +235,18 @@ def test_values_that_become_equal_under_the_temperature(sonic, oracle, temperatu
     dev = sonic.DeviceSample(w)
     dev.run()
     compare_sample(dev.results(), oracle.sample(w), w, max_near=6)
+
+
+@pytest.mark.parametrize("B", [8, 80])                             # row kernel (k up to 2048), streaming chain
+@pytest.mark.parametrize("k", [513, 1024, 2048, 3000])
+def test_sorts_with_hundreds_of_equal_values(sonic, oracle, B, k):
+    # a dozen distinct values among the wanted ones, hundreds of each: buckets beyond what a warp sorts, most candidates unwanted
+    V = 65536
+    rng = np.random.default_rng(k + B)
+    x = (np.round(rng.standard_normal((B, V)) * 8) / 8).astype(np.float32)
+    x[1::3] = np.round(x[1::3] * 2) / 2
+    x[2::3, rng.choice(V, k // 2, replace=False)] += np.float32(40.0)
+    tw = wl.TopKWorkload(name="t", B=B, V=V, dtype=wl.DTYPE_F32, logits=x)
+    dev = sonic.DeviceTopK(tw, k)
+    dev.run()
+    compare_topk(*dev.results(), *oracle.topk(x, k))
