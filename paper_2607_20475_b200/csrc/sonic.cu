@@ -152,6 +152,9 @@ static const GroupTable &group_table(int V) {
 }
 
 static int g_sm_count[64];
+// Clusters of C CTAs of the row kernel that are resident at once, per device (a cluster has to fit into one GPC, so that they are
+// fewer than the CTA slots divide into: 71, 33 and 14 of 4, 8 and 16 CTAs on a B200, where 296 slots make 74, 37 and 18).
+static int g_row_clusters[64][ROW_CMAX + 1];
 
 static int configure_once(int *sm_count, int *device) {
     static std::once_flag once[64];
@@ -181,6 +184,22 @@ static int configure_once(int *sm_count, int *device) {
         set((const void *)sonic_row_kernel<1>, ROW_DYN_SMEM);
         for (const void *f : {(const void *)sonic_row_kernel<0>, (const void *)sonic_row_kernel<1>})
             if (r == cudaSuccess) r = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);      // (clusters of up to 16)
+        for (int c = ROW_CMIN; c <= ROW_CMAX && r == cudaSuccess; ++c) {
+            cudaLaunchConfig_t cfg;
+            memset(&cfg, 0, sizeof(cfg));
+            cfg.gridDim = dim3(c);
+            cfg.blockDim = dim3(ROW_THREADS);
+            cfg.dynamicSmemBytes = ROW_DYN_SMEM;
+            cudaLaunchAttribute attr;
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = c; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+            cfg.attrs = &attr;
+            cfg.numAttrs = 1;
+            int n0 = 0, n1 = 0;                       // (a size that cannot be launched is resident 0 times and never chosen)
+            if (cudaOccupancyMaxActiveClusters(&n0, (const void *)sonic_row_kernel<0>, &cfg) != cudaSuccess ||
+                cudaOccupancyMaxActiveClusters(&n1, (const void *)sonic_row_kernel<1>, &cfg) != cudaSuccess) { n0 = 0; cudaGetLastError(); }
+            g_row_clusters[dev][c] = std::min(n0, n1);
+        }
         set((const void *)sonic_exact_kernel<0>, EXACT_SMEM);
         set((const void *)sonic_exact_kernel<1>, EXACT_SMEM);
         int n = 0;
@@ -246,34 +265,42 @@ static SideStream *side_stream_for(int dev, cudaStream_t st) {
     return &S;
 }
 
-// Whether a call goes to the row kernel as a whole: when all of its rows' clusters are resident at once (two CTAs per SM).
-// Measured (us per call, streaming chain against row kernel): one bf16 row of 131072 with top-k 25.5 -> 13.6; 4 fp32 rows
-// of 32768, one of each kind, 29.9 -> 23.2; 3 x 3 verification rows of 32003 50.4 -> 25.7; 37 fp32 rows of 50021 of every
-// kind 64.3 -> 36.4; 32 bf16 rows of 100003 without top-k 73.9 -> 49.3; 8 bf16 rows of 65536 with k = 50 22.7 -> 14.4.
-// With 64 rows of 131072 (1.7 times what is resident) the chain is ahead, 58 against 64: its persistent CTAs keep loading
-// while the rows' selections wait for one another.  sonic_topk beyond ROW_KMAX: the chain.
-static bool row_route(const KParams &P, int sm_count) {
+// CTAs per row of a call that goes to the row kernel as a whole; 0: the call takes the streaming chain.  Measured (us per call):
+// As many CTAs as keep the rows' clusters resident, so that a CTA has few elements (a step costs 64 cycles per instruction and
+// 8192 elements), within what a slice can be.  Rows behind the resident ones wait for whole rows: 17 fp32 rows of 50021 with k = 300
+// 32 in clusters of 16 (14 are resident), 21 in clusters of 8; 37 rows 32 in clusters of 8, 23 of 4; 18 fp32 rows of 65536 of every
+// kind 37 and 33, with top-p 48 and 33.
+// Sampling calls take clusters of up to 8 CTAs as far as the CTA slots reach, beyond the resident ones: rows of different kinds take
+// different times, and the last ones fit in between (36 fp32 rows of 50021 of every kind 33 in clusters of 8, 37 of 4; 37 rows of
+// 131072 38 to 42, 39 to 40 through the chain, 60 and 70 with top-p in bf16).  Rows of sonic_topk are all alike (37 fp32 rows of
+// 131072 with k = 100 37, 20 through the chain), but in clusters of 4, of short vocabularies, where the chain proves few rows (74 rows of
+// 9000 with k = 50 21 and 100).  Larger clusters never wait: 18 rows of 262144 of every kind 50 and 36 through the chain.
+// The chain before there was a row kernel: one bf16 row of 131072 with top-k 25.5 -> 13.6; 4 fp32 rows of 32768, one of each kind, 29.9
+// -> 23.2; 3 x 3 verification rows of 32003 50.4 -> 25.7; 32 bf16 rows of 100003 without top-k 73.9 -> 49.3.  64 rows of 131072 are 58 in
+// the chain and 64 here: its persistent CTAs keep loading while the rows' selections wait for one another.  What the line costs: 34 to
+// 37 and 72 to 74 fp32 rows of up to 65536, all of them with top-p, are up to a fifth slower than the chain (41 and 46).
+static int row_ctas(const KParams &P, int sm_count, int dev) {
 #ifdef SONIC_TRACE
-    return false;                                 // (this variant exists to look into the streaming chain)
+    return 0;                                     // (this variant exists to look into the streaming chain)
 #else
 #ifdef SONIC_TEST_WITHHOLD
-    if (!getenv("SONIC_TEST_ROW")) return false;  // (this one into the waits of both)
+    if (!getenv("SONIC_TEST_ROW")) return 0;      // (this one into the waits of both)
 #endif
-    if (P.op == OP_TOPK && P.ktop > ROW_KMAX) return false;
-    const int c = std::max(ROW_CMIN, (P.V + ROW_SLICE_MAX - 1) / ROW_SLICE_MAX);
-    return (long long)P.rows * c <= 2ll * sm_count;
+    if (P.op == OP_TOPK && P.ktop > ROW_KMAX) return 0;
+    const int cmin = std::max(ROW_CMIN, (P.V + ROW_SLICE_MAX - 1) / ROW_SLICE_MAX);
+    const int cmax = std::min(ROW_CMAX, std::max(cmin, (P.V + ROW_UNIT - 1) / ROW_UNIT));
+    auto fits = [&](int c) {
+        const int resident = g_row_clusters[dev][c];
+        if (P.rows <= resident) return true;
+        return resident > 0 && (long long)P.rows * c <= 2ll * sm_count && c <= (P.op == OP_TOPK ? ROW_CMIN : 8);
+    };
+    for (int c = ROW_CMAX; c >= ROW_CMIN; c /= 2)
+        if (c >= cmin && c <= cmax && fits(c)) return c;
+    return fits(cmin) ? cmin : 0;
 #endif
 }
 
-// CTAs of a row's cluster: as many as are resident for this number of rows, so that every CTA has few elements (a step
-// costs 64 cycles per instruction and 8192 elements), within what a slice can be.
-static cudaError_t launch_rows(const KParams &P, cudaStream_t st, int sm_count) {
-    const int cmin = std::max(ROW_CMIN, (P.V + ROW_SLICE_MAX - 1) / ROW_SLICE_MAX);
-    const int cmax = std::min(ROW_CMAX, std::max(cmin, (P.V + ROW_UNIT - 1) / ROW_UNIT));
-    const int fit = (int)(2ll * sm_count / P.rows);
-    int C = 1;
-    while (C * 2 <= std::min(fit, cmax)) C *= 2;
-    C = std::max(C, cmin);
+static cudaError_t launch_rows(const KParams &P, cudaStream_t st, int C) {
     const int per = (P.V + C - 1) / C, slice = (per + ROW_UNIT - 1) / ROW_UNIT * ROW_UNIT;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
@@ -328,9 +355,9 @@ static int launch_all(KParams &P, void *ws, size_t ws_bytes, cudaStream_t st, in
         P.ykeys = reinterpret_cast<unsigned int *>(base + L.ykeys);
     }
 
-    if (row_route(P, sm_count)) {
+    if (const int ctas = row_ctas(P, sm_count, dev)) {
         P.fresh = clear ? 1 : 0;
-        cudaError_t e = launch_rows(P, st, sm_count);
+        cudaError_t e = launch_rows(P, st, ctas);
         if (e != cudaSuccess) return fail_cuda(e, "row kernel launch");
         g_err[0] = 0;
         return SONIC_OK;

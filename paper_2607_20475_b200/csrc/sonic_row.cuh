@@ -48,7 +48,11 @@ constexpr int ROW_COPIES = 8;                     // copies of the bins, by lane
 constexpr int ROW_XBINS = 128;                    // bins of a level over (value, index) pairs (exchanged as 64-bit words)
 constexpr int ROW_LAND = 2944;                    // elements CTA 0 can receive
 constexpr int ROW_MEMBERS = ROW_THREADS;          // ... of a top-p row's crossing bin (one per thread)
-constexpr int ROW_GMAX = 512;                     // group maxima that are exchanged directly (one per thread)
+constexpr int ROW_GMAX = 256;                     // group maxima that are exchanged directly (a thread of kth_max counts half of them;
+                                                  // with 512 it counts all: 8 bf16 rows of 50021 with k = 64 23 us, 15 with 256)
+constexpr int ROW_DIRECT = 88;                    // largest k they serve: 108 of 256 groups' elements reach the bound then, give or take 8,
+                                                  // and 128 are what the short finish takes (k = 100 reaches 127 and lies with the maxima of the lanes:
+                                                  // 8 fp32 rows of 50021 23 -> 17 us)
 constexpr int ROW_KMAX = 2048;                    // largest top-k finished from gathered elements
 static_assert(ROW_SLICE_MAX * 4 >= MERGE_CAP * 8, "the epilogue's buffers take the values' place in CTA 0");
 static_assert(ROW_KMAX <= KFAST_SAMPLE, "the epilogue's layout");
@@ -700,7 +704,7 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
         sh.land_n = 0u; sh.land_min = 0xFFFFFFFFu; sh.land_max = 0u;
     }
     if (tid < ROW_CMAX) sh.late[tid] = 0u;
-    sh.gmax[tid] = 0u;                                              // (ROW_GMAX == ROW_THREADS)
+    if (tid < ROW_GMAX) sh.gmax[tid] = 0u;
     if (P.bitmask) {
         const int w = (x.base >> 5) + tid;
         if (tid < slice / 32) mask[tid] = (w < ((P.V + 31) >> 5)) ? __ldg(P.bitmask + (size_t)row * P.bitmask_stride + w) : 0u;
@@ -791,7 +795,7 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
     int gpw = 1;                                                    // groups per warp
     while (2 * gpw * x.ncta * ROW_WARPS <= ROW_GMAX && 2 * gpw * x.ncta * ROW_WARPS <= 8 * c.k) gpw *= 2;
     const int ngroups = gpw * x.ncta * ROW_WARPS;
-    const bool direct = !dense && !greedy && 2 * c.k <= ngroups && c.k <= 100;
+    const bool direct = !dense && !greedy && 2 * c.k <= ngroups && c.k <= ROW_DIRECT;
     const bool masked = (c.z & M_GRAMMAR) != 0;
     float lmax = -CUDART_INF_F, lmin = CUDART_INF_F;                 // maximum, and smallest finite value
     auto process = [&](bool divide, bool first) {

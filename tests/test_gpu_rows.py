@@ -250,3 +250,20 @@ def test_sorts_with_hundreds_of_equal_values(sonic, oracle, B, k):
     dev = sonic.DeviceTopK(tw, k)
     dev.run()
     compare_topk(*dev.results(), *oracle.topk(x, k))
+
+
+@pytest.mark.parametrize("B,V", [(14, 40000), (15, 40000), (18, 245761), (17, 200003), (33, 20001), (34, 20001), (37, 131072), (71, 9000), (74, 9000), (75, 9000)])
+@pytest.mark.parametrize("dtype", [wl.DTYPE_F32, wl.DTYPE_BF16])
+def test_row_counts_at_the_edges_of_the_cluster_sizes(sonic, oracle, B, V, dtype):
+    # as many rows as there are clusters of 16, 8 or 4 CTAs at once, one more, as many as there are CTA slots for; top-k at both
+    # sides of what the group maxima serve
+    w = rows_of_every_class(np.random.default_rng(B * 7 + V), B, V, dtype)
+    dev = sonic.DeviceSample(w)
+    dev.run()
+    compare_sample(dev.results(), oracle.sample(w), w, max_near=B)
+    tw = wl.TopKWorkload(name="t", B=B, V=V, dtype=dtype, logits=w.logits)
+    vals, idx = oracle.topk(tw.logits_f32(), 101)
+    for k in (2, 63, 65, 88, 89, 101):
+        dev = sonic.DeviceTopK(tw, k)
+        dev.run()
+        compare_topk(*dev.results(), vals[:, :k].copy(), idx[:, :k].copy())
