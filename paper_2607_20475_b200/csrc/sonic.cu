@@ -154,7 +154,7 @@ static const GroupTable &group_table(int V) {
 static int g_sm_count[64];
 // Clusters of C CTAs of the row kernel that are resident at once, per device (a cluster has to fit into one GPC, so that they are
 // fewer than the CTA slots divide into: 71, 33 and 14 of 4, 8 and 16 CTAs on a B200, where 296 slots make 74, 37 and 18).
-static int g_row_clusters[64][ROW_CMAX + 1];
+[[maybe_unused]] static int g_row_clusters[64][ROW_CMAX + 1];
 
 static int configure_once(int *sm_count, int *device) {
     static std::once_flag once[64];

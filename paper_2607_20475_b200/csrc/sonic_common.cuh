@@ -90,7 +90,7 @@ struct __align__(16) TileRec {                // written by the tile's CTA in th
 constexpr int DBINS = 2048;                   // bins of the mass histogram, uniform in (M - y)
 constexpr int MEMBER_CAP = 4096;              // elements of the crossing bin that can be listed
 struct __align__(16) DenseRow {
-    unsigned int ticket_h, ticket_c, ticket_r, nmembers;     // items that have finished a pass; listed members
+    unsigned int nmembers, unused[3];                         // listed members
     unsigned int kmin, kmax, overflow, state;                // key span of the members; an item could not stage its members; 1 = collect pass wanted
     unsigned int Mkey, tk, klo, khi;                         // row maximum; min-p key threshold (0 = none); keys of the crossing bin: klo .. khi (empty if klo > khi)
     unsigned long long target;                               // mass the ranking prefix must reach (0: top-p does not decide inside the bin)

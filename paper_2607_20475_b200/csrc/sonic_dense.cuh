@@ -4,19 +4,18 @@
 //
 // The streaming kernel leaves, per row of this class, the ordered keys of the processed logits (read once from
 // HBM, written once, re-read from L2 by the passes below) and per-tile maxima / minima.  Then, every pass a
-// grid-wide launch whose CTAs take (row, tile) items and whose last-arriving CTA of a row (a ticket counter, no
-// waiting) does the row-level step:
+// grid-wide launch whose CTAs take (row, tile) items, and one launch with a CTA per row for the row-level steps at the end:
 //   pass H  (rows with top-p): fixed-point probability mass per bin, 2048 bins uniform in (M - y) that just cover
-//           the row's finite range; the last arriver scans the bins from the top for the bin where the
-//           cumulative mass reaches p * Z (the "crossing bin").  The min-p threshold M + ln(theta) is a key
+//           the row's finite range; every CTA of pass C that meets the row scans the bins from the top for the
+//           bin where the cumulative mass reaches p * Z (the "crossing bin").  The min-p threshold M + ln(theta) is a key
 //           threshold and names a bin as well; the higher of the two bins decides.
 //   pass C  per tile: mass and number of the elements above the crossing bin, and the elements inside it listed
-//           as (key << 32 | ~index); the last arriver resolves the exact cut among the listed elements (a radix
-//           descent over the composite keys weighted by mass; ties by lowest index), then draws: tile-level
-//           CDF from the per-tile masses, one tile re-read for the element.  Rows without top-p know their cut
-//           once the row maximum is known and run pass C in place of pass H.
+//           as (key << 32 | ~index).  Rows without top-p know their cut once the row maximum is known and run
+//           pass C in place of pass H.
+//   finish  the exact cut among the listed elements (by rank; ties by lowest index), then the draw: tile, chunk
+//           and element from the per-tile and per-chunk masses, one chunk re-read for the element.
 //   pass R  (verification rows whose draft was rejected): per-tile sums of the residual max(0, p - q) in fp64,
-//           the last arriver draws from it.
+//           a CTA per row draws from it.
 // This is the truncation epilogue and token selection of the paper's Algorithm "Stage 2" (TopP, MinP; Appendix
 // "Probability Truncation", "Sampling", "Speculative Verification") for supports far beyond the paper's
 // k <= 128 bound (Section 3.3).  Masses are 2^-40 fixed point, sums are integer and order-independent.
@@ -51,7 +50,7 @@ struct DenseShared {
     unsigned int nstage, kmin, kmax, base;
     unsigned int Mkey, mkey, Nf, bad;
     unsigned int cnt_above, nb;
-    int flag, last, digit;
+    int flag, digit;
 };
 
 // Bin of a finite key: larger bin = larger logit; bin DBINS-1 holds the row maximum.
@@ -185,23 +184,8 @@ __device__ __forceinline__ void dense_load_keys(const KParams &P, const DenseIte
     for (int k = 0; k < DENSE_NV; ++k) kv[k] = (k < nv) ? src[k] : make_uint4(KEY_NEG_INF, KEY_NEG_INF, KEY_NEG_INF, KEY_NEG_INF);
 }
 
-// Ticket of a pass: a CTA reports `cnt` finished items of a row at once; true in every thread of the CTA whose report
-// completes the row's `items` (its reads then see what the others wrote).
-__device__ __forceinline__ bool dense_arrive(unsigned int *ticket, int cnt, int items, DenseShared &sm, int tid) {
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-        const unsigned int t = atomicAdd(ticket, (unsigned int)cnt);
-        sm.last = (t + (unsigned int)cnt == (unsigned int)items) ? 1 : 0;
-        if (sm.last) __threadfence();
-    }
-    __syncthreads();
-    return sm.last != 0;
-}
-
 // The items of a pass are dealt in contiguous ranges, so that a CTA's items mostly belong to one row: the row's
-// parameters are loaded once, its ticket is drawn once, and the rows a CTA turns out to complete are finished after
-// all of its items (another row's items never wait behind a finish).
+// parameters are loaded once.
 struct DenseRange { int lo, hi; };
 __device__ __forceinline__ DenseRange dense_range(int n_items, int cta, int ncta) {
     const int per = (n_items + ncta - 1) / ncta;
@@ -210,7 +194,6 @@ __device__ __forceinline__ DenseRange dense_range(int n_items, int cta, int ncta
     r.hi = min(n_items, r.lo + per);
     return r;
 }
-constexpr int DENSE_FIN_MAX = 8;              // rows one CTA can have to finish (a range spans few rows)
 
 // ---------------------------------------------------------------- pass H
 // Mass histogram of one item, added to the row's histogram in global memory.
@@ -564,7 +547,7 @@ __device__ __forceinline__ void smem_add_u64(unsigned long long *p, unsigned lon
     if (hi + carry) atomicAdd(q + 1, hi + carry);
 }
 
-// Last arriver of pass C: the exact cut, the support's size and mass, then the draw or the accept test.
+// The row's finish, behind pass C: the exact cut, the support's size and mass, then the draw or the accept test.
 // dyn: DENSE_DYN_SMEM bytes; cells: the row's two Philox cells.  Returns false if the row must go to the cluster kernel.
 __device__ bool dense_finish(const KParams &P, const RowCfg &c, int row, int tiles, DenseShared &sm, unsigned long long *dyn, int tid,
                              uint32_t Mkey, bool listed, unsigned long long target, uint32_t tk, uint2 cells, int draft, float q_draft) {

@@ -191,15 +191,15 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
             return it;
         };
         int item = current_item();
-        // lane 0: the tile's bulk copy, with the arrival on full[s] (arrive == true) or with the bytes announced only
-        // (the arrival then follows once the stage's description is written)
-        auto issue_copy = [&](int row, int tile, int s, bool arrive) {
+        // lane 0: the tile's bulk copy, with its bytes announced on full[s] (the arrival follows once the stage's description is
+        // written)
+        auto issue_copy = [&](int row, int tile, int s) {
             const int first = tile * CTA_TILE;
             const int elems = min(CTA_TILE, ((P.V - first) + VEC - 1) / VEC * VEC);
             const unsigned int bytes = (unsigned int)elems * ELT;
             const unsigned char *src = reinterpret_cast<const unsigned char *>(P.logits) +
                                        ((size_t)row * (size_t)P.row_stride + (size_t)first) * ELT;
-            if (arrive) mbar_arrive_expect_tx(&sh.full[s], bytes); else mbar_expect_tx(&sh.full[s], bytes);
+            mbar_expect_tx(&sh.full[s], bytes);
 #ifdef SONIC_TEST_WITHHOLD
             // test-only build: the bytes of one chosen tile are announced but its copy is never issued, so the waits
             // on this stage run out (consumers, then the producer) and the call reports it
@@ -210,7 +210,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         // The CTA's first tile is requested at once, before its row's parameters and lists are known (they take two
         // rounds of global loads): the copy's latency hides behind them.  (A row of the cluster kernel's class gets
         // a copy nobody reads: such rows are rare.)
-        if (item >= 0 && lane == 0) issue_copy(item / tiles, item % tiles, 0, false);
+        if (item >= 0 && lane == 0) issue_copy(item / tiles, item % tiles, 0);
         // The record of a tile that every consumer warp has left: candidates, cutoff, argmax, bad list ids.
         auto retire = [&](int s) {
             const int row = sh.meta[s].row, tile = sh.meta[s].tile;
@@ -252,7 +252,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                         return;
                     }
                     // (the first tiles' copies are under way; nothing is copied for rows of the cluster kernel's class)
-                    if (item >= 0 && !skip && lane == 0) issue_copy(row, tile, s, false);
+                    if (item >= 0 && !skip && lane == 0) issue_copy(row, tile, s);
                     retire(s);
                 }
                 if (item < 0) {                            // out of work: tell the consumers
@@ -262,7 +262,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 advance();
                 const int hint = current_item();           // the tile that follows
                 if (lane == 0) {
-                    if (n > 0 && n < NSTAGE && !skip) issue_copy(row, tile, s, false);
+                    if (n > 0 && n < NSTAGE && !skip) issue_copy(row, tile, s);
                     StageMeta &m = sh.meta[s];
                     m.row = row; m.tile = tile; m.slot = cur_slot; m.skip = skip ? 1 : 0;
                     m.stop = 0;
@@ -310,12 +310,9 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
         if (meta.stop) { KERNEL_T1(0); break; }
         const int row = meta.row, tile = meta.tile;
         const int tile_base = tile * CTA_TILE;
-        uint32_t mword = 0xFFFFFFFFu;
-        if (P.bitmask) {
-            mword = (row == pre_row && tile == pre_tile) ? mword_pre : load_mask_words(row, tile);
-            pre_row = meta.next_row; pre_tile = meta.next_tile;
-            if (pre_row >= 0) mword_pre = load_mask_words(pre_row, pre_tile);
-        }
+        const uint32_t mword = (row == pre_row && tile == pre_tile) ? mword_pre : load_mask_words(row, tile);
+        pre_row = meta.next_row; pre_tile = meta.next_tile;
+        if (pre_row >= 0) mword_pre = load_mask_words(pre_row, pre_tile);
         if (!meta.skip) {
             const unsigned char *stage = stages + (size_t)s * STAGE_BYTES;
             const RowSlot &slot = sh.slot[meta.slot];
@@ -412,7 +409,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                     for (int i = tid; i < DBINS / 2; i += STREAM_THREADS) h[i] = make_uint4(0u, 0u, 0u, 0u);
                     if (tid == 0) {
                         DenseRow *dr = P.drow + row;
-                        dr->ticket_h = 0u; dr->ticket_c = 0u; dr->ticket_r = 0u; dr->nmembers = 0u;
+                        dr->nmembers = 0u;
                         dr->kmin = 0xFFFFFFFFu; dr->kmax = 0u; dr->overflow = 0u; dr->state = 0u;
                         P.dlist[atomicAdd(&P.error[WS_NDENSE], 1u)] = row;
                     }

@@ -1498,7 +1498,7 @@ sonic_stream_kernel(const KParams P, const int tiles, const int nitems, const in
                 for (int i = tid; i < DBINS / 2; i += STREAM_THREADS) h[i] = make_uint4(0u, 0u, 0u, 0u);
                 if (tid == 0) {
                     DenseRow *dr = P.drow + row;
-                    dr->ticket_h = 0u; dr->ticket_c = 0u; dr->ticket_r = 0u; dr->nmembers = 0u;
+                    dr->nmembers = 0u;
                     dr->kmin = 0xFFFFFFFFu; dr->kmax = 0u; dr->overflow = 0u; dr->state = 0u;
                     P.dlist[atomicAdd(&P.error[WS_NDENSE], 1u)] = row;
                 }
