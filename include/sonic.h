@@ -178,9 +178,10 @@ int sonic_topk(const void *logits, int dtype, int B, int V, int64_t row_stride, 
  *
  * The first call on each device resolves the array's device address and configures the
  * kernels; that first call should come before any stream capture is begun.  All calls on a device share
- * the one array, which keeps the contents of the previous call: each call first clears
- * the control words it needs at zero (a memset enqueued on `stream`), and two calls that
- * overlap on the device (different streams, or graphs replayed concurrently) race on it.
+ * the one array, which keeps the contents of the previous call: a call that needs
+ * control words at zero (k beyond 2048) first clears them (a memset enqueued on `stream`),
+ * and two calls that overlap on the device (different streams, or graphs replayed
+ * concurrently) race on it.
  */
 #define SONIC_STATIC_MAX_ROWS 8
 int sonic_topk_static(const void *logits, int dtype, int B, int V, int64_t row_stride, int k,
