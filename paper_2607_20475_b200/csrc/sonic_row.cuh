@@ -131,6 +131,14 @@ struct RowCtx {
     float Mf;                                     // row maximum
 };
 
+// The bound of a row's small top-k where its quotient by the temperature is far from the ordinary (subnormal, overflowing, or none).
+// Ordinary quotients that are equal come from values within 2^-22 of each other; with the exact bound on that path as well a bf16 row of
+// 131072 takes 13.8 instead of 13.0 us.  (One division and two searches for a neighbour: code that runs once, fetched cold.)
+__device__ __noinline__ float row_bound_before_div(float t, float tau) {
+    const float low = first_finite_quotient(tau);
+    return t > low ? fmaxf(bound_before_div(t, tau), low) : low;
+}
+
 // Four elements at a time over the warp's part, index order across the lanes: f(value, vocabulary index).
 template <typename F>
 __device__ __forceinline__ void row_each(const RowCtx &x, F f) {
@@ -859,9 +867,8 @@ sonic_row_kernel(const __grid_constant__ KParams P, const int slice) {
         // Everything that reaches the bound goes to CTA 0.  With a temperature a value a little below the bound may become
         // equal to it when divided, and then the index decides: the bound is what can divide to as much as it does.  (What
         // divides to -inf is masked by that.)
-        const float low = divide ? first_finite_quotient(c.tau) : s.vmin;
-        float t = max(unkey(tk), low);
-        if (divide && t > low) t = fmaxf(bound_before_div(t, c.tau), low);
+        float t = max(unkey(tk), s.vmin);
+        if (divide) t = (fabsf(t) > c.tau * 0x1p-100f && fabsf(t) < c.tau * 0x1p100f) ? t - fabsf(t) * 0x1p-21f : row_bound_before_div(t, c.tau);
         if (__any_sync(0xFFFFFFFFu, lmax >= t)) {
             unsigned long long *land = cl_map(row_land(), 0);
             unsigned int mine = 0u;
