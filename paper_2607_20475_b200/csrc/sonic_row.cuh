@@ -25,8 +25,8 @@
 // whatever its values.
 // What it measured, against the chain of kernels of large calls (us per call): a bf16 row of 131072 with top-k 50, top-p
 // 0.9 13.6 (25.5); 32 bf16 rows of 100003 with top-p or min-p only 49.3 (73.9); 37 fp32 rows of 50021 of every kind 36.4
-// (64.3).  Its stalls are instruction fetch (7.4 of 23.5 cycles between two instructions of a warp), barriers (4.9), loads
-// (2.5) and fences (2.4): serial code, not bytes.
+// (64.3).  Its stalls are instruction fetch (8.1 of 23.1 cycles between two instructions of a warp, four rows of four kinds), barriers
+// (3.6), loads (2.5) and fences (2.4): serial code, not bytes.
 // Masses are integers, 2^-44 of the largest weight: sums do not depend on the order, replays are bit-identical.
 #pragma once
 #include <cooperative_groups.h>
